@@ -313,8 +313,8 @@ size_t sbr_synth_ws_bytes(const sbr_radar_cfg* radar, int64_t path_cap);
  * per CTA are reduced in a fixed order.  SBR_PHASE_SPLIT with N_s <= 512 and
  * at least 65536 record slots (path_cap * n_virt) is evaluated as a type-1
  * non-uniform FFT (spreading onto 2 N_s grid points with a width-8
- * exponential-of-semicircle kernel, one FFT, deconvolution; ~1e-6 relative to
- * the FP64 sum), term by term otherwise.  SBR_PHASE_FP64 forms each
+ * Kaiser-Bessel kernel, one FFT, deconvolution; below 1e-6 relative to the FP64
+ * sum), term by term otherwise.  SBR_PHASE_FP64 forms each
  * sample's phase in FP64 from paths->path_len; SBR_PHASE_NAIVE rounds the delay
  * to FP32.  With SBR_SYNTH_MOVING OR'ed into mode (paths traced on a scene with
  * motion) every chirp c is synthesised from the delays tau + c chirp_rep

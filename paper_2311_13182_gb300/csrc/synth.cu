@@ -5,10 +5,10 @@
 //
 // Split-phase mode, N_s <= 512 (sbr_synthesize's default path): a type-1
 // non-uniform FFT.  Each (path, antenna) is spread onto a periodic grid of
-// 2 N_s points with a width-8 exponential-of-semicircle kernel, one FFT per
-// antenna follows, and the kernel's Fourier transform is divided out: 8 grid
-// updates per (path, antenna) instead of N_s phasors, about 1e-6 from the FP64
-// sum (details at k_nufft_spread).
+// 2 N_s points with a width-8 Kaiser-Bessel kernel, one FFT per antenna follows,
+// and the kernel's Fourier transform is divided out: 8 grid updates per (path,
+// antenna) instead of N_s phasors, less than 1e-6 from the FP64 sum (details at
+// k_nufft_spread).
 //
 // Tensor-core kernel (N_s = 256 or 512, run by the allocation-free entry
 // point): with n = 16 a + b (b < 16), Eq. 8 factorises per path into
@@ -38,6 +38,7 @@
 #include <limits.h>
 #include <math.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "common.cuh"
@@ -516,215 +517,292 @@ __global__ void __launch_bounds__(256) k_synth_bwd(const float4* __restrict__ pr
 
 // ---- non-uniform FFT forward kernel -----------------------------------------
 //
-// For the split-phase mode with N_s <= 512 the samples are computed as a type-1
-// non-uniform FFT (Dutt & Rokhlin 1993; kernel of Barnett, Magland & af Klinteberg
-// 2019) instead of term by term.  With n = n' + N_s / 2 (n' in [-N_s/2, N_s/2)),
+// The samples are computed as a type-1 non-uniform FFT (Dutt & Rokhlin 1993;
+// Kaiser-Bessel kernel, Greengard & Lee 2004, Barnett et al. 2019) instead of
+// term by term.  With n = n' + N_s / 2 (n' in [-N_s/2, N_s/2)),
 //   S[n] = sum_p c_p e^{j 2 pi n' delta_p},  c_p = A_p e^{j 2 pi (phi0_p + (N_s/2) delta_p)},
 // every path is spread onto a periodic grid of M = 2 N_s points, u_p = M delta_p,
-//   b[l] = sum_p c_p psi(l - u_p),  psi(x) = exp(beta (sqrt(1 - (2x/w)^2) - 1)), |x| < w/2,
+//   b[l] = sum_p c_p psi(l - u_p),  psi(x) = I0(beta sqrt(1 - (2x/w)^2)) / I0(beta), |x| < w/2,
 // then B[k] = sum_l b[l] e^{+j 2 pi k l / M} (one M-point FFT) and, by Poisson
 // summation, S[n' + N_s/2] = B[n'] / Psi(n'/M) with Psi the Fourier transform of
-// psi, up to the aliasing terms Psi(n'/M - k), k != 0 (about 1e-7 relative for
-// w = 8, beta = 2.3 w at upsampling 2).  Per (path, antenna) that is w = 8 kernel
-// values instead of N_s phasors.
+// psi, up to the aliasing terms Psi(n'/M - k), k != 0 (7e-8 relative rms over
+// the band for w = 8, beta = 2.3 w at upsampling 2).  Per (path, antenna) that
+// is w = 8 kernel values instead of N_s phasors.
 //
 // The grid position keeps the split phase's precision: M delta_hi is exact in
-// FP32 (delta_hi is a multiple of 2^-12, M <= 1024), so the offset of the path
-// from its grid cell, t = (M delta_hi - floor(M delta_hi)) + M delta_lo, carries
-// about 2^-24 of one grid step.
+// FP32 (delta_hi is a multiple of 2^-12, M <= 8192), so the offset t of the path
+// from its grid cell carries about 2^-24 of one grid step.  With t = s + 1/2 the
+// eight values psi((j - 7/2) - s) are polynomials of degree 8 in s (1.2e-8 of the
+// peak), mirrored in pairs, psi_j(s) = E_j(s^2) + s O_j(s^2) = psi_{7-j}(-s): 37
+// FMAs for the eight, and no square root or exponential.
 //
-// Each warp spreads into its own grid in shared memory (no atomics): its lanes
-// form four groups of w = 8, one grid point per lane; each group takes eight
-// consecutive paths of the warp's batch of 32 in turn.  Neighbouring rays sit
-// at nearly the same range, so consecutive paths mostly share a grid cell: a
-// lane keeps the sum for its point of the current cell in registers and adds
-// it to the grid only when its group's cell changes (and once after the warp's
-// last batch), the flushing groups one after the other, as their cells may
-// overlap.
-// The warps' grids are added in a fixed order, and the CTAs' grids by the
-// finishing kernel in a fixed order, so the result is bitwise reproducible.
-constexpr int kNuW = 8;             // kernel width in grid points
-constexpr int kNuWarps = 8;         // warps per CTA, one grid each
-constexpr int kNuThreads = 32 * kNuWarps;
-constexpr int kNuMaxSamples = 512;  // grids of up to 1024 points (8 KB per warp)
-constexpr int kNuQuad = 32;         // Gauss-Legendre nodes for Psi
+// One lane takes one record, and its sixteen additions go to the CTA's grid in
+// shared memory as integer atomics: the sums are then exact, do not depend on
+// the order, and are bitwise reproducible.  A grid word has kNuCopies copies,
+// one per lane pair (l, l + 16), and the lower half of a warp adds real parts
+// while the upper adds imaginary parts (then the other way round), so the 32
+// lanes of an atomic always hit 32 different banks, whatever the cells are:
+// neighbouring rays share cells, and consecutive records jump between a ray's
+// bounces.  A term is rounded to 2^-kNuTermBits of the power of two above the
+// chunk's largest amplitude, so that a chunk's additions to one copy stay below
+// 2^31; after each chunk the copies of the touched cells (a flag per eight
+// cells) are summed, scaled and added to the CTA's FP32 grid, each point by one
+// thread.  The CTAs' grids are added in a fixed order by the finishing kernel.
+//
+// Bound by issue slots (58 % active) and the chunks' barriers.  12 antennas x
+// 367,500 records x 256 samples: 49 us against 109 us for sums kept in registers
+// per run of equal cells (8 lanes a record, each warp its own FP32 grid), which a
+// changing cell flushes one group at a time; 93 us for the same with the chunk
+// first sorted by cell.  Error against FP64 over the same records 2e-7 (1.3e-6 with
+// the approximate sine, square root and exponential of the former kernel).
+constexpr int kNuW = 8;         // kernel width in grid points
+constexpr int kNuCopies = 16;   // copies of a grid word
+constexpr int kNuBlock = 1024;  // cells a CTA's grid holds at once; larger grids block by block
+constexpr double kNuBeta = 2.3 * kNuW;
 
-__device__ __forceinline__ float ex2_approx(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-__device__ __forceinline__ float sqrt_approx(float x) {
-  float y;
-  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
+struct NufftCoef {
+  float e[4][5], o[4][4];  // psi((j - 7/2) - s) = sum_k e[j][k] s^(2k) + s sum_k o[j][k] s^(2k), j < 4, |s| <= 1/2
+  float inv[9];            // 1 / Psi(n'/M) = sum_k inv[k] (2 n' / N_s)^(2k)
+};
 
 struct NufftArg {
-  float half_n;    // N_s / 2
-  float m;         // M = 2 N_s
-  float beta_l2e;  // beta log2(e)
   int log_m;
+  float half_n, m;           // N_s / 2, M = 2 N_s
+  double f0_c, b_cn, m_d;    // FP64 phase: f_c / c and B / (c N_s) per metre, M
+  int V, Q, chirps, chirp0;  // antennas, CTAs per antenna and chirp, chirps of this launch, the first of them
+  double per_chirp;          // moving scenes: change of path length per chirp per (m/s) of dL/dt
 };
 
-// Psi(xi) = sum_i wpsi[i] cos(2 pi xi x[i]): Gauss-Legendre on [0, w/2] of 2 psi(x) cos(2 pi xi x)
-struct PsiQuad {
-  float x[kNuQuad];
-  float wpsi[kNuQuad];
-};
+// 2^e for -126 <= e <= 127
+__device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) << 23); }
 
-// CTA (v, q) spreads antenna v; the warps of the Q CTAs take contiguous ranges
-// of batches of 32 paths.  Writes the CTA's grid: grids[(q V + v) M + l].
-__global__ void __launch_bounds__(kNuThreads) k_nufft_spread(const float4* __restrict__ prep, int64_t cap,
-                                                            const int32_t* __restrict__ d_P, int V, int Q,
-                                                            NufftArg na, float2* __restrict__ grids,
-                                                            unsigned int* __restrict__ fin_cnt,
-                                                            const float* __restrict__ rate = nullptr,
-                                                            float cnu = 0.f, float ceps = 0.f) {
-  extern __shared__ float2 wgrid[];  // [warp][M]
-  if (blockIdx.x == 0 && threadIdx.x < V) fin_cnt[threadIdx.x] = 0u;  // the finishing kernel's counters
-  const int M = 1 << na.log_m;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, grp = lane >> 3, j = lane & 7;
-  float2* g = wgrid + (size_t)warp * M;
-  for (int i = lane; i < M; i += 32) g[i] = make_float2(0.f, 0.f);
-  __syncwarp();
-  const int v = blockIdx.x % V, q = blockIdx.x / V;
+// Cells a CTA's grid holds, and its points: the cells and w - 1 more to the right
+// (folded back, or into the neighbouring block, when the chunk is added up).
+__host__ __device__ constexpr int nu_cells(int M) { return M < kNuBlock ? M : kNuBlock; }
+__host__ __device__ constexpr int nu_points(int M) { return nu_cells(M) + kNuW; }
+
+// x such that `adds` terms of at most 2^x (and rounding) sum to less than 2^31.
+constexpr int nu_term_bits(int adds) { return adds <= 1 ? 30 : nu_term_bits((adds + 1) / 2) - 1; }
+
+// CTA (q, v, chirp) spreads its share of antenna v's records, P/Q consecutive
+// ones.  Writes the CTA's grid, grids[CTA][l].
+template <bool kFp64, bool kMoving, int kThreads, int kItems>
+__global__ void __launch_bounds__(kThreads, kThreads == 256 ? 3 : 1)
+    k_nufft_spread(const float4* __restrict__ prep, const float2* __restrict__ plen, const float* __restrict__ phase_ofs,
+                   const float* __restrict__ rate, int64_t cap, const int32_t* __restrict__ d_P, const NufftArg na,
+                   const __grid_constant__ NufftCoef co, float2* __restrict__ grids, unsigned int* __restrict__ fin_cnt) {
+  constexpr int kChunk = kThreads * kItems, kBits = nu_term_bits(kChunk / kNuCopies);
+  extern __shared__ int4 nsm[];
+  __shared__ uint32_t wmax[kThreads / 32], wblk[kThreads / 32];
+  __shared__ int flag[kNuBlock / 8 + 2];  // flag[1 + o]: a record of cells 8 o .. 8 o + 7 in this chunk
+  const int M = 1 << na.log_m, bs = nu_cells(M), npts = nu_points(M);
+  int* grid = reinterpret_cast<int*>(nsm);                            // [npts][re, im][kNuCopies]
+  float* sum = reinterpret_cast<float*>(grid + npts * 2 * kNuCopies); // [npts][re, im]: finished chunks
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (blockIdx.x == 0)
+    for (int i = tid; i < na.V * na.chirps; i += kThreads) fin_cnt[i] = 0u;  // the finishing kernel's counters
+  const int cl = blockIdx.x % na.chirps, v = (blockIdx.x / na.chirps) % na.V, q = blockIdx.x / (na.chirps * na.V);
+  const double dt = kMoving ? (double)(na.chirp0 + cl) * na.per_chirp : 0.0;  // path length change per (m/s)
+  const float cnu = (float)(dt * na.f0_c), ceps = (float)(dt * na.b_cn);
+  float2* out = grids + (size_t)blockIdx.x * M;
+  for (int i = tid; i < npts * (2 * kNuCopies / 4); i += kThreads) nsm[i] = make_int4(0, 0, 0, 0);
+  for (int i = tid; i < 2 * npts; i += kThreads) sum[i] = 0.f;
+  for (int i = tid; i < kNuBlock / 8 + 2; i += kThreads) flag[i] = 0;
+  if (M > bs)
+    for (int i = tid; i < M; i += kThreads) out[i] = make_float2(0.f, 0.f);
   const int64_t P = *d_P;
-  const float4* pv = prep + (size_t)v * cap;
-  const float xo = (float)(j - (kNuW / 2 - 1));  // this lane's grid point minus floor(u), before t
-  // each warp takes a contiguous range of batches of 32 paths, so that a group's
-  // register sums carry over from one batch to the next (neighbouring rays)
-  const int64_t nbat = (P + 31) / 32, nw = (int64_t)Q * kNuWarps, wi = (int64_t)q * kNuWarps + warp;
-  const int64_t b0 = nbat * wi / nw, b1 = nbat * (wi + 1) / nw;
-  float ax = 0.f, ay = 0.f;
-  int cur = INT_MIN;
-  for (int64_t b = b0; b < b1; ++b) {
-    const int64_t p = b * 32 + lane;  // lane prepares path p
-    float cre = 0.f, cim = 0.f, t = 0.f;
-    int i0 = 0;
-    if (p < P) {
-      float4 r = __ldg(&pv[p]);  // phi0, delta_hi, delta_lo, A
-      if (rate) {
-        // a moving scene's chirp: phi0 + dL/dt cnu and delta + dL/dt ceps, whole multiples of
-        // 2^-12 of the delta shift moved into delta_hi (which stays exact)
-        const float ld = __ldg(&rate[(size_t)v * cap + p]);
-        float ph = fmaf(ld, cnu, r.x);
-        r.x = ph - rintf(ph);
-        const float dl = fmaf(ld, ceps, r.z);
-        const float kq = rintf(dl * 4096.f);
-        const float dh = r.y + kq * (1.f / 4096.f);
-        r.y = dh - rintf(dh);
-        r.z = dl - kq * (1.f / 4096.f);
-      }
-      float x = na.half_n * r.y;       // exact
-      x -= rintf(x);
-      x = fmaf(na.half_n, r.z, x) + r.x;
-      x -= rintf(x);
-      float sn, cs;
-      __sincosf(kTwoPiF * x, &sn, &cs);
-      cre = r.w * cs;
-      cim = r.w * sn;
-      const float uh = na.m * r.y;  // exact
-      const float fl = floorf(uh);
-      t = fmaf(na.m, r.z, uh - fl);
-      i0 = (int)fl;
-      if (t < 0.f) {
-        t += 1.f;
-        --i0;
-      } else if (t >= 1.f) {
-        t -= 1.f;
-        ++i0;
-      }
+  const int64_t r0 = P * q / na.Q;
+  const int n = (int)(P * (q + 1) / na.Q - r0);
+  const size_t at = (size_t)v * cap + r0;
+  const float4* pv = prep + at;
+  const bool upper = lane >= 16;
+  int* mine = grid + (lane & 15);
+  int blk = 0;       // block of cells the grid holds
+  bool bad = false;  // a record that is not finite: the antenna's samples are NaN
+  // the finished sums of block blk into the CTA's output (several blocks only)
+  auto store_block = [&]() {
+    for (int i = tid; i < npts; i += kThreads) {
+      float2* o = out + ((blk * bs + i - (kNuW / 2 - 1)) & (M - 1));
+      *o = make_float2(o->x + sum[2 * i], o->y + sum[2 * i + 1]);
+      sum[2 * i] = sum[2 * i + 1] = 0.f;
     }
-    const int nb = (int)min((int64_t)32, P - b * 32);
-    // group grp takes paths 8 grp .. 8 grp + 7 in turn; a lane keeps the sum for its
-    // point of the current cell in registers and adds it to the grid when the cell changes
-    for (int st = 0; st < 8; ++st) {
-      const int src = 8 * grp + st;
-      const bool live = src < nb;
-      const float pr = __shfl_sync(0xffffffffu, cre, src), pi = __shfl_sync(0xffffffffu, cim, src);
-      const float pt = __shfl_sync(0xffffffffu, t, src);
-      const int pl = __shfl_sync(0xffffffffu, i0, src);
-      const bool flush = live && pl != cur && cur != INT_MIN;
-      unsigned fg = __ballot_sync(0xffffffffu, flush) & 0x01010101u;  // lane 8 g flags group g
-      if (fg) {  // the flushing groups in turn: their cells may overlap
-        const int lc = (cur + j - (kNuW / 2 - 1)) & (M - 1);
-        do {
-          const int gg = (__ffs(fg) - 1) >> 3;
-          if (grp == gg) {
-            float2 o = g[lc];
-            o.x += ax;
-            o.y += ay;
-            g[lc] = o;
-          }
-          __syncwarp();
-          fg &= fg - 1;
-        } while (fg);
-      }
-      if (live && pl != cur) {
-        ax = 0.f;
-        ay = 0.f;
-        cur = pl;
-      }
-      if (live) {
-        const float z = (xo - pt) * (2.f / kNuW);
-        // psi = exp(beta (sqrt(1 - z^2) - 1)); |z| <= 1 on the 8 points
-        const float psi = ex2_approx(na.beta_l2e * (sqrt_approx(fmaxf(fmaf(-z, z, 1.f), 0.f)) - 1.f));
-        ax = fmaf(psi, pr, ax);
-        ay = fmaf(psi, pi, ay);
-      }
-    }
-  }
-  {  // the last cells
-    const int lc = (cur + j - (kNuW / 2 - 1)) & (M - 1);
-    for (int gg = 0; gg < 4; ++gg) {
-      if (grp == gg && cur != INT_MIN) {
-        float2 o = g[lc];
-        o.x += ax;
-        o.y += ay;
-        g[lc] = o;
-      }
-      __syncwarp();
-    }
-  }
+  };
   __syncthreads();
-  float2* out = grids + ((size_t)q * V + v) * M;
-  for (int i = threadIdx.x; i < M; i += blockDim.x) {
-    float2 acc = wgrid[i];
-    for (int w = 1; w < kNuWarps; ++w) {
-      const float2 x = wgrid[(size_t)w * M + i];
-      acc.x += x.x;
-      acc.y += x.y;
+  for (int c0 = 0; c0 < n; c0 += kChunk) {
+    float4 rec[kItems];  // c re, c im over A, s, A
+    int cell[kItems];
+    uint32_t am = 0, blocks = 0;
+#pragma unroll
+    for (int u = 0; u < kItems; ++u) {
+      const int p = c0 + tid + u * kThreads;
+      rec[u] = p < n ? __ldg(&pv[p]) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    out[i] = acc;
+#pragma unroll
+    for (int u = 0; u < kItems; ++u) {
+      const int p = c0 + tid + u * kThreads;
+      float4 r = rec[u];
+      float x, t, fl;
+      int ce;
+      if (kFp64) {
+        float2 L2 = make_float2(0.f, 0.f);
+        double L = 0.0, po = 0.0;
+        if (p < n) {
+          L2 = __ldg(&plen[at + p]);
+          po = (double)__ldg(&phase_ofs[r0 + p]);
+          if (kMoving) L = dt * (double)__ldg(&rate[at + p]);
+        }
+        L += (double)L2.x + (double)L2.y;
+        double d = na.b_cn * L;
+        d -= rint(d);
+        double ph = fma((double)na.half_n, d, na.f0_c * L + po);
+        ph -= rint(ph);
+        x = (float)ph;
+        const double ud = na.m_d * d, fd = floor(ud);
+        t = (float)(ud - fd);
+        ce = (int)fd;
+      } else {
+        if (kMoving) {
+          // phi0 + dL/dt cnu and delta + dL/dt ceps, whole multiples of 2^-12 of the delta
+          // shift moved into delta_hi (which stays exact)
+          const float ld = p < n ? __ldg(&rate[at + p]) : 0.f;
+          const float ph = fmaf(ld, cnu, r.x);
+          r.x = ph - rintf(ph);
+          const float dl = fmaf(ld, ceps, r.z), kq = rintf(dl * 4096.f), dh = r.y + kq * (1.f / 4096.f);
+          r.y = dh - rintf(dh);
+          r.z = dl - kq * (1.f / 4096.f);
+        }
+        x = na.half_n * r.y;  // exact
+        x -= rintf(x);
+        x = fmaf(na.half_n, r.z, x) + r.x;
+        const float uh = na.m * r.y;  // exact
+        fl = floorf(uh);
+        t = fmaf(na.m, r.z, uh - fl);
+        ce = (int)fl;
+      }
+      bad |= !isfinite(x + t + r.w);
+      fl = floorf(t);
+      t -= fl;
+      ce = (ce + (int)fl) & (M - 1);
+      float sn, cs;
+      sincospif(2.f * x, &sn, &cs);
+      rec[u] = make_float4(cs, sn, t - 0.5f, r.w);
+      cell[u] = ce;
+      am = max(am, __float_as_uint(fabsf(r.w)));
+      if (p < n) blocks |= 1u << (ce / kNuBlock);
+    }
+    am = __reduce_max_sync(0xffffffffu, am);
+    blocks = __reduce_or_sync(0xffffffffu, blocks);
+    if (lane == 0) {
+      wmax[warp] = am;
+      wblk[warp] = blocks;
+    }
+    __syncthreads();
+    am = wmax[0];
+    blocks = wblk[0];
+#pragma unroll
+    for (int w = 1; w < kThreads / 32; ++w) {
+      am = max(am, wmax[w]);
+      blocks |= wblk[w];
+    }
+    const int ex = max((int)(am >> 23) - 126, -80);  // |A| < 2^ex
+    const float scale = pow2f(kBits - ex);
+    const float unit = pow2f(ex - kBits);
+    while (blocks) {
+      const int b = __ffs(blocks) - 1;
+      blocks &= blocks - 1;
+      if (b != blk) {  // the same for the whole CTA; sum is complete (the barrier after each chunk's addition)
+        store_block();
+        blk = b;
+        __syncthreads();
+      }
+#pragma unroll
+      for (int u = 0; u < kItems; ++u) {
+        const int idx = cell[u] - b * bs;
+        if ((unsigned)idx >= (unsigned)bs || rec[u].w == 0.f) continue;
+        const float s = rec[u].z, s2 = s * s, a = rec[u].w * scale;
+        const float c1 = a * (upper ? rec[u].y : rec[u].x), c2 = a * (upper ? rec[u].x : rec[u].y);
+        int* g1 = mine + idx * (2 * kNuCopies) + (upper ? kNuCopies : 0);
+        int* g2 = mine + idx * (2 * kNuCopies) + (upper ? 0 : kNuCopies);
+        flag[1 + (idx >> 3)] = 1;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          float E = co.e[j][4], O = co.o[j][3];
+#pragma unroll
+          for (int k = 3; k >= 0; --k) E = fmaf(E, s2, co.e[j][k]);
+#pragma unroll
+          for (int k = 2; k >= 0; --k) O = fmaf(O, s2, co.o[j][k]);
+          const float pl = fmaf(O, s, E), pr = fmaf(-O, s, E);  // points j and 7 - j
+          atomicAdd(g1 + j * (2 * kNuCopies), __float2int_rn(c1 * pl));
+          atomicAdd(g2 + j * (2 * kNuCopies), __float2int_rn(c2 * pl));
+          atomicAdd(g1 + (7 - j) * (2 * kNuCopies), __float2int_rn(c1 * pr));
+          atomicAdd(g2 + (7 - j) * (2 * kNuCopies), __float2int_rn(c2 * pr));
+        }
+      }
+      __syncthreads();
+      // the chunk's sums: point i / 2, part i & 1; its copies' four 16-byte words in an order
+      // that gives the eight lanes of a shared-memory phase different banks
+      for (int i = tid; i < 2 * npts; i += kThreads) {
+        const int o = i >> 4;  // points 8 o .. 8 o + 7 take records of cells of octets o - 1 and o
+        if (!(flag[o] | flag[o + 1])) continue;
+        long long t = 0;
+#pragma unroll
+        for (int k = 0; k < kNuCopies / 4; ++k) {
+          const int w = i * (kNuCopies / 4) + ((k + (i >> 1)) & (kNuCopies / 4 - 1));
+          const int4 x = nsm[w];
+          nsm[w] = make_int4(0, 0, 0, 0);
+          t += (long long)x.x + x.y + ((long long)x.z + x.w);
+        }
+        sum[i] = fmaf((float)t, unit, sum[i]);
+      }
+      __syncthreads();
+      for (int i = tid; i < kNuBlock / 8 + 2; i += kThreads) flag[i] = 0;
+      __syncthreads();
+    }
+  }
+  bad = __syncthreads_or(bad);
+  if (M > bs) {
+    store_block();
+  } else {  // the points past the grid's end fold back
+    for (int i = tid; i < M; i += kThreads) {
+      float re = sum[2 * i], im = sum[2 * i + 1];
+      for (int k = i + M; k < npts; k += M) {
+        re += sum[2 * k];
+        im += sum[2 * k + 1];
+      }
+      out[(i - (kNuW / 2 - 1)) & (M - 1)] = make_float2(re, im);
+    }
+  }
+  if (bad) {
+    __syncthreads();
+    for (int i = tid; i < M; i += kThreads) out[i] = make_float2(NAN, NAN);
   }
 }
 
-// Finishing, kNuFinSlice grid points per CTA: CTA (v, s) adds slice s of the Q
-// CTAs' grids of antenna v in a fixed order (kNuFinThreads / slice threads per
-// point, each over every such CTA with four interleaved sums, then the threads'
-// sums in order) into bsum; the last CTA of the antenna to finish (a counter per
-// antenna, zeroed by the spreading kernel) runs the M-point FFT and the division
-// by Psi(n'/M) and writes S[v][n] into the cube: chirp `only` (a moving scene),
+// Finishing, kNuFinSlice grid points per CTA: CTA (row, s) adds slice s of the Q
+// CTAs' grids of a row (antenna and chirp) in a fixed order (kNuFinThreads / slice
+// threads per point, each over every such CTA with four interleaved sums, then the
+// threads' sums in order) into bsum; the last CTA of the row to finish (a counter
+// per row, zeroed by the spreading kernel) runs the M-point FFT and the division
+// by Psi(n'/M) and writes S[v][n] into the cube: the row's chirp of a moving scene,
 // else every chirp (a static scene's chirps are equal).
 constexpr int kNuFinThreads = 1024;
 constexpr int kNuFinSlice = 128;
-__global__ void __launch_bounds__(kNuFinThreads) k_nufft_finish(const float2* __restrict__ grids, int V, int Q,
-                                                                int Ns, int log_m, PsiQuad pq,
+__global__ void __launch_bounds__(kNuFinThreads) k_nufft_finish(const float2* __restrict__ grids, const NufftArg na,
+                                                                const __grid_constant__ NufftCoef co,
                                                                 float2* __restrict__ bsum,
                                                                 unsigned int* __restrict__ cnt,
-                                                                float2* __restrict__ cube, int C, int only) {
+                                                                float2* __restrict__ cube, int C, bool moving) {
   extern __shared__ float2 sg[];  // [M] grid, [M / 2] twiddles, [kNuFinThreads] per-thread sums
   __shared__ int s_last;
-  const int M = 1 << log_m, slice = M < kNuFinSlice ? M : kNuFinSlice, S = M / slice;
-  const int v = blockIdx.x / S, sl = blockIdx.x - v * S;
+  const int log_m = na.log_m, M = 1 << log_m, slice = M < kNuFinSlice ? M : kNuFinSlice, S = M / slice;
+  const int row = blockIdx.x / S, sl = blockIdx.x - row * S, rows = na.V * na.chirps, Q = na.Q;
   float2* tw = sg + M;
   float2* part = tw + M / 2;
   const int parts = blockDim.x / slice, li = threadIdx.x % slice, k0 = threadIdx.x / slice;
   const int l = sl * slice + li;
   float2 a0 = make_float2(0.f, 0.f), a1 = a0, a2 = a0, a3 = a0;
-  const float2* src = grids + (size_t)v * M + l;
-  const size_t qs = (size_t)V * M;  // from one CTA's grid to the next
+  const float2* src = grids + (size_t)row * M + l;
+  const size_t qs = (size_t)rows * M;  // from one CTA's grid to the next
   int q = k0;
   for (; q + 3 * parts < Q; q += 4 * parts) {  // four loads in flight, four interleaved sums
     const float2 x0 = __ldcg(src + (size_t)q * qs), x1 = __ldcg(src + (size_t)(q + parts) * qs);
@@ -751,75 +829,93 @@ __global__ void __launch_bounds__(kNuFinThreads) k_nufft_finish(const float2* __
       acc.x += part[k * slice + li].x;
       acc.y += part[k * slice + li].y;
     }
-    bsum[(size_t)v * M + l] = acc;
+    bsum[(size_t)row * M + l] = acc;
   }
   __threadfence();
   __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(&cnt[v], 1u) == (unsigned)(S - 1);
+  if (threadIdx.x == 0) s_last = atomicAdd(&cnt[row], 1u) == (unsigned)(S - 1);
   __syncthreads();
   if (!s_last) return;
   __threadfence();
   fft::fill_twiddles(tw, M, 1.f, blockDim.x, threadIdx.x);
-  for (int i = threadIdx.x; i < M; i += blockDim.x) sg[fft::bitrev(i, log_m)] = __ldcg(&bsum[(size_t)v * M + i]);
+  for (int i = threadIdx.x; i < M; i += blockDim.x) sg[fft::bitrev(i, log_m)] = __ldcg(&bsum[(size_t)row * M + i]);
   __syncthreads();
   fft::smem_fft(sg, tw, log_m, blockDim.x, threadIdx.x);
-  const int h = Ns >> 1;
+  const int Ns = M >> 1, h = Ns >> 1;
+  // rows are (antenna, chirp of the launch), the chirp fastest
+  const int v = row / na.chirps;
+  const int c0 = moving ? na.chirp0 + row - v * na.chirps : 0, c1 = moving ? c0 + 1 : C;
   for (int n = threadIdx.x; n < Ns; n += blockDim.x) {
-    const float xi = (float)(n - h) / (float)M;
-    float ph = 0.f;
-#pragma unroll 8
-    for (int i = 0; i < kNuQuad; ++i) ph = fmaf(pq.wpsi[i], cospif(2.f * xi * pq.x[i]), ph);
+    const float xi = (float)(n - h) / (float)h, y = xi * xi;
+    float inv = co.inv[8];
+#pragma unroll
+    for (int k = 7; k >= 0; --k) inv = fmaf(inv, y, co.inv[k]);
     const float2 B = sg[(n - h) & (M - 1)];
-    const float inv = 1.f / ph;
     const float2 val = make_float2(B.x * inv, B.y * inv);
-    if (only >= 0) {
-      cube[((size_t)v * C + only) * Ns + n] = val;
-    } else {
-      for (int c = 0; c < C; ++c) cube[((size_t)v * C + c) * Ns + n] = val;
-    }
+    for (int c = c0; c < c1; ++c) cube[((size_t)v * C + c) * Ns + n] = val;
   }
 }
 
-// Gauss-Legendre nodes and weights on [-1, 1] (Newton on the three-term
-// recurrence of the Legendre polynomials), mapped to Psi's quadrature.
-PsiQuad make_psi_quad(double beta) {
-  PsiQuad pq{};
-  const int n = kNuQuad;
-  const double half_w = 0.5 * kNuW;
-  for (int i = 0; i < n; ++i) {
-    double z = cos(M_PI * (i + 0.75) / (n + 0.5)), dp = 1.0;
-    for (int it = 0; it < 100; ++it) {
-      double p0 = 1.0, p1 = z;
-      for (int k = 2; k <= n; ++k) {
-        const double p2 = ((2.0 * k - 1.0) * z * p1 - (k - 1.0) * p0) / k;
-        p0 = p1;
-        p1 = p2;
-      }
-      dp = n * (z * p1 - p0) / (z * z - 1.0);
-      const double dz = p1 / dp;
-      z -= dz;
-      if (fabs(dz) < 1e-15) break;
-    }
-    const double wgt = 2.0 / ((1.0 - z * z) * dp * dp);
-    // [-1, 1] -> [0, w/2]; Psi(xi) = 2 int_0^{w/2} psi(x) cos(2 pi xi x) dx
-    const double x = 0.5 * half_w * (1.0 + z);
-    const double zz = x / half_w;
-    const double psi = exp(beta * (sqrt(1.0 - zz * zz) - 1.0));
-    pq.x[i] = (float)x;
-    pq.wpsi[i] = (float)(2.0 * 0.5 * half_w * wgt * psi);
+// I0 by its power series (the terms are positive: no cancellation; beta < 20).
+double bessel_i0(double x) {
+  double t = 1.0, s = 1.0;
+  for (int k = 1; k < 200 && t > 1e-18 * s; ++k) {
+    t *= (0.5 * x / k) * (0.5 * x / k);
+    s += t;
   }
-  return pq;
+  return s;
 }
 
-constexpr double kNuBeta = 2.3 * kNuW;
+double kb_kernel(double x) {
+  const double z = 2.0 * x / kNuW, y = 1.0 - z * z;
+  return y > 0.0 ? bessel_i0(kNuBeta * sqrt(y)) / bessel_i0(kNuBeta) : (y < 0.0 ? 0.0 : 1.0 / bessel_i0(kNuBeta));
+}
 
-const PsiQuad& psi_quad() {
-  static const PsiQuad pq = make_psi_quad(kNuBeta);
-  return pq;
+// Monomial coefficients of the degree-n interpolant of f at the Chebyshev nodes of
+// [0, b] (Newton's divided differences, expanded).
+template <int n, class F>
+void fit_poly(F f, double b, float* out) {
+  double x[n + 1], d[n + 1], m[n + 1] = {};
+  for (int i = 0; i <= n; ++i) {
+    x[i] = 0.5 * b * (1.0 + cos(M_PI * (i + 0.5) / (n + 1)));
+    d[i] = f(x[i]);
+  }
+  for (int k = 1; k <= n; ++k)
+    for (int i = n; i >= k; --i) d[i] = (d[i] - d[i - 1]) / (x[i] - x[i - k]);
+  for (int k = n; k >= 0; --k) {  // m <- m (x - x_k) + d_k
+    for (int i = n; i >= 1; --i) m[i] = m[i - 1] - x[k] * m[i];
+    m[0] = -x[k] * m[0] + d[k];
+  }
+  for (int i = 0; i <= n; ++i) out[i] = (float)m[i];
+}
+
+NufftCoef make_nufft_coef() {
+  NufftCoef c{};
+  for (int j = 0; j < 4; ++j) {  // the even and odd parts of psi_j in y = s^2
+    const double a = j - 0.5 * (kNuW - 1);
+    fit_poly<4>([&](double y) { return 0.5 * (kb_kernel(a - sqrt(y)) + kb_kernel(a + sqrt(y))); }, 0.25, c.e[j]);
+    fit_poly<3>([&](double y) { return 0.5 * (kb_kernel(a - sqrt(y)) - kb_kernel(a + sqrt(y))) / sqrt(y); }, 0.25,
+                c.o[j]);
+  }
+  // Psi(xi) = w / I0(beta) sinh(r) / r, r = sqrt(beta^2 - (pi w xi)^2), real on the band
+  // |xi| <= 1/4; its reciprocal in y = (4 xi)^2 = (2 n' / N_s)^2
+  fit_poly<8>(
+      [&](double y) {
+        const double a = M_PI * kNuW * 0.25, r = sqrt(kNuBeta * kNuBeta - a * a * y);
+        return bessel_i0(kNuBeta) * r / (kNuW * sinh(r));
+      },
+      1.0, c.inv);
+  return c;
+}
+
+const NufftCoef& nufft_coef() {
+  static const NufftCoef c = make_nufft_coef();
+  return c;
 }
 
 // Few (path, antenna) records: the direct kernels, whose one pass over the records
 // costs less than the non-uniform FFT's spreading, finishing sum and FFT chain.
+constexpr int kNuMaxSamples = 512;
 #ifndef SBR_NUFFT_MIN_RECORDS
 #define SBR_NUFFT_MIN_RECORDS 65536
 #endif
@@ -907,11 +1003,24 @@ void grid_shape(int V, int Ns, int64_t cap, int* Q) {
   *Q = (int)q;
 }
 
-// dynamic shared memory of the spreading kernel: one grid of M = 2 N_s points per warp
-inline size_t nufft_smem(int Ns) { return sizeof(float2) * kNuWarps * 2 * (size_t)Ns; }
+// dynamic shared memory of the spreading kernel: the grid's copies and its sums
+inline size_t nufft_smem(int Ns) { return (2 * kNuCopies * sizeof(int) + 2 * sizeof(float)) * (size_t)nu_points(2 * Ns); }
+inline size_t nufft_fin_smem(int Ns) { return sizeof(float2) * (3 * (size_t)Ns + kNuFinThreads); }
+
+// Grids of up to 512 points take 71 KB: three CTAs of 256 threads per SM; larger ones
+// (a block of 1024 cells takes 141 KB) one CTA of 1024.
+inline bool nufft_wide(int Ns) { return 2 * Ns > 512; }
+inline int nufft_threads(int Ns) { return nufft_wide(Ns) ? 1024 : 256; }
+
+using NufftSpread = void (*)(const float4*, const float2*, const float*, const float*, int64_t, const int32_t*, NufftArg,
+                             NufftCoef, float2*, unsigned int*);
+inline NufftSpread nufft_kernel(int Ns, bool moving) {
+  if (nufft_wide(Ns)) return moving ? k_nufft_spread<false, true, 1024, 1> : k_nufft_spread<false, false, 1024, 1>;
+  return moving ? k_nufft_spread<false, true, 256, 4> : k_nufft_spread<false, false, 256, 4>;
+}
 
 // resident spreading CTAs per SM (shared memory and registers decide); raises
-// the kernel's shared-memory limit once where the grids pass 48 KB
+// the kernels' shared-memory limits once where they pass 48 KB
 int nufft_per_sm(int Ns) {
   static int cache[kDevCache][16] = {};
   int lg = 0;
@@ -919,10 +1028,16 @@ int nufft_per_sm(int Ns) {
   const int dev = current_device();
   if (dev < kDevCache && cache[dev][lg]) return cache[dev][lg];
   const size_t sm = nufft_smem(Ns);
-  if (sm > 48 * 1024) cudaFuncSetAttribute(k_nufft_spread, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  int n = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_nufft_spread, kNuThreads, sm);
-  n = n > 0 ? n : 1;
+  int n = 32;
+  for (int moving = 0; moving < 2; ++moving) {
+    const NufftSpread k = nufft_kernel(Ns, moving != 0);
+    if (sm > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    int m = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&m, k, nufft_threads(Ns), sm);
+    n = std::min(n, m > 0 ? m : 1);
+  }
+  if (nufft_fin_smem(Ns) > 48 * 1024)
+    cudaFuncSetAttribute(k_nufft_finish, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)nufft_fin_smem(Ns));
   if (dev < kDevCache) cache[dev][lg] = n;
   return n;
 }
@@ -930,7 +1045,7 @@ int nufft_per_sm(int Ns) {
 // CTAs per antenna of the spreading kernel: one wave, at most one per 256 paths
 void nufft_shape(int V, int Ns, int64_t cap, int* Qn) {
   int64_t q = ((int64_t)sm_count() * nufft_per_sm(Ns)) / V;
-  const int64_t batches = (cap + 32 * kNuWarps - 1) / (32 * kNuWarps);
+  const int64_t batches = (cap + 255) / 256;
   if (q > batches) q = batches;
   if (q < 1) q = 1;
   *Qn = (int)q;
@@ -996,6 +1111,37 @@ sbr_status bind_ws(const sbr_radar_cfg* radar, int64_t cap, void* ws, size_t byt
   return SBR_OK;
 }
 
+// The non-uniform FFT of chirps [c0, c0 + chirps) of a moving scene, or of a static
+// scene's one chirp, written to all of them: spread, then finish.
+void launch_nufft(const sbr_paths* p, const sbr_radar_cfg* r, const SynthWs& w, bool moving, int c0, int chirps,
+                  float2* cube, cudaStream_t st) {
+  const int V = p->n_virt, Ns = r->n_samples, M = 2 * Ns;
+  NufftArg na{};
+  while ((1 << na.log_m) < M) ++na.log_m;
+  na.half_n = 0.5f * (float)Ns;
+  na.m = (float)M;
+  na.f0_c = r->f0 / kC;
+  na.b_cn = r->bandwidth / (kC * Ns);
+  na.m_d = (double)M;
+  na.V = V;
+  na.Q = w.Qn;
+  na.chirps = chirps;
+  na.chirp0 = c0;
+  na.per_chirp = r->chirp_rep;
+  nufft_per_sm(Ns);  // sets the shared-memory limits before the first launch
+  const NufftCoef& co = nufft_coef();
+  const float4* prep = reinterpret_cast<const float4*>(p->prep);
+  const float2* plen = reinterpret_cast<const float2*>(p->path_len);
+  const int grid = V * w.Qn * chirps;
+  ::sbr::note_launch();
+  nufft_kernel(Ns, moving)<<<grid, nufft_threads(Ns), nufft_smem(Ns), st>>>(
+      prep, plen, p->phase_ofs, p->path_rate, p->path_cap, p->count, na, co, w.grids, w.fin_cnt);
+  const int slices = M < kNuFinSlice ? 1 : M / kNuFinSlice;
+  ::sbr::note_launch();
+  k_nufft_finish<<<V * chirps * slices, kNuFinThreads, nufft_fin_smem(Ns), st>>>(w.grids, na, co, w.bsum, w.fin_cnt, cube,
+                                                                                r->n_chirps, moving);
+}
+
 // A moving scene: every chirp synthesised from its own delays (split phase by the
 // non-uniform FFT up to 512 samples, or the FP64 phase), chirp by chirp.
 sbr_status launch_moving(sbr_phase_mode mode, const sbr_paths* p, const sbr_radar_cfg* r, const SynthWs& w,
@@ -1003,21 +1149,7 @@ sbr_status launch_moving(sbr_phase_mode mode, const sbr_paths* p, const sbr_rada
   const int V = p->n_virt, Ns = r->n_samples, C = r->n_chirps;
   const double per_chirp = r->chirp_rep / kC;  // delay change per chirp per (m/s) of dL/dt
   if (mode == SBR_PHASE_SPLIT && Ns <= kNuMaxSamples) {
-    int log_m = 0;
-    while ((1 << log_m) < 2 * Ns) ++log_m;
-    NufftArg na{0.5f * (float)Ns, 2.f * (float)Ns, (float)(kNuBeta * 1.4426950408889634), log_m};
-    nufft_per_sm(Ns);
-    const int M = 2 * Ns, slices = M < kNuFinSlice ? 1 : M / kNuFinSlice;
-    for (int c = 0; c < C; ++c) {
-      const float cnu = (float)(c * per_chirp * r->f0), ceps = (float)(c * per_chirp * r->bandwidth / Ns);
-      ::sbr::note_launch();
-      k_nufft_spread<<<V * w.Qn, kNuThreads, nufft_smem(Ns), st>>>(reinterpret_cast<const float4*>(p->prep),
-                                                                   p->path_cap, p->count, V, w.Qn, na, w.grids,
-                                                                   w.fin_cnt, p->path_rate, cnu, ceps);
-      ::sbr::note_launch();
-      k_nufft_finish<<<V * slices, kNuFinThreads, sizeof(float2) * (3 * (size_t)Ns + kNuFinThreads), st>>>(
-          w.grids, V, w.Qn, Ns, log_m, psi_quad(), w.bsum, w.fin_cnt, cube, C, c);
-    }
+    for (int c = 0; c < C; ++c) launch_nufft(p, r, w, true, c, 1, cube, st);
     return SBR_OK;
   }
   if (mode == SBR_PHASE_FP64) {
@@ -1042,23 +1174,6 @@ sbr_status launch_moving(sbr_phase_mode mode, const sbr_paths* p, const sbr_rada
   set_error("sbr_synthesize: SBR_SYNTH_MOVING supports SBR_PHASE_SPLIT up to %d samples and SBR_PHASE_FP64",
             kNuMaxSamples);
   return SBR_ERR_UNSUPPORTED;
-}
-
-// Split-phase samples by the non-uniform FFT: spread, then finish (one chirp, written to all chirps).
-void launch_nufft(const sbr_paths* p, const sbr_radar_cfg* r, const SynthWs& w, float2* cube, cudaStream_t st) {
-  const int V = p->n_virt, Ns = r->n_samples;
-  int log_m = 0;
-  while ((1 << log_m) < 2 * Ns) ++log_m;
-  NufftArg na{0.5f * (float)Ns, 2.f * (float)Ns, (float)(kNuBeta * 1.4426950408889634), log_m};
-  nufft_per_sm(Ns);  // sets the shared-memory limit before the first launch
-  ::sbr::note_launch();
-  k_nufft_spread<<<V * w.Qn, kNuThreads, nufft_smem(Ns), st>>>(reinterpret_cast<const float4*>(p->prep),
-                                                               p->path_cap, p->count, V, w.Qn, na, w.grids,
-                                                               w.fin_cnt);
-  const int M = 2 * Ns, slices = M < kNuFinSlice ? 1 : M / kNuFinSlice;
-  ::sbr::note_launch();
-  k_nufft_finish<<<V * slices, kNuFinThreads, sizeof(float2) * (3 * (size_t)Ns + kNuFinThreads), st>>>(
-      w.grids, V, w.Qn, Ns, log_m, psi_quad(), w.bsum, w.fin_cnt, cube, r->n_chirps, -1);
 }
 
 template <int M>
@@ -1113,7 +1228,7 @@ extern "C" sbr_status sbr_synthesize(const sbr_paths* paths, const sbr_radar_cfg
     return SBR_OK;
   }
   if (nufft_for(mode, Ns, paths->path_cap * paths->n_virt)) {
-    launch_nufft(paths, radar, w, reinterpret_cast<float2*>(d_cube), st);
+    launch_nufft(paths, radar, w, false, 0, 1, reinterpret_cast<float2*>(d_cube), st);
     SBR_CUDA(cudaGetLastError());
     return SBR_OK;
   }

@@ -1,0 +1,103 @@
+"""sbr_synthesize on given path records against the same sum in FP64 (Eq. 8).
+
+The records are seeded and written into the path buffers directly, so the comparison holds the
+synthesis alone: sample counts over the whole range, record counts around the kernels' chunks
+(256 threads, 1024 records), cells at the ends of the spreading grid and of its blocks.
+
+Tolerance of the non-uniform FFT, relative L2 over the cube, rms contributions: carrier phase
+rounded to 2^-25 cycles 1.1e-7, kernel polynomials and products 6e-8, aliasing 7e-8, terms
+rounded to 2^-23 of twice the largest amplitude 2.6e-7 (amplitudes uniform in [0.1, 1]),
+transform 1e-7: 3.3e-7 together; three times that is 1e-6."""
+import math
+
+import numpy as np
+import pytest
+import torch
+
+from sbr_inputs import C_LIGHT, radar_mimo_3x4, radar_single_tx
+
+pytestmark = pytest.mark.gpu
+
+TOL = 1e-6
+
+
+def bind(sbr, radar, cap, delta, phi, A, rate=None):
+    """Path buffers of ``cap`` slots per antenna holding the records (phi, delta in cycles, FP64)."""
+    P = delta.shape[1]
+    paths = sbr.PathBuffers(cap, 1, radar.n_virt)
+    dhi = np.round(delta * 4096) / 4096
+    rec = np.stack([phi, dhi, delta - dhi, A], -1).astype(np.float32)
+    paths.prep()[:, :P] = torch.from_numpy(rec).cuda()
+    if rate is not None:
+        paths.path_rate()[:, :P] = torch.from_numpy(rate.astype(np.float32)).cuda()
+    paths.count_tensor().fill_(P)
+    rec = rec.astype(np.float64)
+    return paths, rec[..., 0], rec[..., 1] + rec[..., 2], rec[..., 3]
+
+
+def direct(phi, delta, A, ns):
+    n = torch.arange(ns, dtype=torch.float64, device="cuda")
+    out = []
+    for p, d, a in zip(*(torch.from_numpy(x).cuda() for x in (phi, delta, A))):
+        acc = torch.zeros(ns, dtype=torch.complex128, device="cuda")
+        for s in range(0, len(p), 4096):
+            x = p[s:s + 4096, None] + d[s:s + 4096, None] * n
+            x = 2 * math.pi * (x - x.round())
+            acc += (a[s:s + 4096, None] * torch.complex(x.cos(), x.sin())).sum(0)
+        out.append(acc)
+    return torch.stack(out)
+
+
+def rel(cube, ref):
+    got = torch.view_as_complex(cube.double().contiguous())
+    return float((got - ref).norm() / ref.norm())
+
+
+def records(seed, V, P, ns, where="all"):
+    rng = np.random.default_rng(seed)
+    delta = rng.uniform(-0.5, 0.5, (V, P))
+    if where == "edges":  # cells at both ends of the grid and of its 1024-cell blocks, exact cell borders among them
+        M = 2 * ns
+        edge = np.concatenate([[0, M - 1, M // 2, M // 2 - 1], np.arange(1024, M, 1024), np.arange(1024, M, 1024) - 1])
+        cell = rng.choice(edge, (V, P)) + rng.choice([0.0, 0.25, 1 - 2.0 ** -12], (V, P))
+        delta = (cell / M + 0.5) % 1.0 - 0.5
+    if where == "one":
+        delta = np.full((V, P), 0.1234567)
+    return delta, rng.uniform(-0.5, 0.5, (V, P)), rng.uniform(0.1, 1.0, (V, P)) * rng.choice([1, -1], (V, P))
+
+
+@pytest.mark.parametrize("ns,P,where", [
+    (32, 20000, "all"), (64, 16385, "edges"), (128, 17001, "all"), (256, 16384, "all"), (256, 16415, "edges"),
+    (256, 150000, "one"), (256, 3 * 152 * 1024 + 1, "all"), (512, 20011, "edges"), (512, 16384, "all")])
+def test_split_records(sbr, ns, P, where):
+    radar = radar_single_tx(ns, 1)
+    delta, phi, A = records(ns + P, 4, P, ns, where)
+    paths, phi, delta, A = bind(sbr, radar, P + 7, delta, phi, A)
+    cube = sbr.synthesize(paths, radar)
+    again = sbr.synthesize(paths, radar)
+    assert torch.equal(cube, again)
+    assert rel(cube[:, 0], direct(phi, delta, A, ns)) <= TOL
+
+
+def test_split_records_not_finite(sbr):
+    """A record that is not finite makes its antenna's samples NaN, and no others."""
+    radar = radar_single_tx(256, 1)
+    delta, phi, A = records(3, 4, 20000, 256)
+    A[2, 17] = np.inf
+    paths, _, _, _ = bind(sbr, radar, 20000, delta, phi, A)
+    cube = sbr.synthesize(paths, radar)
+    assert torch.isnan(cube[2]).all() and torch.isfinite(cube[[0, 1, 3]]).all()
+
+
+def test_moving_records(sbr):
+    """12 antennas, 16 chirps: every chirp from its own delays."""
+    radar = radar_mimo_3x4(256, 16)
+    delta, phi, A = records(9, 12, 7001, 256)
+    rate = np.random.default_rng(4).uniform(-8.0, 8.0, delta.shape).astype(np.float32)
+    paths, phi, delta, A = bind(sbr, radar, 7001, delta, phi, A, rate)
+    cube = sbr.synthesize(paths, radar, sbr.PHASE_SPLIT | sbr.SYNTH_MOVING)
+    per = radar.chirp_rep / C_LIGHT
+    ref = torch.stack([direct(phi + rate * (c * per * radar.f0), delta + rate * (c * per * radar.bandwidth / 256), A, 256)
+                       for c in range(16)], 1)
+    # the chirp's phase shift (up to 1.3 cycles here) and delta shift are each rounded once more in FP32
+    assert rel(cube, ref) <= 2 * TOL
