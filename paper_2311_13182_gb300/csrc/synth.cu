@@ -3,8 +3,7 @@
 // cube[v, c, n] = sum_p A_{p,v} exp(j 2 pi (f_c tau_{p,v} + mu tau_{p,v} t_n)),
 // t_n = n T / N_s, identical for every chirp c of a static scene.
 //
-// Split-phase mode, N_s <= 512 (sbr_synthesize's default path): a type-1
-// non-uniform FFT.  Each (path, antenna) is spread onto a periodic grid of
+// Split-phase mode (sbr_synthesize's default path): a type-1 non-uniform FFT.  Each (path, antenna) is spread onto a periodic grid of
 // 2 N_s points with a width-8 Kaiser-Bessel kernel, one FFT per antenna follows,
 // and the kernel's Fourier transform is divided out: 8 grid updates per (path,
 // antenna) instead of N_s phasors, less than 1e-6 from the FP64 sum (details at
@@ -22,7 +21,7 @@
 // two per staged chunk so the halves stay in fp16 range (the accumulators are
 // rescaled exactly when the scale drops).
 //
-// Direct FP32 kernel (other sample counts; persistent, one virtual antenna per
+// Direct FP32 kernel (few records, other sample counts; persistent, one virtual antenna per
 // CTA): the CTA's threads own M consecutive samples each and together cover
 // all N_s samples, so the sum over paths accumulates in registers with no
 // cross-thread reduction.  Paths stream through shared memory in chunks; per
@@ -913,15 +912,15 @@ const NufftCoef& nufft_coef() {
   return c;
 }
 
-// Few (path, antenna) records: the direct kernels, whose one pass over the records
-// costs less than the non-uniform FFT's spreading, finishing sum and FFT chain.
-constexpr int kNuMaxSamples = 512;
-#ifndef SBR_NUFFT_MIN_RECORDS
-#define SBR_NUFFT_MIN_RECORDS 65536
-#endif
-constexpr int64_t kNuMinRecords = SBR_NUFFT_MIN_RECORDS;
+// Few (path, antenna) record slots: the direct kernels, whose one pass over the
+// records costs less than the non-uniform FFT's spreading, finishing sum and FFT
+// chain.  Measured crossings (4 antennas, one wave of either): up to 512 samples,
+// where the tensor-core kernel sums directly, 8.5-10 us against 9-14 us at 32,768
+// slots, 11-12 against 11-14 us at 73,728, 23 against 13-15 us at 262,088; above,
+// 10-26 against 17-41 us at 2,048 slots, 19-59 against 17-47 us at 8,192.
+constexpr int kNuMovingMaxSamples = 512;  // the split phase of a moving scene
 inline bool nufft_for(sbr_phase_mode mode, int Ns, int64_t records) {
-  return mode == SBR_PHASE_SPLIT && Ns <= kNuMaxSamples && records >= kNuMinRecords;
+  return mode == SBR_PHASE_SPLIT && records >= (Ns <= 512 ? 65536 : 8192);
 }
 
 // Launch-shape queries are cached per device ordinal (kernel attributes such as
@@ -1058,7 +1057,7 @@ size_t ws_layout(const sbr_radar_cfg* radar, int64_t cap, int* Q, int* Qn = null
   const int V = radar->n_tx * radar->n_rx, Ns = radar->n_samples;
   grid_shape(V, Ns, cap, Q);
   int qn = 0;
-  if (Ns <= kNuMaxSamples) nufft_shape(V, Ns, cap, &qn);
+  nufft_shape(V, Ns, cap, &qn);
   if (Qn) *Qn = qn;
   Carver c(nullptr);
   c.take<float2>((size_t)V * (*Q) * Ns);       // per-CTA partial sums
@@ -1148,7 +1147,7 @@ sbr_status launch_moving(sbr_phase_mode mode, const sbr_paths* p, const sbr_rada
                          float2* cube, cudaStream_t st) {
   const int V = p->n_virt, Ns = r->n_samples, C = r->n_chirps;
   const double per_chirp = r->chirp_rep / kC;  // delay change per chirp per (m/s) of dL/dt
-  if (mode == SBR_PHASE_SPLIT && Ns <= kNuMaxSamples) {
+  if (mode == SBR_PHASE_SPLIT && Ns <= kNuMovingMaxSamples) {
     for (int c = 0; c < C; ++c) launch_nufft(p, r, w, true, c, 1, cube, st);
     return SBR_OK;
   }
@@ -1172,7 +1171,7 @@ sbr_status launch_moving(sbr_phase_mode mode, const sbr_paths* p, const sbr_rada
     return SBR_OK;
   }
   set_error("sbr_synthesize: SBR_SYNTH_MOVING supports SBR_PHASE_SPLIT up to %d samples and SBR_PHASE_FP64",
-            kNuMaxSamples);
+            kNuMovingMaxSamples);
   return SBR_ERR_UNSUPPORTED;
 }
 

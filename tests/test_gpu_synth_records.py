@@ -68,7 +68,9 @@ def records(seed, V, P, ns, where="all"):
 
 @pytest.mark.parametrize("ns,P,where", [
     (32, 20000, "all"), (64, 16385, "edges"), (128, 17001, "all"), (256, 16384, "all"), (256, 16415, "edges"),
-    (256, 150000, "one"), (256, 3 * 152 * 1024 + 1, "all"), (512, 20011, "edges"), (512, 16384, "all")])
+    (256, 150000, "one"), (256, 3 * 152 * 1024 + 1, "all"), (512, 20011, "edges"), (512, 16384, "all"),
+    (1024, 2048, "edges"), (1024, 2047, "all"), (2048, 10007, "edges"), (4096, 2049, "all"), (4096, 70001, "edges"),
+    (4096, 30000, "one")])
 def test_split_records(sbr, ns, P, where):
     radar = radar_single_tx(ns, 1)
     delta, phi, A = records(ns + P, 4, P, ns, where)
