@@ -118,7 +118,7 @@ typedef struct {
 
 typedef enum {
   SBR_PHASE_SPLIT = 0, /* tau in float-float, phase anchors in hi/lo FP32, FP32 rotation */
-  SBR_PHASE_FP64 = 1,  /* per-sample carrier phase f_c tau + mu tau t_n in FP64 */
+  SBR_PHASE_FP64 = 1,  /* phase f_c tau + mu tau t_n from FP64 delays, reduced mod 1 in FP64 */
   SBR_PHASE_NAIVE = 2  /* tau, f_c tau and mu tau t_n all in FP32 */
 } sbr_phase_mode;
 
@@ -315,7 +315,8 @@ size_t sbr_synth_ws_bytes(const sbr_radar_cfg* radar, int64_t path_cap);
  * evaluated as a type-1 non-uniform FFT (spreading onto 2 N_s grid points with a width-8
  * Kaiser-Bessel kernel, one FFT, deconvolution; below 1e-6 relative to the FP64
  * sum), term by term otherwise.  SBR_PHASE_FP64 forms each
- * sample's phase in FP64 from paths->path_len; SBR_PHASE_NAIVE rounds the delay
+ * path's carrier phase and grid position in FP64 from paths->path_len and is
+ * evaluated the same way; SBR_PHASE_NAIVE rounds the delay
  * to FP32.  With SBR_SYNTH_MOVING OR'ed into mode (paths traced on a scene with
  * motion) every chirp c is synthesised from the delays tau + c chirp_rep
  * (dL/dt) / c_0, chirp by chirp; the adjoint below is the static model's. */

@@ -330,16 +330,15 @@ __global__ void __launch_bounds__(kMmaThreads) k_synth_mma(const float4* __restr
   }
 }
 
-// Per-sample phase in FP64: x = f_c tau + (B / N_s) tau n, reduced mod 1.
+// Per-sample phase in FP64, term by term (the allocation-free entry point):
+// x = f_c tau + (B / N_s) tau n, reduced mod 1.
 template <int M>
 __global__ void __launch_bounds__(256) k_synth_fp64(const float4* __restrict__ prep,
                                                     const float2* __restrict__ plen,
                                                     const float* __restrict__ phase_ofs, int64_t cap,
                                                     const int32_t* __restrict__ d_P, int V, int Q,
                                                     int Ns, double f0, double b_over_ns,
-                                                    float2* __restrict__ partial,
-                                                    const float* __restrict__ rate = nullptr,
-                                                    double crep = 0.0) {
+                                                    float2* __restrict__ partial) {
   __shared__ double2 sx[kChunk];
   __shared__ float sa[kChunk];
   const int v = blockIdx.x % V, q = blockIdx.x / V;
@@ -353,8 +352,7 @@ __global__ void __launch_bounds__(256) k_synth_fp64(const float4* __restrict__ p
     __syncthreads();
     for (int j = threadIdx.x; j < cnt; j += blockDim.x) {
       const float2 L = plen[(size_t)v * cap + c0 + j];
-      double t = ((double)L.x + (double)L.y) * (1.0 / kC);
-      if (rate) t += crep * (double)rate[(size_t)v * cap + c0 + j];  // this chirp's delay
+      const double t = ((double)L.x + (double)L.y) * (1.0 / kC);
       const double x0 = f0 * t;
       const double d = b_over_ns * t;
       sx[j] = make_double2(x0 - rint(x0) + (double)phase_ofs[c0 + j], d - rint(d));
@@ -427,7 +425,7 @@ __global__ void __launch_bounds__(256) k_synth_naive(const float4* __restrict__ 
 // the group's chirps (a static scene: every chirp equal).
 constexpr int kRedChirps = 16;
 __global__ void k_reduce(const float2* __restrict__ partial, int V, int Q, int Ns, int C,
-                         float2* __restrict__ cube, int only = -1) {
+                         float2* __restrict__ cube) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= V * Ns) return;
   const int v = i / Ns, n = i - v * Ns;
@@ -436,10 +434,6 @@ __global__ void k_reduce(const float2* __restrict__ partial, int V, int Q, int N
     const float2 x = partial[((size_t)q * V + v) * Ns + n];
     re += x.x;
     im += x.y;
-  }
-  if (only >= 0) {  // a moving scene: this chirp only
-    cube[((size_t)v * C + only) * Ns + n] = make_float2(re, im);
-    return;
   }
   const int c1 = min(C, (int)(blockIdx.y + 1) * kRedChirps);
   for (int c = blockIdx.y * kRedChirps; c < c1; ++c) cube[((size_t)v * C + c) * Ns + n] = make_float2(re, im);
@@ -542,8 +536,7 @@ __global__ void __launch_bounds__(256) k_synth_bwd(const float4* __restrict__ pr
 // while the upper adds imaginary parts (then the other way round), so the 32
 // lanes of an atomic always hit 32 different banks, whatever the cells are:
 // neighbouring rays share cells, and consecutive records jump between a ray's
-// bounces.  A term is rounded to 2^-kNuTermBits of the power of two above the
-// chunk's largest amplitude, so that a chunk's additions to one copy stay below
+// bounces.  A term is rounded to 2^-24 of the chunk's largest amplitude, so that a chunk's additions to one copy stay below
 // 2^31; after each chunk the copies of the touched cells (a flag per eight
 // cells) are summed, scaled and added to the CTA's FP32 grid, each point by one
 // thread.  The CTAs' grids are added in a fixed order by the finishing kernel.
@@ -571,9 +564,6 @@ struct NufftArg {
   int V, Q, chirps, chirp0;  // antennas, CTAs per antenna and chirp, chirps of this launch, the first of them
   double per_chirp;          // moving scenes: change of path length per chirp per (m/s) of dL/dt
 };
-
-// 2^e for -126 <= e <= 127
-__device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) << 23); }
 
 // Cells a CTA's grid holds, and its points: the cells and w - 1 more to the right
 // (folded back, or into the neighbouring block, when the chunk is added up).
@@ -703,9 +693,8 @@ __global__ void __launch_bounds__(kThreads, kThreads == 256 ? 3 : 1)
       am = max(am, wmax[w]);
       blocks |= wblk[w];
     }
-    const int ex = max((int)(am >> 23) - 126, -80);  // |A| < 2^ex
-    const float scale = pow2f(kBits - ex);
-    const float unit = pow2f(ex - kBits);
+    const float top = fmaxf(__uint_as_float(am), 1e-20f);  // terms up to 2^kBits
+    const float scale = (float)(1 << kBits) / top, unit = top * (1.f / (float)(1 << kBits));
     while (blocks) {
       const int b = __ffs(blocks) - 1;
       blocks &= blocks - 1;
@@ -919,7 +908,13 @@ const NufftCoef& nufft_coef() {
 // slots, 11-12 against 11-14 us at 73,728, 23 against 13-15 us at 262,088; above,
 // 10-26 against 17-41 us at 2,048 slots, 19-59 against 17-47 us at 8,192.
 constexpr int kNuMovingMaxSamples = 512;  // the split phase of a moving scene
+// The FP64 phase always goes to the non-uniform FFT, which forms each path's carrier
+// phase and grid position in FP64 and leaves no per-sample FP64 work: 13-46 us
+// against 32-248 us at 512 slots and 64-4096 samples, 29 us against 2.64 ms at
+// 524,288 and 1024, and 1.0-2.6e-7 from FP64 against 3.3e-7-2.7e-6 (the term-by-term
+// kernel's FP32 sums).
 inline bool nufft_for(sbr_phase_mode mode, int Ns, int64_t records) {
+  if (mode == SBR_PHASE_FP64) return true;
   return mode == SBR_PHASE_SPLIT && records >= (Ns <= 512 ? 65536 : 8192);
 }
 
@@ -1013,8 +1008,12 @@ inline int nufft_threads(int Ns) { return nufft_wide(Ns) ? 1024 : 256; }
 
 using NufftSpread = void (*)(const float4*, const float2*, const float*, const float*, int64_t, const int32_t*, NufftArg,
                              NufftCoef, float2*, unsigned int*);
-inline NufftSpread nufft_kernel(int Ns, bool moving) {
-  if (nufft_wide(Ns)) return moving ? k_nufft_spread<false, true, 1024, 1> : k_nufft_spread<false, false, 1024, 1>;
+inline NufftSpread nufft_kernel(int Ns, bool fp64, bool moving) {
+  if (nufft_wide(Ns)) {
+    if (fp64) return moving ? k_nufft_spread<true, true, 1024, 1> : k_nufft_spread<true, false, 1024, 1>;
+    return moving ? k_nufft_spread<false, true, 1024, 1> : k_nufft_spread<false, false, 1024, 1>;
+  }
+  if (fp64) return moving ? k_nufft_spread<true, true, 256, 4> : k_nufft_spread<true, false, 256, 4>;
   return moving ? k_nufft_spread<false, true, 256, 4> : k_nufft_spread<false, false, 256, 4>;
 }
 
@@ -1028,8 +1027,8 @@ int nufft_per_sm(int Ns) {
   if (dev < kDevCache && cache[dev][lg]) return cache[dev][lg];
   const size_t sm = nufft_smem(Ns);
   int n = 32;
-  for (int moving = 0; moving < 2; ++moving) {
-    const NufftSpread k = nufft_kernel(Ns, moving != 0);
+  for (int i = 0; i < 4; ++i) {
+    const NufftSpread k = nufft_kernel(Ns, (i & 2) != 0, (i & 1) != 0);
     if (sm > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     int m = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&m, k, nufft_threads(Ns), sm);
@@ -1112,8 +1111,8 @@ sbr_status bind_ws(const sbr_radar_cfg* radar, int64_t cap, void* ws, size_t byt
 
 // The non-uniform FFT of chirps [c0, c0 + chirps) of a moving scene, or of a static
 // scene's one chirp, written to all of them: spread, then finish.
-void launch_nufft(const sbr_paths* p, const sbr_radar_cfg* r, const SynthWs& w, bool moving, int c0, int chirps,
-                  float2* cube, cudaStream_t st) {
+void launch_nufft(sbr_phase_mode mode, const sbr_paths* p, const sbr_radar_cfg* r, const SynthWs& w, bool moving, int c0,
+                  int chirps, float2* cube, cudaStream_t st) {
   const int V = p->n_virt, Ns = r->n_samples, M = 2 * Ns;
   NufftArg na{};
   while ((1 << na.log_m) < M) ++na.log_m;
@@ -1133,7 +1132,7 @@ void launch_nufft(const sbr_paths* p, const sbr_radar_cfg* r, const SynthWs& w, 
   const float2* plen = reinterpret_cast<const float2*>(p->path_len);
   const int grid = V * w.Qn * chirps;
   ::sbr::note_launch();
-  nufft_kernel(Ns, moving)<<<grid, nufft_threads(Ns), nufft_smem(Ns), st>>>(
+  nufft_kernel(Ns, mode == SBR_PHASE_FP64, moving)<<<grid, nufft_threads(Ns), nufft_smem(Ns), st>>>(
       prep, plen, p->phase_ofs, p->path_rate, p->path_cap, p->count, na, co, w.grids, w.fin_cnt);
   const int slices = M < kNuFinSlice ? 1 : M / kNuFinSlice;
   ::sbr::note_launch();
@@ -1141,33 +1140,12 @@ void launch_nufft(const sbr_paths* p, const sbr_radar_cfg* r, const SynthWs& w, 
                                                                                 r->n_chirps, moving);
 }
 
-// A moving scene: every chirp synthesised from its own delays (split phase by the
-// non-uniform FFT up to 512 samples, or the FP64 phase), chirp by chirp.
+// A moving scene: every chirp synthesised from its own delays (split phase up to 512
+// samples, or the FP64 phase), chirp by chirp.
 sbr_status launch_moving(sbr_phase_mode mode, const sbr_paths* p, const sbr_radar_cfg* r, const SynthWs& w,
                          float2* cube, cudaStream_t st) {
-  const int V = p->n_virt, Ns = r->n_samples, C = r->n_chirps;
-  const double per_chirp = r->chirp_rep / kC;  // delay change per chirp per (m/s) of dL/dt
-  if (mode == SBR_PHASE_SPLIT && Ns <= kNuMovingMaxSamples) {
-    for (int c = 0; c < C; ++c) launch_nufft(p, r, w, true, c, 1, cube, st);
-    return SBR_OK;
-  }
-  if (mode == SBR_PHASE_FP64) {
-    const int T = threads_for(Ns), Mv = Ns / T;
-    const int grid = V * w.Q;
-    const float4* prep = reinterpret_cast<const float4*>(p->prep);
-    const float2* plen = reinterpret_cast<const float2*>(p->path_len);
-    for (int c = 0; c < C; ++c) {
-      ::sbr::note_launch();
-      switch (Mv) {
-        case 1: k_synth_fp64<1><<<grid, T, 0, st>>>(prep, plen, p->phase_ofs, p->path_cap, p->count, V, w.Q, Ns, r->f0, r->bandwidth / Ns, w.partial, p->path_rate, c * per_chirp); break;
-        case 2: k_synth_fp64<2><<<grid, T, 0, st>>>(prep, plen, p->phase_ofs, p->path_cap, p->count, V, w.Q, Ns, r->f0, r->bandwidth / Ns, w.partial, p->path_rate, c * per_chirp); break;
-        case 4: k_synth_fp64<4><<<grid, T, 0, st>>>(prep, plen, p->phase_ofs, p->path_cap, p->count, V, w.Q, Ns, r->f0, r->bandwidth / Ns, w.partial, p->path_rate, c * per_chirp); break;
-        case 8: k_synth_fp64<8><<<grid, T, 0, st>>>(prep, plen, p->phase_ofs, p->path_cap, p->count, V, w.Q, Ns, r->f0, r->bandwidth / Ns, w.partial, p->path_rate, c * per_chirp); break;
-        default: k_synth_fp64<16><<<grid, T, 0, st>>>(prep, plen, p->phase_ofs, p->path_cap, p->count, V, w.Q, Ns, r->f0, r->bandwidth / Ns, w.partial, p->path_rate, c * per_chirp); break;
-      }
-      ::sbr::note_launch();
-      k_reduce<<<dim3((V * Ns + 255) / 256, 1), 256, 0, st>>>(w.partial, V, w.Q, Ns, C, cube, c);
-    }
+  if (mode == SBR_PHASE_FP64 || (mode == SBR_PHASE_SPLIT && r->n_samples <= kNuMovingMaxSamples)) {
+    for (int c = 0; c < r->n_chirps; ++c) launch_nufft(mode, p, r, w, true, c, 1, cube, st);
     return SBR_OK;
   }
   set_error("sbr_synthesize: SBR_SYNTH_MOVING supports SBR_PHASE_SPLIT up to %d samples and SBR_PHASE_FP64",
@@ -1227,7 +1205,7 @@ extern "C" sbr_status sbr_synthesize(const sbr_paths* paths, const sbr_radar_cfg
     return SBR_OK;
   }
   if (nufft_for(mode, Ns, paths->path_cap * paths->n_virt)) {
-    launch_nufft(paths, radar, w, false, 0, 1, reinterpret_cast<float2*>(d_cube), st);
+    launch_nufft(mode, paths, radar, w, false, 0, 1, reinterpret_cast<float2*>(d_cube), st);
     SBR_CUDA(cudaGetLastError());
     return SBR_OK;
   }

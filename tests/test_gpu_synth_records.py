@@ -21,6 +21,22 @@ pytestmark = pytest.mark.gpu
 TOL = 1e-6
 
 
+def bind64(sbr, radar, cap, L, A, rate=None):
+    """Path buffers holding path lengths (float-float pairs) and strengths, for the FP64 phase."""
+    P = L.shape[1]
+    paths = sbr.PathBuffers(cap, 1, radar.n_virt)
+    paths.prep()[:, :P, 3] = torch.from_numpy(A.astype(np.float32)).cuda()
+    paths.phase_ofs().zero_()
+    hi = L.astype(np.float32)
+    at = paths.s.path_len - paths.mem.data_ptr()
+    raw = paths.mem[at:at + 8 * radar.n_virt * cap].view(torch.float32).view(radar.n_virt, cap, 2)
+    raw[:, :P] = torch.from_numpy(np.stack([hi, (L - hi).astype(np.float32)], -1)).cuda()
+    if rate is not None:
+        paths.path_rate()[:, :P] = torch.from_numpy(rate.astype(np.float32)).cuda()
+    paths.count_tensor().fill_(P)
+    return paths, paths.path_len().cpu().numpy()[:, :P], A.astype(np.float32).astype(np.float64)
+
+
 def bind(sbr, radar, cap, delta, phi, A, rate=None):
     """Path buffers of ``cap`` slots per antenna holding the records (phi, delta in cycles, FP64)."""
     P = delta.shape[1]
@@ -103,3 +119,20 @@ def test_moving_records(sbr):
                        for c in range(16)], 1)
     # the chirp's phase shift (up to 1.3 cycles here) and delta shift are each rounded once more in FP32
     assert rel(cube, ref) <= 2 * TOL
+
+
+@pytest.mark.parametrize("ns,P,moving", [(32, 1, False), (64, 1023, False), (256, 1025, True), (1024, 1024, False),
+                                         (2048, 3001, True), (4096, 20000, False)])
+def test_fp64_records(sbr, ns, P, moving):
+    """The FP64 phase over delays of the whole unambiguous range, static and moving (4 chirps)."""
+    radar = radar_single_tx(ns, 4 if moving else 1)
+    rng = np.random.default_rng(ns)
+    L = rng.uniform(0.1, 0.999, (4, P)) * ns * C_LIGHT / radar.bandwidth
+    A = rng.uniform(0.1, 1.0, (4, P))
+    rate = rng.uniform(-30.0, 30.0, (4, P)).astype(np.float32) if moving else None
+    paths, L, A = bind64(sbr, radar, P + 3, L, A, rate)
+    cube = sbr.synthesize(paths, radar, sbr.PHASE_FP64 | (sbr.SYNTH_MOVING if moving else 0))
+    for c in range(radar.n_chirps):
+        Lc = L + (c * radar.chirp_rep * rate if moving else 0.0)
+        phi, delta = radar.f0 / C_LIGHT * Lc, radar.bandwidth / (C_LIGHT * ns) * Lc
+        assert rel(cube[:, c], direct(phi - np.round(phi), delta - np.round(delta), A, ns)) <= TOL
