@@ -33,11 +33,13 @@
 //
 // Every evaluation writes per-CTA partial sums (or grids) that a second kernel
 // adds in a fixed order, so the result is bitwise reproducible.
+#include <cooperative_groups.h>
 #include <cuda_fp16.h>
 #include <limits.h>
 #include <math.h>
 
 #include <algorithm>
+#include <atomic>
 #include <mutex>
 
 #include "common.cuh"
@@ -901,6 +903,152 @@ const NufftCoef& nufft_coef() {
   return c;
 }
 
+// ---- adjoint by the type-2 non-uniform FFT ----------------------------------
+//
+// Eq. 11-12 need, per (path, antenna), sums over the samples of the upstream
+// gradient against the path's phasors.  With h[n'] = conj(g[n' + N_s/2]) and
+// e^{j 2 pi x}, x = phi0 + (N_s/2) delta, the phasor at n' = 0,
+//   Z0 = e^{j 2 pi x} sum_n' h[n'] e^{j 2 pi n' delta},            dL/dA = Re Z0,
+//   Z1 = the same sum with weights 1 + (n' + N_s/2) B / (f_c N_s),  dL/dL = -2 pi A f_c / c Im Z1,
+// and dL/d(phase offset) = -2 pi A Im Z0.  Both sums are band-limited functions of
+// delta, so they are read off a grid of M = 2 N_s points (one M-point FFT each of
+// h / Psi(n'/M)) with the spreading kernel's eight weights: a path costs eight
+// 16-byte reads and 32 FMAs instead of N_s phasors and 6 N_s FMAs.  12 antennas x
+// 367,500 paths x 256 samples, 128 chirps: 43 us (505 us term by term), 16 us of them
+// the records' 16 bytes in and 8 out at the copy rate; error against FP64 2.8e-7
+// (6.8e-7).
+
+constexpr int kAdjThreads = 512;
+constexpr int kAdjMargin = kNuW;  // the grid is stored with its wrap-around: entry i is point i - 3
+
+// One cluster per antenna: its CTAs sum a share of the chirps each (a static scene's
+// chirps see the same paths), CTAs 0 and 1 then transform Z0's and Z1's coefficients
+// and write their halves of the grid's float4 entries.
+__global__ void __launch_bounds__(kAdjThreads) k_adj_grid(const float2* __restrict__ g, int V, int C, int Ns, int log_m,
+                                                          float slope, const __grid_constant__ NufftCoef co,
+                                                          float2* __restrict__ out) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  extern __shared__ float2 sa[];  // [N_s] this CTA's chirps summed, [M] grid, [M / 2] twiddles
+  const int M = 1 << log_m, rank = (int)cluster.block_rank(), ranks = (int)cluster.num_blocks();
+  const int v = blockIdx.x / ranks, h = Ns >> 1;
+  float2* s = sa + Ns;
+  float2* tw = s + M;
+  const int c0 = C * rank / ranks, c1 = C * (rank + 1) / ranks;
+  for (int n = threadIdx.x; n < Ns; n += kAdjThreads) {
+    float2 a = make_float2(0.f, 0.f);
+#pragma unroll 8
+    for (int c = c0; c < c1; ++c) {
+      const float2 x = __ldg(&g[((size_t)v * C + c) * Ns + n]);
+      a.x += x.x;
+      a.y += x.y;
+    }
+    sa[n] = a;
+  }
+  if (rank < 2) {
+    fft::fill_twiddles(tw, M, 1.f, kAdjThreads, threadIdx.x);
+    for (int i = threadIdx.x; i < M; i += kAdjThreads) s[i] = make_float2(0.f, 0.f);
+  }
+  cluster.sync();
+  if (rank < 2) {
+    for (int n = threadIdx.x; n < Ns; n += kAdjThreads) {
+      float2 a = make_float2(0.f, 0.f);
+      for (int r = 0; r < ranks; ++r) {
+        const float2 x = cluster.map_shared_rank(sa, r)[n];
+        a.x += x.x;
+        a.y += x.y;
+      }
+      const float xi = (float)(n - h) / (float)h, y = xi * xi;
+      float w = co.inv[8];
+#pragma unroll
+      for (int k = 7; k >= 0; --k) w = fmaf(w, y, co.inv[k]);
+      if (rank == 1) w *= fmaf((float)n, slope, 1.f);
+      s[fft::bitrev((n - h) & (M - 1), log_m)] = make_float2(a.x * w, -a.y * w);
+    }
+    __syncthreads();
+    fft::smem_fft(s, tw, log_m, kAdjThreads, threadIdx.x);
+    float2* o = out + 2 * (size_t)v * (M + kAdjMargin) + rank;
+    for (int i = threadIdx.x; i < M + kAdjMargin; i += kAdjThreads) o[2 * i] = s[(i - (kNuW / 2 - 1)) & (M - 1)];
+  }
+  cluster.sync();  // no CTA leaves while another may read its shared memory
+}
+
+// One record per thread at a time, the grid's CTAs striding over antenna blockIdx.y's
+// records.  The grid (8 KB to 131 KB per antenna) is read through L1, where the
+// neighbouring rays of a warp share lines.
+__global__ void __launch_bounds__(256) k_synth_bwd_nufft(const float4* __restrict__ prep, int64_t cap,
+                                                         const int32_t* __restrict__ d_P, int log_m,
+                                                         const __grid_constant__ NufftCoef co,
+                                                         const float4* __restrict__ grid, float inv_lambda,
+                                                         float* __restrict__ glen, float* __restrict__ gamp,
+                                                         float* __restrict__ gphase) {
+  const int v = blockIdx.y, M = 1 << log_m, P = *d_P;
+  const float m = (float)M, half_n = 0.25f * m;
+  const size_t row = (size_t)v * cap;
+  const float4* gv = grid + (size_t)v * (M + kAdjMargin);
+  for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < P; p += (int64_t)gridDim.x * blockDim.x) {
+    const float4 r = __ldg(&prep[row + p]);
+    float x = half_n * r.y;  // exact
+    x -= rintf(x);
+    x = fmaf(half_n, r.z, x) + r.x;
+    const float uh = m * r.y;  // exact
+    float fl = floorf(uh);
+    float t = fmaf(m, r.z, uh - fl);
+    int cell = (int)fl;
+    fl = floorf(t);
+    t -= fl;
+    cell = (cell + (int)fl) & (M - 1);
+    const float s = t - 0.5f, s2 = s * s;
+    float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+    auto add = [&](float w, float4 q) {
+      z.x = fmaf(w, q.x, z.x);
+      z.y = fmaf(w, q.y, z.y);
+      z.z = fmaf(w, q.z, z.z);
+      z.w = fmaf(w, q.w, z.w);
+    };
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {  // outermost points first: the smallest weights
+      const float4 ql = __ldg(&gv[cell + j]), qr = __ldg(&gv[cell + 7 - j]);
+      float E = co.e[j][4], O = co.o[j][3];
+#pragma unroll
+      for (int k = 3; k >= 0; --k) E = fmaf(E, s2, co.e[j][k]);
+#pragma unroll
+      for (int k = 2; k >= 0; --k) O = fmaf(O, s2, co.o[j][k]);
+      add(fmaf(O, s, E), ql);
+      add(fmaf(-O, s, E), qr);
+    }
+    float sn, cs;
+    sincospif(2.f * x, &sn, &cs);
+    gamp[row + p] = cs * z.x - sn * z.y;
+    glen[row + p] = -kTwoPiF * r.w * inv_lambda * (cs * z.w + sn * z.z);
+    if (gphase) gphase[row + p] = -kTwoPiF * r.w * (cs * z.y + sn * z.x);
+  }
+}
+
+inline size_t adj_smem(int Ns) { return sizeof(float2) * 4 * (size_t)Ns; }
+
+cudaError_t adj_attr(int Ns) {
+  static std::atomic<uint64_t> done{0};  // bit per device ordinal below 64
+  if (adj_smem(Ns) <= 48 * 1024) return cudaSuccess;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 64 && ((done.load() >> dev) & 1u)) return cudaSuccess;
+  e = cudaFuncSetAttribute(k_adj_grid, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)adj_smem(4096));
+  if (e == cudaSuccess && dev < 64) done.fetch_or(1ull << dev);
+  return e;
+}
+
+// When the grids beat the direct kernel (k_chirp_sum, k_synth_bwd), by record slots
+// (path_cap x antennas), measured: 256 samples, one chirp, 6.9 against 6.5 us at
+// 32,768 and 7.0 against 10.4 us at 64,800; 64 samples 6.5 against 4.3 us at 131,072
+// and 7.2 against 9.1 us at 524,288; 1024 samples 12.1 against 14.0 us at 512
+// already; 128 chirps (whose sum the direct kernel's one CTA per antenna waits for)
+// 9.3 against 11.4 us at 1,536.
+inline bool adj_nufft_for(int Ns, int C, int64_t records) {
+  return Ns >= 1024 || C >= 8 || records * Ns >= (3 << 22);
+}
+
 // Few (path, antenna) record slots: the direct kernels, whose one pass over the
 // records costs less than the non-uniform FFT's spreading, finishing sum and FFT
 // chain.  Measured crossings (4 antennas, one wave of either): up to 512 samples,
@@ -1064,6 +1212,7 @@ size_t ws_layout(const sbr_radar_cfg* radar, int64_t cap, int* Q, int* Qn = null
   c.take<float2>((size_t)V * qn * 2 * Ns);     // non-uniform FFT: the CTAs' grids
   c.take<float2>((size_t)V * 2 * Ns);          // non-uniform FFT: the summed grids
   c.take<unsigned int>((size_t)V);             // non-uniform FFT: finishing counters
+  c.take<float4>((size_t)V * (2 * Ns + kAdjMargin));  // adjoint: the antennas' grids
   return c.bytes();
 }
 
@@ -1085,6 +1234,7 @@ struct SynthWs {
   float2* grids;
   float2* bsum;
   unsigned int* fin_cnt;
+  float4* adj;
   int Q, Qn;
 };
 
@@ -1104,6 +1254,7 @@ sbr_status bind_ws(const sbr_radar_cfg* radar, int64_t cap, void* ws, size_t byt
   w->grids = c.take<float2>((size_t)V * Qn * 2 * Ns);
   w->bsum = c.take<float2>((size_t)V * 2 * Ns);
   w->fin_cnt = c.take<unsigned int>((size_t)V);
+  w->adj = c.take<float4>((size_t)V * (2 * Ns + kAdjMargin));
   w->Q = Q;
   w->Qn = Qn;
   return SBR_OK;
@@ -1314,6 +1465,36 @@ extern "C" sbr_status sbr_synthesize_bwd(const sbr_paths* paths, const sbr_radar
   if (rs != SBR_OK) return rs;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const int V = paths->n_virt, Ns = radar->n_samples, C = radar->n_chirps;
+  const double lam_inv = radar->f0 / kC;
+  if (paths->path_cap > 0 && adj_nufft_for(Ns, C, paths->path_cap * V)) {
+    int log_m = 0;
+    while ((1 << log_m) < 2 * Ns) ++log_m;
+    SBR_CUDA(adj_attr(Ns));
+    cudaLaunchConfig_t lc{};
+    cudaLaunchAttribute at{};
+    const unsigned ranks = C >= 8 ? 8 : 2;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = ranks;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    lc.gridDim = dim3(V * ranks);
+    lc.blockDim = dim3(kAdjThreads);
+    lc.dynamicSmemBytes = adj_smem(Ns);
+    lc.stream = st;
+    lc.attrs = &at;
+    lc.numAttrs = 1;
+    const NufftCoef& co = nufft_coef();
+    ::sbr::note_launch();
+    SBR_CUDA(cudaLaunchKernelEx(&lc, k_adj_grid, reinterpret_cast<const float2*>(d_gcube), V, C, Ns, log_m,
+                                (float)(radar->bandwidth / (radar->f0 * Ns)), co, reinterpret_cast<float2*>(w.adj)));
+    // a wave of CTAs at most, at least one per antenna
+    const int64_t need = (paths->path_cap + 255) / 256, wave = std::max(1, 8 * sm_count() / V);
+    ::sbr::note_launch();
+    k_synth_bwd_nufft<<<dim3((unsigned)std::min(need, wave), V), 256, 0, st>>>(
+        reinterpret_cast<const float4*>(paths->prep), paths->path_cap, paths->count, log_m, co, w.adj, (float)lam_inv,
+        d_glen, d_gamp, d_gphase);
+    SBR_CUDA(cudaGetLastError());
+    return SBR_OK;
+  }
   // the upstream gradient summed over the (equal) chirps; one chirp needs no sum
   const float2* gs = reinterpret_cast<const float2*>(d_gcube);
   if (C > 1) {
@@ -1324,7 +1505,6 @@ extern "C" sbr_status sbr_synthesize_bwd(const sbr_paths* paths, const sbr_radar
   const int64_t cap = paths->path_cap;
   if (cap > 0) {
     dim3 grid((unsigned)((cap + 255) / 256), (unsigned)V);
-    const double lam_inv = radar->f0 / kC;
     const double bcn = radar->bandwidth / (kC * Ns);
     ::sbr::note_launch();
     k_synth_bwd<<<grid, 256, Ns * sizeof(float2), st>>>(

@@ -136,3 +136,31 @@ def test_fp64_records(sbr, ns, P, moving):
         Lc = L + (c * radar.chirp_rep * rate if moving else 0.0)
         phi, delta = radar.f0 / C_LIGHT * Lc, radar.bandwidth / (C_LIGHT * ns) * Lc
         assert rel(cube[:, c], direct(phi - np.round(phi), delta - np.round(delta), A, ns)) <= TOL
+
+
+@pytest.mark.parametrize("ns,nc,P,where", [
+    (32, 8, 1, "all"), (64, 1, 50001, "edges"), (256, 1, 12288, "all"), (256, 1, 12289, "edges"), (256, 128, 255, "all"),
+    (512, 4, 6200, "one"), (1024, 1, 257, "edges"), (2048, 16, 513, "all"), (4096, 1, 4099, "edges")])
+def test_adjoint_records(sbr, ns, nc, P, where):
+    """sbr_synthesize_bwd (dL/dlength, dL/dA, dL/dphase) on given records against FP64 sums."""
+    radar = radar_single_tx(ns, nc)
+    delta, phi, A = records(ns + P, 4, P, ns, where)
+    paths, phi, delta, A = bind(sbr, radar, P + 5, delta, phi, A)
+    gen = torch.Generator(device="cuda").manual_seed(P)
+    gcube = torch.randn(4, nc, ns, 2, generator=gen, device="cuda")
+    got = sbr.synthesize_bwd(paths, radar, gcube, phase=True)
+    g = torch.view_as_complex(gcube.double()).sum(1)
+    n = torch.arange(ns, dtype=torch.float64, device="cuda")
+    k0, k1 = radar.f0 / C_LIGHT, radar.bandwidth / (C_LIGHT * ns)
+    ref = torch.empty(3, 4, P, dtype=torch.float64, device="cuda")
+    for v in range(4):
+        p, d, a = (torch.from_numpy(x[v]).cuda() for x in (phi, delta, A))
+        for s in range(0, P, 4096):
+            x = p[s:s + 4096, None] + d[s:s + 4096, None] * n
+            e = torch.polar(torch.ones_like(x), 2 * math.pi * (x - x.round()))
+            z0, z1 = (e * g[v].conj()).sum(1), (e * (g[v].conj() * n)).sum(1)
+            ref[0, v, s:s + 4096] = -2 * math.pi * a[s:s + 4096] * (k0 * z0.imag + k1 * z1.imag)
+            ref[1, v, s:s + 4096] = z0.real
+            ref[2, v, s:s + 4096] = -2 * math.pi * a[s:s + 4096] * z0.imag
+    for x, y in zip(got, ref):
+        assert float((x[:, :P].double() - y).norm() / y.norm()) <= TOL
