@@ -96,8 +96,60 @@ __host__ inline int ceil_log2(int64_t n) {
 __device__ inline int fix_exp(unsigned int max_bits, int log2n) {
   return 62 - log2n - ((int)((max_bits >> 23) & 0xffu) - 126);
 }
+// x 2^E rounded to the nearest integer (ties to even) on the integer pipe: the FP64
+// pipe, where ldexp and the conversion would run, has a small fraction of its rate.
+// Not finite: the values a saturating conversion gives.
+__device__ inline long long fix_ll(float x, int E) {
+  const unsigned b = __float_as_uint(x), ex = (b >> 23) & 0xffu;
+  const long long m = (long long)((b & 0x7fffffu) | (ex ? 0x800000u : 0u));
+  const int sh = (int)(ex ? ex : 1u) - 150 + E;
+  long long r;
+  if (ex == 255u) {
+    return x > 0.f ? 0x7fffffffffffffffll : (long long)0x8000000000000000ull;
+  } else if (sh >= 0) {
+    r = m << min(sh, 39);
+  } else if (sh < -25) {
+    r = 0;
+  } else {
+    const long long q = m >> -sh;
+    r = (m + ((1ll << (-sh - 1)) - 1) + (q & 1)) >> -sh;
+  }
+  return (b >> 31) ? -r : r;
+}
 __device__ inline void fix_add(unsigned long long* acc, float x, int E) {
-  atomicAdd(acc, (unsigned long long)__double2ll_rn(ldexp((double)x, E)));
+  atomicAdd(acc, (unsigned long long)fix_ll(x, E));
+}
+
+// Sum of x over the lanes of `peers` (all of them call with the same mask): three
+// 32-bit warp sums of 26, 26 and 12 bits.
+__device__ inline long long peer_sum(unsigned peers, long long x) {
+  constexpr unsigned kLow = (1u << 26) - 1u;
+  const unsigned lo = __reduce_add_sync(peers, (unsigned)x & kLow);
+  const unsigned mid = __reduce_add_sync(peers, (unsigned)(x >> 26) & kLow);
+  const int hi = __reduce_add_sync(peers, (int)(x >> 52));
+  return (long long)lo + ((long long)mid << 26) + (long long)((unsigned long long)(long long)hi << 52);
+}
+
+// Adds the calling lanes' values x[0 .. n) to acc[n i + c], lanes with the same i as
+// one: rays of a warp mostly hit the same few triangles, and a large triangle's
+// corners take contributions from most of the launch, whose atomics would queue at one
+// address.  Integer sums: the result is that of one atomic per lane.  Each group of
+// peers runs its warp sums on its own, so small groups go straight to the atomics.
+constexpr int kPeersDirect = 4;
+template <int n>
+__device__ inline void fix_add_peers(unsigned long long* acc, int i, const float* x, int E) {
+  const unsigned peers = __match_any_sync(__activemask(), i);
+  if (__popc(peers) <= kPeersDirect) {
+#pragma unroll
+    for (int c = 0; c < n; ++c) fix_add(&acc[(size_t)n * i + c], x[c], E);
+    return;
+  }
+  const bool lead = (int)(threadIdx.x & 31) == __ffs(peers) - 1;
+#pragma unroll
+  for (int c = 0; c < n; ++c) {
+    const long long v = peer_sum(peers, fix_ll(x[c], E));
+    if (lead) atomicAdd(&acc[(size_t)n * i + c], (unsigned long long)v);
+  }
 }
 __device__ inline float fix_get(unsigned long long a, int E) { return (float)ldexp((double)(long long)a, -E); }
 // Warp-reduced max of |x| over the calling warp's lanes (all 32 must call), one atomic per warp.

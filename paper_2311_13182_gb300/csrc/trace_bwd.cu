@@ -29,6 +29,11 @@
 // order-independent fixed-point scatter of common.cuh (two passes over the rays:
 // the largest contribution, then the integer sums), so the gradient is bitwise
 // the same on every run.
+// What bounds it where many rays share a triangle (a ground plane's two) is the queue
+// of 64-bit atomics at its corners, so the lanes of a warp that add to one vertex add
+// as one (fix_add_peers), at the same bounce: 523,000 rays on 20,002 triangles,
+// integer pass 1214 -> 84 us; 4,096 rays on 5,120 triangles, where few lanes share a
+// vertex, 11.5 -> 11.9 us (38 us if groups of up to four were summed too).
 #include <math.h>
 
 #include "scene.cuh"
@@ -62,9 +67,8 @@ __device__ inline void scatter(const FixScatter& fs, int E, float& lmax, int vi,
   if (kPass == 0) {
     lmax = fmaxf(lmax, fmaxf(fabsf(d.x), fmaxf(fabsf(d.y), fabsf(d.z))));
   } else {
-    fix_add(&fs.acc[3 * vi], d.x, E);
-    fix_add(&fs.acc[3 * vi + 1], d.y, E);
-    fix_add(&fs.acc[3 * vi + 2], d.z, E);
+    const float x[3] = {d.x, d.y, d.z};
+    fix_add_peers<3>(fs.acc, vi, x, E);
   }
 }
 
@@ -74,8 +78,8 @@ __device__ inline void scatter_eps(const FixScatter& fe, int Ee, float& emax, in
   if (kPass == 0) {
     emax = fmaxf(emax, fmaxf(fabsf(dre), fabsf(dim)));
   } else {
-    fix_add(&fe.acc[2 * m], dre, Ee);
-    fix_add(&fe.acc[2 * m + 1], dim, Ee);
+    const float x[2] = {dre, dim};
+    fix_add_peers<2>(fe.acc, m, x, Ee);
   }
 }
 
@@ -217,7 +221,8 @@ __device__ void ray_adjoint(int i, const float* __restrict__ verts, int nv, cons
   // reverse sweep over bounces
   float3 db_next = f3(0.f, 0.f, 0.f);  // adjoint of d_{k+1}
   float3 ob_next = f3(0.f, 0.f, 0.f);  // adjoint of o_{k+1} = h_k
-  for (int k = m - 1; k >= 0; --k) {
+  for (int k = K - 1; k >= 0; --k) {  // the warp's rays at the same bounce: they share triangles
+    if (k >= m) continue;
     float3 db = f3(0.f, 0.f, 0.f), nb = f3(0.f, 0.f, 0.f);
     // |d.n|
     const float cbar = cb[k] * (cdn[k] >= 0.f ? 1.f : -1.f);
