@@ -404,15 +404,43 @@ __device__ inline uint32_t detect_key(const float* __restrict__ Pw, const CfarAr
   return w >= c.w_min ? 0xffffffffu - __float_as_uint(w) : 0xffffffffu;
 }
 
-__global__ void k_detect(const float* __restrict__ Pw, CfarArg c, const unsigned long long* __restrict__ amax_key,
-                         int32_t* __restrict__ amax, int32_t* __restrict__ flag, uint32_t* __restrict__ key) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+// Detections of 256 consecutive cells per CTA, appended in cell order to the CTA's
+// list (keys and cells at 256 blockIdx.x, their number in cnt), or, when flag is
+// given, marked per cell for the multi-kernel selection.
+constexpr int kDetThreads = 256;
+__global__ void __launch_bounds__(kDetThreads) k_detect(const float* __restrict__ Pw, CfarArg c,
+                                                        const unsigned long long* __restrict__ amax_key,
+                                                        int32_t* __restrict__ amax, int32_t* __restrict__ flag,
+                                                        uint32_t* __restrict__ key, int32_t* __restrict__ cell,
+                                                        int32_t* __restrict__ cnt) {
+  __shared__ int wn[kDetThreads / 32];
+  const int i = blockIdx.x * kDetThreads + threadIdx.x;  // cells come in multiples of 256
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int am = amax_cell(amax_key);
   if (i == 0) *amax = am;
-  if (i >= c.E * c.A * c.Ns) return;
-  const uint32_t kk = detect_key(Pw, c, i, c.floor_rel * Pw[am]);
-  if (flag) flag[i] = kk != 0xffffffffu ? 1 : 0;
-  key[i] = kk;
+  const bool in = i < c.E * c.A * c.Ns;
+  const uint32_t kk = in ? detect_key(Pw, c, i, c.floor_rel * Pw[am]) : 0xffffffffu;
+  const bool hit = kk != 0xffffffffu;
+  if (flag) {
+    if (in) {
+      flag[i] = hit ? 1 : 0;
+      key[i] = kk;
+    }
+    return;
+  }
+  const unsigned m = __ballot_sync(0xffffffffu, hit);
+  if (lane == 0) wn[warp] = __popc(m);
+  __syncthreads();
+  int pos = blockIdx.x * kDetThreads + __popc(m & ((1u << lane) - 1u)), n = 0;
+  for (int w = 0; w < kDetThreads / 32; ++w) {
+    if (w < warp) pos += wn[w];
+    n += wn[w];
+  }
+  if (hit) {
+    key[pos] = kk;
+    cell[pos] = i;
+  }
+  if (threadIdx.x == 0) cnt[blockIdx.x] = n;
 }
 
 __global__ void k_compact(const int32_t* __restrict__ flag, const int32_t* __restrict__ off,
@@ -512,71 +540,96 @@ __global__ void k_points(const float* __restrict__ Pw, PointArg pa, const int32_
   cell_out[i] = cell;
 }
 
-// Steps 7-9 in one CTA when the map has at most kSortOneCta cells: compaction
-// of k_detect's keys in cell order (rounds of 4096 cells, four per thread, one
-// block scan per round places them), the stable sort by weight, and the points.  Same
-// results as scan, k_compact, the sort and k_points, in one launch instead of four.
+// Steps 7-9 in one CTA: k_detect's lists joined in cell order, the stable sort by
+// weight, and the points.  A map has a few hundred detections whatever its size, so
+// the joined list is what this costs (a scan over the CTAs' counts and a direct
+// ranking); the multi-kernel compaction and eight-pass sort of maps above 65,536
+// cells took 140 us for 262,144 cells against 14 us.  A map of noise can have tens
+// of thousands: then a radix selection first keeps the k_max that are emitted.
 constexpr int kSelThreads = 1024;
+constexpr int kSelMax = 4096;  // points a selection from a map of any size may keep
 constexpr int kRankMax = 256;  // candidates k_select ranks directly (shared memory: 2 KB)
 static_assert(2 * kRankMax <= cta::kSortSmemWords, "the rank buffers share the sort's shared memory");
+
+// The k smallest of n (key, cell) pairs, equal keys in list order, moved to (ko, vo) in list order.
+__device__ inline void select_smallest(const uint32_t* k0, const int32_t* v0, int n, int k, uint32_t* ko, int32_t* vo,
+                                       uint32_t* sm, uint32_t* wt) {
+  uint32_t* hist = sm;  // [256]
+  __shared__ uint32_t s_prefix, s_left;
+  const int t = threadIdx.x;
+  uint32_t prefix = 0, left = (uint32_t)k;  // the k-th smallest key's leading digits; its rank among keys sharing them
+  for (int d = 3; d >= 0; --d) {
+    if (t < 256) hist[t] = 0u;
+    __syncthreads();
+    const uint32_t mask = d == 3 ? 0u : 0xffffffffu << (8 * (d + 1));
+    for (int i = t; i < n; i += kSelThreads) {
+      const uint32_t key = k0[i];
+      if ((key & mask) == prefix) atomicAdd(&hist[(key >> (8 * d)) & 255u], 1u);
+    }
+    __syncthreads();
+    if (t == 0) {
+      uint32_t b = 0;
+      while (left > hist[b]) left -= hist[b++];
+      s_prefix = prefix | (b << (8 * d));
+      s_left = left;
+    }
+    __syncthreads();
+    prefix = s_prefix;
+    left = s_left;
+  }
+  uint32_t base = 0, ties = 0;  // kept so far; keys equal to the k-th smallest met so far
+  for (int r = 0; r < n; r += kSelThreads) {
+    const int i = r + t;
+    const uint32_t key = i < n ? k0[i] : 0xffffffffu;
+    uint32_t tot;
+    const uint32_t tie = block_exclusive_sel(i < n && key == prefix, &tot, wt) + ties;
+    ties += tot;
+    const bool keep = i < n && (key < prefix || (key == prefix && tie < left));
+    const uint32_t pos = base + block_exclusive_sel(keep, &tot, wt);
+    base += tot;
+    if (keep) {
+      ko[pos] = key;
+      vo[pos] = v0[i];
+    }
+  }
+  __syncthreads();
+}
+
 __global__ void __launch_bounds__(kSelThreads) k_select(const float* __restrict__ Pw, PointArg pa,
                                                         const unsigned long long* __restrict__ amax_key,
                                                         const uint32_t* __restrict__ key,
+                                                        const int32_t* __restrict__ list, const int32_t* __restrict__ cnt,
                                                         uint32_t* k0, int32_t* v0, uint32_t* k1, int32_t* v1,
                                                         float4* __restrict__ pts, int32_t* __restrict__ cell_out,
                                                         int32_t* __restrict__ n_out) {
   extern __shared__ __align__(16) uint32_t sel_sm[];  // cta::kSortSmemWords
   __shared__ uint32_t wt[32];
   const CfarArg& c = pa.c;
-  const int cells = c.E * c.A * c.Ns, t = threadIdx.x;
+  const int lists = c.E * c.A * c.Ns / kDetThreads, t = threadIdx.x;
   const float floor_v = c.floor_rel * Pw[amax_cell(amax_key)];
-  // rounds of 4 x kSelThreads cells (cells is a multiple of 8): thread t loads
-  // cells 4t .. 4t + 3 of the round as one coalesced 16-B load, up to four
-  // rounds' loads in flight before the first scan
-  constexpr int kRound = 4 * kSelThreads, kBatch = 4;
-  const uint4* key4 = reinterpret_cast<const uint4*>(key);
-  uint32_t base = 0;
-  for (int r0 = 0; r0 < cells; r0 += kBatch * kRound) {
-    uint4 q[kBatch];
-#pragma unroll
-    for (int b = 0; b < kBatch; ++b) {
-      const int cell = r0 + b * kRound + 4 * t;
-      q[b] = cell < cells ? __ldcg(&key4[cell >> 2]) : make_uint4(~0u, ~0u, ~0u, ~0u);
-    }
-#pragma unroll
-    for (int b = 0; b < kBatch; ++b) {
-      if (r0 + b * kRound >= cells) break;  // the same for every thread
-      const uint32_t kq[4] = {q[b].x, q[b].y, q[b].z, q[b].w};
-      uint32_t mine = 0;
-#pragma unroll
-      for (int e = 0; e < 4; ++e) mine += kq[e] != 0xffffffffu;
-      uint32_t total;
-      uint32_t pos = base + block_exclusive_sel(mine, &total, wt);
-      const int cell = r0 + b * kRound + 4 * t;
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        if (kq[e] != 0xffffffffu) {
-          k0[pos] = kq[e];
-          v0[pos] = cell + e;
-          ++pos;
-        }
-      }
-      base += total;
+  const int per = (lists + kSelThreads - 1) / kSelThreads, l0 = min(t * per, lists), l1 = min(l0 + per, lists);
+  uint32_t mine = 0, total;
+  for (int l = l0; l < l1; ++l) mine += (uint32_t)cnt[l];
+  uint32_t pos = block_exclusive_sel(mine, &total, wt);
+  uint32_t* rk = sel_sm;
+  int32_t* rv = reinterpret_cast<int32_t*>(sel_sm + kRankMax);
+  const bool direct = total <= (uint32_t)kRankMax;  // joined in shared memory
+  uint32_t* jk = direct ? rk : k0;
+  int32_t* jv = direct ? rv : v0;
+  for (int l = l0; l < l1 && mine; ++l) {
+    const int m = cnt[l];
+    for (int e = 0; e < m; ++e, ++pos) {
+      jk[pos] = key[l * kDetThreads + e];
+      jv[pos] = list[l * kDetThreads + e];
     }
   }
-  const uint32_t total = base;
-  __syncthreads();  // the compacted candidates are visible to the whole CTA
-  if (total <= (uint32_t)kRankMax) {
+  __syncthreads();  // the joined candidates are visible to the whole CTA
+  const int n = min((int)total, pa.k_max);
+  const int32_t* sorted = v0;
+  if (direct) {
     // few candidates: each one's rank is the number of smaller keys plus the equal keys
     // before it (they are in cell order), i.e. its place in the stable sort, found with
     // two barriers instead of the sort network's dozens
-    uint32_t* rk = sel_sm;
-    int32_t* rv = reinterpret_cast<int32_t*>(sel_sm + kRankMax);
-    for (int i = t; i < (int)total; i += kSelThreads) {
-      rk[i] = k0[i];
-      rv[i] = v0[i];
-    }
-    __syncthreads();
     if (t < (int)total) {
       const uint32_t ki = rk[t];
       int r = 0;
@@ -586,18 +639,21 @@ __global__ void __launch_bounds__(kSelThreads) k_select(const float* __restrict_
       }
       v0[r] = rv[t];
     }
+  } else if ((int)total > n && total > (uint32_t)cta::kRankRound) {
+    select_smallest(k0, v0, (int)total, n, k1, v1, sel_sm, wt);
+    cta::sort_pairs(k1, v1, k0, v0, n, 32, nullptr, sel_sm);
+    sorted = v1;
   } else {
     cta::sort_pairs(k0, v0, k1, v1, (int64_t)total, 32, nullptr, sel_sm);
   }
   __syncthreads();
-  const int n = min((int)total, pa.k_max);
   if (t == 0) *n_out = n;
   for (int i = t; i < pa.k_max; i += kSelThreads) {
     if (i >= n) {
       pts[i] = make_float4(0.f, 0.f, 0.f, 0.f);
       cell_out[i] = -1;
     } else {
-      const int cell = v0[i];
+      const int cell = sorted[i];
       pts[i] = emit_point(Pw, pa, floor_v, cell);
       cell_out[i] = cell;
     }
@@ -1041,12 +1097,14 @@ extern "C" sbr_status sbr_pointcloud(const float* d_cube, const sbr_radar_cfg* r
   // 5-9: soft CFAR, peaks, compaction in cell order, stable sort by weight, points
   const CfarArg ca = cfar_arg(radar, cfar);
   PointArg pa{ca, cfar->k_max, (float)(kC / (2.0 * radar->bandwidth))};
-  if (cells <= kSortOneCta) {
+  // one CTA selects, except from a large map asked for more points than its radix
+  // selection bounds the sort by
+  if (cells <= kSortOneCta || cfar->k_max <= kSelMax) {
     SBR_CUDA(select_attr());
     ::sbr::note_launch();
-    k_detect<<<(cells + 255) / 256, 256, 0, st>>>(L.power, ca, L.amax_key, L.argmax, nullptr, L.key);
+    k_detect<<<cells / kDetThreads, kDetThreads, 0, st>>>(L.power, ca, L.amax_key, L.argmax, nullptr, L.key, L.flag, L.off);
     ::sbr::note_launch();
-    k_select<<<1, kSelThreads, cta::kSortSmemBytes, st>>>(L.power, pa, L.amax_key, L.key, L.skeys[0],
+    k_select<<<1, kSelThreads, cta::kSortSmemBytes, st>>>(L.power, pa, L.amax_key, L.key, L.flag, L.off, L.skeys[0],
                                                            L.svals[0], L.skeys[1], L.svals[1],
                                                            reinterpret_cast<float4*>(d_points), L.peak_cell,
                                                            L.n_points);
@@ -1054,7 +1112,7 @@ extern "C" sbr_status sbr_pointcloud(const float* d_cube, const sbr_radar_cfg* r
     return SBR_OK;
   }
   ::sbr::note_launch();
-  k_detect<<<(cells + 255) / 256, 256, 0, st>>>(L.power, ca, L.amax_key, L.argmax, L.flag, L.key);
+  k_detect<<<cells / kDetThreads, kDetThreads, 0, st>>>(L.power, ca, L.amax_key, L.argmax, L.flag, L.key, nullptr, nullptr);
   SBR_CUDA(exclusive_scan(L.flag, L.off, cells, nullptr, L.scan_scr, st));
   ::sbr::note_launch();
   k_compact<<<(cells + 255) / 256, 256, 0, st>>>(L.flag, L.off, L.key, cells, L.skeys[0], L.svals[0]);
