@@ -30,27 +30,41 @@ namespace {
 
 using namespace fft;
 
-// FFT along the contiguous last axis: one CTA per row of n points.
-__global__ void k_fft_rows(const float2* __restrict__ in, float2* __restrict__ out, int n, int logn,
-                           float sign) {
-  extern __shared__ float2 s[];  // [n] points, [n / 2] twiddles
-  float2* tw = s + n;
-  const size_t row = blockIdx.x;
+// FFT along the contiguous last axis: 2^logb rows of n points per CTA, eight points
+// per thread.  clear: words the first CTA zeroes for later kernels of the call, or NULL.
+__global__ void k_fft_rows(const float2* __restrict__ in, float2* __restrict__ out, int rows, int logn, int logb,
+                           float sign, unsigned long long* clear) {
+  extern __shared__ float2 s[];  // [2^logb] rows of slots(n) points, slots(n / 2) twiddles
+  const int n = 1 << logn, ld = slots(n);
+  float2* tw = s + (ld << logb);
+  if (clear && blockIdx.x == 0 && threadIdx.x < 2) clear[threadIdx.x] = 0ull;
+  const size_t at = (size_t)blockIdx.x << (logn + logb);
+  const int cnt = min(1 << logb, rows - ((int)blockIdx.x << logb)) << logn;  // points of this CTA's rows
+  float2 x[8];  // in flight while the twiddles are computed: the CTA holds eight points per thread
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const int i = threadIdx.x + u * blockDim.x;
+    x[u] = i < cnt ? in[at + i] : make_float2(0.f, 0.f);
+  }
   fill_twiddles(tw, n, sign, blockDim.x, threadIdx.x);
-  for (int i = threadIdx.x; i < n; i += blockDim.x) s[bitrev(i, logn)] = in[row * n + i];
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const int i = threadIdx.x + u * blockDim.x;
+    if (i < cnt) s[(i >> logn) * ld + slot(bitrev(i & (n - 1), logn))] = x[u];
+  }
   __syncthreads();
-  smem_fft(s, tw, logn, blockDim.x, threadIdx.x);
-  for (int i = threadIdx.x; i < n; i += blockDim.x) out[row * n + i] = s[i];
+  smem_fft_rows<false>(s, ld, logb, tw, logn, blockDim.x, threadIdx.x);
+  for (int i = threadIdx.x; i < cnt; i += blockDim.x) out[at + i] = s[(i >> logn) * ld + slot(i & (n - 1))];
 }
 
-constexpr int kColTile = 16;
+constexpr int kLogColTile = 4, kColTile = 1 << kLogColTile;
 
 // FFT along the chirp axis of [V][C][N_s]: one CTA per (v, 16 consecutive k).
-// Columns sit C + 1 points apart in shared memory, so the 16 columns of one
-// chirp fall in different banks.
+// Columns sit an odd number of points apart in shared memory, so the 16 columns of
+// one chirp fall in different banks.
 __global__ void k_fft_cols(float2* __restrict__ x, int C, int logc, int Ns, float sign) {
-  extern __shared__ float2 s[];  // [kColTile][C + 1] points, [C / 2] twiddles
-  const int ld = C + 1;
+  extern __shared__ float2 s[];  // [kColTile][slots(C) | 1] points, slots(C / 2) twiddles
+  const int ld = slots(C) | 1;
   float2* tw = s + kColTile * ld;
   const int tiles = Ns / kColTile;
   const int v = blockIdx.x / tiles, k0 = (blockIdx.x - v * tiles) * kColTile;
@@ -58,27 +72,13 @@ __global__ void k_fft_cols(float2* __restrict__ x, int C, int logc, int Ns, floa
   fill_twiddles(tw, C, sign, blockDim.x, threadIdx.x);
   for (int i = threadIdx.x; i < C * kColTile; i += blockDim.x) {
     const int c = i / kColTile, kk = i - c * kColTile;
-    s[kk * ld + bitrev(c, logc)] = base[(size_t)c * Ns + kk];
+    s[kk * ld + slot(bitrev(c, logc))] = base[(size_t)c * Ns + kk];
   }
   __syncthreads();
-  const int hc = C >> 1;
-  for (int m = 1; m <= logc; ++m) {
-    const int half = 1 << (m - 1);
-    for (int u = threadIdx.x; u < kColTile * hc; u += blockDim.x) {
-      const int col = u >> (logc - 1), w = u & (hc - 1);
-      const int j = w & (half - 1);
-      float2* sc = s + col * ld;
-      const int i0 = ((w >> (m - 1)) << m) + j, i1 = i0 + half;
-      const float2 t = cmul(sc[i1], tw[j << (logc - m)]);
-      const float2 a = sc[i0];
-      sc[i0] = make_float2(a.x + t.x, a.y + t.y);
-      sc[i1] = make_float2(a.x - t.x, a.y - t.y);
-    }
-    __syncthreads();
-  }
+  smem_fft_rows<true>(s, ld, kLogColTile, tw, logc, blockDim.x, threadIdx.x);
   for (int i = threadIdx.x; i < C * kColTile; i += blockDim.x) {
     const int c = i / kColTile, kk = i - c * kColTile;
-    base[(size_t)c * Ns + kk] = s[kk * ld + c];
+    base[(size_t)c * Ns + kk] = s[kk * ld + slot(c)];
   }
 }
 
@@ -948,21 +948,27 @@ void launch_angle_bwd(const float2* X, const Steer& xl, const float* dpw, const 
   k_angle_bwd<APT><<<grid, 256, sm, st>>>(X, xl, dpw, fs, V, C, Ns, dX);
 }
 
-cudaError_t fft_rows(const float2* in, float2* out, int rows, int n, float sign, cudaStream_t st) {
-  const int threads = n / 2 < 256 ? (n / 2 < 32 ? 32 : n / 2) : 256;
-  const size_t sm = sizeof(float2) * (n + n / 2);
+// Eight points per thread: as many short rows per CTA as 256 threads hold (32 to 256
+// threads measured the same within 0.2 us).
+constexpr int kRowThreads = 256;
+cudaError_t fft_rows(const float2* in, float2* out, int rows, int n, float sign, cudaStream_t st,
+                     unsigned long long* clear = nullptr) {
+  const int threads = n <= 8 * kRowThreads ? kRowThreads : n / 8, logn = ilog2(n);
+  int logb = ilog2(threads * 8 / n);
+  while (logb > 0 && (1 << (logb - 1)) >= rows) --logb;  // no more than the rows there are
+  const size_t sm = sizeof(float2) * ((size_t)(slots(n) << logb) + slots(n / 2));
   if (sm > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(k_fft_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
   }
   ::sbr::note_launch();
-  k_fft_rows<<<rows, threads, sm, st>>>(in, out, n, ilog2(n), sign);
+  k_fft_rows<<<(rows + (1 << logb) - 1) >> logb, threads, sm, st>>>(in, out, rows, logn, logb, sign, clear);
   return cudaGetLastError();
 }
 
 cudaError_t fft_cols(float2* x, int V, int C, int Ns, float sign, cudaStream_t st) {
   if (C == 1) return cudaSuccess;
-  const size_t sm = sizeof(float2) * ((size_t)(C + 1) * kColTile + C / 2);
+  const size_t sm = sizeof(float2) * ((size_t)(slots(C) | 1) * kColTile + slots(C / 2));
   if (sm > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(k_fft_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
@@ -1035,10 +1041,10 @@ sbr_status power_map_impl(const float* d_cube, const sbr_radar_cfg* radar, const
   const int cells = R * Ns;
   const Steer xl = steering_table(radar, cfar);
   // 1-2: range FFT over samples, Doppler FFT over chirps
-  SBR_CUDA(fft_rows(reinterpret_cast<const float2*>(d_cube), L.spec, V * C, Ns, -1.f, st));
+  SBR_CUDA(fft_rows(reinterpret_cast<const float2*>(d_cube), L.spec, V * C, Ns, -1.f, st, L.amax_key));
   SBR_CUDA(fft_cols(L.spec, V, C, Ns, -1.f, st));
-  // 3-4: angle DFT and power map (partials per Doppler group, fixed-order sum)
-  SBR_CUDA(cudaMemsetAsync(L.amax_key, 0, 2 * sizeof(unsigned long long), st));
+  // 3-4: angle DFT and power map (partials per Doppler group, fixed-order sum; the
+  // argmax key and the error word were zeroed by the first transform)
   if (angle_tc_ok(R, V, Ns)) {
     SBR_CUDA(angle_tc_attr());
     ::sbr::note_launch();

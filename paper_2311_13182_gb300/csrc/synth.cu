@@ -782,12 +782,12 @@ __global__ void __launch_bounds__(kNuFinThreads) k_nufft_finish(const float2* __
                                                                 float2* __restrict__ bsum,
                                                                 unsigned int* __restrict__ cnt,
                                                                 float2* __restrict__ cube, int C, bool moving) {
-  extern __shared__ float2 sg[];  // [M] grid, [M / 2] twiddles, [kNuFinThreads] per-thread sums
+  extern __shared__ float2 sg[];  // slots(M) grid, slots(M / 2) twiddles, [kNuFinThreads] per-thread sums
   __shared__ int s_last;
   const int log_m = na.log_m, M = 1 << log_m, slice = M < kNuFinSlice ? M : kNuFinSlice, S = M / slice;
   const int row = blockIdx.x / S, sl = blockIdx.x - row * S, rows = na.V * na.chirps, Q = na.Q;
-  float2* tw = sg + M;
-  float2* part = tw + M / 2;
+  float2* tw = sg + fft::slots(M);
+  float2* part = tw + fft::slots(M / 2);
   const int parts = blockDim.x / slice, li = threadIdx.x % slice, k0 = threadIdx.x / slice;
   const int l = sl * slice + li;
   float2 a0 = make_float2(0.f, 0.f), a1 = a0, a2 = a0, a3 = a0;
@@ -828,7 +828,7 @@ __global__ void __launch_bounds__(kNuFinThreads) k_nufft_finish(const float2* __
   if (!s_last) return;
   __threadfence();
   fft::fill_twiddles(tw, M, 1.f, blockDim.x, threadIdx.x);
-  for (int i = threadIdx.x; i < M; i += blockDim.x) sg[fft::bitrev(i, log_m)] = __ldcg(&bsum[(size_t)row * M + i]);
+  for (int i = threadIdx.x; i < M; i += blockDim.x) sg[fft::slot(fft::bitrev(i, log_m))] = __ldcg(&bsum[(size_t)row * M + i]);
   __syncthreads();
   fft::smem_fft(sg, tw, log_m, blockDim.x, threadIdx.x);
   const int Ns = M >> 1, h = Ns >> 1;
@@ -840,7 +840,7 @@ __global__ void __launch_bounds__(kNuFinThreads) k_nufft_finish(const float2* __
     float inv = co.inv[8];
 #pragma unroll
     for (int k = 7; k >= 0; --k) inv = fmaf(inv, y, co.inv[k]);
-    const float2 B = sg[(n - h) & (M - 1)];
+    const float2 B = sg[fft::slot((n - h) & (M - 1))];
     const float2 val = make_float2(B.x * inv, B.y * inv);
     for (int c = c0; c < c1; ++c) cube[((size_t)v * C + c) * Ns + n] = val;
   }
@@ -929,11 +929,11 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_grid(const float2* __restri
                                                           float2* __restrict__ out) {
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
-  extern __shared__ float2 sa[];  // [N_s] this CTA's chirps summed, [M] grid, [M / 2] twiddles
+  extern __shared__ float2 sa[];  // [N_s] this CTA's chirps summed, slots(M) grid, slots(M / 2) twiddles
   const int M = 1 << log_m, rank = (int)cluster.block_rank(), ranks = (int)cluster.num_blocks();
   const int v = blockIdx.x / ranks, h = Ns >> 1;
   float2* s = sa + Ns;
-  float2* tw = s + M;
+  float2* tw = s + fft::slots(M);
   const int c0 = C * rank / ranks, c1 = C * (rank + 1) / ranks;
   for (int n = threadIdx.x; n < Ns; n += kAdjThreads) {
     float2 a = make_float2(0.f, 0.f);
@@ -947,7 +947,7 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_grid(const float2* __restri
   }
   if (rank < 2) {
     fft::fill_twiddles(tw, M, 1.f, kAdjThreads, threadIdx.x);
-    for (int i = threadIdx.x; i < M; i += kAdjThreads) s[i] = make_float2(0.f, 0.f);
+    for (int i = threadIdx.x; i < fft::slots(M); i += kAdjThreads) s[i] = make_float2(0.f, 0.f);
   }
   cluster.sync();
   if (rank < 2) {
@@ -963,12 +963,12 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_grid(const float2* __restri
 #pragma unroll
       for (int k = 7; k >= 0; --k) w = fmaf(w, y, co.inv[k]);
       if (rank == 1) w *= fmaf((float)n, slope, 1.f);
-      s[fft::bitrev((n - h) & (M - 1), log_m)] = make_float2(a.x * w, -a.y * w);
+      s[fft::slot(fft::bitrev((n - h) & (M - 1), log_m))] = make_float2(a.x * w, -a.y * w);
     }
     __syncthreads();
     fft::smem_fft(s, tw, log_m, kAdjThreads, threadIdx.x);
     float2* o = out + 2 * (size_t)v * (M + kAdjMargin) + rank;
-    for (int i = threadIdx.x; i < M + kAdjMargin; i += kAdjThreads) o[2 * i] = s[(i - (kNuW / 2 - 1)) & (M - 1)];
+    for (int i = threadIdx.x; i < M + kAdjMargin; i += kAdjThreads) o[2 * i] = s[fft::slot((i - (kNuW / 2 - 1)) & (M - 1))];
   }
   cluster.sync();  // no CTA leaves while another may read its shared memory
 }
@@ -1025,7 +1025,7 @@ __global__ void __launch_bounds__(256) k_synth_bwd_nufft(const float4* __restric
   }
 }
 
-inline size_t adj_smem(int Ns) { return sizeof(float2) * 4 * (size_t)Ns; }
+inline size_t adj_smem(int Ns) { return sizeof(float2) * (size_t)(Ns + fft::slots(2 * Ns) + fft::slots(Ns)); }
 
 cudaError_t adj_attr(int Ns) {
   static std::atomic<uint64_t> done{0};  // bit per device ordinal below 64
@@ -1147,7 +1147,7 @@ void grid_shape(int V, int Ns, int64_t cap, int* Q) {
 
 // dynamic shared memory of the spreading kernel: the grid's copies and its sums
 inline size_t nufft_smem(int Ns) { return (2 * kNuCopies * sizeof(int) + 2 * sizeof(float)) * (size_t)nu_points(2 * Ns); }
-inline size_t nufft_fin_smem(int Ns) { return sizeof(float2) * (3 * (size_t)Ns + kNuFinThreads); }
+inline size_t nufft_fin_smem(int Ns) { return sizeof(float2) * (size_t)(fft::slots(2 * Ns) + fft::slots(Ns) + kNuFinThreads); }
 
 // Grids of up to 512 points take 71 KB: three CTAs of 256 threads per SM; larger ones
 // (a block of 1024 cells takes 141 KB) one CTA of 1024.
