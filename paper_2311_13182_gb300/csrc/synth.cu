@@ -1210,8 +1210,8 @@ size_t ws_layout(const sbr_radar_cfg* radar, int64_t cap, int* Q, int* Qn = null
   c.take<float2>((size_t)V * (*Q) * Ns);       // per-CTA partial sums
   c.take<float2>((size_t)V * Ns);              // chirp-summed upstream gradient
   c.take<float2>((size_t)V * qn * 2 * Ns);     // non-uniform FFT: the CTAs' grids
-  c.take<float2>((size_t)V * 2 * Ns);          // non-uniform FFT: the summed grids
-  c.take<unsigned int>((size_t)V);             // non-uniform FFT: finishing counters
+  c.take<float2>((size_t)V * qn * 2 * Ns);     // non-uniform FFT: the rows' summed grids (a moving scene: V * chirps)
+  c.take<unsigned int>((size_t)V * qn);        // non-uniform FFT: finishing counters
   c.take<float4>((size_t)V * (2 * Ns + kAdjMargin));  // adjoint: the antennas' grids
   return c.bytes();
 }
@@ -1252,8 +1252,8 @@ sbr_status bind_ws(const sbr_radar_cfg* radar, int64_t cap, void* ws, size_t byt
   w->partial = c.take<float2>((size_t)V * Q * Ns);
   w->gsum = c.take<float2>((size_t)V * Ns);
   w->grids = c.take<float2>((size_t)V * Qn * 2 * Ns);
-  w->bsum = c.take<float2>((size_t)V * 2 * Ns);
-  w->fin_cnt = c.take<unsigned int>((size_t)V);
+  w->bsum = c.take<float2>((size_t)V * Qn * 2 * Ns);
+  w->fin_cnt = c.take<unsigned int>((size_t)V * Qn);
   w->adj = c.take<float4>((size_t)V * (2 * Ns + kAdjMargin));
   w->Q = Q;
   w->Qn = Qn;
@@ -1261,9 +1261,10 @@ sbr_status bind_ws(const sbr_radar_cfg* radar, int64_t cap, void* ws, size_t byt
 }
 
 // The non-uniform FFT of chirps [c0, c0 + chirps) of a moving scene, or of a static
-// scene's one chirp, written to all of them: spread, then finish.
-void launch_nufft(sbr_phase_mode mode, const sbr_paths* p, const sbr_radar_cfg* r, const SynthWs& w, bool moving, int c0,
-                  int chirps, float2* cube, cudaStream_t st) {
+// scene's one chirp, written to all of them: spread by Q CTAs per antenna and chirp
+// (Q * chirps <= w.Qn), then finish.
+void launch_nufft(sbr_phase_mode mode, const sbr_paths* p, const sbr_radar_cfg* r, const SynthWs& w, bool moving, int Q,
+                  int c0, int chirps, float2* cube, cudaStream_t st) {
   const int V = p->n_virt, Ns = r->n_samples, M = 2 * Ns;
   NufftArg na{};
   while ((1 << na.log_m) < M) ++na.log_m;
@@ -1273,7 +1274,7 @@ void launch_nufft(sbr_phase_mode mode, const sbr_paths* p, const sbr_radar_cfg* 
   na.b_cn = r->bandwidth / (kC * Ns);
   na.m_d = (double)M;
   na.V = V;
-  na.Q = w.Qn;
+  na.Q = Q;
   na.chirps = chirps;
   na.chirp0 = c0;
   na.per_chirp = r->chirp_rep;
@@ -1281,7 +1282,7 @@ void launch_nufft(sbr_phase_mode mode, const sbr_paths* p, const sbr_radar_cfg* 
   const NufftCoef& co = nufft_coef();
   const float4* prep = reinterpret_cast<const float4*>(p->prep);
   const float2* plen = reinterpret_cast<const float2*>(p->path_len);
-  const int grid = V * w.Qn * chirps;
+  const int grid = V * Q * chirps;
   ::sbr::note_launch();
   nufft_kernel(Ns, mode == SBR_PHASE_FP64, moving)<<<grid, nufft_threads(Ns), nufft_smem(Ns), st>>>(
       prep, plen, p->phase_ofs, p->path_rate, p->path_cap, p->count, na, co, w.grids, w.fin_cnt);
@@ -1292,11 +1293,29 @@ void launch_nufft(sbr_phase_mode mode, const sbr_paths* p, const sbr_radar_cfg* 
 }
 
 // A moving scene: every chirp synthesised from its own delays (split phase up to 512
-// samples, or the FP64 phase), chirp by chirp.
+// samples, or the FP64 phase), a group of chirps per launch.  A launch is one wave of
+// Q CTAs per antenna and chirp; fewer CTAs per chirp mean fewer launches and the same
+// records per CTA in all, so Q is the one whose launches / Q, the chirps' share of a
+// wave each, is least (12 antennas x 128 chirps: 2 CTAs each, 7 launches of 19 chirps,
+// 3.5 against the ideal 3.4; the records are then read from L2 by the chirps of a
+// launch).  One launch pair per chirp took 7.85 ms for 12 x 367,500 records x 128
+// chirps, groups took 6.3 ms.
 sbr_status launch_moving(sbr_phase_mode mode, const sbr_paths* p, const sbr_radar_cfg* r, const SynthWs& w,
                          float2* cube, cudaStream_t st) {
   if (mode == SBR_PHASE_FP64 || (mode == SBR_PHASE_SPLIT && r->n_samples <= kNuMovingMaxSamples)) {
-    for (int c = 0; c < r->n_chirps; ++c) launch_nufft(mode, p, r, w, true, c, 1, cube, st);
+    const int C = r->n_chirps;
+    int best = 1, group = 1;
+    double cost = 1e30;
+    for (int q = 1; q <= w.Qn; ++q) {
+      const int most = std::min(C, w.Qn / q), launches = (C + most - 1) / most;
+      if (launches < cost * q) {
+        cost = (double)launches / q;
+        best = q;
+        group = (C + launches - 1) / launches;
+      }
+    }
+    for (int c = 0; c < C; c += group)
+      launch_nufft(mode, p, r, w, true, best, c, std::min(group, C - c), cube, st);
     return SBR_OK;
   }
   set_error("sbr_synthesize: SBR_SYNTH_MOVING supports SBR_PHASE_SPLIT up to %d samples and SBR_PHASE_FP64",
@@ -1356,7 +1375,7 @@ extern "C" sbr_status sbr_synthesize(const sbr_paths* paths, const sbr_radar_cfg
     return SBR_OK;
   }
   if (nufft_for(mode, Ns, paths->path_cap * paths->n_virt)) {
-    launch_nufft(mode, paths, radar, w, false, 0, 1, reinterpret_cast<float2*>(d_cube), st);
+    launch_nufft(mode, paths, radar, w, false, w.Qn, 0, 1, reinterpret_cast<float2*>(d_cube), st);
     SBR_CUDA(cudaGetLastError());
     return SBR_OK;
   }
