@@ -538,31 +538,44 @@ __global__ void __launch_bounds__(256) k_synth_bwd(const float4* __restrict__ pr
 // while the upper adds imaginary parts (then the other way round), so the 32
 // lanes of an atomic always hit 32 different banks, whatever the cells are:
 // neighbouring rays share cells, and consecutive records jump between a ray's
-// bounces.  A term is rounded to 2^-24 of the chunk's largest amplitude, so that a chunk's additions to one copy stay below
-// 2^31; after each chunk the copies of the touched cells (a flag per eight
-// cells) are summed, scaled and added to the CTA's FP32 grid, each point by one
-// thread.  The CTAs' grids are added in a fixed order by the finishing kernel.
+// bounces.  A term is rounded to 2^-24 of the chunk's largest amplitude, so that
+// a chunk's additions to one copy stay below 2^30; after each chunk the copies of
+// the touched cells (a flag per eight cells) are summed, scaled and added to the
+// CTA's FP32 grid, each point by one thread.  The CTAs' grids are added in a fixed
+// order by the finishing kernel.
 //
-// Bound by issue slots (58 % active) and the chunks' barriers.  12 antennas x
-// 367,500 records x 256 samples: 49 us against 109 us for sums kept in registers
-// per run of equal cells (8 lanes a record, each warp its own FP32 grid), which a
-// changing cell flushes one group at a time; 93 us for the same with the chunk
-// first sorted by cell.  Error against FP64 over the same records 2e-7 (1.3e-6 with
-// the approximate sine, square root and exponential of the former kernel).
-constexpr int kNuW = 8;         // kernel width in grid points
-constexpr int kNuCopies = 16;   // copies of a grid word
-constexpr int kNuBlock = 1024;  // cells a CTA's grid holds at once; larger grids block by block
+// A CTA has a barrier for a chunk's maximum and one before its sums are added up;
+// the next chunk's records are in flight meanwhile, and its preparation needs none.
+// Bound by issue slots (212 instructions per 32 records) and the conversion unit,
+// three CTAs per SM: 12 antennas x 367,500 records x 256 samples 35 us (109 us when
+// each warp kept runs of equal cells in registers, eight lanes to a record, and
+// flushed them to its own FP32 grid, one group at a time; 93 us with the chunk sorted
+// by cell first), 71 MB of records at 2 TB/s.  A block of 512 cells, so that long
+// chirps keep three CTAs per SM too: 4 antennas x 3.1 M records x 4096 samples 250 ->
+// 124 us against a block of 1024 in one CTA of 1024 threads.  Error against FP64 over
+// the same records 2e-7 (1.3e-6 with the former kernel's approximate sine, square root
+// and exponential).
+constexpr int kNuW = 8;        // kernel width in grid points
+constexpr int kNuCopies = 16;  // copies of a grid word
+constexpr int kNuBlock = 512;  // cells a CTA's grid holds at once (71 KB: three CTAs per SM); larger grids block by block
+constexpr int kNuThreads = 256;
+constexpr int kNuItems = 4;    // records per thread and chunk
+constexpr int kNuChunk = kNuThreads * kNuItems;
+constexpr int kNuBits = 24;    // 2 kNuChunk / 32 additions per copy of terms up to 0.98 2^24: below 2^30
+static_assert(kNuChunk / kNuCopies <= 1 << (30 - kNuBits), "a chunk's additions to one copy");
 constexpr double kNuBeta = 2.3 * kNuW;
 
 struct NufftCoef {
-  float e[4][5], o[4][4];  // psi((j - 7/2) - s) = sum_k e[j][k] s^(2k) + s sum_k o[j][k] s^(2k), j < 4, |s| <= 1/2
-  float inv[9];            // 1 / Psi(n'/M) = sum_k inv[k] (2 n' / N_s)^(2k)
+  // psi((j - 7/2) - s) = sum_k e[k][j] s^(2k) + s sum_k o[k][j] s^(2k), j < 4, |s| <= 1/2
+  float e[5][4], o[4][4];
+  float inv[9];  // 1 / Psi(n'/M) = sum_k inv[k] (2 n' / N_s)^(2k)
 };
 
 struct NufftArg {
   int log_m;
   float half_n, m;           // N_s / 2, M = 2 N_s
-  double f0_c, b_cn, m_d;    // FP64 phase: f_c / c and B / (c N_s) per metre, M
+  double cyc, cell;          // FP64 phase: carrier cycles at n' = 0 and grid cells per metre of path
+  double f0_c, b_cn;         // f_c / c and B / (c N_s) per metre
   int V, Q, chirps, chirp0;  // antennas, CTAs per antenna and chirp, chirps of this launch, the first of them
   double per_chirp;          // moving scenes: change of path length per chirp per (m/s) of dL/dt
 };
@@ -572,35 +585,66 @@ struct NufftArg {
 __host__ __device__ constexpr int nu_cells(int M) { return M < kNuBlock ? M : kNuBlock; }
 __host__ __device__ constexpr int nu_points(int M) { return nu_cells(M) + kNuW; }
 
-// x such that `adds` terms of at most 2^x (and rounding) sum to less than 2^31.
-constexpr int nu_term_bits(int adds) { return adds <= 1 ? 30 : nu_term_bits((adds + 1) / 2) - 1; }
+// The eight weights psi((j - 7/2) - s): left[j] of point j and right[j] of point 7 - j,
+// j < 4, two points per packed FMA.
+__device__ __forceinline__ void nu_weights(const NufftCoef& co, float s, float (&left)[4], float (&right)[4]) {
+  const float2 s2 = make_float2(s * s, s * s), ss = make_float2(s, s);
+#pragma unroll
+  for (int j = 0; j < 4; j += 2) {
+    float2 E = make_float2(co.e[4][j], co.e[4][j + 1]), O = make_float2(co.o[3][j], co.o[3][j + 1]);
+#pragma unroll
+    for (int k = 3; k >= 0; --k) E = __ffma2_rn(E, s2, make_float2(co.e[k][j], co.e[k][j + 1]));
+#pragma unroll
+    for (int k = 2; k >= 0; --k) O = __ffma2_rn(O, s2, make_float2(co.o[k][j], co.o[k][j + 1]));
+    O = __fmul2_rn(O, ss);
+    left[j] = E.x + O.x;
+    left[j + 1] = E.y + O.y;
+    right[j] = E.x - O.x;
+    right[j + 1] = E.y - O.y;
+  }
+}
+
+// c w rounded to an integer.  Below 2^22 (the outer points: psi <= 0.085 from two
+// grid steps on) by one FMA against 1.5 2^23 and the bits' difference, which leaves
+// the conversion unit, a quarter of the FMA pipe's rate, to the inner points.
+constexpr int kNuSmall = 2;  // outer points on either side
+__device__ __forceinline__ int nu_term(float c, float w, bool small) {
+  return small ? __float_as_int(fmaf(c, w, 12582912.f)) - 0x4B400000 : __float2int_rn(c * w);
+}
+
+// x = rint(x) + the returned fraction in [-1/2, 1/2], |x| < 2^50; n gets rint(x) mod 2^32.
+__device__ __forceinline__ double split_rint(double x, int& n) {
+  const double k = x + 6755399441055744.0;  // 1.5 2^52: the integer in the low word
+  n = __double2loint(k);
+  return x - (k - 6755399441055744.0);
+}
 
 // CTA (q, v, chirp) spreads its share of antenna v's records, P/Q consecutive
-// ones.  Writes the CTA's grid, grids[CTA][l].
-template <bool kFp64, bool kMoving, int kThreads, int kItems>
-__global__ void __launch_bounds__(kThreads, kThreads == 256 ? 3 : 1)
+// ones.  Writes the CTA's grid, grids[CTA][l].  kBlocks: M > kNuBlock.
+template <bool kFp64, bool kMoving, bool kBlocks>
+__global__ void __launch_bounds__(kNuThreads, 3)
     k_nufft_spread(const float4* __restrict__ prep, const float2* __restrict__ plen, const float* __restrict__ phase_ofs,
                    const float* __restrict__ rate, int64_t cap, const int32_t* __restrict__ d_P, const NufftArg na,
                    const __grid_constant__ NufftCoef co, float2* __restrict__ grids, unsigned int* __restrict__ fin_cnt) {
-  constexpr int kChunk = kThreads * kItems, kBits = nu_term_bits(kChunk / kNuCopies);
   extern __shared__ int4 nsm[];
-  __shared__ uint32_t wmax[kThreads / 32], wblk[kThreads / 32];
-  __shared__ int flag[kNuBlock / 8 + 2];  // flag[1 + o]: a record of cells 8 o .. 8 o + 7 in this chunk
+  __shared__ uint32_t s_max[2], s_blk[2];     // by the parity of the chunk
+  __shared__ int flag[2][kNuBlock / 8];       // by the parity of the pass: a record of cells 8 o .. 8 o + 7
   const int M = 1 << na.log_m, bs = nu_cells(M), npts = nu_points(M);
   int* grid = reinterpret_cast<int*>(nsm);                            // [npts][re, im][kNuCopies]
   float* sum = reinterpret_cast<float*>(grid + npts * 2 * kNuCopies); // [npts][re, im]: finished chunks
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31;
   if (blockIdx.x == 0)
-    for (int i = tid; i < na.V * na.chirps; i += kThreads) fin_cnt[i] = 0u;  // the finishing kernel's counters
+    for (int i = tid; i < na.V * na.chirps; i += kNuThreads) fin_cnt[i] = 0u;  // the finishing kernel's counters
   const int cl = blockIdx.x % na.chirps, v = (blockIdx.x / na.chirps) % na.V, q = blockIdx.x / (na.chirps * na.V);
   const double dt = kMoving ? (double)(na.chirp0 + cl) * na.per_chirp : 0.0;  // path length change per (m/s)
   const float cnu = (float)(dt * na.f0_c), ceps = (float)(dt * na.b_cn);
   float2* out = grids + (size_t)blockIdx.x * M;
-  for (int i = tid; i < npts * (2 * kNuCopies / 4); i += kThreads) nsm[i] = make_int4(0, 0, 0, 0);
-  for (int i = tid; i < 2 * npts; i += kThreads) sum[i] = 0.f;
-  for (int i = tid; i < kNuBlock / 8 + 2; i += kThreads) flag[i] = 0;
-  if (M > bs)
-    for (int i = tid; i < M; i += kThreads) out[i] = make_float2(0.f, 0.f);
+  for (int i = tid; i < npts * (2 * kNuCopies / 4); i += kNuThreads) nsm[i] = make_int4(0, 0, 0, 0);
+  for (int i = tid; i < 2 * npts; i += kNuThreads) sum[i] = 0.f;
+  for (int i = tid; i < 2 * (kNuBlock / 8); i += kNuThreads) (&flag[0][0])[i] = 0;
+  if (tid < 2) s_max[tid] = s_blk[tid] = 0u;
+  if (kBlocks)
+    for (int i = tid; i < M; i += kNuThreads) out[i] = make_float2(0.f, 0.f);
   const int64_t P = *d_P;
   const int64_t r0 = P * q / na.Q;
   const int n = (int)(P * (q + 1) / na.Q - r0);
@@ -609,48 +653,49 @@ __global__ void __launch_bounds__(kThreads, kThreads == 256 ? 3 : 1)
   const bool upper = lane >= 16;
   int* mine = grid + (lane & 15);
   int blk = 0;       // block of cells the grid holds
+  int pass = 0;      // passes so far (a chunk has one per block of cells it touches)
   bool bad = false;  // a record that is not finite: the antenna's samples are NaN
   // the finished sums of block blk into the CTA's output (several blocks only)
   auto store_block = [&]() {
-    for (int i = tid; i < npts; i += kThreads) {
+    for (int i = tid; i < npts; i += kNuThreads) {
       float2* o = out + ((blk * bs + i - (kNuW / 2 - 1)) & (M - 1));
       *o = make_float2(o->x + sum[2 * i], o->y + sum[2 * i + 1]);
       sum[2 * i] = sum[2 * i + 1] = 0.f;
     }
   };
-  __syncthreads();
-  for (int c0 = 0; c0 < n; c0 += kChunk) {
-    float4 rec[kItems];  // c re, c im over A, s, A
-    int cell[kItems];
-    uint32_t am = 0, blocks = 0;
+  float4 rec[kNuItems];  // a chunk's records; then cos, sin of the carrier phase at n' = 0, s, A
+  auto load = [&](int c0) {
 #pragma unroll
-    for (int u = 0; u < kItems; ++u) {
-      const int p = c0 + tid + u * kThreads;
+    for (int u = 0; u < kNuItems; ++u) {
+      const int p = c0 + tid + u * kNuThreads;
       rec[u] = p < n ? __ldg(&pv[p]) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
+  };
+  load(0);
+  __syncthreads();
+  for (int c0 = 0, chunk = 0; c0 < n; c0 += kNuChunk, ++chunk) {
+    int cell[kNuItems];
+    uint32_t am = 0, blocks = 0;
 #pragma unroll
-    for (int u = 0; u < kItems; ++u) {
-      const int p = c0 + tid + u * kThreads;
+    for (int u = 0; u < kNuItems; ++u) {
+      const int p = c0 + tid + u * kNuThreads;
       float4 r = rec[u];
-      float x, t, fl;
+      float x, t;
       int ce;
       if (kFp64) {
         float2 L2 = make_float2(0.f, 0.f);
-        double L = 0.0, po = 0.0;
+        float po = 0.f, ld = 0.f;
         if (p < n) {
           L2 = __ldg(&plen[at + p]);
-          po = (double)__ldg(&phase_ofs[r0 + p]);
-          if (kMoving) L = dt * (double)__ldg(&rate[at + p]);
+          po = __ldg(&phase_ofs[r0 + p]);
+          if (kMoving) ld = __ldg(&rate[at + p]);
         }
-        L += (double)L2.x + (double)L2.y;
-        double d = na.b_cn * L;
-        d -= rint(d);
-        double ph = fma((double)na.half_n, d, na.f0_c * L + po);
-        ph -= rint(ph);
-        x = (float)ph;
-        const double ud = na.m_d * d, fd = floor(ud);
-        t = (float)(ud - fd);
-        ce = (int)fd;
+        double L = (double)L2.x + (double)L2.y;
+        if (kMoving) L = fma(dt, (double)ld, L);
+        int whole;
+        x = (float)split_rint(na.cyc * L, whole) + po;
+        t = (float)split_rint(fma(na.cell, L, -0.5), ce);  // the cell is rint(u - 1/2), s the rest
+        bad |= !isfinite(x + t + r.w);
       } else {
         if (kMoving) {
           // phi0 + dL/dt cnu and delta + dL/dt ceps, whole multiples of 2^-12 of the delta
@@ -666,94 +711,96 @@ __global__ void __launch_bounds__(kThreads, kThreads == 256 ? 3 : 1)
         x -= rintf(x);
         x = fmaf(na.half_n, r.z, x) + r.x;
         const float uh = na.m * r.y;  // exact
-        fl = floorf(uh);
+        float fl = floorf(uh);
         t = fmaf(na.m, r.z, uh - fl);
         ce = (int)fl;
+        bad |= !isfinite(x + t + r.w);
+        fl = floorf(t);
+        t = (t - fl) - 0.5f;
+        ce += (int)fl;
       }
-      bad |= !isfinite(x + t + r.w);
-      fl = floorf(t);
-      t -= fl;
-      ce = (ce + (int)fl) & (M - 1);
+      ce &= M - 1;
       float sn, cs;
       sincospif(2.f * x, &sn, &cs);
-      rec[u] = make_float4(cs, sn, t - 0.5f, r.w);
+      rec[u] = make_float4(cs, sn, t, r.w);
       cell[u] = ce;
       am = max(am, __float_as_uint(fabsf(r.w)));
-      if (p < n) blocks |= 1u << (ce / kNuBlock);
+      if (kBlocks && p < n) blocks |= 1u << (ce / kNuBlock);
     }
     am = __reduce_max_sync(0xffffffffu, am);
-    blocks = __reduce_or_sync(0xffffffffu, blocks);
+    if (kBlocks) blocks = __reduce_or_sync(0xffffffffu, blocks);
     if (lane == 0) {
-      wmax[warp] = am;
-      wblk[warp] = blocks;
+      atomicMax(&s_max[chunk & 1], am);
+      if (kBlocks) atomicOr(&s_blk[chunk & 1], blocks);
     }
-    __syncthreads();
-    am = wmax[0];
-    blocks = wblk[0];
-#pragma unroll
-    for (int w = 1; w < kThreads / 32; ++w) {
-      am = max(am, wmax[w]);
-      blocks |= wblk[w];
-    }
-    const float top = fmaxf(__uint_as_float(am), 1e-20f);  // terms up to 2^kBits
-    const float scale = (float)(1 << kBits) / top, unit = top * (1.f / (float)(1 << kBits));
+    __syncthreads();  // the chunk's maximum; the previous chunk is added up
+    const float top = fmaxf(__uint_as_float(s_max[chunk & 1]), 1e-20f);  // terms up to 0.98 2^kNuBits
+    const float scale = 0.98f * (float)(1 << kNuBits) / top, unit = top * (1.f / (0.98f * (float)(1 << kNuBits)));
+    blocks = kBlocks ? s_blk[chunk & 1] : 1u;
     while (blocks) {
-      const int b = __ffs(blocks) - 1;
+      const int b = kBlocks ? __ffs(blocks) - 1 : 0;
       blocks &= blocks - 1;
-      if (b != blk) {  // the same for the whole CTA; sum is complete (the barrier after each chunk's addition)
+      if (kBlocks && b != blk) {  // the same for the whole CTA
         store_block();
         blk = b;
         __syncthreads();
       }
+      int* fl = flag[pass & 1];
+      // read before this pass: the other parity's flags, the previous chunk's maximum
+      if (tid < kNuBlock / 8) flag[~pass & 1][tid] = 0;
+      if (tid == 0) s_max[~chunk & 1] = s_blk[~chunk & 1] = 0u;
 #pragma unroll
-      for (int u = 0; u < kItems; ++u) {
-        const int idx = cell[u] - b * bs;
-        if ((unsigned)idx >= (unsigned)bs || rec[u].w == 0.f) continue;
-        const float s = rec[u].z, s2 = s * s, a = rec[u].w * scale;
+      for (int u = 0; u < kNuItems; ++u) {
+        const int idx = kBlocks ? cell[u] - b * bs : cell[u];
+        if ((kBlocks && (unsigned)idx >= (unsigned)bs) || rec[u].w == 0.f) continue;
+        const float a = rec[u].w * scale;
         const float c1 = a * (upper ? rec[u].y : rec[u].x), c2 = a * (upper ? rec[u].x : rec[u].y);
         int* g1 = mine + idx * (2 * kNuCopies) + (upper ? kNuCopies : 0);
         int* g2 = mine + idx * (2 * kNuCopies) + (upper ? 0 : kNuCopies);
-        flag[1 + (idx >> 3)] = 1;
+        fl[idx >> 3] = 1;
+        float wl[4], wr[4];
+        nu_weights(co, rec[u].z, wl, wr);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          float E = co.e[j][4], O = co.o[j][3];
-#pragma unroll
-          for (int k = 3; k >= 0; --k) E = fmaf(E, s2, co.e[j][k]);
-#pragma unroll
-          for (int k = 2; k >= 0; --k) O = fmaf(O, s2, co.o[j][k]);
-          const float pl = fmaf(O, s, E), pr = fmaf(-O, s, E);  // points j and 7 - j
-          atomicAdd(g1 + j * (2 * kNuCopies), __float2int_rn(c1 * pl));
-          atomicAdd(g2 + j * (2 * kNuCopies), __float2int_rn(c2 * pl));
-          atomicAdd(g1 + (7 - j) * (2 * kNuCopies), __float2int_rn(c1 * pr));
-          atomicAdd(g2 + (7 - j) * (2 * kNuCopies), __float2int_rn(c2 * pr));
+          atomicAdd(g1 + j * (2 * kNuCopies), nu_term(c1, wl[j], j < kNuSmall));
+          atomicAdd(g2 + j * (2 * kNuCopies), nu_term(c2, wl[j], j < kNuSmall));
+          atomicAdd(g1 + (7 - j) * (2 * kNuCopies), nu_term(c1, wr[j], j < kNuSmall));
+          atomicAdd(g2 + (7 - j) * (2 * kNuCopies), nu_term(c2, wr[j], j < kNuSmall));
         }
       }
+      if (!kBlocks || !blocks) load(c0 + kNuChunk);  // in flight while this chunk is added up
       __syncthreads();
-      // the chunk's sums: point i / 2, part i & 1; its copies' four 16-byte words in an order
-      // that gives the eight lanes of a shared-memory phase different banks
-      for (int i = tid; i < 2 * npts; i += kThreads) {
-        const int o = i >> 4;  // points 8 o .. 8 o + 7 take records of cells of octets o - 1 and o
-        if (!(flag[o] | flag[o + 1])) continue;
+      // Add the chunk up: half-warp h takes the octets of points o = h mod 16, which records
+      // of the cells of octets o - 1 and o reach, one thread per point and part; the copies'
+      // four 16-byte words in an order that gives the lanes of a shared-memory phase
+      // different banks.
+      const unsigned m0 = __ballot_sync(0xffffffffu, fl[lane] != 0), m1 = __ballot_sync(0xffffffffu, fl[32 + lane] != 0);
+      const unsigned long long cells = (unsigned long long)m1 << 32 | m0, lit = cells | cells << 1;
+#pragma unroll
+      for (int r = 0; r < kNuBlock / 8 / 16 + 1; ++r) {
+        const int o = r * 16 + (tid >> 4);
+        const bool on = o < 64 ? (lit >> (o & 63)) & 1ull : o == 64 && (cells >> 63) != 0ull;
+        if (!on) continue;
+        const int i = o * 16 + (tid & 15);  // point i / 2, part i & 1
         long long t = 0;
 #pragma unroll
         for (int k = 0; k < kNuCopies / 4; ++k) {
           const int w = i * (kNuCopies / 4) + ((k + (i >> 1)) & (kNuCopies / 4 - 1));
           const int4 x = nsm[w];
           nsm[w] = make_int4(0, 0, 0, 0);
-          t += (long long)x.x + x.y + ((long long)x.z + x.w);
+          t += (long long)(x.x + x.y) + (long long)(x.z + x.w);
         }
         sum[i] = fmaf((float)t, unit, sum[i]);
       }
-      __syncthreads();
-      for (int i = tid; i < kNuBlock / 8 + 2; i += kThreads) flag[i] = 0;
-      __syncthreads();
+      ++pass;
+      if (kBlocks && blocks) __syncthreads();  // before the next block's additions (else: the next chunk's barrier)
     }
   }
   bad = __syncthreads_or(bad);
-  if (M > bs) {
+  if (kBlocks) {
     store_block();
   } else {  // the points past the grid's end fold back
-    for (int i = tid; i < M; i += kThreads) {
+    for (int i = tid; i < M; i += kNuThreads) {
       float re = sum[2 * i], im = sum[2 * i + 1];
       for (int k = i + M; k < npts; k += M) {
         re += sum[2 * k];
@@ -764,7 +811,7 @@ __global__ void __launch_bounds__(kThreads, kThreads == 256 ? 3 : 1)
   }
   if (bad) {
     __syncthreads();
-    for (int i = tid; i < M; i += kThreads) out[i] = make_float2(NAN, NAN);
+    for (int i = tid; i < M; i += kNuThreads) out[i] = make_float2(NAN, NAN);
   }
 }
 
@@ -883,9 +930,11 @@ NufftCoef make_nufft_coef() {
   NufftCoef c{};
   for (int j = 0; j < 4; ++j) {  // the even and odd parts of psi_j in y = s^2
     const double a = j - 0.5 * (kNuW - 1);
-    fit_poly<4>([&](double y) { return 0.5 * (kb_kernel(a - sqrt(y)) + kb_kernel(a + sqrt(y))); }, 0.25, c.e[j]);
-    fit_poly<3>([&](double y) { return 0.5 * (kb_kernel(a - sqrt(y)) - kb_kernel(a + sqrt(y))) / sqrt(y); }, 0.25,
-                c.o[j]);
+    float e[5], o[4];
+    fit_poly<4>([&](double y) { return 0.5 * (kb_kernel(a - sqrt(y)) + kb_kernel(a + sqrt(y))); }, 0.25, e);
+    fit_poly<3>([&](double y) { return 0.5 * (kb_kernel(a - sqrt(y)) - kb_kernel(a + sqrt(y))) / sqrt(y); }, 0.25, o);
+    for (int k = 0; k < 5; ++k) c.e[k][j] = e[k];
+    for (int k = 0; k < 4; ++k) c.o[k][j] = o[k];
   }
   // Psi(xi) = w / I0(beta) sinh(r) / r, r = sqrt(beta^2 - (pi w xi)^2), real on the band
   // |xi| <= 1/4; its reciprocal in y = (4 xi)^2 = (2 n' / N_s)^2
@@ -998,7 +1047,8 @@ __global__ void __launch_bounds__(256) k_synth_bwd_nufft(const float4* __restric
     fl = floorf(t);
     t -= fl;
     cell = (cell + (int)fl) & (M - 1);
-    const float s = t - 0.5f, s2 = s * s;
+    float wl[4], wr[4];
+    nu_weights(co, t - 0.5f, wl, wr);
     float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
     auto add = [&](float w, float4 q) {
       z.x = fmaf(w, q.x, z.x);
@@ -1008,14 +1058,8 @@ __global__ void __launch_bounds__(256) k_synth_bwd_nufft(const float4* __restric
     };
 #pragma unroll
     for (int j = 0; j < 4; ++j) {  // outermost points first: the smallest weights
-      const float4 ql = __ldg(&gv[cell + j]), qr = __ldg(&gv[cell + 7 - j]);
-      float E = co.e[j][4], O = co.o[j][3];
-#pragma unroll
-      for (int k = 3; k >= 0; --k) E = fmaf(E, s2, co.e[j][k]);
-#pragma unroll
-      for (int k = 2; k >= 0; --k) O = fmaf(O, s2, co.o[j][k]);
-      add(fmaf(O, s, E), ql);
-      add(fmaf(-O, s, E), qr);
+      add(wl[j], __ldg(&gv[cell + j]));
+      add(wr[j], __ldg(&gv[cell + 7 - j]));
     }
     float sn, cs;
     sincospif(2.f * x, &sn, &cs);
@@ -1149,20 +1193,15 @@ void grid_shape(int V, int Ns, int64_t cap, int* Q) {
 inline size_t nufft_smem(int Ns) { return (2 * kNuCopies * sizeof(int) + 2 * sizeof(float)) * (size_t)nu_points(2 * Ns); }
 inline size_t nufft_fin_smem(int Ns) { return sizeof(float2) * (size_t)(fft::slots(2 * Ns) + fft::slots(Ns) + kNuFinThreads); }
 
-// Grids of up to 512 points take 71 KB: three CTAs of 256 threads per SM; larger ones
-// (a block of 1024 cells takes 141 KB) one CTA of 1024.
-inline bool nufft_wide(int Ns) { return 2 * Ns > 512; }
-inline int nufft_threads(int Ns) { return nufft_wide(Ns) ? 1024 : 256; }
-
 using NufftSpread = void (*)(const float4*, const float2*, const float*, const float*, int64_t, const int32_t*, NufftArg,
                              NufftCoef, float2*, unsigned int*);
+template <bool kBlocks>
+NufftSpread nufft_kernel_of(bool fp64, bool moving) {
+  if (fp64) return moving ? k_nufft_spread<true, true, kBlocks> : k_nufft_spread<true, false, kBlocks>;
+  return moving ? k_nufft_spread<false, true, kBlocks> : k_nufft_spread<false, false, kBlocks>;
+}
 inline NufftSpread nufft_kernel(int Ns, bool fp64, bool moving) {
-  if (nufft_wide(Ns)) {
-    if (fp64) return moving ? k_nufft_spread<true, true, 1024, 1> : k_nufft_spread<true, false, 1024, 1>;
-    return moving ? k_nufft_spread<false, true, 1024, 1> : k_nufft_spread<false, false, 1024, 1>;
-  }
-  if (fp64) return moving ? k_nufft_spread<true, true, 256, 4> : k_nufft_spread<true, false, 256, 4>;
-  return moving ? k_nufft_spread<false, true, 256, 4> : k_nufft_spread<false, false, 256, 4>;
+  return 2 * Ns > kNuBlock ? nufft_kernel_of<true>(fp64, moving) : nufft_kernel_of<false>(fp64, moving);
 }
 
 // resident spreading CTAs per SM (shared memory and registers decide); raises
@@ -1179,7 +1218,7 @@ int nufft_per_sm(int Ns) {
     const NufftSpread k = nufft_kernel(Ns, (i & 2) != 0, (i & 1) != 0);
     if (sm > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     int m = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&m, k, nufft_threads(Ns), sm);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&m, k, kNuThreads, sm);
     n = std::min(n, m > 0 ? m : 1);
   }
   if (nufft_fin_smem(Ns) > 48 * 1024)
@@ -1272,7 +1311,8 @@ void launch_nufft(sbr_phase_mode mode, const sbr_paths* p, const sbr_radar_cfg* 
   na.m = (float)M;
   na.f0_c = r->f0 / kC;
   na.b_cn = r->bandwidth / (kC * Ns);
-  na.m_d = (double)M;
+  na.cyc = na.f0_c + 0.5 * Ns * na.b_cn;  // N_s / 2 is whole: delta need not be reduced first
+  na.cell = M * na.b_cn;
   na.V = V;
   na.Q = Q;
   na.chirps = chirps;
@@ -1284,7 +1324,7 @@ void launch_nufft(sbr_phase_mode mode, const sbr_paths* p, const sbr_radar_cfg* 
   const float2* plen = reinterpret_cast<const float2*>(p->path_len);
   const int grid = V * Q * chirps;
   ::sbr::note_launch();
-  nufft_kernel(Ns, mode == SBR_PHASE_FP64, moving)<<<grid, nufft_threads(Ns), nufft_smem(Ns), st>>>(
+  nufft_kernel(Ns, mode == SBR_PHASE_FP64, moving)<<<grid, kNuThreads, nufft_smem(Ns), st>>>(
       prep, plen, p->phase_ofs, p->path_rate, p->path_cap, p->count, na, co, w.grids, w.fin_cnt);
   const int slices = M < kNuFinSlice ? 1 : M / kNuFinSlice;
   ::sbr::note_launch();
