@@ -893,6 +893,82 @@ __global__ void __launch_bounds__(kNuFinThreads) k_nufft_finish(const float2* __
   }
 }
 
+// Finishing of grids of up to kNuClusterPoints points: a cluster of eight CTAs per row.
+// CTA r adds the r-th eighth of the Q grids (as many threads per point as there are,
+// then the threads' sums in order), the CTAs exchange their eighths through each
+// other's shared memory, and each that has chirps of the row to write transforms the
+// whole grid (three or four passes: cheaper than handing the result on) and writes
+// its share of them.  A chain of latencies, so it is the links that count: no partial
+// sums through L2, no fence and counter, a static scene's chirps written by 8 V CTAs
+// instead of V (12 antennas x 128 chirps x 256 samples: about 10 -> 6 us).
+// Above 1024 points a CTA's eighth leaves too few threads per point for the grids' sum
+// (2048 points: 109 us for a synthesis that takes 105 with the kernel above).
+constexpr int kNuClusterPoints = 1024;
+constexpr int kNuRanks = 8;
+constexpr int kNuClThreads = 512;
+__global__ void __cluster_dims__(kNuRanks, 1, 1) __launch_bounds__(kNuClThreads)
+    k_nufft_finish_cluster(const float2* __restrict__ grids, const NufftArg na, const __grid_constant__ NufftCoef co,
+                           float2* __restrict__ cube, int C, bool moving) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  extern __shared__ float2 sg[];  // slots(M) grid, slots(M / 2) twiddles, [kNuClThreads] per-thread sums, [M / 8] this eighth
+  const int log_m = na.log_m, M = 1 << log_m, pts = M / kNuRanks, rank = (int)cluster.block_rank();
+  const int row = blockIdx.x / kNuRanks, rows = na.V * na.chirps, Q = na.Q, tid = threadIdx.x;
+  float2* tw = sg + fft::slots(M);
+  float2* part = tw + fft::slots(M / 2);
+  float2* mine = part + kNuClThreads;
+  const int parts = kNuClThreads / pts, li = tid % pts, k0 = tid / pts;  // pts <= 128
+  const float2* src = grids + (size_t)row * M + rank * pts + li;
+  const size_t qs = (size_t)rows * M;  // from one CTA's grid to the next
+  float2 a0 = make_float2(0.f, 0.f), a1 = a0, a2 = a0, a3 = a0;
+  int q = k0;
+  for (; q + 3 * parts < Q; q += 4 * parts) {  // four loads in flight, four interleaved sums
+    const float2 x0 = __ldcg(src + (size_t)q * qs), x1 = __ldcg(src + (size_t)(q + parts) * qs);
+    const float2 x2 = __ldcg(src + (size_t)(q + 2 * parts) * qs), x3 = __ldcg(src + (size_t)(q + 3 * parts) * qs);
+    a0 = make_float2(a0.x + x0.x, a0.y + x0.y);
+    a1 = make_float2(a1.x + x1.x, a1.y + x1.y);
+    a2 = make_float2(a2.x + x2.x, a2.y + x2.y);
+    a3 = make_float2(a3.x + x3.x, a3.y + x3.y);
+  }
+  for (; q < Q; q += parts) {
+    const float2 x = __ldcg(src + (size_t)q * qs);
+    a0 = make_float2(a0.x + x.x, a0.y + x.y);
+  }
+  part[tid] = make_float2((a0.x + a1.x) + (a2.x + a3.x), (a0.y + a1.y) + (a2.y + a3.y));
+  const int c0 = moving ? (rank == 0 ? 0 : 1) : C * rank / kNuRanks, c1 = moving ? 1 : C * (rank + 1) / kNuRanks;
+  if (c0 < c1) fft::fill_twiddles(tw, M, 1.f, kNuClThreads, tid);
+  __syncthreads();
+  if (tid < pts) {
+    float2 acc = part[tid];
+    for (int k = 1; k < parts; ++k) acc = make_float2(acc.x + part[k * pts + tid].x, acc.y + part[k * pts + tid].y);
+    mine[tid] = acc;
+  }
+  cluster.sync();
+  if (c0 < c1) {
+    for (int i = tid; i < M; i += kNuClThreads)
+      sg[fft::slot(fft::bitrev(i, log_m))] = cluster.map_shared_rank(mine, i / pts)[i % pts];
+  }
+  cluster.sync();  // every eighth has been read: a CTA may leave
+  if (c0 >= c1) return;
+  fft::smem_fft(sg, tw, log_m, kNuClThreads, tid);
+  // rows are (antenna, chirp of the launch), the chirp fastest
+  const int Ns = M >> 1, h = Ns >> 1, v = row / na.chirps, first = moving ? na.chirp0 + row - v * na.chirps : c0;
+  const int last = moving ? first + 1 : c1;
+  // threads over samples, then over chirps; one 8-byte store each (a cube need not be
+  // aligned to more)
+  float2* out = cube + (size_t)v * C * Ns;
+  const int groups = kNuClThreads / Ns > 0 ? kNuClThreads / Ns : 1, g = tid / Ns;
+  for (int n = tid % Ns; n < Ns && g < groups; n += kNuClThreads) {
+    const float xi = (float)(n - h) / (float)h, y = xi * xi;
+    float inv = co.inv[8];
+#pragma unroll
+    for (int k = 7; k >= 0; --k) inv = fmaf(inv, y, co.inv[k]);
+    const float2 B = sg[fft::slot((n - h) & (M - 1))];
+    const float2 val = make_float2(B.x * inv, B.y * inv);
+    for (int c = first + g; c < last; c += groups) out[(size_t)c * Ns + n] = val;
+  }
+}
+
 // I0 by its power series (the terms are positive: no cancellation; beta < 20).
 double bessel_i0(double x) {
   double t = 1.0, s = 1.0;
@@ -1191,6 +1267,9 @@ void grid_shape(int V, int Ns, int64_t cap, int* Q) {
 
 // dynamic shared memory of the spreading kernel: the grid's copies and its sums
 inline size_t nufft_smem(int Ns) { return (2 * kNuCopies * sizeof(int) + 2 * sizeof(float)) * (size_t)nu_points(2 * Ns); }
+inline size_t nufft_cl_smem(int Ns) {
+  return sizeof(float2) * (size_t)(fft::slots(2 * Ns) + fft::slots(Ns) + kNuClThreads + 2 * Ns / kNuRanks);
+}
 inline size_t nufft_fin_smem(int Ns) { return sizeof(float2) * (size_t)(fft::slots(2 * Ns) + fft::slots(Ns) + kNuFinThreads); }
 
 using NufftSpread = void (*)(const float4*, const float2*, const float*, const float*, int64_t, const int32_t*, NufftArg,
@@ -1326,8 +1405,13 @@ void launch_nufft(sbr_phase_mode mode, const sbr_paths* p, const sbr_radar_cfg* 
   ::sbr::note_launch();
   nufft_kernel(Ns, mode == SBR_PHASE_FP64, moving)<<<grid, kNuThreads, nufft_smem(Ns), st>>>(
       prep, plen, p->phase_ofs, p->path_rate, p->path_cap, p->count, na, co, w.grids, w.fin_cnt);
-  const int slices = M < kNuFinSlice ? 1 : M / kNuFinSlice;
   ::sbr::note_launch();
+  if (M <= kNuClusterPoints) {
+    k_nufft_finish_cluster<<<V * chirps * kNuRanks, kNuClThreads, nufft_cl_smem(Ns), st>>>(w.grids, na, co, cube,
+                                                                                          r->n_chirps, moving);
+    return;
+  }
+  const int slices = M / kNuFinSlice;
   k_nufft_finish<<<V * chirps * slices, kNuFinThreads, nufft_fin_smem(Ns), st>>>(w.grids, na, co, w.bsum, w.fin_cnt, cube,
                                                                                 r->n_chirps, moving);
 }

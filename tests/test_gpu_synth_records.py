@@ -97,6 +97,23 @@ def test_split_records(sbr, ns, P, where):
     assert rel(cube[:, 0], direct(phi, delta, A, ns)) <= TOL
 
 
+@pytest.mark.parametrize("nc,ns", [(1, 256), (4, 32), (16, 256), (128, 64), (8, 2048)])
+def test_chirps_and_cube_alignment(sbr, nc, ns):
+    """Every chirp of a static scene equal, in a cube that starts 8 bytes past a 16-byte boundary
+    and in an aligned one."""
+    radar = radar_single_tx(ns, nc)
+    delta, phi, A = records(nc + ns, 4, 17000, ns)
+    paths, phi, delta, A = bind(sbr, radar, 17000, delta, phi, A)
+    n = 4 * nc * ns * 2
+    buf = torch.full((n + 4,), 7.0, device="cuda")
+    sbr.synthesize(paths, radar, out=buf[2:n + 2].view(4, nc, ns, 2))
+    cube = sbr.synthesize(paths, radar)
+    host = buf.cpu()
+    assert torch.equal(host[2:n + 2].view(4, nc, ns, 2), cube.cpu()) and bool((cube == cube[:, :1]).all())
+    assert bool((host[:2] == 7).all()) and bool((host[n + 2:] == 7).all())
+    assert rel(cube[:, 0], direct(phi, delta, A, ns)) <= TOL
+
+
 def test_split_records_not_finite(sbr):
     """A record that is not finite makes its antenna's samples NaN, and no others."""
     radar = radar_single_tx(256, 1)
