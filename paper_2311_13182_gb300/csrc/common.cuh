@@ -14,6 +14,39 @@ void set_error(const char* fmt, ...);
 // Host-side count of kernel launches issued by the library (sbr_launch_count).
 void note_launch();
 
+// ---- launches of a chain of dependent kernels ------------------------------
+//
+// Most calls are chains of kernels of a few microseconds, between which a plain
+// launch leaves about 2 us (the previous grid drains, the next is dispatched).  A
+// kernel launched by launch_after may be dispatched while the kernel before it in
+// the stream still runs; it must not touch global memory before after_previous(),
+// which returns once that kernel has finished and its writes are visible.  Every
+// thread of such a kernel calls it, so a kernel's end implies the end of all before
+// it.  next_may_start() lets the next kernel be dispatched from the moment all CTAs
+// of this one have begun; long kernels leave it out, as waiting CTAs hold registers
+// and shared memory that other streams could use.
+template <class T>
+struct same_type {
+  using type = T;
+};
+template <class... P>
+inline cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                                typename same_type<P>::type... args) {
+  cudaLaunchConfig_t c{};
+  cudaLaunchAttribute a{};
+  a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  a.val.programmaticStreamSerializationAllowed = 1;
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.dynamicSmemBytes = smem;
+  c.stream = st;
+  c.attrs = &a;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, kernel, args...);
+}
+__device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void next_may_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 constexpr double kC = 299792458.0;  // m/s
 constexpr double kTwoPi = 6.283185307179586476925286766559;
 constexpr int kAlign = 256;

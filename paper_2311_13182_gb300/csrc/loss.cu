@@ -41,6 +41,8 @@ __device__ inline float block_sum(float v, float* red) {
 __global__ void __launch_bounds__(1024) k_chamfer(const float4* __restrict__ P, const int32_t* __restrict__ d_n,
                                                   int cap, const float4* __restrict__ Q, int m,
                                                   float* __restrict__ loss, float4* __restrict__ gP) {
+  next_may_start();
+  after_previous();
   __shared__ int nn_p[kChamferMax], nn_q[kChamferMax];
   __shared__ float d2_p[kChamferMax], d2_q[kChamferMax];
   __shared__ float red[32];
@@ -121,6 +123,8 @@ __global__ void __launch_bounds__(kLapThreads) k_lap_delta(const float* __restri
                                                            const int32_t* __restrict__ off,
                                                            const int32_t* __restrict__ adj, float* __restrict__ delta,
                                                            float* __restrict__ partial) {
+  next_may_start();
+  after_previous();
   __shared__ float red[32];
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   float sq = 0.f;
@@ -162,6 +166,8 @@ __global__ void __launch_bounds__(kLapThreads) k_lap_grad(const float* __restric
                                                           const int32_t* __restrict__ adj, float scale,
                                                           float* __restrict__ g, const float* __restrict__ partial,
                                                           int nb, float lscale, float* __restrict__ loss) {
+  next_may_start();
+  after_previous();
   __shared__ float red[32];
   if (blockIdx.x == 0) {
     float s = 0.f;
@@ -200,6 +206,8 @@ __global__ void __launch_bounds__(kLapThreads) k_lap_grad(const float* __restric
 __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
                        float* __restrict__ v, int64_t n, const int32_t* __restrict__ step, float lr, float b1,
                        float b2, float eps) {
+  next_may_start();
+  after_previous();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const float t = (float)(*step + 1);
@@ -212,7 +220,11 @@ __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float
   p[i] -= lr * (mi * c1) / (sqrtf(vi * c2) + eps);
 }
 
-__global__ void k_step_inc(int32_t* step) { *step += 1; }
+__global__ void k_step_inc(int32_t* step) {
+  next_may_start();
+  after_previous();
+  *step += 1;
+}
 
 }  // namespace
 }  // namespace sbr
@@ -229,9 +241,7 @@ extern "C" sbr_status sbr_chamfer(const float* d_pred, const int32_t* d_n_pred, 
           "sbr_chamfer: n_target=%d outside [0, %d]", n_target, kChamferMax);
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   ::sbr::note_launch();
-  k_chamfer<<<1, 1024, 0, st>>>(reinterpret_cast<const float4*>(d_pred), d_n_pred, pred_cap,
-                                reinterpret_cast<const float4*>(d_target), n_target, d_loss,
-                                reinterpret_cast<float4*>(d_gpred));
+  launch_after(k_chamfer, 1, 1024, 0, st, reinterpret_cast<const float4*>(d_pred), d_n_pred, pred_cap, reinterpret_cast<const float4*>(d_target), n_target, d_loss, reinterpret_cast<float4*>(d_gpred));
   SBR_CUDA(cudaGetLastError());
   return SBR_OK;
 }
@@ -288,10 +298,9 @@ extern "C" sbr_status sbr_laplacian(const float* d_verts, int32_t nv, const int3
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const int b = (nv + kLapThreads - 1) / kLapThreads;
   ::sbr::note_launch();
-  k_lap_delta<<<b, kLapThreads, 0, st>>>(d_verts, nv, d_off, d_adj, delta, partial);
+  launch_after(k_lap_delta, b, kLapThreads, 0, st, d_verts, nv, d_off, d_adj, delta, partial);
   ::sbr::note_launch();
-  k_lap_grad<<<b, kLapThreads, 0, st>>>(delta, nv, d_off, d_adj, 2.f * weight / (float)nv, d_gverts, partial, b,
-                                        weight / (float)nv, d_loss);
+  launch_after(k_lap_grad, b, kLapThreads, 0, st, delta, nv, d_off, d_adj, 2.f * weight / (float)nv, d_gverts, partial, b, weight / (float)nv, d_loss);
   SBR_CUDA(cudaGetLastError());
   return SBR_OK;
 }
@@ -304,11 +313,10 @@ extern "C" sbr_status sbr_adam_step(float* d_params, const float* d_grad, float*
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   if (n > 0) {
     ::sbr::note_launch();
-    k_adam<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(d_params, d_grad, d_m, d_v, n, d_step, lr, beta1, beta2,
-                                                         eps);
+    launch_after(k_adam, (unsigned)((n + 255) / 256), 256, 0, st, d_params, d_grad, d_m, d_v, n, d_step, lr, beta1, beta2, eps);
   }
   ::sbr::note_launch();
-  k_step_inc<<<1, 1, 0, st>>>(d_step);
+  launch_after(k_step_inc, 1, 1, 0, st, d_step);
   SBR_CUDA(cudaGetLastError());
   return SBR_OK;
 }

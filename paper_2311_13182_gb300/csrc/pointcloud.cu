@@ -34,19 +34,21 @@ using namespace fft;
 // per thread.  clear: words the first CTA zeroes for later kernels of the call, or NULL.
 __global__ void k_fft_rows(const float2* __restrict__ in, float2* __restrict__ out, int rows, int logn, int logb,
                            float sign, unsigned long long* clear) {
+  next_may_start();
   extern __shared__ float2 s[];  // [2^logb] rows of slots(n) points, slots(n / 2) twiddles
   const int n = 1 << logn, ld = slots(n);
   float2* tw = s + (ld << logb);
+  fill_twiddles(tw, n, sign, blockDim.x, threadIdx.x);
+  after_previous();
   if (clear && blockIdx.x == 0 && threadIdx.x < 2) clear[threadIdx.x] = 0ull;
   const size_t at = (size_t)blockIdx.x << (logn + logb);
   const int cnt = min(1 << logb, rows - ((int)blockIdx.x << logb)) << logn;  // points of this CTA's rows
-  float2 x[8];  // in flight while the twiddles are computed: the CTA holds eight points per thread
+  float2 x[8];  // the CTA holds eight points per thread
 #pragma unroll
   for (int u = 0; u < 8; ++u) {
     const int i = threadIdx.x + u * blockDim.x;
     x[u] = i < cnt ? in[at + i] : make_float2(0.f, 0.f);
   }
-  fill_twiddles(tw, n, sign, blockDim.x, threadIdx.x);
 #pragma unroll
   for (int u = 0; u < 8; ++u) {
     const int i = threadIdx.x + u * blockDim.x;
@@ -63,6 +65,7 @@ constexpr int kLogColTile = 4, kColTile = 1 << kLogColTile;
 // Columns sit an odd number of points apart in shared memory, so the 16 columns of
 // one chirp fall in different banks.
 __global__ void k_fft_cols(float2* __restrict__ x, int C, int logc, int Ns, float sign) {
+  next_may_start();
   extern __shared__ float2 s[];  // [kColTile][slots(C) | 1] points, slots(C / 2) twiddles
   const int ld = slots(C) | 1;
   float2* tw = s + kColTile * ld;
@@ -70,6 +73,7 @@ __global__ void k_fft_cols(float2* __restrict__ x, int C, int logc, int Ns, floa
   const int v = blockIdx.x / tiles, k0 = (blockIdx.x - v * tiles) * kColTile;
   float2* base = x + (size_t)v * C * Ns + k0;
   fill_twiddles(tw, C, sign, blockDim.x, threadIdx.x);
+  after_previous();
   for (int i = threadIdx.x; i < C * kColTile; i += blockDim.x) {
     const int c = i / kColTile, kk = i - c * kColTile;
     s[kk * ld + slot(bitrev(c, logc))] = base[(size_t)c * Ns + kk];
@@ -118,6 +122,8 @@ template <int APT>
 __global__ void __launch_bounds__(256) k_angle_power(const float2* __restrict__ X,
                                                      const Steer xl, int V, int C,
                                                      int Ns, int dpg, float* __restrict__ part) {
+  next_may_start();
+  after_previous();
   extern __shared__ float2 sm[];
   constexpr int R = 8 * APT;
   float2* sw = sm;                // [R][V]
@@ -215,6 +221,7 @@ template <int NR>
 __global__ void __launch_bounds__(kTcThreads) k_angle_tc(const float2* __restrict__ X, const Steer xl, int R,
                                                          int V, int C, int Ns, float* __restrict__ part,
                                                          int* __restrict__ err) {
+  next_may_start();
   constexpr int kN = 2 * NR;                         // MMA N
   constexpr int kCols = tc_cols<NR>();
   constexpr uint32_t kTileW = (uint32_t)kN * kTcK * 4;  // steering operand bytes (hi or lo)
@@ -233,15 +240,7 @@ __global__ void __launch_bounds__(kTcThreads) k_angle_tc(const float2* __restric
     tc::tmem_relinquish();
   }
   if (tid == 0) tc::mbar_init(mbar, 1);
-  // A: thread t takes range bin k0 + t; per Doppler bin and antenna pair one 16-byte chunk
-  // (Re, Im of antenna 2j, Re, Im of antenna 2j + 1); antennas >= V and bins >= nd are zero.
-  // Every load is issued before the steering matrix is generated, which hides their latency.
-  float2 xv[kTcDG][kTcK / 2];
-#pragma unroll
-  for (int dd = 0; dd < kTcDG; ++dd)
-#pragma unroll
-    for (int v = 0; v < kTcK / 2; ++v)
-      xv[dd][v] = (dd < nd && v < V) ? X[((size_t)v * C + d0 + dd) * Ns + k0 + tid] : make_float2(0.f, 0.f);
+  // The steering matrix needs no input: it is made while the transforms before this kernel end.
   // B: row pair (2a, 2a + 1) of angle row a, antenna pair j: one 16-byte chunk per row
   for (int i = tid; i < NR * (kTcK / 4); i += kTcThreads) {
     const int a = i >> 3, j = i & 7;
@@ -253,6 +252,15 @@ __global__ void __launch_bounds__(kTcThreads) k_angle_tc(const float2* __restric
     tc_put4(sw_hi, sw_lo, tc_off(2 * a, 4 * j), make_float4(c0, -s0, c1, -s1));
     tc_put4(sw_hi, sw_lo, tc_off(2 * a + 1, 4 * j), make_float4(s0, c0, s1, c1));
   }
+  after_previous();
+  // A: thread t takes range bin k0 + t; per Doppler bin and antenna pair one 16-byte chunk
+  // (Re, Im of antenna 2j, Re, Im of antenna 2j + 1); antennas >= V and bins >= nd are zero.
+  float2 xv[kTcDG][kTcK / 2];
+#pragma unroll
+  for (int dd = 0; dd < kTcDG; ++dd)
+#pragma unroll
+    for (int v = 0; v < kTcK / 2; ++v)
+      xv[dd][v] = (dd < nd && v < V) ? X[((size_t)v * C + d0 + dd) * Ns + k0 + tid] : make_float2(0.f, 0.f);
 #pragma unroll
   for (int dd = 0; dd < kTcDG; ++dd) {
     unsigned char* xh = sx_hi + 2 * (size_t)kTcTile * dd;
@@ -322,6 +330,8 @@ __global__ void __launch_bounds__(kTcThreads) k_angle_tc(const float2* __restric
 // amax_key must be 0 on entry.
 __global__ void k_power_reduce(const float* __restrict__ part, int groups, int cells, float* __restrict__ Pw,
                                unsigned long long* __restrict__ amax_key) {
+  next_may_start();
+  after_previous();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   unsigned long long key = 0ull;
   if (i < cells) {
@@ -413,6 +423,8 @@ __global__ void __launch_bounds__(kDetThreads) k_detect(const float* __restrict_
                                                         int32_t* __restrict__ amax, int32_t* __restrict__ flag,
                                                         uint32_t* __restrict__ key, int32_t* __restrict__ cell,
                                                         int32_t* __restrict__ cnt) {
+  next_may_start();
+  after_previous();
   __shared__ int wn[kDetThreads / 32];
   const int i = blockIdx.x * kDetThreads + threadIdx.x;  // cells come in multiples of 256
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -446,6 +458,8 @@ __global__ void __launch_bounds__(kDetThreads) k_detect(const float* __restrict_
 __global__ void k_compact(const int32_t* __restrict__ flag, const int32_t* __restrict__ off,
                           const uint32_t* __restrict__ key, int cells, uint32_t* __restrict__ ko,
                           int32_t* __restrict__ vo) {
+  next_may_start();
+  after_previous();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= cells || !flag[i]) return;
   ko[off[i]] = key[i];
@@ -526,6 +540,8 @@ __global__ void k_points(const float* __restrict__ Pw, PointArg pa, const int32_
                          const int32_t* __restrict__ cand, const int32_t* __restrict__ n_cand,
                          float4* __restrict__ pts, int32_t* __restrict__ cell_out,
                          int32_t* __restrict__ n_out) {
+  next_may_start();
+  after_previous();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int n = min(*n_cand, pa.k_max);
   if (i == 0) *n_out = n;
@@ -602,6 +618,8 @@ __global__ void __launch_bounds__(kSelThreads) k_select(const float* __restrict_
                                                         uint32_t* k0, int32_t* v0, uint32_t* k1, int32_t* v1,
                                                         float4* __restrict__ pts, int32_t* __restrict__ cell_out,
                                                         int32_t* __restrict__ n_out) {
+  next_may_start();
+  after_previous();
   extern __shared__ __align__(16) uint32_t sel_sm[];  // cta::kSortSmemWords
   __shared__ uint32_t wt[32];
   const CfarArg& c = pa.c;
@@ -752,6 +770,8 @@ template <int kPass>
 __global__ void k_points_bwd(const float* __restrict__ Pw, PointArg pa, const int32_t* __restrict__ amax,
                              const int32_t* __restrict__ cells, const int32_t* __restrict__ n_pts,
                              const float4* __restrict__ gpts, FixScatter fs) {
+  next_may_start();
+  after_previous();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   float lmax = 0.f;
   const DpwScatter<kPass> sc{fs, kPass == 0 ? 0 : fix_exp(*fs.max_bits, fs.log2n), lmax};
@@ -767,6 +787,8 @@ __global__ void __launch_bounds__(256) k_angle_bwd(const float2* __restrict__ X,
                                                    const Steer xl,
                                                    const float* __restrict__ dPw, FixScatter fs, int V, int C,
                                                    int Ns, float2* __restrict__ dX) {
+  next_may_start();
+  after_previous();
   extern __shared__ float2 sm[];
   constexpr int R = 8 * APT;
   float2* sw = sm;               // [R][V]
@@ -933,7 +955,7 @@ void launch_angle_power(const float2* X, const Steer& xl, int V, int C, int Ns, 
   const size_t sm = sizeof(float2) * ((size_t)R * V + (size_t)V * kKT);
   dim3 grid(Ns / kKT, groups);
   ::sbr::note_launch();
-  k_angle_power<APT><<<grid, 256, sm, st>>>(X, xl, V, C, Ns, (C + groups - 1) / groups, part);
+  launch_after(k_angle_power<APT>, grid, 256, sm, st, X, xl, V, C, Ns, (C + groups - 1) / groups, part);
 }
 
 template <int APT>
@@ -945,7 +967,7 @@ void launch_angle_bwd(const float2* X, const Steer& xl, const float* dpw, const 
   dim3 grid(Ns / kKT, C);
   if (sm > 48 * 1024) cudaFuncSetAttribute(k_angle_bwd<APT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   ::sbr::note_launch();
-  k_angle_bwd<APT><<<grid, 256, sm, st>>>(X, xl, dpw, fs, V, C, Ns, dX);
+  launch_after(k_angle_bwd<APT>, grid, 256, sm, st, X, xl, dpw, fs, V, C, Ns, dX);
 }
 
 // Eight points per thread: as many short rows per CTA as 256 threads hold (32 to 256
@@ -962,7 +984,7 @@ cudaError_t fft_rows(const float2* in, float2* out, int rows, int n, float sign,
     if (e != cudaSuccess) return e;
   }
   ::sbr::note_launch();
-  k_fft_rows<<<(rows + (1 << logb) - 1) >> logb, threads, sm, st>>>(in, out, rows, logn, logb, sign, clear);
+  launch_after(k_fft_rows, (rows + (1 << logb) - 1) >> logb, threads, sm, st, in, out, rows, logn, logb, sign, clear);
   return cudaGetLastError();
 }
 
@@ -974,7 +996,7 @@ cudaError_t fft_cols(float2* x, int V, int C, int Ns, float sign, cudaStream_t s
     if (e != cudaSuccess) return e;
   }
   ::sbr::note_launch();
-  k_fft_cols<<<V * (Ns / kColTile), 256, sm, st>>>(x, C, ilog2(C), Ns, sign);
+  launch_after(k_fft_cols, V * (Ns / kColTile), 256, sm, st, x, C, ilog2(C), Ns, sign);
   return cudaGetLastError();
 }
 
@@ -1050,9 +1072,9 @@ sbr_status power_map_impl(const float* d_cube, const sbr_radar_cfg* radar, const
     ::sbr::note_launch();
     const dim3 grid(Ns / kTcM, L.groups);
     if (angle_tc_rows(R) == 64)
-      k_angle_tc<64><<<grid, kTcThreads, tc_smem<64>(), st>>>(L.spec, xl, R, V, C, Ns, L.part, L.err);
+      launch_after(k_angle_tc<64>, grid, kTcThreads, tc_smem<64>(), st, L.spec, xl, R, V, C, Ns, L.part, L.err);
     else
-      k_angle_tc<128><<<grid, kTcThreads, tc_smem<128>(), st>>>(L.spec, xl, R, V, C, Ns, L.part, L.err);
+      launch_after(k_angle_tc<128>, grid, kTcThreads, tc_smem<128>(), st, L.spec, xl, R, V, C, Ns, L.part, L.err);
   } else switch (R / 8) {
     case 1: launch_angle_power<1>(L.spec, xl, V, C, Ns, L.groups, L.part, st); break;
     case 2: launch_angle_power<2>(L.spec, xl, V, C, Ns, L.groups, L.part, st); break;
@@ -1064,7 +1086,7 @@ sbr_status power_map_impl(const float* d_cube, const sbr_radar_cfg* radar, const
   }
   SBR_CUDA(cudaGetLastError());
   ::sbr::note_launch();
-  k_power_reduce<<<(cells + 255) / 256, 256, 0, st>>>(L.part, L.groups, cells, L.power, L.amax_key);
+  launch_after(k_power_reduce, (cells + 255) / 256, 256, 0, st, L.part, L.groups, cells, L.power, L.amax_key);
   SBR_CUDA(cudaGetLastError());
   return SBR_OK;
 }
@@ -1108,26 +1130,21 @@ extern "C" sbr_status sbr_pointcloud(const float* d_cube, const sbr_radar_cfg* r
   if (cells <= kSortOneCta || cfar->k_max <= kSelMax) {
     SBR_CUDA(select_attr());
     ::sbr::note_launch();
-    k_detect<<<cells / kDetThreads, kDetThreads, 0, st>>>(L.power, ca, L.amax_key, L.argmax, nullptr, L.key, L.flag, L.off);
+    launch_after(k_detect, cells / kDetThreads, kDetThreads, 0, st, L.power, ca, L.amax_key, L.argmax, nullptr, L.key, L.flag, L.off);
     ::sbr::note_launch();
-    k_select<<<1, kSelThreads, cta::kSortSmemBytes, st>>>(L.power, pa, L.amax_key, L.key, L.flag, L.off, L.skeys[0],
-                                                           L.svals[0], L.skeys[1], L.svals[1],
-                                                           reinterpret_cast<float4*>(d_points), L.peak_cell,
-                                                           L.n_points);
+    launch_after(k_select, 1, kSelThreads, cta::kSortSmemBytes, st, L.power, pa, L.amax_key, L.key, L.flag, L.off, L.skeys[0], L.svals[0], L.skeys[1], L.svals[1], reinterpret_cast<float4*>(d_points), L.peak_cell, L.n_points);
     SBR_CUDA(cudaGetLastError());
     return SBR_OK;
   }
   ::sbr::note_launch();
-  k_detect<<<cells / kDetThreads, kDetThreads, 0, st>>>(L.power, ca, L.amax_key, L.argmax, L.flag, L.key, nullptr, nullptr);
+  launch_after(k_detect, cells / kDetThreads, kDetThreads, 0, st, L.power, ca, L.amax_key, L.argmax, L.flag, L.key, nullptr, nullptr);
   SBR_CUDA(exclusive_scan(L.flag, L.off, cells, nullptr, L.scan_scr, st));
   ::sbr::note_launch();
-  k_compact<<<(cells + 255) / 256, 256, 0, st>>>(L.flag, L.off, L.key, cells, L.skeys[0], L.svals[0]);
+  launch_after(k_compact, (cells + 255) / 256, 256, 0, st, L.flag, L.off, L.key, cells, L.skeys[0], L.svals[0]);
   SBR_CUDA(radix_sort_pairs(L.skeys, L.svals, cells, L.off + cells, 32, L.sort_scr, st));
   // 8-9: refine and emit points
   ::sbr::note_launch();
-  k_points<<<(cfar->k_max + 255) / 256, 256, 0, st>>>(L.power, pa, L.argmax, L.svals[0], L.off + cells,
-                                                       reinterpret_cast<float4*>(d_points), L.peak_cell,
-                                                       L.n_points);
+  launch_after(k_points, (cfar->k_max + 255) / 256, 256, 0, st, L.power, pa, L.argmax, L.svals[0], L.off + cells, reinterpret_cast<float4*>(d_points), L.peak_cell, L.n_points);
   SBR_CUDA(cudaGetLastError());
   return SBR_OK;
 }
@@ -1186,6 +1203,8 @@ constexpr int kMseThreads = 1024;
 __global__ void __launch_bounds__(kMseThreads) k_image_mse(const float* __restrict__ Pw, const float* __restrict__ T,
                                                            int cells, float* __restrict__ loss,
                                                            float* __restrict__ dpw) {
+  next_may_start();
+  after_previous();
   __shared__ float red[kMseThreads / 32];
   const float inv_n = 1.f / (float)cells;
   float s = 0.f;
@@ -1219,7 +1238,7 @@ extern "C" sbr_status sbr_image_loss(const sbr_radar_cfg* radar, const sbr_cfar_
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const int cells = angle_rows(cfar) * radar->n_samples;
   ::sbr::note_launch();
-  k_image_mse<<<1, kMseThreads, 0, st>>>(L.power, d_target, cells, d_loss, d_gcube ? L.dpw : nullptr);
+  launch_after(k_image_mse, 1, kMseThreads, 0, st, L.power, d_target, cells, d_loss, d_gcube ? L.dpw : nullptr);
   SBR_CUDA(cudaGetLastError());
   if (!d_gcube) return SBR_OK;
   return cube_adjoint(radar, cfar, L, FixScatter{nullptr, nullptr, 0}, d_gcube, st);
@@ -1249,8 +1268,8 @@ extern "C" sbr_status sbr_pointcloud_bwd(const sbr_radar_cfg* radar, const sbr_c
   const float4* gp = reinterpret_cast<const float4*>(d_gpoints);
   const int nb = (cfar->k_max + 255) / 256;
   ::sbr::note_launch();
-  k_points_bwd<0><<<nb, 256, 0, st>>>(L.power, pa, L.argmax, L.peak_cell, L.n_points, gp, fs);
+  launch_after(k_points_bwd<0>, nb, 256, 0, st, L.power, pa, L.argmax, L.peak_cell, L.n_points, gp, fs);
   ::sbr::note_launch();
-  k_points_bwd<1><<<nb, 256, 0, st>>>(L.power, pa, L.argmax, L.peak_cell, L.n_points, gp, fs);
+  launch_after(k_points_bwd<1>, nb, 256, 0, st, L.power, pa, L.argmax, L.peak_cell, L.n_points, gp, fs);
   return cube_adjoint(radar, cfar, L, fs, d_gcube, st);
 }

@@ -53,6 +53,8 @@ __device__ inline uint32_t block_exclusive(uint32_t v, uint32_t* total, uint32_t
 
 __global__ void k_tile_sums(const int32_t* __restrict__ in, int64_t cap, const int32_t* d_n,
                             int32_t* __restrict__ sums) {
+  next_may_start();
+  after_previous();
   __shared__ uint32_t wt[32];
   const int64_t n = clamp_n(cap, d_n);
   const int64_t base = (int64_t)blockIdx.x * kTile + (int64_t)threadIdx.x * kItems;
@@ -67,6 +69,8 @@ __global__ void k_tile_sums(const int32_t* __restrict__ in, int64_t cap, const i
 
 // In-place exclusive scan of m values with one CTA (m up to a few million).
 __global__ void k_scan_single(int32_t* __restrict__ a, int64_t m) {
+  next_may_start();
+  after_previous();
   __shared__ uint32_t wt[32];
   uint32_t carry = 0;
   for (int64_t base = 0; base < m; base += blockDim.x) {
@@ -81,6 +85,8 @@ __global__ void k_scan_single(int32_t* __restrict__ a, int64_t m) {
 
 __global__ void k_tile_scan(const int32_t* __restrict__ in, int32_t* __restrict__ out, int64_t cap,
                             const int32_t* d_n, const int32_t* __restrict__ sums) {
+  next_may_start();
+  after_previous();
   __shared__ uint32_t wt[32];
   const int64_t n = clamp_n(cap, d_n);
   if (n == 0) {
@@ -109,6 +115,8 @@ __global__ void k_tile_scan(const int32_t* __restrict__ in, int32_t* __restrict_
 
 __global__ void k_digit_hist(const uint32_t* __restrict__ keys, int64_t cap, const int32_t* d_n,
                              int shift, int32_t* __restrict__ hist, int ntiles) {
+  next_may_start();
+  after_previous();
   __shared__ uint32_t cnt[16];
   if (threadIdx.x < 16) cnt[threadIdx.x] = 0;
   __syncthreads();
@@ -128,6 +136,8 @@ __global__ void k_digit_scatter(const uint32_t* __restrict__ kin, const int32_t*
                                 uint32_t* __restrict__ kout, int32_t* __restrict__ vout,
                                 int64_t cap, const int32_t* d_n, int shift,
                                 const int32_t* __restrict__ hist, int ntiles) {
+  next_may_start();
+  after_previous();
   __shared__ uint32_t wt[32];
   __shared__ int32_t tile_off[16];
   if (threadIdx.x < 16) tile_off[threadIdx.x] = hist[threadIdx.x * ntiles + blockIdx.x];
@@ -192,6 +202,8 @@ using cta::kSortSmemBytes;
 __global__ void __launch_bounds__(kSmallThreads) k_scan_small(const int32_t* __restrict__ in,
                                                               int32_t* __restrict__ out, int64_t cap,
                                                               const int32_t* d_n) {
+  next_may_start();
+  after_previous();
   __shared__ uint32_t wt[32];
   const int64_t n = clamp_n(cap, d_n);
   uint32_t carry = 0;
@@ -219,6 +231,8 @@ __global__ void __launch_bounds__(kSmallThreads) k_scan_small(const int32_t* __r
 __global__ void __launch_bounds__(kSmallThreads) k_sort_small(uint32_t* k0, int32_t* v0, uint32_t* k1,
                                                               int32_t* v1, int64_t cap, const int32_t* d_n,
                                                               int bits, const uint32_t* __restrict__ d_hist) {
+  next_may_start();
+  after_previous();
   extern __shared__ __align__(16) uint32_t sm[];  // kSortSmemWords
   cta::sort_pairs(k0, v0, k1, v1, clamp_n(cap, d_n), bits, d_hist, sm);
 }
@@ -245,17 +259,17 @@ cudaError_t exclusive_scan(const int32_t* in, int32_t* out, int64_t n, const int
                            void* scratch, cudaStream_t s) {
   if (n <= kSmall) {
     ::sbr::note_launch();
-    k_scan_small<<<1, kSmallThreads, 0, s>>>(in, out, n, d_n);
+    launch_after(k_scan_small, 1, kSmallThreads, 0, s, in, out, n, d_n);
     return cudaGetLastError();
   }
   const int nt = tiles_for(n < 1 ? 1 : n);
   int32_t* sums = static_cast<int32_t*>(scratch);
   ::sbr::note_launch();
-  k_tile_sums<<<nt, kThreads, 0, s>>>(in, n, d_n, sums);
+  launch_after(k_tile_sums, nt, kThreads, 0, s, in, n, d_n, sums);
   ::sbr::note_launch();
-  k_scan_single<<<1, 1024, 0, s>>>(sums, nt);
+  launch_after(k_scan_single, 1, 1024, 0, s, sums, nt);
   ::sbr::note_launch();
-  k_tile_scan<<<nt, kThreads, 0, s>>>(in, out, n, d_n, sums);
+  launch_after(k_tile_scan, nt, kThreads, 0, s, in, out, n, d_n, sums);
   return cudaGetLastError();
 }
 
@@ -269,8 +283,7 @@ cudaError_t radix_sort_pairs(uint32_t* keys[2], int32_t* vals[2], int64_t n, con
     cudaError_t e = sort_small_attr();
     if (e != cudaSuccess) return e;
     ::sbr::note_launch();
-    k_sort_small<<<1, kSmallThreads, kSortSmemBytes, s>>>(keys[0], vals[0], keys[1], vals[1], n, d_n, bits,
-                                                          d_hist);
+    launch_after(k_sort_small, 1, kSmallThreads, kSortSmemBytes, s, keys[0], vals[0], keys[1], vals[1], n, d_n, bits, d_hist);
     return cudaGetLastError();
   }
   const int passes = (bits + 3) / 4;
@@ -280,12 +293,11 @@ cudaError_t radix_sort_pairs(uint32_t* keys[2], int32_t* vals[2], int64_t n, con
   for (int p = 0; p < passes; ++p) {
     const int shift = 4 * p;
     ::sbr::note_launch();
-    k_digit_hist<<<nt, kThreads, 0, s>>>(keys[cur], n, d_n, shift, hist, nt);
+    launch_after(k_digit_hist, nt, kThreads, 0, s, keys[cur], n, d_n, shift, hist, nt);
     ::sbr::note_launch();
-    k_scan_single<<<1, 1024, 0, s>>>(hist, (int64_t)16 * nt);
+    launch_after(k_scan_single, 1, 1024, 0, s, hist, (int64_t)16 * nt);
     ::sbr::note_launch();
-    k_digit_scatter<<<nt, kThreads, 0, s>>>(keys[cur], vals[cur], keys[cur ^ 1], vals[cur ^ 1], n,
-                                            d_n, shift, hist, nt);
+    launch_after(k_digit_scatter, nt, kThreads, 0, s, keys[cur], vals[cur], keys[cur ^ 1], vals[cur ^ 1], n, d_n, shift, hist, nt);
     cur ^= 1;
   }
   if (cur == 1) {  // odd number of passes: copy back so the result is in buffer 0

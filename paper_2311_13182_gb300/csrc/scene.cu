@@ -27,6 +27,8 @@ __device__ inline int32_t ord(float f) {
 __device__ inline float unord(int32_t i) { return __int_as_float(i >= 0 ? i : i ^ 0x7fffffff); }
 
 __global__ void k_init_bounds(int32_t* b, int32_t* err, uint32_t* hist) {
+  next_may_start();
+  after_previous();
   if (threadIdx.x < 3) b[threadIdx.x] = 0x7fffffff;           // min x, y, z
   else if (threadIdx.x < 6) b[threadIdx.x] = (int32_t)0x80000000;  // max x, y, z
   else if (threadIdx.x == 6) b[6] = 0;                        // max |coord| (ordered, >= 0)
@@ -48,6 +50,8 @@ __device__ inline float3 vload(const float* v, int i) { return f3(v[3 * i], v[3 
 
 __global__ void k_bounds(const float* __restrict__ verts, int nv, const int32_t* __restrict__ faces,
                          int nt, int32_t* bounds, int32_t* err) {
+  next_may_start();
+  after_previous();
   int f = blockIdx.x * blockDim.x + threadIdx.x;
   float3 lo = f3(INFINITY, INFINITY, INFINITY), hi = f3(-INFINITY, -INFINITY, -INFINITY);
   float mabs = 0.f;
@@ -117,6 +121,8 @@ __global__ void __launch_bounds__(256) k_morton(const float* __restrict__ verts,
                                                 const int32_t* __restrict__ faces, int nt,
                                                 const int32_t* __restrict__ bounds, uint32_t* keys,
                                                 int32_t* vals, uint32_t* hist, int32_t* err) {
+  next_may_start();
+  after_previous();
   __shared__ uint32_t h[4 * 256];
   for (int i = threadIdx.x; i < 4 * 256; i += blockDim.x) h[i] = 0u;
   __syncthreads();
@@ -146,6 +152,8 @@ __global__ void __launch_bounds__(256) k_morton(const float* __restrict__ verts,
 __global__ void k_pack(const float* __restrict__ verts, int nv, const int32_t* __restrict__ faces,
                        int nt, const int32_t* __restrict__ order, float4* __restrict__ tris,
                        int32_t* err) {
+  next_may_start();
+  after_previous();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= nt) return;
   int f = order[i];
@@ -195,6 +203,8 @@ __device__ inline void karras_node(const KeyAt& key, int n, int i, int* left, in
 }
 
 __global__ void k_karras(const uint32_t* __restrict__ keys, int n, Node* nodes, int32_t* parent) {
+  next_may_start();
+  after_previous();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n - 1) return;
   int left, right, lo, hi;
@@ -230,6 +240,8 @@ __device__ inline Box node_box(const Node* nodes, int i) {
 __global__ void k_refit(const float4* __restrict__ tris, int n, Node* nodes,
                         const int32_t* __restrict__ parent, uint32_t* visits,
                         const int32_t* __restrict__ bounds) {
+  next_may_start();
+  after_previous();
   int l = blockIdx.x * blockDim.x + threadIdx.x;
   if (l >= n) return;
   // conservative pad: covers the FP32 ray's deviation from its FP64 source and
@@ -881,6 +893,8 @@ __device__ inline void node_children(const Node* nodes, int i, Box& l, Box& r, i
 // Entry i of the 4-wide tree: binary node i's grandchildren, then greedy
 // expansion of the largest internal slot while fewer than four slots are used.
 __global__ void k_collapse4(const Node* __restrict__ nodes, int n, Node4* __restrict__ out) {
+  next_may_start();
+  after_previous();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n - 1) return;
   Box bx[4];
@@ -1034,7 +1048,7 @@ sbr_status rebuild(sbr_scene* s, const float* verts, cudaStream_t st, bool refit
       if (refit) SBR_CUDA(cudaLaunchKernelEx(&cfg, k_build_scene<true>, verts, nv, faces, nt, B, slots, true));
       else SBR_CUDA(cudaLaunchKernelEx(&cfg, k_build_scene<false>, verts, nv, faces, nt, B, slots, true));
       ::sbr::note_launch();
-      k_collapse4<<<blocks(nt - 1, 128), 128, 0, st>>>(s->nodes, nt, s->nodes4);
+      launch_after(k_collapse4, blocks(nt - 1, 128), 128, 0, st, s->nodes, nt, s->nodes4);
       if (kTopLevels > 0) {
         ::sbr::note_launch();
         k_top_table<<<1, 128, 0, st>>>(s->nodes4, nt, s->top, s->top_n);
@@ -1049,7 +1063,7 @@ sbr_status rebuild(sbr_scene* s, const float* verts, cudaStream_t st, bool refit
     SBR_CUDA(cudaLaunchCooperativeKernel(refit ? (const void*)k_build_scene<true> : (const void*)k_build_scene<false>,
                                          dim3(blocks(nt, kBuildTile)), dim3(kBuildTile), args, build_smem(nt), st));
     ::sbr::note_launch();
-    k_collapse4<<<blocks(nt - 1, 128), 128, 0, st>>>(s->nodes, nt, s->nodes4);
+    launch_after(k_collapse4, blocks(nt - 1, 128), 128, 0, st, s->nodes, nt, s->nodes4);
     if (kTopLevels > 0) {
       ::sbr::note_launch();
       k_top_table<<<1, 128, 0, st>>>(s->nodes4, nt, s->top, s->top_n);
@@ -1058,32 +1072,30 @@ sbr_status rebuild(sbr_scene* s, const float* verts, cudaStream_t st, bool refit
     return SBR_OK;
   }
   ::sbr::note_launch();
-  k_init_bounds<<<1, 256, 0, st>>>(s->bounds, s->err, s->hist);
+  launch_after(k_init_bounds, 1, 256, 0, st, s->bounds, s->err, s->hist);
   if (nt == 0) {
     SBR_CUDA(cudaGetLastError());
     return SBR_OK;
   }
   ::sbr::note_launch();
-  k_bounds<<<blocks(nt, 256), 256, 0, st>>>(verts, nv, s->faces, nt, s->bounds, s->err);
+  launch_after(k_bounds, blocks(nt, 256), 256, 0, st, verts, nv, s->faces, nt, s->bounds, s->err);
   if (!refit) {
     ::sbr::note_launch();
-    k_morton<<<blocks(nt, 256), 256, 0, st>>>(verts, nv, s->faces, nt, s->bounds, s->keys[0],
-                                              s->vals[0], s->hist, s->err);
+    launch_after(k_morton, blocks(nt, 256), 256, 0, st, verts, nv, s->faces, nt, s->bounds, s->keys[0], s->vals[0], s->hist, s->err);
     SBR_CUDA(radix_sort_pairs(s->keys, s->vals, nt, nullptr, 31, s->sort_scratch, st, s->hist));
   }
   ::sbr::note_launch();
-  k_pack<<<blocks(nt, 256), 256, 0, st>>>(verts, nv, s->faces, nt, s->vals[0], s->tris, s->err);
+  launch_after(k_pack, blocks(nt, 256), 256, 0, st, verts, nv, s->faces, nt, s->vals[0], s->tris, s->err);
   if (nt > 1) {
     if (!refit) {
       ::sbr::note_launch();
-      k_karras<<<blocks(nt - 1, 256), 256, 0, st>>>(s->keys[0], nt, s->nodes, s->parent);
+      launch_after(k_karras, blocks(nt - 1, 256), 256, 0, st, s->keys[0], nt, s->nodes, s->parent);
     }
     SBR_CUDA(cudaMemsetAsync(s->visits, 0, sizeof(uint32_t) * (nt - 1), st));
     ::sbr::note_launch();
-    k_refit<<<blocks(nt, 256), 256, 0, st>>>(s->tris, nt, s->nodes, s->parent, s->visits,
-                                             s->bounds);
+    launch_after(k_refit, blocks(nt, 256), 256, 0, st, s->tris, nt, s->nodes, s->parent, s->visits, s->bounds);
     ::sbr::note_launch();
-    k_collapse4<<<blocks(nt - 1, 128), 128, 0, st>>>(s->nodes, nt, s->nodes4);
+    launch_after(k_collapse4, blocks(nt - 1, 128), 128, 0, st, s->nodes, nt, s->nodes4);
   }
   if (kTopLevels > 0) {
     ::sbr::note_launch();
@@ -1177,7 +1189,7 @@ extern "C" sbr_status sbr_scene_create(const float* d_verts, int32_t nv, const i
     if (e == cudaSuccess) e = cudaMemsetAsync(s->done, 0, sizeof(uint32_t), cs);
     if (e == cudaSuccess) {
       ::sbr::note_launch();
-      k_init_bounds<<<1, 256, 0, cs>>>(s->bounds, s->err, s->hist);
+      launch_after(k_init_bounds, 1, 256, 0, cs, s->bounds, s->err, s->hist);
       e = cudaGetLastError();
     }
     if (e != cudaSuccess) {

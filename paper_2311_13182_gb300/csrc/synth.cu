@@ -71,6 +71,7 @@ template <int M>
 __global__ void __launch_bounds__(kSplitThreads) k_synth_split(const float4* __restrict__ prep, int64_t cap,
                                                                const int32_t* __restrict__ d_P, int V,
                                                                int Q, int Ns, float2* __restrict__ partial) {
+  after_previous();
   __shared__ float4 sp[kChunk];
   __shared__ float4 sstep[kChunk];  // cos w, sin w, 2 cos w
   extern __shared__ float2 red[];   // [M][kSplitThreads] when G > 1
@@ -174,6 +175,7 @@ template <int MT>
 __global__ void __launch_bounds__(kMmaThreads) k_synth_mma(const float4* __restrict__ prep, int64_t cap,
                                                            const int32_t* __restrict__ d_P, int V, int Q,
                                                            float2* __restrict__ partial) {
+  after_previous();
   constexpr int Ns = 256 * MT, NU = 2 * MT;  // U values per (thread, path): a = g + 8 i
   constexpr int kWarps = kMmaThreads / 32;
   // staged records and steps; at the end the warps' sums ([warp][n][Re, Im])
@@ -341,6 +343,7 @@ __global__ void __launch_bounds__(256) k_synth_fp64(const float4* __restrict__ p
                                                     const int32_t* __restrict__ d_P, int V, int Q,
                                                     int Ns, double f0, double b_over_ns,
                                                     float2* __restrict__ partial) {
+  after_previous();
   __shared__ double2 sx[kChunk];
   __shared__ float sa[kChunk];
   const int v = blockIdx.x % V, q = blockIdx.x / V;
@@ -388,6 +391,7 @@ __global__ void __launch_bounds__(256) k_synth_naive(const float4* __restrict__ 
                                                      const int32_t* __restrict__ d_P, int V, int Q,
                                                      int Ns, float f0, float mu, float dt,
                                                      float2* __restrict__ partial) {
+  after_previous();
   __shared__ float2 sx[kChunk];
   __shared__ float so[kChunk];
   const int v = blockIdx.x % V, q = blockIdx.x / V;
@@ -428,6 +432,8 @@ __global__ void __launch_bounds__(256) k_synth_naive(const float4* __restrict__ 
 constexpr int kRedChirps = 16;
 __global__ void k_reduce(const float2* __restrict__ partial, int V, int Q, int Ns, int C,
                          float2* __restrict__ cube) {
+  next_may_start();
+  after_previous();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= V * Ns) return;
   const int v = i / Ns, n = i - v * Ns;
@@ -449,6 +455,8 @@ inline dim3 reduce_grid(int V, int Ns, int C) {
 
 __global__ void k_chirp_sum(const float2* __restrict__ g, int V, int C, int Ns,
                             float2* __restrict__ gs) {
+  next_may_start();
+  after_previous();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= V * Ns) return;
   const int v = i / Ns, n = i - v * Ns;
@@ -470,6 +478,8 @@ __global__ void __launch_bounds__(256) k_synth_bwd(const float4* __restrict__ pr
                                                    const float2* __restrict__ gs, float inv_lambda,
                                                    float b_over_cns, float* __restrict__ glen,
                                                    float* __restrict__ gamp, float* __restrict__ gphase) {
+  next_may_start();
+  after_previous();
   extern __shared__ float2 sg[];
   const int v = blockIdx.y;
   for (int n = threadIdx.x; n < Ns; n += blockDim.x) sg[n] = gs[(size_t)v * Ns + n];
@@ -633,8 +643,6 @@ __global__ void __launch_bounds__(kNuThreads, 3)
   int* grid = reinterpret_cast<int*>(nsm);                            // [npts][re, im][kNuCopies]
   float* sum = reinterpret_cast<float*>(grid + npts * 2 * kNuCopies); // [npts][re, im]: finished chunks
   const int tid = threadIdx.x, lane = tid & 31;
-  if (blockIdx.x == 0)
-    for (int i = tid; i < na.V * na.chirps; i += kNuThreads) fin_cnt[i] = 0u;  // the finishing kernel's counters
   const int cl = blockIdx.x % na.chirps, v = (blockIdx.x / na.chirps) % na.V, q = blockIdx.x / (na.chirps * na.V);
   const double dt = kMoving ? (double)(na.chirp0 + cl) * na.per_chirp : 0.0;  // path length change per (m/s)
   const float cnu = (float)(dt * na.f0_c), ceps = (float)(dt * na.b_cn);
@@ -643,6 +651,9 @@ __global__ void __launch_bounds__(kNuThreads, 3)
   for (int i = tid; i < 2 * npts; i += kNuThreads) sum[i] = 0.f;
   for (int i = tid; i < 2 * (kNuBlock / 8); i += kNuThreads) (&flag[0][0])[i] = 0;
   if (tid < 2) s_max[tid] = s_blk[tid] = 0u;
+  after_previous();
+  if (blockIdx.x == 0)
+    for (int i = tid; i < na.V * na.chirps; i += kNuThreads) fin_cnt[i] = 0u;  // the finishing kernel's counters
   if (kBlocks)
     for (int i = tid; i < M; i += kNuThreads) out[i] = make_float2(0.f, 0.f);
   const int64_t P = *d_P;
@@ -829,6 +840,8 @@ __global__ void __launch_bounds__(kNuFinThreads) k_nufft_finish(const float2* __
                                                                 float2* __restrict__ bsum,
                                                                 unsigned int* __restrict__ cnt,
                                                                 float2* __restrict__ cube, int C, bool moving) {
+  next_may_start();
+  after_previous();
   extern __shared__ float2 sg[];  // slots(M) grid, slots(M / 2) twiddles, [kNuFinThreads] per-thread sums
   __shared__ int s_last;
   const int log_m = na.log_m, M = 1 << log_m, slice = M < kNuFinSlice ? M : kNuFinSlice, S = M / slice;
@@ -909,6 +922,7 @@ constexpr int kNuClThreads = 512;
 __global__ void __cluster_dims__(kNuRanks, 1, 1) __launch_bounds__(kNuClThreads)
     k_nufft_finish_cluster(const float2* __restrict__ grids, const NufftArg na, const __grid_constant__ NufftCoef co,
                            float2* __restrict__ cube, int C, bool moving) {
+  next_may_start();
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
   extern __shared__ float2 sg[];  // slots(M) grid, slots(M / 2) twiddles, [kNuClThreads] per-thread sums, [M / 8] this eighth
@@ -920,6 +934,10 @@ __global__ void __cluster_dims__(kNuRanks, 1, 1) __launch_bounds__(kNuClThreads)
   const int parts = kNuClThreads / pts, li = tid % pts, k0 = tid / pts;  // pts <= 128
   const float2* src = grids + (size_t)row * M + rank * pts + li;
   const size_t qs = (size_t)rows * M;  // from one CTA's grid to the next
+  // this CTA's chirps of the row (of a moving scene's one chirp: all of it to CTA 0)
+  const int c0 = moving ? (rank == 0 ? 0 : 1) : C * rank / kNuRanks, c1 = moving ? 1 : C * (rank + 1) / kNuRanks;
+  if (c0 < c1) fft::fill_twiddles(tw, M, 1.f, kNuClThreads, tid);
+  after_previous();
   float2 a0 = make_float2(0.f, 0.f), a1 = a0, a2 = a0, a3 = a0;
   int q = k0;
   for (; q + 3 * parts < Q; q += 4 * parts) {  // four loads in flight, four interleaved sums
@@ -935,8 +953,6 @@ __global__ void __cluster_dims__(kNuRanks, 1, 1) __launch_bounds__(kNuClThreads)
     a0 = make_float2(a0.x + x.x, a0.y + x.y);
   }
   part[tid] = make_float2((a0.x + a1.x) + (a2.x + a3.x), (a0.y + a1.y) + (a2.y + a3.y));
-  const int c0 = moving ? (rank == 0 ? 0 : 1) : C * rank / kNuRanks, c1 = moving ? 1 : C * (rank + 1) / kNuRanks;
-  if (c0 < c1) fft::fill_twiddles(tw, M, 1.f, kNuClThreads, tid);
   __syncthreads();
   if (tid < pts) {
     float2 acc = part[tid];
@@ -1052,6 +1068,7 @@ constexpr int kAdjMargin = kNuW;  // the grid is stored with its wrap-around: en
 __global__ void __launch_bounds__(kAdjThreads) k_adj_grid(const float2* __restrict__ g, int V, int C, int Ns, int log_m,
                                                           float slope, const __grid_constant__ NufftCoef co,
                                                           float2* __restrict__ out) {
+  next_may_start();
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
   extern __shared__ float2 sa[];  // [N_s] this CTA's chirps summed, slots(M) grid, slots(M / 2) twiddles
@@ -1060,6 +1077,11 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_grid(const float2* __restri
   float2* s = sa + Ns;
   float2* tw = s + fft::slots(M);
   const int c0 = C * rank / ranks, c1 = C * (rank + 1) / ranks;
+  if (rank < 2) {
+    fft::fill_twiddles(tw, M, 1.f, kAdjThreads, threadIdx.x);
+    for (int i = threadIdx.x; i < fft::slots(M); i += kAdjThreads) s[i] = make_float2(0.f, 0.f);
+  }
+  after_previous();
   for (int n = threadIdx.x; n < Ns; n += kAdjThreads) {
     float2 a = make_float2(0.f, 0.f);
 #pragma unroll 8
@@ -1069,10 +1091,6 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_grid(const float2* __restri
       a.y += x.y;
     }
     sa[n] = a;
-  }
-  if (rank < 2) {
-    fft::fill_twiddles(tw, M, 1.f, kAdjThreads, threadIdx.x);
-    for (int i = threadIdx.x; i < fft::slots(M); i += kAdjThreads) s[i] = make_float2(0.f, 0.f);
   }
   cluster.sync();
   if (rank < 2) {
@@ -1107,6 +1125,7 @@ __global__ void __launch_bounds__(256) k_synth_bwd_nufft(const float4* __restric
                                                          const float4* __restrict__ grid, float inv_lambda,
                                                          float* __restrict__ glen, float* __restrict__ gamp,
                                                          float* __restrict__ gphase) {
+  after_previous();
   const int v = blockIdx.y, M = 1 << log_m, P = *d_P;
   const float m = (float)M, half_n = 0.25f * m;
   const size_t row = (size_t)v * cap;
@@ -1403,17 +1422,15 @@ void launch_nufft(sbr_phase_mode mode, const sbr_paths* p, const sbr_radar_cfg* 
   const float2* plen = reinterpret_cast<const float2*>(p->path_len);
   const int grid = V * Q * chirps;
   ::sbr::note_launch();
-  nufft_kernel(Ns, mode == SBR_PHASE_FP64, moving)<<<grid, kNuThreads, nufft_smem(Ns), st>>>(
-      prep, plen, p->phase_ofs, p->path_rate, p->path_cap, p->count, na, co, w.grids, w.fin_cnt);
+  launch_after(nufft_kernel(Ns, mode == SBR_PHASE_FP64, moving), grid, kNuThreads, nufft_smem(Ns), st, prep, plen,
+               p->phase_ofs, p->path_rate, p->path_cap, p->count, na, co, w.grids, w.fin_cnt);
   ::sbr::note_launch();
   if (M <= kNuClusterPoints) {
-    k_nufft_finish_cluster<<<V * chirps * kNuRanks, kNuClThreads, nufft_cl_smem(Ns), st>>>(w.grids, na, co, cube,
-                                                                                          r->n_chirps, moving);
+    launch_after(k_nufft_finish_cluster, V * chirps * kNuRanks, kNuClThreads, nufft_cl_smem(Ns), st, w.grids, na, co, cube, r->n_chirps, moving);
     return;
   }
   const int slices = M / kNuFinSlice;
-  k_nufft_finish<<<V * chirps * slices, kNuFinThreads, nufft_fin_smem(Ns), st>>>(w.grids, na, co, w.bsum, w.fin_cnt, cube,
-                                                                                r->n_chirps, moving);
+  launch_after(k_nufft_finish, V * chirps * slices, kNuFinThreads, nufft_fin_smem(Ns), st, w.grids, na, co, w.bsum, w.fin_cnt, cube, r->n_chirps, moving);
 }
 
 // A moving scene: every chirp synthesised from its own delays (split phase up to 512
@@ -1455,22 +1472,18 @@ void launch_fwd(sbr_phase_mode mode, const sbr_paths* p, const sbr_radar_cfg* r,
   const float4* prep = reinterpret_cast<const float4*>(p->prep);
   if (mode == SBR_PHASE_SPLIT && (Ns == 256 || Ns == 512)) {
     ::sbr::note_launch();
-    if (Ns == 256) k_synth_mma<1><<<grid, kMmaThreads, 0, st>>>(prep, p->path_cap, p->count, V, w.Q, w.partial);
-    else k_synth_mma<2><<<grid, kMmaThreads, 0, st>>>(prep, p->path_cap, p->count, V, w.Q, w.partial);
+    if (Ns == 256) launch_after(k_synth_mma<1>, grid, kMmaThreads, 0, st, prep, p->path_cap, p->count, V, w.Q, w.partial);
+    else launch_after(k_synth_mma<2>, grid, kMmaThreads, 0, st, prep, p->path_cap, p->count, V, w.Q, w.partial);
   } else if (mode == SBR_PHASE_SPLIT) {
     ::sbr::note_launch();
-    k_synth_split<M><<<grid, kSplitThreads, split_smem(Ns), st>>>(prep, p->path_cap, p->count, V, w.Q, Ns,
-                                                                   w.partial);
+    launch_after(k_synth_split<M>, grid, kSplitThreads, split_smem(Ns), st, prep, p->path_cap, p->count, V, w.Q, Ns, w.partial);
   } else if (mode == SBR_PHASE_FP64) {
     ::sbr::note_launch();
-    k_synth_fp64<M><<<grid, T, 0, st>>>(prep, reinterpret_cast<const float2*>(p->path_len), p->phase_ofs,
-                                        p->path_cap, p->count, V, w.Q, Ns, r->f0, r->bandwidth / Ns, w.partial);
+    launch_after(k_synth_fp64<M>, grid, T, 0, st, prep, reinterpret_cast<const float2*>(p->path_len), p->phase_ofs, p->path_cap, p->count, V, w.Q, Ns, r->f0, r->bandwidth / Ns, w.partial);
   } else {
     const double mu = r->bandwidth / r->chirp_time, dt = r->chirp_time / Ns;
     ::sbr::note_launch();
-    k_synth_naive<M><<<grid, T, 0, st>>>(prep, reinterpret_cast<const float2*>(p->path_len), p->phase_ofs,
-                                         p->path_cap, p->count, V, w.Q, Ns, (float)r->f0, (float)mu, (float)dt,
-                                         w.partial);
+    launch_after(k_synth_naive<M>, grid, T, 0, st, prep, reinterpret_cast<const float2*>(p->path_len), p->phase_ofs, p->path_cap, p->count, V, w.Q, Ns, (float)r->f0, (float)mu, (float)dt, w.partial);
   }
 }
 }  // namespace
@@ -1514,8 +1527,7 @@ extern "C" sbr_status sbr_synthesize(const sbr_paths* paths, const sbr_radar_cfg
   SBR_CUDA(cudaGetLastError());
   const int V = paths->n_virt;
   ::sbr::note_launch();
-  k_reduce<<<reduce_grid(V, Ns, radar->n_chirps), 256, 0, st>>>(w.partial, V, w.Q, Ns, radar->n_chirps,
-                                                  reinterpret_cast<float2*>(d_cube));
+  launch_after(k_reduce, reduce_grid(V, Ns, radar->n_chirps), 256, 0, st, w.partial, V, w.Q, Ns, radar->n_chirps, reinterpret_cast<float2*>(d_cube));
   SBR_CUDA(cudaGetLastError());
   return SBR_OK;
 }
@@ -1590,8 +1602,7 @@ extern "C" sbr_status sbr_synthesize_noalloc(const sbr_paths* paths, const sbr_r
   }
   SBR_CUDA(cudaGetLastError());
   ::sbr::note_launch();
-  k_reduce<<<reduce_grid(V, Ns, radar->n_chirps), 256, 0, st>>>(w.partial, V, w.Q, Ns, radar->n_chirps,
-                                                  reinterpret_cast<float2*>(d_cube));
+  launch_after(k_reduce, reduce_grid(V, Ns, radar->n_chirps), 256, 0, st, w.partial, V, w.Q, Ns, radar->n_chirps, reinterpret_cast<float2*>(d_cube));
   SBR_CUDA(cudaGetLastError());
   return SBR_OK;
 }
@@ -1614,17 +1625,19 @@ extern "C" sbr_status sbr_synthesize_bwd(const sbr_paths* paths, const sbr_radar
     while ((1 << log_m) < 2 * Ns) ++log_m;
     SBR_CUDA(adj_attr(Ns));
     cudaLaunchConfig_t lc{};
-    cudaLaunchAttribute at{};
+    cudaLaunchAttribute at[2] = {};
     const unsigned ranks = C >= 8 ? 8 : 2;
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = ranks;
-    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = ranks;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // as launch_after
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     lc.gridDim = dim3(V * ranks);
     lc.blockDim = dim3(kAdjThreads);
     lc.dynamicSmemBytes = adj_smem(Ns);
     lc.stream = st;
-    lc.attrs = &at;
-    lc.numAttrs = 1;
+    lc.attrs = at;
+    lc.numAttrs = 2;
     const NufftCoef& co = nufft_coef();
     ::sbr::note_launch();
     SBR_CUDA(cudaLaunchKernelEx(&lc, k_adj_grid, reinterpret_cast<const float2*>(d_gcube), V, C, Ns, log_m,
@@ -1632,9 +1645,7 @@ extern "C" sbr_status sbr_synthesize_bwd(const sbr_paths* paths, const sbr_radar
     // a wave of CTAs at most, at least one per antenna
     const int64_t need = (paths->path_cap + 255) / 256, wave = std::max(1, 8 * sm_count() / V);
     ::sbr::note_launch();
-    k_synth_bwd_nufft<<<dim3((unsigned)std::min(need, wave), V), 256, 0, st>>>(
-        reinterpret_cast<const float4*>(paths->prep), paths->path_cap, paths->count, log_m, co, w.adj, (float)lam_inv,
-        d_glen, d_gamp, d_gphase);
+    launch_after(k_synth_bwd_nufft, dim3((unsigned)std::min(need, wave), V), 256, 0, st, reinterpret_cast<const float4*>(paths->prep), paths->path_cap, paths->count, log_m, co, w.adj, (float)lam_inv, d_glen, d_gamp, d_gphase);
     SBR_CUDA(cudaGetLastError());
     return SBR_OK;
   }
@@ -1642,7 +1653,7 @@ extern "C" sbr_status sbr_synthesize_bwd(const sbr_paths* paths, const sbr_radar
   const float2* gs = reinterpret_cast<const float2*>(d_gcube);
   if (C > 1) {
     ::sbr::note_launch();
-    k_chirp_sum<<<(V * Ns + 255) / 256, 256, 0, st>>>(gs, V, C, Ns, w.gsum);
+    launch_after(k_chirp_sum, (V * Ns + 255) / 256, 256, 0, st, gs, V, C, Ns, w.gsum);
     gs = w.gsum;
   }
   const int64_t cap = paths->path_cap;
@@ -1650,9 +1661,7 @@ extern "C" sbr_status sbr_synthesize_bwd(const sbr_paths* paths, const sbr_radar
     dim3 grid((unsigned)((cap + 255) / 256), (unsigned)V);
     const double bcn = radar->bandwidth / (kC * Ns);
     ::sbr::note_launch();
-    k_synth_bwd<<<grid, 256, Ns * sizeof(float2), st>>>(
-        reinterpret_cast<const float4*>(paths->prep), cap, paths->count, Ns, gs,
-        (float)lam_inv, (float)bcn, d_glen, d_gamp, d_gphase);
+    launch_after(k_synth_bwd, grid, 256, Ns * sizeof(float2), st, reinterpret_cast<const float4*>(paths->prep), cap, paths->count, Ns, gs, (float)lam_inv, (float)bcn, d_glen, d_gamp, d_gphase);
   }
   SBR_CUDA(cudaGetLastError());
   return SBR_OK;

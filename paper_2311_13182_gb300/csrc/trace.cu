@@ -576,6 +576,7 @@ __global__ void __launch_bounds__(128, SBR_TRACE_MIN_BLOCKS) k_trace(const float
                                                RayDump* __restrict__ dumps, unsigned int* __restrict__ n_dumps,
                                                unsigned long long* __restrict__ counts,
                                                const Node4* __restrict__ top, const int32_t* __restrict__ top_n) {
+  after_previous();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   int n_nodes = 0, n_tris = 0, n_trav = 0;
   if (kTopLevels > 0) {  // every thread of the CTA, before any may return
@@ -759,6 +760,7 @@ __global__ void __launch_bounds__(128) k_trace_coop(const float4* __restrict__ t
                                                     unsigned int* __restrict__ work, sbr_hit* __restrict__ hits,
                                                     float4* __restrict__ hit_pos, int32_t* __restrict__ nvalid,
                                                     unsigned long long* __restrict__ counts) {
+  after_previous();
   __shared__ int lists[4][kCoopList];
   const int lane = threadIdx.x & 31;
   int* list = lists[threadIdx.x >> 5];
@@ -852,6 +854,8 @@ __global__ void __launch_bounds__(128) k_trace_warp(const float4* __restrict__ t
                                                     sbr_hit* __restrict__ hits, float4* __restrict__ hit_pos,
                                                     float* __restrict__ ray_w, int32_t* __restrict__ nvalid,
                                                     unsigned long long* __restrict__ counts) {
+  next_may_start();
+  after_previous();
   __shared__ int lists[4][kCoopList];
   const int lane = threadIdx.x & 31;
   int* list = lists[threadIdx.x >> 5];
@@ -927,6 +931,7 @@ __global__ void k_prep(const float4* __restrict__ hit_pos, const sbr_hit* __rest
                        RadarArg rd, MatArg mat, MotionArg mot, int64_t cap, float4* __restrict__ prep,
                        float2* __restrict__ plen, int32_t* __restrict__ path_ray, float* __restrict__ phase_ofs,
                        float* __restrict__ path_rate) {
+  after_previous();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int lane = threadIdx.x & 31;
   int p0 = 0, nh = 0;
@@ -1058,29 +1063,19 @@ void launch_prep(int nb, cudaStream_t st, const float4* hp4, const sbr_paths* pa
                  const RadarArg& rd, const MatArg& mat, const MotionArg& mot, float4* prep, float2* plen) {
   switch (rd.ntx) {
     case 1:
-      k_prep<1, kMotion><<<nb, 128, 0, st>>>(hp4, paths->hits, paths->ray_weight, paths->ray_first, (int)R, K, rd,
-                                              mat, mot, paths->path_cap, prep, plen, paths->path_ray,
-                                              paths->phase_ofs, paths->path_rate);
+      launch_after(k_prep<1, kMotion>, nb, 128, 0, st, hp4, paths->hits, paths->ray_weight, paths->ray_first, (int)R, K, rd, mat, mot, paths->path_cap, prep, plen, paths->path_ray, paths->phase_ofs, paths->path_rate);
       break;
     case 2:
-      k_prep<2, kMotion><<<nb, 128, 0, st>>>(hp4, paths->hits, paths->ray_weight, paths->ray_first, (int)R, K, rd,
-                                              mat, mot, paths->path_cap, prep, plen, paths->path_ray,
-                                              paths->phase_ofs, paths->path_rate);
+      launch_after(k_prep<2, kMotion>, nb, 128, 0, st, hp4, paths->hits, paths->ray_weight, paths->ray_first, (int)R, K, rd, mat, mot, paths->path_cap, prep, plen, paths->path_ray, paths->phase_ofs, paths->path_rate);
       break;
     case 3:
-      k_prep<3, kMotion><<<nb, 128, 0, st>>>(hp4, paths->hits, paths->ray_weight, paths->ray_first, (int)R, K, rd,
-                                              mat, mot, paths->path_cap, prep, plen, paths->path_ray,
-                                              paths->phase_ofs, paths->path_rate);
+      launch_after(k_prep<3, kMotion>, nb, 128, 0, st, hp4, paths->hits, paths->ray_weight, paths->ray_first, (int)R, K, rd, mat, mot, paths->path_cap, prep, plen, paths->path_ray, paths->phase_ofs, paths->path_rate);
       break;
     case 4:
-      k_prep<4, kMotion><<<nb, 128, 0, st>>>(hp4, paths->hits, paths->ray_weight, paths->ray_first, (int)R, K, rd,
-                                              mat, mot, paths->path_cap, prep, plen, paths->path_ray,
-                                              paths->phase_ofs, paths->path_rate);
+      launch_after(k_prep<4, kMotion>, nb, 128, 0, st, hp4, paths->hits, paths->ray_weight, paths->ray_first, (int)R, K, rd, mat, mot, paths->path_cap, prep, plen, paths->path_ray, paths->phase_ofs, paths->path_rate);
       break;
     default:
-      k_prep<0, kMotion><<<nb, 128, 0, st>>>(hp4, paths->hits, paths->ray_weight, paths->ray_first, (int)R, K, rd,
-                                              mat, mot, paths->path_cap, prep, plen, paths->path_ray,
-                                              paths->phase_ofs, paths->path_rate);
+      launch_after(k_prep<0, kMotion>, nb, 128, 0, st, hp4, paths->hits, paths->ray_weight, paths->ray_first, (int)R, K, rd, mat, mot, paths->path_cap, prep, plen, paths->path_ray, paths->phase_ofs, paths->path_rate);
   }
 }
 
@@ -1238,36 +1233,26 @@ static sbr_status trace_impl(const sbr_scene* scene, const sbr_radar_cfg* radar,
   }
   RayDump* dumps = dump_records(paths);
   unsigned int* dctr = dump_counters(paths);
-  SBR_CUDA(cudaMemsetAsync(dctr, 0, 2 * sizeof(unsigned int), st));
+  if (R > kWarpRaysMax) SBR_CUDA(cudaMemsetAsync(dctr, 0, 2 * sizeof(unsigned int), st));  // the hand-over's
   float4* hp = reinterpret_cast<float4*>(paths->hit_pos);
   if (d_counts) SBR_CUDA(cudaMemsetAsync(d_counts, 0, 4 * sizeof(unsigned long long), st));
   if (R <= kWarpRaysMax) {  // one warp per ray (no hand-over needed)
     const int nbw = blocks(R * 32, 128);
     ::sbr::note_launch();
     if (d_counts)
-      k_trace_warp<true><<<nbw, 128, 0, st>>>(scene->tris, scene->nodes4, scene->nt, g, d_ray_ids, (int)R,
-                                               max_bounces, paths->hits, hp, paths->ray_weight, paths->ray_first,
-                                               d_counts);
+      launch_after(k_trace_warp<true>, nbw, 128, 0, st, scene->tris, scene->nodes4, scene->nt, g, d_ray_ids, (int)R, max_bounces, paths->hits, hp, paths->ray_weight, paths->ray_first, d_counts);
     else
-      k_trace_warp<false><<<nbw, 128, 0, st>>>(scene->tris, scene->nodes4, scene->nt, g, d_ray_ids, (int)R,
-                                                max_bounces, paths->hits, hp, paths->ray_weight, paths->ray_first,
-                                                nullptr);
+      launch_after(k_trace_warp<false>, nbw, 128, 0, st, scene->tris, scene->nodes4, scene->nt, g, d_ray_ids, (int)R, max_bounces, paths->hits, hp, paths->ray_weight, paths->ray_first, nullptr);
   } else if (d_counts) {
     ::sbr::note_launch();
-    k_trace<true><<<blocks(R, 128), 128, 0, st>>>(scene->tris, scene->nodes4, scene->nt, g, d_ray_ids, (int)R,
-                                                  max_bounces, paths->hits, hp, paths->ray_weight, paths->ray_first,
-                                                  dumps, dctr, d_counts, scene->top, scene->top_n);
+    launch_after(k_trace<true>, blocks(R, 128), 128, 0, st, scene->tris, scene->nodes4, scene->nt, g, d_ray_ids, (int)R, max_bounces, paths->hits, hp, paths->ray_weight, paths->ray_first, dumps, dctr, d_counts, scene->top, scene->top_n);
     ::sbr::note_launch();
-    k_trace_coop<true><<<coop_grid(), 128, 0, st>>>(scene->tris, scene->nodes4, scene->nt, g, max_bounces, dumps,
-                                                    dctr, dctr + 1, paths->hits, hp, paths->ray_first, d_counts);
+    launch_after(k_trace_coop<true>, coop_grid(), 128, 0, st, scene->tris, scene->nodes4, scene->nt, g, max_bounces, dumps, dctr, dctr + 1, paths->hits, hp, paths->ray_first, d_counts);
   } else {
     ::sbr::note_launch();
-    k_trace<false><<<blocks(R, 128), 128, 0, st>>>(scene->tris, scene->nodes4, scene->nt, g, d_ray_ids, (int)R,
-                                                   max_bounces, paths->hits, hp, paths->ray_weight,
-                                                   paths->ray_first, dumps, dctr, nullptr, scene->top, scene->top_n);
+    launch_after(k_trace<false>, blocks(R, 128), 128, 0, st, scene->tris, scene->nodes4, scene->nt, g, d_ray_ids, (int)R, max_bounces, paths->hits, hp, paths->ray_weight, paths->ray_first, dumps, dctr, nullptr, scene->top, scene->top_n);
     ::sbr::note_launch();
-    k_trace_coop<false><<<coop_grid(), 128, 0, st>>>(scene->tris, scene->nodes4, scene->nt, g, max_bounces, dumps,
-                                                     dctr, dctr + 1, paths->hits, hp, paths->ray_first, nullptr);
+    launch_after(k_trace_coop<false>, coop_grid(), 128, 0, st, scene->tris, scene->nodes4, scene->nt, g, max_bounces, dumps, dctr, dctr + 1, paths->hits, hp, paths->ray_first, nullptr);
   }
   SBR_CUDA(cudaGetLastError());
   SBR_CUDA(exclusive_scan(paths->ray_first, paths->ray_first, R, nullptr, paths->scratch, st));

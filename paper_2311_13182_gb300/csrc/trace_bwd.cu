@@ -282,6 +282,7 @@ __global__ void __launch_bounds__(128) k_trace_bwd(
     const float4* __restrict__ hit_pos, const int32_t* __restrict__ first,
     const float4* __restrict__ prep, int64_t cap, const float* __restrict__ glen,
     const float* __restrict__ gamp, const float* __restrict__ gphase, bool reparam, FixScatter fs, FixScatter fe) {
+  after_previous();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int E = kPass == 0 ? 0 : fix_exp(*fs.max_bits, fs.log2n);
   const int Ee = kPass == 0 ? 0 : fix_exp(*fe.max_bits, fe.log2n);
@@ -297,6 +298,8 @@ __global__ void __launch_bounds__(128) k_trace_bwd(
 
 // gverts[i] += acc[i] 2^-E
 __global__ void k_fix_finish_add(FixScatter fs, int n, float* __restrict__ gverts) {
+  next_may_start();
+  after_previous();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   gverts[i] += fix_get(fs.acc[i], fix_exp(*fs.max_bits, fs.log2n));
@@ -383,21 +386,17 @@ extern "C" sbr_status sbr_trace_bwd(const sbr_scene* scene, const float* d_verts
   const float4* hp = reinterpret_cast<const float4*>(paths->hit_pos);
   const float4* pr = reinterpret_cast<const float4*>(paths->prep);
   ::sbr::note_launch();
-  k_trace_bwd<0><<<(R + 127) / 128, 128, 0, st>>>(d_verts, scene->nv, scene->faces, g, rd, mat, d_ray_ids, R,
-                                                   paths->max_bounces, paths->hits, hp, paths->ray_first, pr,
-                                                   paths->path_cap, d_glen, d_gamp, d_gphase, reparam, w.fs, w.fe);
+  launch_after(k_trace_bwd<0>, (R + 127) / 128, 128, 0, st, d_verts, scene->nv, scene->faces, g, rd, mat, d_ray_ids, R, paths->max_bounces, paths->hits, hp, paths->ray_first, pr, paths->path_cap, d_glen, d_gamp, d_gphase, reparam, w.fs, w.fe);
   ::sbr::note_launch();
-  k_trace_bwd<1><<<(R + 127) / 128, 128, 0, st>>>(d_verts, scene->nv, scene->faces, g, rd, mat, d_ray_ids, R,
-                                                   paths->max_bounces, paths->hits, hp, paths->ray_first, pr,
-                                                   paths->path_cap, d_glen, d_gamp, d_gphase, reparam, w.fs, w.fe);
+  launch_after(k_trace_bwd<1>, (R + 127) / 128, 128, 0, st, d_verts, scene->nv, scene->faces, g, rd, mat, d_ray_ids, R, paths->max_bounces, paths->hits, hp, paths->ray_first, pr, paths->path_cap, d_glen, d_gamp, d_gphase, reparam, w.fs, w.fe);
   const int n3 = 3 * scene->nv;
   if (n3 > 0) {
     ::sbr::note_launch();
-    k_fix_finish_add<<<(n3 + 255) / 256, 256, 0, st>>>(w.fs, n3, d_gverts);
+    launch_after(k_fix_finish_add, (n3 + 255) / 256, 256, 0, st, w.fs, n3, d_gverts);
   }
   if (mat.n > 0 && d_geps) {
     ::sbr::note_launch();
-    k_fix_finish_add<<<1, 64, 0, st>>>(w.fe, 2 * mat.n, d_geps);
+    launch_after(k_fix_finish_add, 1, 64, 0, st, w.fe, 2 * mat.n, d_geps);
   }
   SBR_CUDA(cudaGetLastError());
   return SBR_OK;
