@@ -37,3 +37,24 @@ def test_few_rays_match_many(sbr, kind, n):
     assert torch.equal(few.hit_pos(), full.hit_pos()[at])
     assert torch.equal(few.ray_weight(), full.ray_weight()[at])
     assert few.count() == int((few.hits()[0] >= 0).sum())
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 31, 33, 500, 512, 513, 1023, 1024])
+def test_one_tile_build(sbr, n):
+    """A mesh of at most 1024 triangles (one sort in one CTA) against the same triangles with others
+    behind the radar added (several tiles): the same hits."""
+    v, f, _ = superquadric(8, 24, 24, center=(0.0, 0.0, 1.0))
+    f = f[np.random.default_rng(n).permutation(len(f))[:n]]
+    w, g = icosphere(3, 0.2, (0.0, 0.0, -1.0))
+    both = merge_meshes((v, f), (w, g))
+    radar = radar_single_tx(256, 1)
+    grid = ray_grid_for_sphere((0.0, 0.0, 1.0), 0.5, 100)
+    out = []
+    for mesh_v, mesh_f in ((v, f), both):
+        scene = sbr.Scene(torch.from_numpy(mesh_v).cuda(), torch.from_numpy(mesh_f).cuda())
+        out.append(sbr.trace(scene, radar, grid, 3))
+        scene.check()
+    hit = out[0].hits()[0]
+    same = (hit == out[1].hits()[0]).all(1)  # a ray reflected back may meet the others
+    assert bool((same | (out[1].hits()[0] >= n).any(1)).all())
+    assert n < 500 or bool((hit >= 0).any())
