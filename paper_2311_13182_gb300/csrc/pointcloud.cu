@@ -74,9 +74,19 @@ __global__ void k_fft_cols(float2* __restrict__ x, int C, int logc, int Ns, floa
   float2* base = x + (size_t)v * C * Ns + k0;
   fill_twiddles(tw, C, sign, blockDim.x, threadIdx.x);
   after_previous();
-  for (int i = threadIdx.x; i < C * kColTile; i += blockDim.x) {
-    const int c = i / kColTile, kk = i - c * kColTile;
-    s[kk * ld + slot(bitrev(c, logc))] = base[(size_t)c * Ns + kk];
+  constexpr int kAhead = 8;  // loads in flight per thread
+  for (int i0 = threadIdx.x; i0 < C * kColTile; i0 += kAhead * blockDim.x) {
+    float2 y[kAhead];
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+      const int i = i0 + u * blockDim.x, c = i / kColTile;
+      y[u] = i < C * kColTile ? base[(size_t)c * Ns + (i - c * kColTile)] : make_float2(0.f, 0.f);
+    }
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+      const int i = i0 + u * blockDim.x, c = i / kColTile;
+      if (i < C * kColTile) s[(i - c * kColTile) * ld + slot(bitrev(c, logc))] = y[u];
+    }
   }
   __syncthreads();
   smem_fft_rows<true>(s, ld, kLogColTile, tw, logc, blockDim.x, threadIdx.x);
@@ -369,10 +379,19 @@ __device__ inline void noise_cells(const CfarArg& c, int k, int& lo0, int& lo1, 
 __device__ inline float cfar_noise(const float* __restrict__ row, const CfarArg& c, int k, int* cnt) {
   int lo0, lo1, hi0, hi1;
   noise_cells(c, k, lo0, lo1, hi0, hi1);
+  const int nl = max(lo1 - lo0, 0), n = nl + max(hi1 - hi0, 0);
   float s = 0.f;
-  int n = 0;
-  for (int j = lo0; j < lo1; ++j, ++n) s += row[j];
-  for (int j = hi0; j < hi1; ++j, ++n) s += row[j];
+  constexpr int kAhead = 16;  // cells in flight, added in order
+  for (int j0 = 0; j0 < n; j0 += kAhead) {
+    float y[kAhead];
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+      const int j = j0 + u;
+      y[u] = j < n ? row[j < nl ? lo0 + j : hi0 + (j - nl)] : 0.f;
+    }
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) s += y[u];
+  }
   *cnt = n;
   return n ? s / (float)n : 0.f;
 }
@@ -395,19 +414,23 @@ __device__ inline uint32_t detect_key(const float* __restrict__ Pw, const CfarAr
   const int e = rho / c.A, a = rho - e * c.A;
   const float p = Pw[i];
   bool peak = p > floor_v;
-  for (int de = -1; de <= 1 && peak; ++de)
-    for (int da = -1; da <= 1 && peak; ++da)
-      for (int dk = -1; dk <= 1; ++dk) {
-        if (de == 0 && da == 0 && dk == 0) continue;
-        const int ee = e + de, aa = a + da, kk = k + dk;
-        if (ee < 0 || ee >= c.E || aa < 0 || aa >= c.A || kk < 0 || kk >= c.Ns) continue;
-        const int j = ((ee * c.A) + aa) * c.Ns + kk;
-        const float q = Pw[j];
-        if (j < i ? !(p > q) : !(p >= q)) {
-          peak = false;
-          break;
-        }
-      }
+  if (!peak) return 0xffffffffu;
+  for (int de = c.E > 1 ? -1 : 0; de <= (c.E > 1 ? 1 : 0) && peak; ++de) {
+    const int ee = e + de;
+    if (ee < 0 || ee >= c.E) continue;
+    float q[9];  // the bin's 3 x 3 cells in flight together
+#pragma unroll
+    for (int u = 0; u < 9; ++u) {
+      const int aa = a + u / 3 - 1, kk = k + u % 3 - 1;
+      const bool in = aa >= 0 && aa < c.A && kk >= 0 && kk < c.Ns;
+      q[u] = in ? Pw[(ee * c.A + aa) * c.Ns + kk] : -INFINITY;
+    }
+#pragma unroll
+    for (int u = 0; u < 9; ++u) {
+      const int j = (ee * c.A + a + u / 3 - 1) * c.Ns + k + u % 3 - 1;
+      if (q[u] != -INFINITY && j != i && (j < i ? !(p > q[u]) : !(p >= q[u]))) peak = false;
+    }
+  }
   if (!peak) return 0xffffffffu;
   int cnt;
   const float w = soft_w(Pw, c, rho, k, floor_v, nullptr, nullptr, &cnt);
