@@ -826,6 +826,156 @@ __global__ void __launch_bounds__(kNuThreads, 3)
   }
 }
 
+// The split phase of a moving scene whose grid a CTA holds whole: CTA (q, v) spreads
+// its records for the launch's chirps, up to kTile.  From one chirp to the next a
+// record's phasor turns by a constant and its grid position moves by a constant, so the
+// preparation (two sines, the split phase) is paid once per tile, from that chirp's own
+// delays, and a chirp costs a complex product and the sixteen additions: 12 antennas x
+// 367,500 records x 128 chirps 3.5 ms
+// against 5.0 in groups chirp by chirp (8 chirps at a time 3.9, 4 at a time 4.6; a
+// third of it adds the chunks' copies up).  The rounding of up to kTile - 1 turns adds
+// about 1e-7.  A chunk's sums go to the chirp's grid in global memory (L2), each
+// point by one thread; kTile copies in shared memory would cost a resident CTA.
+constexpr int kTile = 16;  // chirps per launch
+__global__ void __launch_bounds__(kNuThreads, 3)
+    k_nufft_spread_chirps(const float4* __restrict__ prep, const float* __restrict__ rate, int64_t cap,
+                          const int32_t* __restrict__ d_P, const NufftArg na, const __grid_constant__ NufftCoef co, float2* __restrict__ grids) {
+  extern __shared__ int4 nsm[];  // [npts][re, im][kNuCopies]
+  __shared__ uint32_t s_max[2];
+  __shared__ int flag[2][kNuBlock / 8];
+  const int M = 1 << na.log_m, npts = nu_points(M), oct = M >> 3;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int v = blockIdx.x % na.V, q = blockIdx.x / na.V, nc = na.chirps;
+  const double dt = (double)na.chirp0 * na.per_chirp;  // path length change per (m/s)
+  const float cnu = (float)(dt * na.f0_c), ceps = (float)(dt * na.b_cn);
+  const float turn = (float)(na.per_chirp * na.cyc), move = (float)(na.per_chirp * na.cell);  // per (m/s) and chirp
+  float2* out = grids + (size_t)(q * na.V + v) * nc * M;
+  for (int i = tid; i < npts * (2 * kNuCopies / 4); i += kNuThreads) nsm[i] = make_int4(0, 0, 0, 0);
+  for (int i = tid; i < 2 * (kNuBlock / 8); i += kNuThreads) (&flag[0][0])[i] = 0;
+  if (tid < 2) s_max[tid] = 0u;
+  after_previous();
+  for (int i = tid; i < nc * M; i += kNuThreads) out[i] = make_float2(0.f, 0.f);
+  const int64_t P = *d_P;
+  const int64_t r0 = P * q / na.Q;
+  const int n = (int)(P * (q + 1) / na.Q - r0);
+  const size_t at = (size_t)v * cap + r0;
+  const bool upper = lane >= 16;
+  int* mine = reinterpret_cast<int*>(nsm) + (lane & 15);
+  int pass = 0;
+  bool bad = false;  // a record that is not finite: the antenna's samples are NaN
+  __syncthreads();
+  for (int c0 = 0, chunk = 0; c0 < n; c0 += kNuChunk, ++chunk) {
+    float c1[kNuItems], c2[kNuItems], wr[kNuItems], wi[kNuItems], s[kNuItems], ds[kNuItems];
+    int cell[kNuItems];
+    uint32_t am = 0;
+#pragma unroll
+    for (int u = 0; u < kNuItems; ++u) {
+      const int p = c0 + tid + u * kNuThreads;
+      const float4 r = p < n ? __ldg(&prep[at + p]) : make_float4(0.f, 0.f, 0.f, 0.f);
+      const float ld = p < n ? __ldg(&rate[at + p]) : 0.f;
+      // the tile's first chirp: phi0 + dL/dt cnu and delta + dL/dt ceps, whole multiples of
+      // 2^-12 of the delta shift moved into delta_hi (which stays exact)
+      const float ph = fmaf(ld, cnu, r.x);
+      const float dl = fmaf(ld, ceps, r.z), kq = rintf(dl * 4096.f);
+      float dh = r.y + kq * (1.f / 4096.f);
+      dh -= rintf(dh);
+      const float dlo = dl - kq * (1.f / 4096.f);
+      float x = na.half_n * dh;  // exact
+      x -= rintf(x);
+      x = fmaf(na.half_n, dlo, x) + (ph - rintf(ph));
+      const float uh = na.m * dh;  // exact
+      float fl = floorf(uh);
+      float t = fmaf(na.m, dlo, uh - fl);
+      int ce = (int)fl;
+      bad |= !isfinite(x + t + r.w + ld);
+      fl = floorf(t);
+      s[u] = (t - fl) - 0.5f;
+      cell[u] = (ce + (int)fl) & (M - 1);
+      ds[u] = ld * move;
+      float sn, cs;
+      sincospif(2.f * x, &sn, &cs);
+      // the lower half of a warp adds real parts first, the upper imaginary ones: with the turn's
+      // sine negated, the swapped pair turns by the same formula
+      c1[u] = r.w * (upper ? sn : cs);
+      c2[u] = r.w * (upper ? cs : sn);
+      sincospif(2.f * (ld * turn), &sn, &cs);
+      wr[u] = cs;
+      wi[u] = upper ? -sn : sn;
+      am = max(am, __float_as_uint(fabsf(r.w)));
+    }
+    am = __reduce_max_sync(0xffffffffu, am);
+    if (lane == 0) atomicMax(&s_max[chunk & 1], am);
+    __syncthreads();
+    const float top = fmaxf(__uint_as_float(s_max[chunk & 1]), 1e-20f);  // terms up to 0.98 2^kNuBits
+    const float scale = 0.98f * (float)(1 << kNuBits) / top, unit = top * (1.f / (0.98f * (float)(1 << kNuBits)));
+#pragma unroll
+    for (int u = 0; u < kNuItems; ++u) {
+      c1[u] *= scale;
+      c2[u] *= scale;
+    }
+    for (int k = 0; k < nc; ++k, ++pass) {
+      int* fl = flag[pass & 1];
+      if (tid < kNuBlock / 8) flag[~pass & 1][tid] = 0;  // read before this pass
+      if (tid == 0) s_max[~chunk & 1] = 0u;
+#pragma unroll
+      for (int u = 0; u < kNuItems; ++u) {
+        if (c1[u] != 0.f || c2[u] != 0.f) {
+          int* g1 = mine + cell[u] * (2 * kNuCopies) + (upper ? kNuCopies : 0);
+          int* g2 = mine + cell[u] * (2 * kNuCopies) + (upper ? 0 : kNuCopies);
+          fl[cell[u] >> 3] = 1;
+          float wl[4], wrt[4];
+          nu_weights(co, s[u], wl, wrt);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            atomicAdd(g1 + j * (2 * kNuCopies), nu_term(c1[u], wl[j], j < kNuSmall));
+            atomicAdd(g2 + j * (2 * kNuCopies), nu_term(c2[u], wl[j], j < kNuSmall));
+            atomicAdd(g1 + (7 - j) * (2 * kNuCopies), nu_term(c1[u], wrt[j], j < kNuSmall));
+            atomicAdd(g2 + (7 - j) * (2 * kNuCopies), nu_term(c2[u], wrt[j], j < kNuSmall));
+          }
+        }
+        // the next chirp
+        const float a = c1[u];
+        c1[u] = fmaf(a, wr[u], -c2[u] * wi[u]);
+        c2[u] = fmaf(c2[u], wr[u], a * wi[u]);
+        const float sh = s[u] + ds[u], f = floorf(sh + 0.5f);
+        s[u] = sh - f;
+        cell[u] = (cell[u] + (int)f) & (M - 1);
+      }
+      __syncthreads();
+      // half-warp h adds up the octets of points o = h mod 16 (as k_nufft_spread), into the
+      // chirp's grid; the points past the grid's end belong to octet 0
+      const unsigned m0 = __ballot_sync(0xffffffffu, fl[lane] != 0), m1 = __ballot_sync(0xffffffffu, fl[32 + lane] != 0);
+      const unsigned long long cells = (unsigned long long)m1 << 32 | m0, last = cells >> (oct - 1) & 1ull,
+                               lit = cells | cells << 1 | last;
+      float* to = reinterpret_cast<float*>(out + (size_t)k * M);
+#pragma unroll
+      for (int r = 0; r < kNuBlock / 8 / 16; ++r) {
+        const int o = r * 16 + (tid >> 4);
+        if (o >= oct || !((lit >> o) & 1ull)) continue;
+        const int i = o * 16 + (tid & 15);  // point i / 2, part i & 1
+        float* g = to + 2 * (((i >> 1) - (kNuW / 2 - 1)) & (M - 1)) + (i & 1);
+        const float old = *g;
+        long long t = 0;
+        for (int h = 0; h < (o == 0 ? 2 : 1); ++h) {
+          const int ii = i + h * 2 * M;
+#pragma unroll
+          for (int w4 = 0; w4 < kNuCopies / 4; ++w4) {
+            const int w = ii * (kNuCopies / 4) + ((w4 + (ii >> 1)) & (kNuCopies / 4 - 1));
+            const int4 x = nsm[w];
+            nsm[w] = make_int4(0, 0, 0, 0);
+            t += (long long)(x.x + x.y) + (long long)(x.z + x.w);
+          }
+        }
+        *g = fmaf((float)t, unit, old);
+      }
+      __syncthreads();
+    }
+  }
+  bad = __syncthreads_or(bad);
+  if (bad)
+    for (int i = tid; i < nc * M; i += kNuThreads) out[i] = make_float2(NAN, NAN);
+}
+
 // Finishing, kNuFinSlice grid points per CTA: CTA (row, s) adds slice s of the Q
 // CTAs' grids of a row (antenna and chirp) in a fixed order (kNuFinThreads / slice
 // threads per point, each over every such CTA with four interleaved sums, then the
@@ -1286,6 +1436,7 @@ void grid_shape(int V, int Ns, int64_t cap, int* Q) {
 
 // dynamic shared memory of the spreading kernel: the grid's copies and its sums
 inline size_t nufft_smem(int Ns) { return (2 * kNuCopies * sizeof(int) + 2 * sizeof(float)) * (size_t)nu_points(2 * Ns); }
+inline size_t nufft_chirps_smem(int Ns) { return 2 * kNuCopies * sizeof(int) * (size_t)nu_points(2 * Ns); }
 inline size_t nufft_cl_smem(int Ns) {
   return sizeof(float2) * (size_t)(fft::slots(2 * Ns) + fft::slots(Ns) + kNuClThreads + 2 * Ns / kNuRanks);
 }
@@ -1319,6 +1470,8 @@ int nufft_per_sm(int Ns) {
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&m, k, kNuThreads, sm);
     n = std::min(n, m > 0 ? m : 1);
   }
+  if (nufft_chirps_smem(Ns) > 48 * 1024)
+    cudaFuncSetAttribute(k_nufft_spread_chirps, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)nufft_chirps_smem(Ns));
   if (nufft_fin_smem(Ns) > 48 * 1024)
     cudaFuncSetAttribute(k_nufft_finish, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)nufft_fin_smem(Ns));
   if (dev < kDevCache) cache[dev][lg] = n;
@@ -1334,6 +1487,21 @@ void nufft_shape(int V, int Ns, int64_t cap, int* Qn) {
   *Qn = (int)q;
 }
 
+// Moving scenes whose chirps go in tiles: a grid that a CTA holds whole, and chirps
+// enough to pay for the slower inner loop (2 chirps x 114,000 records: 20.7 us in tiles,
+// 17.3 in a group; 16 chirps: 80 against 130; 16 x 950 records: 28 against 109).
+inline bool nufft_tiles(int C, int Ns) { return 2 * Ns <= kNuBlock && C >= 4; }
+
+// Grids per antenna in the workspace: one per spreading CTA, and for the chirps of a moving
+// scene a tile's from each (at most 30 MB) or, in groups, a wave's (a group is then not
+// held to the few CTAs that few paths ask for: 512 samples, 128 chirps x 950 records 1.01 -> 0.13 ms).
+inline int nufft_wave(int V, int qn, int C, int Ns) {
+  return (int)std::max<int64_t>(qn, std::min<int64_t>((int64_t)qn * C, (int64_t)sm_count() * nufft_per_sm(Ns) / V));
+}
+inline int nufft_grids(int V, int qn, int C, int Ns) {
+  return nufft_tiles(C, Ns) ? qn * std::min(C, kTile) : nufft_wave(V, qn, C, Ns);
+}
+
 // Workspace: per-CTA partial sums of the direct kernels, the chirp-summed
 // upstream gradient of the adjoint, and, for the non-uniform FFT, the CTAs'
 // grids, their sum and the finishing counters.
@@ -1346,9 +1514,10 @@ size_t ws_layout(const sbr_radar_cfg* radar, int64_t cap, int* Q, int* Qn = null
   Carver c(nullptr);
   c.take<float2>((size_t)V * (*Q) * Ns);       // per-CTA partial sums
   c.take<float2>((size_t)V * Ns);              // chirp-summed upstream gradient
-  c.take<float2>((size_t)V * qn * 2 * Ns);     // non-uniform FFT: the CTAs' grids
-  c.take<float2>((size_t)V * qn * 2 * Ns);     // non-uniform FFT: the rows' summed grids (a moving scene: V * chirps)
-  c.take<unsigned int>((size_t)V * qn);        // non-uniform FFT: finishing counters
+  const int qg = nufft_grids(V, qn, radar->n_chirps, Ns);
+  c.take<float2>((size_t)V * qg * 2 * Ns);     // non-uniform FFT: the CTAs' grids
+  c.take<float2>((size_t)V * qg * 2 * Ns);     // non-uniform FFT: the rows' summed grids (a moving scene: V * chirps)
+  c.take<unsigned int>((size_t)V * qg);        // non-uniform FFT: finishing counters
   c.take<float4>((size_t)V * (2 * Ns + kAdjMargin));  // adjoint: the antennas' grids
   return c.bytes();
 }
@@ -1372,7 +1541,7 @@ struct SynthWs {
   float2* bsum;
   unsigned int* fin_cnt;
   float4* adj;
-  int Q, Qn;
+  int Q, Qn, Qg;
 };
 
 sbr_status bind_ws(const sbr_radar_cfg* radar, int64_t cap, void* ws, size_t bytes, SynthWs* w,
@@ -1388,21 +1557,19 @@ sbr_status bind_ws(const sbr_radar_cfg* radar, int64_t cap, void* ws, size_t byt
   Carver c(ws);
   w->partial = c.take<float2>((size_t)V * Q * Ns);
   w->gsum = c.take<float2>((size_t)V * Ns);
-  w->grids = c.take<float2>((size_t)V * Qn * 2 * Ns);
-  w->bsum = c.take<float2>((size_t)V * Qn * 2 * Ns);
-  w->fin_cnt = c.take<unsigned int>((size_t)V * Qn);
+  w->Qg = nufft_grids(V, Qn, radar->n_chirps, Ns);
+  w->grids = c.take<float2>((size_t)V * w->Qg * 2 * Ns);
+  w->bsum = c.take<float2>((size_t)V * w->Qg * 2 * Ns);
+  w->fin_cnt = c.take<unsigned int>((size_t)V * w->Qg);
   w->adj = c.take<float4>((size_t)V * (2 * Ns + kAdjMargin));
   w->Q = Q;
   w->Qn = Qn;
   return SBR_OK;
 }
 
-// The non-uniform FFT of chirps [c0, c0 + chirps) of a moving scene, or of a static
-// scene's one chirp, written to all of them: spread by Q CTAs per antenna and chirp
-// (Q * chirps <= w.Qn), then finish.
-void launch_nufft(sbr_phase_mode mode, const sbr_paths* p, const sbr_radar_cfg* r, const SynthWs& w, bool moving, int Q,
-                  int c0, int chirps, float2* cube, cudaStream_t st) {
-  const int V = p->n_virt, Ns = r->n_samples, M = 2 * Ns;
+// The launch's constants; sets the kernels' shared-memory limits before their first launch.
+NufftArg nufft_arg(const sbr_paths* p, const sbr_radar_cfg* r, int Q, int c0, int chirps) {
+  const int Ns = r->n_samples, M = 2 * Ns;
   NufftArg na{};
   while ((1 << na.log_m) < M) ++na.log_m;
   na.half_n = 0.5f * (float)Ns;
@@ -1411,12 +1578,22 @@ void launch_nufft(sbr_phase_mode mode, const sbr_paths* p, const sbr_radar_cfg* 
   na.b_cn = r->bandwidth / (kC * Ns);
   na.cyc = na.f0_c + 0.5 * Ns * na.b_cn;  // N_s / 2 is whole: delta need not be reduced first
   na.cell = M * na.b_cn;
-  na.V = V;
+  na.V = p->n_virt;
   na.Q = Q;
   na.chirps = chirps;
   na.chirp0 = c0;
   na.per_chirp = r->chirp_rep;
-  nufft_per_sm(Ns);  // sets the shared-memory limits before the first launch
+  nufft_per_sm(Ns);
+  return na;
+}
+
+// The non-uniform FFT of chirps [c0, c0 + chirps) of a moving scene, or of a static
+// scene's one chirp, written to all of them: spread by Q CTAs per antenna and chirp
+// (Q * chirps <= w.Qg), then finish.
+void launch_nufft(sbr_phase_mode mode, const sbr_paths* p, const sbr_radar_cfg* r, const SynthWs& w, bool moving, int Q,
+                  int c0, int chirps, float2* cube, cudaStream_t st) {
+  const int V = p->n_virt, Ns = r->n_samples, M = 2 * Ns;
+  const NufftArg na = nufft_arg(p, r, Q, c0, chirps);
   const NufftCoef& co = nufft_coef();
   const float4* prep = reinterpret_cast<const float4*>(p->prep);
   const float2* plen = reinterpret_cast<const float2*>(p->path_len);
@@ -1433,22 +1610,43 @@ void launch_nufft(sbr_phase_mode mode, const sbr_paths* p, const sbr_radar_cfg* 
   launch_after(k_nufft_finish, V * chirps * slices, kNuFinThreads, nufft_fin_smem(Ns), st, w.grids, na, co, w.bsum, w.fin_cnt, cube, r->n_chirps, moving);
 }
 
+// The chirps of a moving scene, kTile at a time: a launch is one wave of CTAs, each with
+// its share of the records and all chirps of the tile.
+void launch_chirps(const sbr_paths* p, const sbr_radar_cfg* r, const SynthWs& w, float2* cube, cudaStream_t st) {
+  const int V = p->n_virt, Ns = r->n_samples, C = r->n_chirps;
+  for (int c = 0; c < C; c += kTile) {
+    const NufftArg na = nufft_arg(p, r, w.Qn, c, std::min(kTile, C - c));
+    ::sbr::note_launch();
+    launch_after(k_nufft_spread_chirps, V * w.Qn, kNuThreads, nufft_chirps_smem(Ns), st,
+                 reinterpret_cast<const float4*>(p->prep), p->path_rate, p->path_cap, p->count, na, nufft_coef(), w.grids);
+    ::sbr::note_launch();
+    launch_after(k_nufft_finish_cluster, V * na.chirps * kNuRanks, kNuClThreads, nufft_cl_smem(Ns), st, w.grids, na,
+                 nufft_coef(), cube, C, true);
+  }
+}
+
 // A moving scene: every chirp synthesised from its own delays (split phase up to 512
-// samples, or the FP64 phase), a group of chirps per launch.  A launch is one wave of
-// Q CTAs per antenna and chirp; fewer CTAs per chirp mean fewer launches and the same
+// samples, or the FP64 phase), in tiles of chirps or (two blocks of cells, the FP64
+// phase, few chirps) a group of chirps per launch.  A group's launch is one wave of Q
+// CTAs per antenna and chirp; fewer CTAs per chirp mean fewer launches and the same
 // records per CTA in all, so Q is the one whose launches / Q, the chirps' share of a
 // wave each, is least (12 antennas x 128 chirps: 2 CTAs each, 7 launches of 19 chirps,
 // 3.5 against the ideal 3.4; the records are then read from L2 by the chirps of a
-// launch).  One launch pair per chirp took 7.85 ms for 12 x 367,500 records x 128
-// chirps, groups took 6.3 ms.
+// launch).  256 samples, 12 x 367,500 records x 128 chirps: 7.85 ms with one launch
+// pair per chirp, 6.3 in groups (both before the leaner spreading; 5.0 after it).
 sbr_status launch_moving(sbr_phase_mode mode, const sbr_paths* p, const sbr_radar_cfg* r, const SynthWs& w,
                          float2* cube, cudaStream_t st) {
   if (mode == SBR_PHASE_FP64 || (mode == SBR_PHASE_SPLIT && r->n_samples <= kNuMovingMaxSamples)) {
     const int C = r->n_chirps;
+    if (mode == SBR_PHASE_SPLIT && nufft_tiles(C, r->n_samples)) {
+      launch_chirps(p, r, w, cube, st);
+      return SBR_OK;
+    }
+    const int wave = std::min(w.Qg, nufft_wave(p->n_virt, w.Qn, C, r->n_samples));
     int best = 1, group = 1;
     double cost = 1e30;
     for (int q = 1; q <= w.Qn; ++q) {
-      const int most = std::min(C, w.Qn / q), launches = (C + most - 1) / most;
+      const int most = std::min(C, wave / q), launches = (C + most - 1) / most;
       if (launches < cost * q) {
         cost = (double)launches / q;
         best = q;

@@ -124,17 +124,20 @@ def test_split_records_not_finite(sbr):
     assert torch.isnan(cube[2]).all() and torch.isfinite(cube[[0, 1, 3]]).all()
 
 
-def test_moving_records(sbr):
-    """12 antennas, 16 chirps: every chirp from its own delays."""
-    radar = radar_mimo_3x4(256, 16)
-    delta, phi, A = records(9, 12, 7001, 256)
+@pytest.mark.parametrize("ns,nc,P", [(256, 16, 7001), (32, 2, 1025), (64, 128, 300), (128, 64, 2049), (512, 4, 5000)])
+def test_moving_records(sbr, ns, nc, P):
+    """Every chirp from its own delays: chirps in tiles (up to 256 samples) and one by one (512)."""
+    radar = radar_mimo_3x4(ns, nc)
+    delta, phi, A = records(9 + ns, 12, P, ns)
     rate = np.random.default_rng(4).uniform(-8.0, 8.0, delta.shape).astype(np.float32)
-    paths, phi, delta, A = bind(sbr, radar, 7001, delta, phi, A, rate)
+    rate[:, ::5] = 0.0
+    paths, phi, delta, A = bind(sbr, radar, P + 2, delta, phi, A, rate)
     cube = sbr.synthesize(paths, radar, sbr.PHASE_SPLIT | sbr.SYNTH_MOVING)
+    assert torch.equal(cube, sbr.synthesize(paths, radar, sbr.PHASE_SPLIT | sbr.SYNTH_MOVING))
     per = radar.chirp_rep / C_LIGHT
-    ref = torch.stack([direct(phi + rate * (c * per * radar.f0), delta + rate * (c * per * radar.bandwidth / 256), A, 256)
-                       for c in range(16)], 1)
-    # the chirp's phase shift (up to 1.3 cycles here) and delta shift are each rounded once more in FP32
+    ref = torch.stack([direct(phi + rate * (c * per * radar.f0), delta + rate * (c * per * radar.bandwidth / ns), A, ns)
+                       for c in range(nc)], 1)
+    # the chirp's phase shift (up to 10 cycles here), delta shift and turns are each rounded once more in FP32
     assert rel(cube, ref) <= 2 * TOL
 
 
