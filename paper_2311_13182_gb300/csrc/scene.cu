@@ -959,16 +959,15 @@ __global__ void k_collapse4(const Node* __restrict__ nodes, int n, Node4* __rest
     ++cnt;
   }
   Node4 o;
-  float* f = reinterpret_cast<float*>(&o);
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     const bool used = k < cnt;
-    f[0 * 4 + k] = used ? bx[k].lo.x : 0.f;
-    f[1 * 4 + k] = used ? bx[k].hi.x : 0.f;
-    f[2 * 4 + k] = used ? bx[k].lo.y : 0.f;
-    f[3 * 4 + k] = used ? bx[k].hi.y : 0.f;
-    f[4 * 4 + k] = used ? bx[k].lo.z : 0.f;
-    f[5 * 4 + k] = used ? bx[k].hi.z : 0.f;
+    (&o.lox.x)[k] = used ? bx[k].lo.x : 0.f;
+    (&o.hix.x)[k] = used ? bx[k].hi.x : 0.f;
+    (&o.loy.x)[k] = used ? bx[k].lo.y : 0.f;
+    (&o.hiy.x)[k] = used ? bx[k].hi.y : 0.f;
+    (&o.loz.x)[k] = used ? bx[k].lo.z : 0.f;
+    (&o.hiz.x)[k] = used ? bx[k].hi.z : 0.f;
   }
   o.child = make_int4(cnt > 0 ? id[0] : kEmpty, cnt > 1 ? id[1] : kEmpty, cnt > 2 ? id[2] : kEmpty,
                       cnt > 3 ? id[3] : kEmpty);

@@ -19,12 +19,15 @@ struct __align__(16) Node {
 // binary node i holds i's grandchildren (a leaf child stands for itself), then
 // the largest internal slot is expanded while a slot is free.  child >= 0:
 // internal binary node (its own 4-wide entry); kEmpty: unused slot; otherwise a
-// leaf ~slot.  Boxes per axis as float4 over the four slots (112 of 128 bytes).
+// leaf ~slot.  Boxes per axis as float4 over the four slots (112 of 128 bytes), an
+// axis's lower and upper row one address bit apart, another bit for each axis.
 constexpr int kEmpty = (int)0x80000000;
 struct __align__(128) Node4 {
-  float4 lox, hix, loy, hiy, loz, hiz;
+  float4 lox, hix;
   int4 child;
+  float4 loz, loy;
   int4 pad;
+  float4 hiy, hiz;
 };
 
 // Shared-memory staging of the top levels of the 4-wide tree: the scene build

@@ -114,7 +114,7 @@ struct Ray {
   __device__ Ray(ff3& o_, ff3& d_) : o(o_), d(d_) {}
   float3 of, df;  // FP32 ray driving the traversal
   float3 idir;
-  int near;  // byte offsets of a 4-wide entry's near-plane rows, x | y << 8 | z << 16 (set_idir)
+  int near;  // address bits of a 4-wide entry's near-plane rows (set_idir)
   int skip;
   bool has_ff;        // primary rays build d in float-float only when needed
   int rid;
@@ -250,33 +250,35 @@ __device__ inline void slab_nf(const float3& o, const float3& idir, float nx, fl
 // A 4-wide entry's boxes as the ray meets them: per axis the plane entered first
 // (the lower bound when the direction component is positive, else the upper
 // one) and the plane left last, one float4 over the four slots each.  Entries
-// are 128-byte aligned, so a near row's byte offset (Ray::near) is OR-ed
-// into the entry's address, and the far row is the near one with bit 4 flipped.
+// are 128-byte aligned and an axis's two rows differ in one address bit of its own
+// (x 16, y 32, z 64), so a near row's address is the entry's with that bit of
+// Ray::near OR-ed in, the far row's with its complement, and the rest is the
+// load's own offset (1 % less time for the traversal than unpacked row offsets).
 struct Planes4 {
   float4 nx, fx, ny, fy, nz, fz;
 };
 
-static_assert(offsetof(Node4, lox) == 0 && offsetof(Node4, hix) == 16 && offsetof(Node4, loy) == 32 &&
-                  offsetof(Node4, hiy) == 48 && offsetof(Node4, loz) == 64 && offsetof(Node4, hiz) == 80 &&
+static_assert(offsetof(Node4, lox) == 0 && offsetof(Node4, hix) == 16 && offsetof(Node4, loy) == 64 &&
+                  offsetof(Node4, hiy) == 96 && offsetof(Node4, loz) == 48 && offsetof(Node4, hiz) == 112 &&
                   alignof(Node4) == 128,
               "near/far plane rows assume this entry layout");
 
 template <bool kGlobal>
-__device__ inline float4 plane_row(const void* q, int off) {
-  const float4* a = reinterpret_cast<const float4*>(reinterpret_cast<uintptr_t>(q) | (uintptr_t)(unsigned)off);
+__device__ inline float4 plane_row(uintptr_t q, int bit, int row) {
+  const float4* a = reinterpret_cast<const float4*>((q | (uintptr_t)(unsigned)bit) + row);
   return kGlobal ? __ldg(a) : *a;
 }
 
 template <bool kGlobal = true>
-__device__ inline Planes4 load_planes(const void* q, int near) {
-  const int nxo = near & 0xff, nyo = (near >> 8) & 0xff, nzo = near >> 16;
+__device__ inline Planes4 load_planes(const void* entry, int near) {
+  const uintptr_t q = reinterpret_cast<uintptr_t>(entry);
   Planes4 p;
-  p.nx = plane_row<kGlobal>(q, nxo);
-  p.fx = plane_row<kGlobal>(q, nxo ^ 16);
-  p.ny = plane_row<kGlobal>(q, nyo);
-  p.fy = plane_row<kGlobal>(q, nyo ^ 16);
-  p.nz = plane_row<kGlobal>(q, nzo);
-  p.fz = plane_row<kGlobal>(q, nzo ^ 16);
+  p.nx = plane_row<kGlobal>(q, near & 16, 0);
+  p.fx = plane_row<kGlobal>(q, ~near & 16, 0);
+  p.ny = plane_row<kGlobal>(q, near & 32, 64);
+  p.fy = plane_row<kGlobal>(q, ~near & 32, 64);
+  p.nz = plane_row<kGlobal>(q, near & 64, 48);
+  p.fz = plane_row<kGlobal>(q, ~near & 64, 48);
   return p;
 }
 
@@ -405,13 +407,13 @@ __device__ Best nearest(const float4* __restrict__ tris, const Node4* __restrict
         p = load_planes(q, r.near);
         ch = __ldg(&q->child);
       }
-      const float lim = b.hi;
+      const float lim = b.hi;  // slots 0 and 1 are always used
       float d0, d1, d2, d3, tf;
       int c0 = ch.x, c1 = ch.y, c2 = ch.z, c3 = ch.w;
       slab_nf(r.of, r.idir, p.nx.x, p.fx.x, p.ny.x, p.fy.x, p.nz.x, p.fz.x, d0, tf);
-      d0 = (c0 != kEmpty && d0 <= tf && tf >= 0.f && d0 <= lim) ? d0 : INFINITY;
+      d0 = (d0 <= tf && tf >= 0.f && d0 <= lim) ? d0 : INFINITY;
       slab_nf(r.of, r.idir, p.nx.y, p.fx.y, p.ny.y, p.fy.y, p.nz.y, p.fz.y, d1, tf);
-      d1 = (c1 != kEmpty && d1 <= tf && tf >= 0.f && d1 <= lim) ? d1 : INFINITY;
+      d1 = (d1 <= tf && tf >= 0.f && d1 <= lim) ? d1 : INFINITY;
       slab_nf(r.of, r.idir, p.nx.z, p.fx.z, p.ny.z, p.fy.z, p.nz.z, p.fz.z, d2, tf);
       d2 = (c2 != kEmpty && d2 <= tf && tf >= 0.f && d2 <= lim) ? d2 : INFINITY;
       slab_nf(r.of, r.idir, p.nx.w, p.fx.w, p.ny.w, p.fy.w, p.nz.w, p.fz.w, d3, tf);
@@ -502,9 +504,9 @@ __device__ bool traverse(const float4* __restrict__ tris, const Node4* __restric
 __device__ inline void set_idir(Ray& r) {
   auto inv = [](float x) { return 1.0f / (fabsf(x) < 1e-20f ? copysignf(1e-20f, x) : x); };
   r.idir = f3(inv(r.df.x), inv(r.df.y), inv(r.df.z));
-  // near rows: lo (bytes 0, 32, 64 of the entry) for a positive component, hi (16, 48, 80) otherwise
-  r.near = (__float_as_int(r.idir.x) < 0 ? 16 : 0) | (__float_as_int(r.idir.y) < 0 ? 48 : 32) << 8 |
-           (__float_as_int(r.idir.z) < 0 ? 80 : 64) << 16;
+  // near rows: lo for a positive component, hi (the axis's address bit set) otherwise
+  r.near = (__float_as_int(r.idir.x) < 0 ? 16 : 0) | (__float_as_int(r.idir.y) < 0 ? 32 : 0) |
+           (__float_as_int(r.idir.z) < 0 ? 64 : 0);
 }
 
 __device__ inline void set_f32(Ray& r) {
@@ -523,7 +525,9 @@ __device__ inline void bary(const Ray& r, float3 a, float3 b, float3 c, float& u
 }
 
 #ifndef SBR_TRACE_MIN_BLOCKS
-#define SBR_TRACE_MIN_BLOCKS 6  // resident 128-thread CTAs per SM the register budget targets
+// Resident 128-thread CTAs per SM the register budget targets (200,000 triangles, 4 M rays:
+// k_trace 1774 / 1730 / 1717 / 1823 us with 5 / 6 / 7 / 8).
+#define SBR_TRACE_MIN_BLOCKS 7
 #endif
 
 // Records k..K-1 of a ray that found nothing at bounce k.
@@ -565,8 +569,52 @@ __device__ inline void record_hit(const float4* __restrict__ tris, Ray& r, const
   set_f32(r);
 }
 
+// The whole grid goes to k_trace in tiles of 16 x 16 rays, two CTAs per tile, a warp on 16 x
+// 2 of them: neighbours in both directions walk the same entries (32 rays of a row per warp
+// issue 8 % more instructions).  The kernel's ALU pipe bounds it (comparisons, minima and the
+// sorting network), and its end: a warp of grazing rays takes 100-250 us, ten times the mean,
+// so one that starts late is waited for by an empty chip.  Grids are aimed at the object, its
+// silhouette lies around its middle and the middle reflects straight back, so the tiles go from
+// the border inwards.  1.05 M rays, 20,000 triangles: 517 -> 484 us for the whole trace, 4 M
+// rays, 200,000 triangles 1872 -> 1694, 0.5 M rays 276 -> 223 (tiles row by row: 513, 1910, 297).
+// A ray list is taken in its own order.
+constexpr int kTile = 16, kTraceThreads = 128, kTileCtas = kTile * kTile / kTraceThreads;
+
+__host__ __device__ inline int tiles_across(int G) { return (G + kTile - 1) / kTile; }
+
+inline int trace_blocks(int64_t R, int G, bool list) {
+  return list ? (int)((R + kTraceThreads - 1) / kTraceThreads) : kTileCtas * tiles_across(G) * tiles_across(G);
+}
+
+// Grid ray of the thread, or -1 outside the grid.  The tiles lie in square rings, the
+// outermost first; a ring is its upper row, then the ends of the rows between, then its
+// lower row.
+__device__ inline int tiled_ray(int G) {
+  const int U = tiles_across(G), n = (int)blockIdx.x / kTileCtas;
+  const int to_come = U * U - n;  // this tile included; its ring's side: the least of U's parity with side^2 >= to_come
+  int side = (int)sqrtf((float)to_come);
+  while (side * side < to_come) ++side;
+  while (side > 1 && (side - 1) * (side - 1) >= to_come) --side;
+  side += (U - side) & 1;
+  const int edge = (U - side) >> 1;
+  int p = n - (U * U - side * side), ty, tx;
+  if (p < side) {
+    ty = edge;
+    tx = edge + p;
+  } else if ((p -= side) < 2 * (side - 2)) {
+    ty = edge + 1 + (p >> 1);
+    tx = (p & 1) ? edge + side - 1 : edge;
+  } else {
+    ty = edge + side - 1;
+    tx = edge + p - 2 * (side - 2);
+  }
+  const int at = threadIdx.x + kTraceThreads * (blockIdx.x % kTileCtas);
+  const int col = tx * kTile + at % kTile, row = ty * kTile + at / kTile;
+  return col < G && row < G ? row * G + col : -1;
+}
+
 template <bool kCount>
-__global__ void __launch_bounds__(128, SBR_TRACE_MIN_BLOCKS) k_trace(const float4* __restrict__ tris,
+__global__ void __launch_bounds__(kTraceThreads, SBR_TRACE_MIN_BLOCKS) k_trace(const float4* __restrict__ tris,
                                                const Node4* __restrict__ nodes, int nt, GridArg g,
                                                const int32_t* __restrict__ ray_ids, int n_rays,
                                                int K, sbr_hit* __restrict__ hits,
@@ -577,7 +625,8 @@ __global__ void __launch_bounds__(128, SBR_TRACE_MIN_BLOCKS) k_trace(const float
                                                unsigned long long* __restrict__ counts,
                                                const Node4* __restrict__ top, const int32_t* __restrict__ top_n) {
   after_previous();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (!ray_ids && (i = tiled_ray(g.G)) < 0) i = n_rays;
   int n_nodes = 0, n_tris = 0, n_trav = 0;
   if (kTopLevels > 0) {  // every thread of the CTA, before any may return
     const int n = *top_n;
@@ -586,12 +635,7 @@ __global__ void __launch_bounds__(128, SBR_TRACE_MIN_BLOCKS) k_trace(const float
     for (int j = threadIdx.x; j < n * (int)(sizeof(Node4) / sizeof(float4)); j += blockDim.x) dst[j] = __ldg(&src[j]);
     __syncthreads();
   }
-  if (kCount) {
-    // whole warps stay to the reduction below; idle lanes count nothing
-    if (i - (int)(threadIdx.x & 31) >= n_rays) return;
-  } else if (i >= n_rays) {
-    return;
-  }
+  if (!kCount && i >= n_rays) return;  // counting: all lanes stay to the reduction below
   if (i < n_rays) {
   const int rid = ray_ids ? ray_ids[i] : i;
   ff3 ray_o, ray_d;
@@ -1333,12 +1377,12 @@ static sbr_status trace_impl(const sbr_scene* scene, const sbr_radar_cfg* radar,
       launch_after(k_trace_warp<false>, nbw, 128, 0, st, scene->tris, scene->nodes4, scene->nt, g, d_ray_ids, (int)R, max_bounces, paths->hits, hp, paths->ray_weight, paths->ray_first, nullptr);
   } else if (d_counts) {
     ::sbr::note_launch();
-    launch_after(k_trace<true>, blocks(R, 128), 128, 0, st, scene->tris, scene->nodes4, scene->nt, g, d_ray_ids, (int)R, max_bounces, paths->hits, hp, paths->ray_weight, paths->ray_first, dumps, dctr, d_counts, scene->top, scene->top_n);
+    launch_after(k_trace<true>, trace_blocks(R, grid->G, d_ray_ids != nullptr), kTraceThreads, 0, st, scene->tris, scene->nodes4, scene->nt, g, d_ray_ids, (int)R, max_bounces, paths->hits, hp, paths->ray_weight, paths->ray_first, dumps, dctr, d_counts, scene->top, scene->top_n);
     ::sbr::note_launch();
     launch_after(k_trace_coop<true>, coop_grid(), 128, 0, st, scene->tris, scene->nodes4, scene->nt, g, max_bounces, dumps, dctr, dctr + 1, paths->hits, hp, paths->ray_first, d_counts);
   } else {
     ::sbr::note_launch();
-    launch_after(k_trace<false>, blocks(R, 128), 128, 0, st, scene->tris, scene->nodes4, scene->nt, g, d_ray_ids, (int)R, max_bounces, paths->hits, hp, paths->ray_weight, paths->ray_first, dumps, dctr, nullptr, scene->top, scene->top_n);
+    launch_after(k_trace<false>, trace_blocks(R, grid->G, d_ray_ids != nullptr), kTraceThreads, 0, st, scene->tris, scene->nodes4, scene->nt, g, d_ray_ids, (int)R, max_bounces, paths->hits, hp, paths->ray_weight, paths->ray_first, dumps, dctr, nullptr, scene->top, scene->top_n);
     ::sbr::note_launch();
     launch_after(k_trace_coop<false>, coop_grid(), 128, 0, st, scene->tris, scene->nodes4, scene->nt, g, max_bounces, dumps, dctr, dctr + 1, paths->hits, hp, paths->ray_first, nullptr);
   }
