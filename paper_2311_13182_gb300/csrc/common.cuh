@@ -84,7 +84,7 @@ cudaError_t exclusive_scan(const int32_t* in, int32_t* out, int64_t n, const int
 // kSortOneCta keys sort in one CTA with 8-bit digits; d_hist, when not NULL,
 // then holds the caller's counts of every digit place (place p's 256 counts at
 // [256p, 256p + 256), for the live keys), which spares the CTA its counting
-// sweep.  Larger inputs take the multi-CTA path (4-bit digits) and ignore it.
+// sweep.  Larger inputs take the multi-CTA path and ignore it.
 constexpr int64_t kSortOneCta = 65536;
 size_t sort_scratch_bytes(int64_t capacity);
 cudaError_t radix_sort_pairs(uint32_t* keys[2], int32_t* vals[2], int64_t n, const int32_t* d_n,

@@ -12,7 +12,7 @@ struct __align__(16) Node {
   float4 lxy;   // left  lo.x hi.x lo.y hi.y
   float4 rxy;   // right lo.x hi.x lo.y hi.y
   float4 lrz;   // left lo.z hi.z, right lo.z hi.z
-  int4 child;   // left, right, unused, unused
+  int4 child;   // left, right; meshes above the fused build's size: first and last leaf
 };
 
 // 4-wide node for the traversal, collapsed from the binary tree: the entry of
