@@ -569,28 +569,40 @@ __device__ inline void record_hit(const float4* __restrict__ tris, Ray& r, const
   set_f32(r);
 }
 
-// The whole grid goes to k_trace in tiles of 16 x 16 rays, two CTAs per tile, a warp on 16 x
-// 2 of them: neighbours in both directions walk the same entries (32 rays of a row per warp
-// issue 8 % more instructions).  The kernel's ALU pipe bounds it (comparisons, minima and the
-// sorting network), and its end: a warp of grazing rays takes 100-250 us, ten times the mean,
-// so one that starts late is waited for by an empty chip.  Grids are aimed at the object, its
-// silhouette lies around its middle and the middle reflects straight back, so the tiles go from
-// the border inwards.  1.05 M rays, 20,000 triangles: 517 -> 484 us for the whole trace, 4 M
-// rays, 200,000 triangles 1872 -> 1694, 0.5 M rays 276 -> 223 (tiles row by row: 513, 1910, 297).
-// A ray list is taken in its own order.
-constexpr int kTile = 16, kTraceThreads = 128, kTileCtas = kTile * kTile / kTraceThreads;
+// The whole grid goes to k_trace in square tiles, from the border inwards.  The kernel's ALU
+// pipe bounds it (comparisons, minima and the sorting network), and its end: a warp of grazing
+// rays takes 100-250 us, ten times the mean, so one that starts late is waited for by an empty
+// chip.  Grids are aimed at the object, its silhouette lies around its middle and the middle
+// reflects straight back, so the border goes first.  Above kRowWarpRays the tiles have 16 x 16
+// rays and a warp 16 x 2 of them: neighbours in both directions walk the same entries (32 rays
+// of a row per warp issue 8 % more instructions).  1.05 M rays, 20,000 triangles: 517 -> 482 us
+// for the whole trace, 4 M rays, 200,000 triangles 1872 -> 1684, 0.5 M rays 276 -> 218 (tiles
+// of that shape row by row: 513, 1910, 297).  Up to it, about three waves of CTAs, the longest
+// warps decide, and two rows of grazing rays in one warp make them longer: tiles of 32 x 32
+// rays, a warp a row of 32 (250,000 rays on 5,120 triangles, row by row / 32 / 16: 147 / 135 /
+// 125 us; 360,000 on 150,000 triangles, four views: 405 407 426 292 / 363 383 429 308 / 391 409
+// 465 336).  In a single wave (152 SMs x 7 CTAs) nothing starts late, and a ray list is the
+// caller's: both are taken in their order (47,157 triangles, 34,225 rays, the worst of four
+// views: 115 us, 129 in tiles of 32, 148 of 16).
+constexpr int kTraceThreads = 128;
+constexpr int64_t kOneWaveRays = 136192, kRowWarpRays = 400000;
+constexpr int kInOrder = 0;  // in place of a tile size's logarithm
 
-__host__ __device__ inline int tiles_across(int G) { return (G + kTile - 1) / kTile; }
+inline int tile_log2(int64_t R, bool list) {
+  return list || R <= kOneWaveRays ? kInOrder : R <= kRowWarpRays ? 5 : 4;
+}
+__host__ __device__ inline int tiles_across(int G, int log2) { return (G + (1 << log2) - 1) >> log2; }
 
-inline int trace_blocks(int64_t R, int G, bool list) {
-  return list ? (int)((R + kTraceThreads - 1) / kTraceThreads) : kTileCtas * tiles_across(G) * tiles_across(G);
+inline int trace_blocks(int64_t R, int G, int log2) {
+  if (log2 == kInOrder) return (int)((R + kTraceThreads - 1) / kTraceThreads);
+  return ((1 << 2 * log2) / kTraceThreads) * tiles_across(G, log2) * tiles_across(G, log2);
 }
 
 // Grid ray of the thread, or -1 outside the grid.  The tiles lie in square rings, the
 // outermost first; a ring is its upper row, then the ends of the rows between, then its
 // lower row.
-__device__ inline int tiled_ray(int G) {
-  const int U = tiles_across(G), n = (int)blockIdx.x / kTileCtas;
+__device__ inline int tiled_ray(int G, int log2) {
+  const int ctas = (1 << 2 * log2) / kTraceThreads, U = tiles_across(G, log2), n = (int)blockIdx.x / ctas;
   const int to_come = U * U - n;  // this tile included; its ring's side: the least of U's parity with side^2 >= to_come
   int side = (int)sqrtf((float)to_come);
   while (side * side < to_come) ++side;
@@ -608,15 +620,15 @@ __device__ inline int tiled_ray(int G) {
     ty = edge + side - 1;
     tx = edge + p - 2 * (side - 2);
   }
-  const int at = threadIdx.x + kTraceThreads * (blockIdx.x % kTileCtas);
-  const int col = tx * kTile + at % kTile, row = ty * kTile + at / kTile;
+  const int at = threadIdx.x + kTraceThreads * ((int)blockIdx.x - n * ctas);
+  const int col = (tx << log2) + (at & ((1 << log2) - 1)), row = (ty << log2) + (at >> log2);
   return col < G && row < G ? row * G + col : -1;
 }
 
 template <bool kCount>
 __global__ void __launch_bounds__(kTraceThreads, SBR_TRACE_MIN_BLOCKS) k_trace(const float4* __restrict__ tris,
                                                const Node4* __restrict__ nodes, int nt, GridArg g,
-                                               const int32_t* __restrict__ ray_ids, int n_rays,
+                                               const int32_t* __restrict__ ray_ids, int n_rays, int tile,
                                                int K, sbr_hit* __restrict__ hits,
                                                float4* __restrict__ hit_pos,
                                                float* __restrict__ ray_w,
@@ -626,7 +638,7 @@ __global__ void __launch_bounds__(kTraceThreads, SBR_TRACE_MIN_BLOCKS) k_trace(c
                                                const Node4* __restrict__ top, const int32_t* __restrict__ top_n) {
   after_previous();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (!ray_ids && (i = tiled_ray(g.G)) < 0) i = n_rays;
+  if (tile != kInOrder && (i = tiled_ray(g.G, tile)) < 0) i = n_rays;
   int n_nodes = 0, n_tris = 0, n_trav = 0;
   if (kTopLevels > 0) {  // every thread of the CTA, before any may return
     const int n = *top_n;
@@ -1368,6 +1380,7 @@ static sbr_status trace_impl(const sbr_scene* scene, const sbr_radar_cfg* radar,
   if (R > kWarpRaysMax) SBR_CUDA(cudaMemsetAsync(dctr, 0, 2 * sizeof(unsigned int), st));  // the hand-over's
   float4* hp = reinterpret_cast<float4*>(paths->hit_pos);
   if (d_counts) SBR_CUDA(cudaMemsetAsync(d_counts, 0, 4 * sizeof(unsigned long long), st));
+  const int tile = tile_log2(R, d_ray_ids != nullptr);
   if (R <= kWarpRaysMax) {  // a group of lanes per ray (no hand-over needed)
     const int nbw = blocks(R * kGroup, 128);
     ::sbr::note_launch();
@@ -1377,12 +1390,12 @@ static sbr_status trace_impl(const sbr_scene* scene, const sbr_radar_cfg* radar,
       launch_after(k_trace_warp<false>, nbw, 128, 0, st, scene->tris, scene->nodes4, scene->nt, g, d_ray_ids, (int)R, max_bounces, paths->hits, hp, paths->ray_weight, paths->ray_first, nullptr);
   } else if (d_counts) {
     ::sbr::note_launch();
-    launch_after(k_trace<true>, trace_blocks(R, grid->G, d_ray_ids != nullptr), kTraceThreads, 0, st, scene->tris, scene->nodes4, scene->nt, g, d_ray_ids, (int)R, max_bounces, paths->hits, hp, paths->ray_weight, paths->ray_first, dumps, dctr, d_counts, scene->top, scene->top_n);
+    launch_after(k_trace<true>, trace_blocks(R, grid->G, tile), kTraceThreads, 0, st, scene->tris, scene->nodes4, scene->nt, g, d_ray_ids, (int)R, tile, max_bounces, paths->hits, hp, paths->ray_weight, paths->ray_first, dumps, dctr, d_counts, scene->top, scene->top_n);
     ::sbr::note_launch();
     launch_after(k_trace_coop<true>, coop_grid(), 128, 0, st, scene->tris, scene->nodes4, scene->nt, g, max_bounces, dumps, dctr, dctr + 1, paths->hits, hp, paths->ray_first, d_counts);
   } else {
     ::sbr::note_launch();
-    launch_after(k_trace<false>, trace_blocks(R, grid->G, d_ray_ids != nullptr), kTraceThreads, 0, st, scene->tris, scene->nodes4, scene->nt, g, d_ray_ids, (int)R, max_bounces, paths->hits, hp, paths->ray_weight, paths->ray_first, dumps, dctr, nullptr, scene->top, scene->top_n);
+    launch_after(k_trace<false>, trace_blocks(R, grid->G, tile), kTraceThreads, 0, st, scene->tris, scene->nodes4, scene->nt, g, d_ray_ids, (int)R, tile, max_bounces, paths->hits, hp, paths->ray_weight, paths->ray_first, dumps, dctr, nullptr, scene->top, scene->top_n);
     ::sbr::note_launch();
     launch_after(k_trace_coop<false>, coop_grid(), 128, 0, st, scene->tris, scene->nodes4, scene->nt, g, max_bounces, dumps, dctr, dctr + 1, paths->hits, hp, paths->ray_first, nullptr);
   }

@@ -1,5 +1,6 @@
-"""A full grid (tiles of 16 x 16 rays from the border inwards) against the same rays as a list (taken
-in its order): the same records, bit for bit, and every ray traced once."""
+"""A full grid (in order up to one wave of CTAs, then in tiles of 32 x 32 and above 400,000 rays of 16 x
+16 rays from the border inwards) against the same rays as a list (taken in its order): the same
+records, bit for bit, and every ray traced once."""
 import pytest
 import torch
 
@@ -8,8 +9,8 @@ from sbr_inputs import ground_plane, jittered, merge_meshes, radar_single_tx, ra
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("G,jitter", [(182, False), (183, True), (191, False), (192, True), (193, False), (208, True),
-                                      (225, False)])
+@pytest.mark.parametrize("G,jitter", [(182, False), (369, True), (370, False), (383, True), (384, False), (385, True),
+                                      (632, False), (633, True), (640, False), (641, True)])
 def test_tiles_match_list(sbr, G, jitter):
     v, f, _ = superquadric(5, 60, 60, center=(0.0, 0.0, 1.0))
     v, f = (torch.from_numpy(x).cuda() for x in merge_meshes((v, f), ground_plane(-0.2, 0.0, 1.0)))
