@@ -330,7 +330,7 @@ def e2e_arm(sbr, torch, wl, cfg, args, world, flush):
 # what was captured.  Each kernel runs once per stage call.
 COUNTER_STAGES = {
     "trace": ("k_trace", "k_trace_coop", "k_tile_sums", "k_scan_single", "k_tile_scan", "k_scan_small", "k_prep"),
-    "synthesize": ("k_nufft_spread", "k_nufft_finish", "k_reduce"),
+    "synthesize": ("k_nufft_spread", "k_nufft_finish", "k_nufft_finish_cluster", "k_reduce"),
     "pointcloud": ("k_fft_rows", "k_fft_cols", "k_angle_power", "k_angle_tc", "k_power_reduce", "k_detect",
                    "k_select"),
 }
@@ -424,7 +424,7 @@ def rooflines(stage_ms, wl, P, counts, peaks, src):
       antenna) + 4 B per path) per second against the HBM copy rate: the working set is L2-resident,
       so these bytes are served mostly by L1/L2 (a bytes-served rate, not DRAM);
       dram: the call's DRAM bytes (ncu) per second against the HBM copy rate.
-    synthesis (k_nufft_spread + k_nufft_finish; Eq. 8 as a type-1 non-uniform FFT):
+    synthesis (k_nufft_spread + k_nufft_finish_cluster; Eq. 8 as a type-1 non-uniform FFT):
       dram as above; speedup_vs_direct_sum: Eq. 8 terms (path, antenna, sample) per second over the
       FP32-pipe bound of a term-by-term kernel (152 SMs x 128 lanes x f_max / 4 lane-ops per term)."""
     V, Ns = wl.radar.n_virt, wl.radar.n_samples
@@ -462,7 +462,7 @@ def rooflines(stage_ms, wl, P, counts, peaks, src):
     ach, frac = issue("synthesize", t_sy)
     fp32_terms = 152 * 128 * mhz * 1e6 / 4
     rec = P * V * 16
-    synth = {"kernel": "k_nufft_spread (+ k_nufft_finish)", "bound": "alu", "limiter": "issue slots",
+    synth = {"kernel": "k_nufft_spread (+ k_nufft_finish_cluster)", "bound": "alu", "limiter": "issue slots",
              "achieved": ach, "peak": issue_peak, "unit": "warp-inst/s", "frac": frac,
              "inst_per_launch": ctr.get("synthesize", {}).get("inst_per_launch"),
              "traffic": ctr.get("synthesize", {}).get("dram_bytes_per_launch"),

@@ -1,6 +1,6 @@
 // Ray tracing with specular bounces (Section 3.2.1, Eq. 2-3) and path preparation.
 //
-// One thread per ray.  The ray is carried in float-float (ff.cuh): its FP32 hi
+// One thread per ray (up to 32,768 rays eight lanes, k_trace_warp).  The ray is carried in float-float (ff.cuh): its FP32 hi
 // parts drive a stack traversal of the 4-wide BVH collapsed from the LBVH (a
 // node's four child boxes and links as seven float4 loads, triangles as three
 // float4 loads) with the Moller-Trumbore (1997) test.  Every
