@@ -826,24 +826,25 @@ __global__ void __launch_bounds__(kNuThreads, 3)
   }
 }
 
-// The split phase of a moving scene whose grid a CTA holds whole: CTA (q, v) spreads
-// its records for the launch's chirps, up to kTile.  From one chirp to the next a
-// record's phasor turns by a constant and its grid position moves by a constant, so the
-// preparation (two sines, the split phase) is paid once per tile, from that chirp's own
-// delays, and a chirp costs a complex product and the sixteen additions: 12 antennas x
-// 367,500 records x 128 chirps 3.5 ms
-// against 5.0 in groups chirp by chirp (8 chirps at a time 3.9, 4 at a time 4.6; a
-// third of it adds the chunks' copies up).  The rounding of up to kTile - 1 turns adds
-// about 1e-7.  A chunk's sums go to the chirp's grid in global memory (L2), each
-// point by one thread; kTile copies in shared memory would cost a resident CTA.
+// The split phase of a moving scene: CTA (q, v) spreads its records for the launch's
+// chirps, up to kTile, a block of cells at a time (kBlocks: two, 512 samples).  From one
+// chirp to the next a record's phasor turns by a constant and its grid position moves by
+// a constant, so the preparation (two sines, the split phase) is paid once per tile, from
+// that chirp's own delays, and a chirp costs a complex product and the sixteen additions:
+// 12 antennas x 367,500 records x 128 chirps 3.5 ms against 5.0 in groups chirp by chirp
+// (8 chirps at a time 3.9, 4 at a time 4.6; a third of it adds the chunks' copies up), 512
+// samples, 12 x 8,600 records 843 -> 560 us.  The rounding of up to kTile - 1 turns adds
+// about 1e-7.  A chunk's sums go to the chirp's grid in global memory (L2), each point by
+// one thread; kTile copies in shared memory would cost a resident CTA.
 constexpr int kTile = 16;  // chirps per launch
+template <bool kBlocks>
 __global__ void __launch_bounds__(kNuThreads, 3)
     k_nufft_spread_chirps(const float4* __restrict__ prep, const float* __restrict__ rate, int64_t cap,
                           const int32_t* __restrict__ d_P, const NufftArg na, const __grid_constant__ NufftCoef co, float2* __restrict__ grids) {
   extern __shared__ int4 nsm[];  // [npts][re, im][kNuCopies]
   __shared__ uint32_t s_max[2];
   __shared__ int flag[2][kNuBlock / 8];
-  const int M = 1 << na.log_m, npts = nu_points(M), oct = M >> 3;
+  const int M = 1 << na.log_m, bs = nu_cells(M), npts = nu_points(M), oct = bs >> 3;
   const int tid = threadIdx.x, lane = tid & 31;
   const int v = blockIdx.x % na.V, q = blockIdx.x / na.V, nc = na.chirps;
   const double dt = (double)na.chirp0 * na.per_chirp;  // path length change per (m/s)
@@ -913,16 +914,19 @@ __global__ void __launch_bounds__(kNuThreads, 3)
       c1[u] *= scale;
       c2[u] *= scale;
     }
-    for (int k = 0; k < nc; ++k, ++pass) {
+    for (int kb = 0, b = 0; kb < (kBlocks ? nc * (M / bs) : nc); ++kb, ++pass) {
+      const int k = kBlocks ? kb / (M / bs) : kb;
+      if (kBlocks) b = kb - k * (M / bs);
       int* fl = flag[pass & 1];
       if (tid < kNuBlock / 8) flag[~pass & 1][tid] = 0;  // read before this pass
       if (tid == 0) s_max[~chunk & 1] = 0u;
 #pragma unroll
       for (int u = 0; u < kNuItems; ++u) {
-        if (c1[u] != 0.f || c2[u] != 0.f) {
-          int* g1 = mine + cell[u] * (2 * kNuCopies) + (upper ? kNuCopies : 0);
-          int* g2 = mine + cell[u] * (2 * kNuCopies) + (upper ? 0 : kNuCopies);
-          fl[cell[u] >> 3] = 1;
+        const int idx = kBlocks ? cell[u] - b * bs : cell[u];
+        if ((!kBlocks || (unsigned)idx < (unsigned)bs) && (c1[u] != 0.f || c2[u] != 0.f)) {
+          int* g1 = mine + idx * (2 * kNuCopies) + (upper ? kNuCopies : 0);
+          int* g2 = mine + idx * (2 * kNuCopies) + (upper ? 0 : kNuCopies);
+          fl[idx >> 3] = 1;
           float wl[4], wrt[4];
           nu_weights(co, s[u], wl, wrt);
 #pragma unroll
@@ -933,6 +937,7 @@ __global__ void __launch_bounds__(kNuThreads, 3)
             atomicAdd(g2 + (7 - j) * (2 * kNuCopies), nu_term(c2[u], wrt[j], j < kNuSmall));
           }
         }
+        if (kBlocks && (b + 1) * bs < M) continue;
         // the next chirp
         const float a = c1[u];
         c1[u] = fmaf(a, wr[u], -c2[u] * wi[u]);
@@ -943,20 +948,21 @@ __global__ void __launch_bounds__(kNuThreads, 3)
       }
       __syncthreads();
       // half-warp h adds up the octets of points o = h mod 16 (as k_nufft_spread), into the
-      // chirp's grid; the points past the grid's end belong to octet 0
+      // chirp's grid; the points past the grid's end belong to octet 0, those past a block's
+      // end to the next block, whose turn is another pass
       const unsigned m0 = __ballot_sync(0xffffffffu, fl[lane] != 0), m1 = __ballot_sync(0xffffffffu, fl[32 + lane] != 0);
-      const unsigned long long cells = (unsigned long long)m1 << 32 | m0, last = cells >> (oct - 1) & 1ull,
+      const unsigned long long cells = (unsigned long long)m1 << 32 | m0, last = kBlocks ? 0ull : cells >> (oct - 1) & 1ull,
                                lit = cells | cells << 1 | last;
       float* to = reinterpret_cast<float*>(out + (size_t)k * M);
 #pragma unroll
-      for (int r = 0; r < kNuBlock / 8 / 16; ++r) {
+      for (int r = 0; r < kNuBlock / 8 / 16 + (kBlocks ? 1 : 0); ++r) {
         const int o = r * 16 + (tid >> 4);
-        if (o >= oct || !((lit >> o) & 1ull)) continue;
+        if (kBlocks ? o > 64 || !(o < 64 ? lit >> o & 1ull : cells >> 63) : o >= oct || !((lit >> o) & 1ull)) continue;
         const int i = o * 16 + (tid & 15);  // point i / 2, part i & 1
-        float* g = to + 2 * (((i >> 1) - (kNuW / 2 - 1)) & (M - 1)) + (i & 1);
+        float* g = to + 2 * ((b * bs + (i >> 1) - (kNuW / 2 - 1)) & (M - 1)) + (i & 1);
         const float old = *g;
         long long t = 0;
-        for (int h = 0; h < (o == 0 ? 2 : 1); ++h) {
+        for (int h = 0; h < (!kBlocks && o == 0 ? 2 : 1); ++h) {
           const int ii = i + h * 2 * M;
 #pragma unroll
           for (int w4 = 0; w4 < kNuCopies / 4; ++w4) {
@@ -1436,6 +1442,7 @@ void grid_shape(int V, int Ns, int64_t cap, int* Q) {
 
 // dynamic shared memory of the spreading kernel: the grid's copies and its sums
 inline size_t nufft_smem(int Ns) { return (2 * kNuCopies * sizeof(int) + 2 * sizeof(float)) * (size_t)nu_points(2 * Ns); }
+inline auto chirps_kernel(int Ns) { return 2 * Ns > kNuBlock ? k_nufft_spread_chirps<true> : k_nufft_spread_chirps<false>; }
 inline size_t nufft_chirps_smem(int Ns) { return 2 * kNuCopies * sizeof(int) * (size_t)nu_points(2 * Ns); }
 inline size_t nufft_cl_smem(int Ns) {
   return sizeof(float2) * (size_t)(fft::slots(2 * Ns) + fft::slots(Ns) + kNuClThreads + 2 * Ns / kNuRanks);
@@ -1471,7 +1478,7 @@ int nufft_per_sm(int Ns) {
     n = std::min(n, m > 0 ? m : 1);
   }
   if (nufft_chirps_smem(Ns) > 48 * 1024)
-    cudaFuncSetAttribute(k_nufft_spread_chirps, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)nufft_chirps_smem(Ns));
+    cudaFuncSetAttribute(chirps_kernel(Ns), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)nufft_chirps_smem(Ns));
   if (nufft_fin_smem(Ns) > 48 * 1024)
     cudaFuncSetAttribute(k_nufft_finish, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)nufft_fin_smem(Ns));
   if (dev < kDevCache) cache[dev][lg] = n;
@@ -1487,19 +1494,26 @@ void nufft_shape(int V, int Ns, int64_t cap, int* Qn) {
   *Qn = (int)q;
 }
 
-// Moving scenes whose chirps go in tiles: a grid that a CTA holds whole, and chirps
-// enough to pay for the slower inner loop (2 chirps x 114,000 records: 20.7 us in tiles,
-// 17.3 in a group; 16 chirps: 80 against 130; 16 x 950 records: 28 against 109).
-inline bool nufft_tiles(int C, int Ns) { return 2 * Ns <= kNuBlock && C >= 4; }
+// Moving scenes whose chirps go in tiles: records enough to fill the CTAs that every launch
+// of a tile puts to work, chirps enough to pay for the slower inner loop.  Tiles / groups:
+// 12 antennas x 256 samples x 128 chirps, slots per antenna 4,050: 368 / 193 us, 7,200: 378 /
+// 679; 4 antennas, 7,200: 273 / 113, 12,800: 284 / 398, 28,800: 300 / 635; 16 chirps, 12,800:
+// 35 / 16, 28,800: 38 / 81; 2 chirps x 320,000: 20.7 / 17.3; 512 samples x 128 chirps, 4
+// antennas, 28,800: 444 / 800.
+constexpr int64_t kTileSlots = 65536;  // all antennas'
+inline bool nufft_tiles(int V, int C, int Ns, int64_t cap) {
+  return Ns <= kNuMovingMaxSamples && C >= 4 && V * cap >= kTileSlots;
+}
 
 // Grids per antenna in the workspace: one per spreading CTA, and for the chirps of a moving
-// scene a tile's from each (at most 30 MB) or, in groups, a wave's (a group is then not
-// held to the few CTAs that few paths ask for: 512 samples, 128 chirps x 950 records 1.01 -> 0.13 ms).
+// scene a tile's from each (at most 30 MB, 60 with 512 samples) or, in groups, a wave's (a
+// group is then not held to the few CTAs that few paths ask for: 512 samples, 128 chirps x 950
+// records 1.01 -> 0.13 ms).
 inline int nufft_wave(int V, int qn, int C, int Ns) {
   return (int)std::max<int64_t>(qn, std::min<int64_t>((int64_t)qn * C, (int64_t)sm_count() * nufft_per_sm(Ns) / V));
 }
-inline int nufft_grids(int V, int qn, int C, int Ns) {
-  return nufft_tiles(C, Ns) ? qn * std::min(C, kTile) : nufft_wave(V, qn, C, Ns);
+inline int nufft_grids(int V, int qn, int C, int Ns, int64_t cap) {
+  return nufft_tiles(V, C, Ns, cap) ? qn * std::min(C, kTile) : nufft_wave(V, qn, C, Ns);
 }
 
 // Workspace: per-CTA partial sums of the direct kernels, the chirp-summed
@@ -1514,7 +1528,7 @@ size_t ws_layout(const sbr_radar_cfg* radar, int64_t cap, int* Q, int* Qn = null
   Carver c(nullptr);
   c.take<float2>((size_t)V * (*Q) * Ns);       // per-CTA partial sums
   c.take<float2>((size_t)V * Ns);              // chirp-summed upstream gradient
-  const int qg = nufft_grids(V, qn, radar->n_chirps, Ns);
+  const int qg = nufft_grids(V, qn, radar->n_chirps, Ns, cap);
   c.take<float2>((size_t)V * qg * 2 * Ns);     // non-uniform FFT: the CTAs' grids
   c.take<float2>((size_t)V * qg * 2 * Ns);     // non-uniform FFT: the rows' summed grids (a moving scene: V * chirps)
   c.take<unsigned int>((size_t)V * qg);        // non-uniform FFT: finishing counters
@@ -1557,7 +1571,7 @@ sbr_status bind_ws(const sbr_radar_cfg* radar, int64_t cap, void* ws, size_t byt
   Carver c(ws);
   w->partial = c.take<float2>((size_t)V * Q * Ns);
   w->gsum = c.take<float2>((size_t)V * Ns);
-  w->Qg = nufft_grids(V, Qn, radar->n_chirps, Ns);
+  w->Qg = nufft_grids(V, Qn, radar->n_chirps, Ns, cap);
   w->grids = c.take<float2>((size_t)V * w->Qg * 2 * Ns);
   w->bsum = c.take<float2>((size_t)V * w->Qg * 2 * Ns);
   w->fin_cnt = c.take<unsigned int>((size_t)V * w->Qg);
@@ -1617,7 +1631,7 @@ void launch_chirps(const sbr_paths* p, const sbr_radar_cfg* r, const SynthWs& w,
   for (int c = 0; c < C; c += kTile) {
     const NufftArg na = nufft_arg(p, r, w.Qn, c, std::min(kTile, C - c));
     ::sbr::note_launch();
-    launch_after(k_nufft_spread_chirps, V * w.Qn, kNuThreads, nufft_chirps_smem(Ns), st,
+    launch_after(chirps_kernel(Ns), V * w.Qn, kNuThreads, nufft_chirps_smem(Ns), st,
                  reinterpret_cast<const float4*>(p->prep), p->path_rate, p->path_cap, p->count, na, nufft_coef(), w.grids);
     ::sbr::note_launch();
     launch_after(k_nufft_finish_cluster, V * na.chirps * kNuRanks, kNuClThreads, nufft_cl_smem(Ns), st, w.grids, na,
@@ -1626,8 +1640,8 @@ void launch_chirps(const sbr_paths* p, const sbr_radar_cfg* r, const SynthWs& w,
 }
 
 // A moving scene: every chirp synthesised from its own delays (split phase up to 512
-// samples, or the FP64 phase), in tiles of chirps or (two blocks of cells, the FP64
-// phase, few chirps) a group of chirps per launch.  A group's launch is one wave of Q
+// samples, or the FP64 phase), in tiles of chirps or (the FP64 phase, few records, few
+// chirps) a group of chirps per launch.  A group's launch is one wave of Q
 // CTAs per antenna and chirp; fewer CTAs per chirp mean fewer launches and the same
 // records per CTA in all, so Q is the one whose launches / Q, the chirps' share of a
 // wave each, is least (12 antennas x 128 chirps: 2 CTAs each, 7 launches of 19 chirps,
@@ -1638,7 +1652,7 @@ sbr_status launch_moving(sbr_phase_mode mode, const sbr_paths* p, const sbr_rada
                          float2* cube, cudaStream_t st) {
   if (mode == SBR_PHASE_FP64 || (mode == SBR_PHASE_SPLIT && r->n_samples <= kNuMovingMaxSamples)) {
     const int C = r->n_chirps;
-    if (mode == SBR_PHASE_SPLIT && nufft_tiles(C, r->n_samples)) {
+    if (mode == SBR_PHASE_SPLIT && nufft_tiles(p->n_virt, C, r->n_samples, p->path_cap)) {
       launch_chirps(p, r, w, cube, st);
       return SBR_OK;
     }

@@ -124,9 +124,10 @@ def test_split_records_not_finite(sbr):
     assert torch.isnan(cube[2]).all() and torch.isfinite(cube[[0, 1, 3]]).all()
 
 
-@pytest.mark.parametrize("ns,nc,P", [(256, 16, 7001), (32, 2, 1025), (64, 128, 300), (128, 64, 2049), (512, 4, 5000)])
+@pytest.mark.parametrize("ns,nc,P", [(256, 16, 7001), (32, 2, 1025), (64, 128, 300), (128, 64, 2049), (512, 4, 5000),
+                                     (32, 16, 5460), (64, 32, 5459), (128, 64, 6145), (512, 4, 5460), (512, 16, 7001)])
 def test_moving_records(sbr, ns, nc, P):
-    """Every chirp from its own delays: chirps in tiles (up to 256 samples) and one by one (512)."""
+    """Every chirp from its own delays: chirps in tiles (from 65,536 record slots) and in groups."""
     radar = radar_mimo_3x4(ns, nc)
     delta, phi, A = records(9 + ns, 12, P, ns)
     rate = np.random.default_rng(4).uniform(-8.0, 8.0, delta.shape).astype(np.float32)
