@@ -1516,6 +1516,9 @@ inline int nufft_grids(int V, int qn, int C, int Ns, int64_t cap) {
   return nufft_tiles(V, C, Ns, cap) ? qn * std::min(C, kTile) : nufft_wave(V, qn, C, Ns);
 }
 
+// Summed grids per antenna: none where a cluster finishes the rows.
+inline int nufft_sums(int qg, int Ns) { return 2 * Ns <= kNuClusterPoints ? 0 : qg; }
+
 // Workspace: per-CTA partial sums of the direct kernels, the chirp-summed
 // upstream gradient of the adjoint, and, for the non-uniform FFT, the CTAs'
 // grids, their sum and the finishing counters.
@@ -1530,7 +1533,7 @@ size_t ws_layout(const sbr_radar_cfg* radar, int64_t cap, int* Q, int* Qn = null
   c.take<float2>((size_t)V * Ns);              // chirp-summed upstream gradient
   const int qg = nufft_grids(V, qn, radar->n_chirps, Ns, cap);
   c.take<float2>((size_t)V * qg * 2 * Ns);     // non-uniform FFT: the CTAs' grids
-  c.take<float2>((size_t)V * qg * 2 * Ns);     // non-uniform FFT: the rows' summed grids (a moving scene: V * chirps)
+  c.take<float2>((size_t)V * nufft_sums(qg, Ns) * 2 * Ns);  // non-uniform FFT: the rows' summed grids (a moving scene: V * chirps)
   c.take<unsigned int>((size_t)V * qg);        // non-uniform FFT: finishing counters
   c.take<float4>((size_t)V * (2 * Ns + kAdjMargin));  // adjoint: the antennas' grids
   return c.bytes();
@@ -1573,7 +1576,7 @@ sbr_status bind_ws(const sbr_radar_cfg* radar, int64_t cap, void* ws, size_t byt
   w->gsum = c.take<float2>((size_t)V * Ns);
   w->Qg = nufft_grids(V, Qn, radar->n_chirps, Ns, cap);
   w->grids = c.take<float2>((size_t)V * w->Qg * 2 * Ns);
-  w->bsum = c.take<float2>((size_t)V * w->Qg * 2 * Ns);
+  w->bsum = c.take<float2>((size_t)V * nufft_sums(w->Qg, Ns) * 2 * Ns);
   w->fin_cnt = c.take<unsigned int>((size_t)V * w->Qg);
   w->adj = c.take<float4>((size_t)V * (2 * Ns + kAdjMargin));
   w->Q = Q;
