@@ -1460,8 +1460,12 @@ inline NufftSpread nufft_kernel(int Ns, bool fp64, bool moving) {
   return 2 * Ns > kNuBlock ? nufft_kernel_of<true>(fp64, moving) : nufft_kernel_of<false>(fp64, moving);
 }
 
+constexpr int kMaxSamples = 4096;  // check_radar's
+
 // resident spreading CTAs per SM (shared memory and registers decide); raises
-// the kernels' shared-memory limits once where they pass 48 KB
+// the kernels' shared-memory limits once where they pass 48 KB.  A limit belongs to
+// the kernel, whatever the sample count it was raised for, and the counts are cached
+// one by one: each is the most its kernel ever asks for, so none lowers another's.
 int nufft_per_sm(int Ns) {
   static int cache[kDevCache][16] = {};
   int lg = 0;
@@ -1480,7 +1484,7 @@ int nufft_per_sm(int Ns) {
   if (nufft_chirps_smem(Ns) > 48 * 1024)
     cudaFuncSetAttribute(chirps_kernel(Ns), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)nufft_chirps_smem(Ns));
   if (nufft_fin_smem(Ns) > 48 * 1024)
-    cudaFuncSetAttribute(k_nufft_finish, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)nufft_fin_smem(Ns));
+    cudaFuncSetAttribute(k_nufft_finish, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)nufft_fin_smem(kMaxSamples));
   if (dev < kDevCache) cache[dev][lg] = n;
   return n;
 }
