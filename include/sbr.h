@@ -304,7 +304,7 @@ sbr_status sbr_trace_counts(const sbr_scene* scene, const sbr_radar_cfg* radar,
 /* Synthesis (Section 3.2.2, Eq. 8)                                         */
 /* ------------------------------------------------------------------------ */
 
-/* Scratch bytes for sbr_synthesize / sbr_synthesize_bwd. */
+/* Scratch bytes for sbr_synthesize / sbr_synthesize_bwd; 0 for a radar they do not support. */
 size_t sbr_synth_ws_bytes(const sbr_radar_cfg* radar, int64_t path_cap);
 
 /* d_cube [V][C][N_s] complex64 (interleaved re, im) =

@@ -1460,7 +1460,7 @@ inline NufftSpread nufft_kernel(int Ns, bool fp64, bool moving) {
   return 2 * Ns > kNuBlock ? nufft_kernel_of<true>(fp64, moving) : nufft_kernel_of<false>(fp64, moving);
 }
 
-constexpr int kMaxSamples = 4096;  // check_radar's
+constexpr int kMinSamples = 32, kMaxSamples = 4096;  // check_radar's
 
 // resident spreading CTAs per SM (shared memory and registers decide); raises
 // the kernels' shared-memory limits once where they pass 48 KB.  A limit belongs to
@@ -1549,7 +1549,12 @@ size_t ws_layout(const sbr_radar_cfg* radar, int64_t cap, int* Q, int* Qn = null
 using namespace sbr;
 
 extern "C" size_t sbr_synth_ws_bytes(const sbr_radar_cfg* radar, int64_t path_cap) {
-  if (!radar || radar->n_tx < 1 || radar->n_rx < 1 || radar->n_samples < 1) return 0;
+  if (!radar || radar->n_tx < 1 || radar->n_rx < 1) return 0;
+  const int Ns = radar->n_samples;  // the layout asks the device about kernels that exist for these sizes alone
+  if (Ns < kMinSamples || Ns > kMaxSamples || (Ns & (Ns - 1)) != 0) {
+    set_error("sbr_synth_ws_bytes: n_samples=%d must be a power of two in [%d, %d]", Ns, kMinSamples, kMaxSamples);
+    return 0;
+  }
   int Q;
   return ws_layout(radar, path_cap, &Q);
 }

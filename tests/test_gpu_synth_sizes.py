@@ -39,3 +39,17 @@ def test_sample_counts_in_any_order(sizes):
     r = subprocess.run([sys.executable, "-c", SIZES, *map(str, sizes)], cwd=ROOT, capture_output=True, text=True,
                        timeout=300, env={**os.environ, "PYTHONPATH": ROOT})
     assert r.returncode == 0, r.stderr[-2000:]
+
+
+def test_refused_sample_count_leaves_the_next_call_alone(sbr):
+    """A sample count that is refused raises its own error, and no later call inherits one."""
+    import torch
+    from sbr_inputs import radar_single_tx
+    paths = sbr.PathBuffers(3000, 1, 4)
+    paths.mem.zero_()
+    for ns in (16384, 16, 100):
+        assert sbr.synth_ws_bytes(radar_single_tx(ns, 1), paths.cap) == 0
+        with pytest.raises(Exception, match="n_samples"):
+            sbr.synthesize(paths, radar_single_tx(ns, 1))
+        assert float(sbr.synthesize(paths, radar_single_tx(1024, 1)).abs().max()) == 0.0
+    torch.cuda.synchronize()
