@@ -314,7 +314,8 @@ size_t sbr_synth_ws_bytes(const sbr_radar_cfg* radar, int64_t path_cap);
  * least 65536 record slots (path_cap * n_virt; 8192 above 512 samples) is
  * evaluated as a type-1 non-uniform FFT (spreading onto 2 N_s grid points with a width-8
  * Kaiser-Bessel kernel, one FFT, deconvolution; below 1e-6 relative to the FP64
- * sum), term by term otherwise.  SBR_PHASE_FP64 forms each
+ * sum, whatever the amplitudes, as long as that is not small against the root of
+ * their sum of squares), term by term otherwise.  SBR_PHASE_FP64 forms each
  * path's carrier phase and grid position in FP64 from paths->path_len and is
  * evaluated the same way; SBR_PHASE_NAIVE rounds the delay
  * to FP32.  With SBR_SYNTH_MOVING OR'ed into mode (paths traced on a scene with

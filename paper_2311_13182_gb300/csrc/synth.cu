@@ -548,14 +548,14 @@ __global__ void __launch_bounds__(256) k_synth_bwd(const float4* __restrict__ pr
 // while the upper adds imaginary parts (then the other way round), so the 32
 // lanes of an atomic always hit 32 different banks, whatever the cells are:
 // neighbouring rays share cells, and consecutive records jump between a ray's
-// bounces.  A term is rounded to 2^-24 of the chunk's largest amplitude, so that
-// a chunk's additions to one copy stay below 2^30; after each chunk the copies of
-// the touched cells (a flag per eight cells) are summed, scaled and added to the
-// CTA's FP32 grid, each point by one thread.  The CTAs' grids are added in a fixed
-// order by the finishing kernel.
+// bounces.  A term is rounded to 2^-25 to 2^-24 of the largest amplitude of its class
+// (nu_class: nearly always its chunk of 1,024 records), so that a chunk's additions to
+// one copy stay below 2^31; after each class the copies of the touched cells (a flag
+// per eight cells) are summed, scaled and added to the CTA's FP32 grid, each point by
+// one thread.  The CTAs' grids are added in a fixed order by the finishing kernel.
 //
-// A CTA has a barrier for a chunk's maximum and one before its sums are added up;
-// the next chunk's records are in flight meanwhile, and its preparation needs none.
+// A CTA has a barrier for a chunk's largest amplitude and one before its sums are added
+// up; the next chunk's records are in flight meanwhile, and its preparation needs none.
 // Bound by issue slots (212 instructions per 32 records) and the conversion unit,
 // three CTAs per SM: 12 antennas x 367,500 records x 256 samples 35 us (109 us when
 // each warp kept runs of equal cells in registers, eight lanes to a record, and
@@ -571,8 +571,9 @@ constexpr int kNuBlock = 512;  // cells a CTA's grid holds at once (71 KB: three
 constexpr int kNuThreads = 256;
 constexpr int kNuItems = 4;    // records per thread and chunk
 constexpr int kNuChunk = kNuThreads * kNuItems;
-constexpr int kNuBits = 24;    // 2 kNuChunk / 32 additions per copy of terms up to 0.98 2^24: below 2^30
-static_assert(kNuChunk / kNuCopies <= 1 << (30 - kNuBits), "a chunk's additions to one copy");
+constexpr int kNuBits = 25;    // 2 kNuChunk / 32 additions per copy of terms up to 0.98 2^25: below 2^31
+static_assert(kNuChunk / kNuCopies <= 1 << (31 - kNuBits), "a class's additions to one copy");
+constexpr int kNuSpan = 24;    // mean distance of a class's amplitudes from its largest, in eighths of an octave
 constexpr double kNuBeta = 2.3 * kNuW;
 
 struct NufftCoef {
@@ -614,12 +615,86 @@ __device__ __forceinline__ void nu_weights(const NufftCoef& co, float s, float (
   }
 }
 
-// c w rounded to an integer.  Below 2^22 (the outer points: psi <= 0.085 from two
-// grid steps on) by one FMA against 1.5 2^23 and the bits' difference, which leaves
-// the conversion unit, a quarter of the FMA pipe's rate, to the inner points.
+// I0(2 sqrt(q)) by its power series (the terms are positive: no cancellation; q < 100).
+constexpr double bessel_i0_of(double q) {
+  double t = 1.0, s = 1.0;
+  for (int k = 1; k < 200 && t > 1e-18 * s; ++k) {
+    t *= q / ((double)k * k);
+    s += t;
+  }
+  return s;
+}
+
+// c w rounded to an integer.  Below 2^22 (the outer points: psi <= psi(2) = 0.0914 from
+// two grid steps on, terms up to 3.0e6) by one FMA against 1.5 2^23 and the bits'
+// difference, which leaves the conversion unit, a quarter of the FMA pipe's rate, to the
+// inner points.
 constexpr int kNuSmall = 2;  // outer points on either side
+constexpr double nu_outer(double x) {  // psi(x)
+  return bessel_i0_of(0.25 * kNuBeta * kNuBeta * (1.0 - (2.0 * x / kNuW) * (2.0 * x / kNuW))) /
+         bessel_i0_of(0.25 * kNuBeta * kNuBeta);
+}
+static_assert(0.98 * (1 << kNuBits) * nu_outer(kNuW / 2 - kNuSmall) < 0.99 * (1 << 22), "outer terms pass the FMA's range");
 __device__ __forceinline__ int nu_term(float c, float w, bool small) {
   return small ? __float_as_int(fmaf(c, w, 12582912.f)) - 0x4B400000 : __float2int_rn(c * w);
+}
+
+// An amplitude's logarithm in eighths of an octave (2047 and 2046: not finite).
+__device__ __forceinline__ int nu_log(float a) { return (int)((__float_as_uint(a) & 0x7fffffffu) >> 20); }
+constexpr int kNuAll = 2048;  // above every logarithm
+
+// The class of records that one pass rounds on one scale, 2^s for the largest amplitude
+// (its bits: top) to land in (0.49, 0.98] 2^kNuBits: all N that are left if their
+// logarithms (sum: logs) lie within kNuSpan of the largest's on average, else those
+// within kNuSpan of it.  The class's rms amplitude is then an eighth of its largest or
+// more, and the rounding stays near the error of the transform around it; on one scale
+// for all, a chunk's few strong records would cost its weak ones their bits (one record
+// in 1,024 a hundred times the others: 9e-7 to 1.4e-6 from FP64 instead of 1.8e-7; two in
+// 1,024 a thousand times the others and cancelling: 3e-5 instead of 1.9e-7).  Specular
+// returns of one chunk differ little, so more than one class is rare; where it is not it
+// costs passes, not accuracy.  The scale is a power of two, exact; one past a float's
+// range (amplitudes below 1e-31) is applied in two factors.
+// The two words per chunk that this takes, and the copies' sum in 64 bits, cost 12
+// antennas x 367,500 records 42.0 -> 43.0 us for the whole synthesis, 4 antennas x 3.1 M
+// records x 4096 samples 122.8 -> 126.4; moving chirps (no sign extensions in the sum)
+// 3.49 -> 3.41 ms.
+struct NuClass {
+  int floor;   // logarithms from here on belong to the class; 0: every record left
+  bool rare;   // floor or more matter
+  float up, more;    // 2^s = up more, more = 1 but for the smallest amplitudes
+  float down, less;  // their reciprocals
+};
+__device__ __forceinline__ NuClass nu_class(uint32_t top, int logs, int N) {
+  const int l = (int)(top >> 20);
+  NuClass c;
+  c.floor = N * (l - kNuSpan) <= logs ? 0 : max(l - kNuSpan, 0);
+  // exponents of the largest's upper bound: one more from 1.96 on, 1 for all denormal numbers
+  const int s = 126 + kNuBits - max((int)((top + 0x51eb9u) >> 23), 1), a = min(s, 126);
+  c.rare = c.floor != 0 || s != a;
+  c.up = __int_as_float((127 + a) << 23);
+  c.more = __int_as_float((127 + s - a) << 23);
+  c.down = __int_as_float((127 - a) << 23);
+  c.less = __int_as_float((127 - s + a) << 23);
+  return c;
+}
+
+// Grid words in shared memory are kept kNuZero off, so that the copies add up unsigned,
+// with carries and no sign extension.
+constexpr uint32_t kNuZero = 0x80000000u;
+__device__ __forceinline__ uint4 nu_zero() { return make_uint4(kNuZero, kNuZero, kNuZero, kNuZero); }
+
+// The copies of a grid word (at uint4 index w0; the four 16-byte words in an order that
+// gives the lanes of a shared-memory phase different banks) summed and zeroed.
+__device__ __forceinline__ long long nu_add_up(uint4* g, int w0, int turn) {
+  unsigned long long t = 0;
+#pragma unroll
+  for (int k = 0; k < kNuCopies / 4; ++k) {
+    const int w = w0 + ((k + turn) & (kNuCopies / 4 - 1));
+    const uint4 x = g[w];
+    g[w] = nu_zero();
+    t += (unsigned long long)x.x + x.y + x.z + x.w;
+  }
+  return (long long)(t - (unsigned long long)kNuCopies * kNuZero);
 }
 
 // x = rint(x) + the returned fraction in [-1/2, 1/2], |x| < 2^50; n gets rint(x) mod 2^32.
@@ -636,8 +711,9 @@ __global__ void __launch_bounds__(kNuThreads, 3)
     k_nufft_spread(const float4* __restrict__ prep, const float2* __restrict__ plen, const float* __restrict__ phase_ofs,
                    const float* __restrict__ rate, int64_t cap, const int32_t* __restrict__ d_P, const NufftArg na,
                    const __grid_constant__ NufftCoef co, float2* __restrict__ grids, unsigned int* __restrict__ fin_cnt) {
-  extern __shared__ int4 nsm[];
-  __shared__ uint32_t s_max[2], s_blk[2];     // by the parity of the chunk
+  extern __shared__ uint4 nsm[];
+  __shared__ uint32_t s_max[2], s_blk[2];     // by the parity of the chunk: largest amplitude, blocks
+  __shared__ int s_log[2];                    // and the sum of the amplitudes' logarithms
   __shared__ int flag[2][kNuBlock / 8];       // by the parity of the pass: a record of cells 8 o .. 8 o + 7
   const int M = 1 << na.log_m, bs = nu_cells(M), npts = nu_points(M);
   int* grid = reinterpret_cast<int*>(nsm);                            // [npts][re, im][kNuCopies]
@@ -647,10 +723,10 @@ __global__ void __launch_bounds__(kNuThreads, 3)
   const double dt = kMoving ? (double)(na.chirp0 + cl) * na.per_chirp : 0.0;  // path length change per (m/s)
   const float cnu = (float)(dt * na.f0_c), ceps = (float)(dt * na.b_cn);
   float2* out = grids + (size_t)blockIdx.x * M;
-  for (int i = tid; i < npts * (2 * kNuCopies / 4); i += kNuThreads) nsm[i] = make_int4(0, 0, 0, 0);
+  for (int i = tid; i < npts * (2 * kNuCopies / 4); i += kNuThreads) nsm[i] = nu_zero();
   for (int i = tid; i < 2 * npts; i += kNuThreads) sum[i] = 0.f;
   for (int i = tid; i < 2 * (kNuBlock / 8); i += kNuThreads) (&flag[0][0])[i] = 0;
-  if (tid < 2) s_max[tid] = s_blk[tid] = 0u;
+  if (tid < 2) s_max[tid] = s_blk[tid] = 0u, s_log[tid] = 0;
   after_previous();
   if (blockIdx.x == 0)
     for (int i = tid; i < na.V * na.chirps; i += kNuThreads) fin_cnt[i] = 0u;  // the finishing kernel's counters
@@ -684,8 +760,10 @@ __global__ void __launch_bounds__(kNuThreads, 3)
   };
   load(0);
   __syncthreads();
-  for (int c0 = 0, chunk = 0; c0 < n; c0 += kNuChunk, ++chunk) {
-    int cell[kNuItems];
+  // A turn takes a class of a chunk's records: nearly always all of them.
+  int ceil = kNuAll, left = min(kNuChunk, n);  // a chunk's records from ceil on are done, `left` are not
+  for (int c0 = 0, chunk = 0; c0 < n; ++chunk) {
+    int cell[kNuItems], logs = 0;
     uint32_t am = 0, blocks = 0;
 #pragma unroll
     for (int u = 0; u < kNuItems; ++u) {
@@ -735,19 +813,46 @@ __global__ void __launch_bounds__(kNuThreads, 3)
       sincospif(2.f * x, &sn, &cs);
       rec[u] = make_float4(cs, sn, t, r.w);
       cell[u] = ce;
-      am = max(am, __float_as_uint(fabsf(r.w)));
       if (kBlocks && p < n) blocks |= 1u << (ce / kNuBlock);
     }
+    if (ceil != kNuAll) {
+#pragma unroll
+      for (int u = 0; u < kNuItems; ++u)
+        if (nu_log(rec[u].w) >= ceil) rec[u].w = 0.f;
+    }
+#pragma unroll
+    for (int u = 0; u < kNuItems; ++u) {
+      am = max(am, __float_as_uint(fabsf(rec[u].w)));
+      logs += nu_log(rec[u].w);
+    }
     am = __reduce_max_sync(0xffffffffu, am);
+    logs = __reduce_add_sync(0xffffffffu, logs);
     if (kBlocks) blocks = __reduce_or_sync(0xffffffffu, blocks);
     if (lane == 0) {
       atomicMax(&s_max[chunk & 1], am);
+      atomicAdd(&s_log[chunk & 1], logs);
       if (kBlocks) atomicOr(&s_blk[chunk & 1], blocks);
     }
-    __syncthreads();  // the chunk's maximum; the previous chunk is added up
-    const float top = fmaxf(__uint_as_float(s_max[chunk & 1]), 1e-20f);  // terms up to 0.98 2^kNuBits
-    const float scale = 0.98f * (float)(1 << kNuBits) / top, unit = top * (1.f / (0.98f * (float)(1 << kNuBits)));
+    __syncthreads();  // the chunk's words; the turn before is added up
+    const NuClass cls = nu_class(s_max[chunk & 1], s_log[chunk & 1], left);
     blocks = kBlocks ? s_blk[chunk & 1] : 1u;
+    if (cls.rare) {  // the same for the whole CTA
+#pragma unroll
+      for (int u = 0; u < kNuItems; ++u) {
+        const bool in = nu_log(rec[u].w) >= cls.floor;
+        if (cls.floor) left -= __syncthreads_count(in);
+        rec[u].w = in ? rec[u].w * cls.more : 0.f;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kNuItems; ++u) rec[u].w *= cls.up;
+    if (cls.floor) {
+      ceil = cls.floor;
+    } else {
+      ceil = kNuAll;
+      c0 += kNuChunk;
+      left = min(kNuChunk, n - c0);
+    }
     while (blocks) {
       const int b = kBlocks ? __ffs(blocks) - 1 : 0;
       blocks &= blocks - 1;
@@ -757,14 +862,14 @@ __global__ void __launch_bounds__(kNuThreads, 3)
         __syncthreads();
       }
       int* fl = flag[pass & 1];
-      // read before this pass: the other parity's flags, the previous chunk's maximum
+      // read before this pass: the other parity's flags and words
       if (tid < kNuBlock / 8) flag[~pass & 1][tid] = 0;
-      if (tid == 0) s_max[~chunk & 1] = s_blk[~chunk & 1] = 0u;
+      if (tid == 0) s_max[~chunk & 1] = s_blk[~chunk & 1] = 0u, s_log[~chunk & 1] = 0;
 #pragma unroll
       for (int u = 0; u < kNuItems; ++u) {
         const int idx = kBlocks ? cell[u] - b * bs : cell[u];
         if ((kBlocks && (unsigned)idx >= (unsigned)bs) || rec[u].w == 0.f) continue;
-        const float a = rec[u].w * scale;
+        const float a = rec[u].w;
         const float c1 = a * (upper ? rec[u].y : rec[u].x), c2 = a * (upper ? rec[u].x : rec[u].y);
         int* g1 = mine + idx * (2 * kNuCopies) + (upper ? kNuCopies : 0);
         int* g2 = mine + idx * (2 * kNuCopies) + (upper ? 0 : kNuCopies);
@@ -779,12 +884,10 @@ __global__ void __launch_bounds__(kNuThreads, 3)
           atomicAdd(g2 + (7 - j) * (2 * kNuCopies), nu_term(c2, wr[j], j < kNuSmall));
         }
       }
-      if (!kBlocks || !blocks) load(c0 + kNuChunk);  // in flight while this chunk is added up
+      if (!kBlocks || !blocks) load(c0);  // in flight while this turn is added up
       __syncthreads();
-      // Add the chunk up: half-warp h takes the octets of points o = h mod 16, which records
-      // of the cells of octets o - 1 and o reach, one thread per point and part; the copies'
-      // four 16-byte words in an order that gives the lanes of a shared-memory phase
-      // different banks.
+      // Add the turn up: half-warp h takes the octets of points o = h mod 16, which records
+      // of the cells of octets o - 1 and o reach, one thread per point and part.
       const unsigned m0 = __ballot_sync(0xffffffffu, fl[lane] != 0), m1 = __ballot_sync(0xffffffffu, fl[32 + lane] != 0);
       const unsigned long long cells = (unsigned long long)m1 << 32 | m0, lit = cells | cells << 1;
 #pragma unroll
@@ -793,18 +896,11 @@ __global__ void __launch_bounds__(kNuThreads, 3)
         const bool on = o < 64 ? (lit >> (o & 63)) & 1ull : o == 64 && (cells >> 63) != 0ull;
         if (!on) continue;
         const int i = o * 16 + (tid & 15);  // point i / 2, part i & 1
-        long long t = 0;
-#pragma unroll
-        for (int k = 0; k < kNuCopies / 4; ++k) {
-          const int w = i * (kNuCopies / 4) + ((k + (i >> 1)) & (kNuCopies / 4 - 1));
-          const int4 x = nsm[w];
-          nsm[w] = make_int4(0, 0, 0, 0);
-          t += (long long)(x.x + x.y) + (long long)(x.z + x.w);
-        }
-        sum[i] = fmaf((float)t, unit, sum[i]);
+        const long long t = nu_add_up(nsm, i * (kNuCopies / 4), i >> 1);
+        sum[i] = fmaf((float)t * cls.less, cls.down, sum[i]);
       }
       ++pass;
-      if (kBlocks && blocks) __syncthreads();  // before the next block's additions (else: the next chunk's barrier)
+      if (kBlocks && blocks) __syncthreads();  // before the next block's additions (else: the next turn's barrier)
     }
   }
   bad = __syncthreads_or(bad);
@@ -841,8 +937,9 @@ template <bool kBlocks>
 __global__ void __launch_bounds__(kNuThreads, 3)
     k_nufft_spread_chirps(const float4* __restrict__ prep, const float* __restrict__ rate, int64_t cap,
                           const int32_t* __restrict__ d_P, const NufftArg na, const __grid_constant__ NufftCoef co, float2* __restrict__ grids) {
-  extern __shared__ int4 nsm[];  // [npts][re, im][kNuCopies]
-  __shared__ uint32_t s_max[2];
+  extern __shared__ uint4 nsm[];  // [npts][re, im][kNuCopies]
+  __shared__ uint32_t s_max[2];  // by the parity of the turn: largest amplitude
+  __shared__ int s_log[2];       // and the sum of the amplitudes' logarithms
   __shared__ int flag[2][kNuBlock / 8];
   const int M = 1 << na.log_m, bs = nu_cells(M), npts = nu_points(M), oct = bs >> 3;
   const int tid = threadIdx.x, lane = tid & 31;
@@ -851,9 +948,9 @@ __global__ void __launch_bounds__(kNuThreads, 3)
   const float cnu = (float)(dt * na.f0_c), ceps = (float)(dt * na.b_cn);
   const float turn = (float)(na.per_chirp * na.cyc), move = (float)(na.per_chirp * na.cell);  // per (m/s) and chirp
   float2* out = grids + (size_t)(q * na.V + v) * nc * M;
-  for (int i = tid; i < npts * (2 * kNuCopies / 4); i += kNuThreads) nsm[i] = make_int4(0, 0, 0, 0);
+  for (int i = tid; i < npts * (2 * kNuCopies / 4); i += kNuThreads) nsm[i] = nu_zero();
   for (int i = tid; i < 2 * (kNuBlock / 8); i += kNuThreads) (&flag[0][0])[i] = 0;
-  if (tid < 2) s_max[tid] = 0u;
+  if (tid < 2) s_max[tid] = 0u, s_log[tid] = 0;
   after_previous();
   for (int i = tid; i < nc * M; i += kNuThreads) out[i] = make_float2(0.f, 0.f);
   const int64_t P = *d_P;
@@ -865,10 +962,11 @@ __global__ void __launch_bounds__(kNuThreads, 3)
   int pass = 0;
   bool bad = false;  // a record that is not finite: the antenna's samples are NaN
   __syncthreads();
-  for (int c0 = 0, chunk = 0; c0 < n; c0 += kNuChunk, ++chunk) {
+  int ceil = kNuAll, left = min(kNuChunk, n);  // classes in turns, as k_nufft_spread
+  for (int c0 = 0, chunk = 0; c0 < n; ++chunk) {
     float c1[kNuItems], c2[kNuItems], wr[kNuItems], wi[kNuItems], s[kNuItems], ds[kNuItems];
-    int cell[kNuItems];
-    uint32_t am = 0;
+    int cell[kNuItems], logs = 0;
+    uint32_t am = 0, mag[kNuItems];  // mag: the amplitudes' bits
 #pragma unroll
     for (int u = 0; u < kNuItems; ++u) {
       const int p = c0 + tid + u * kNuThreads;
@@ -902,24 +1000,53 @@ __global__ void __launch_bounds__(kNuThreads, 3)
       sincospif(2.f * (ld * turn), &sn, &cs);
       wr[u] = cs;
       wi[u] = upper ? -sn : sn;
-      am = max(am, __float_as_uint(fabsf(r.w)));
+      mag[u] = __float_as_uint(fabsf(r.w));
     }
-    am = __reduce_max_sync(0xffffffffu, am);
-    if (lane == 0) atomicMax(&s_max[chunk & 1], am);
-    __syncthreads();
-    const float top = fmaxf(__uint_as_float(s_max[chunk & 1]), 1e-20f);  // terms up to 0.98 2^kNuBits
-    const float scale = 0.98f * (float)(1 << kNuBits) / top, unit = top * (1.f / (0.98f * (float)(1 << kNuBits)));
+    if (ceil != kNuAll) {
+#pragma unroll
+      for (int u = 0; u < kNuItems; ++u)
+        if ((int)(mag[u] >> 20) >= ceil) c1[u] = c2[u] = 0.f, mag[u] = 0u;
+    }
 #pragma unroll
     for (int u = 0; u < kNuItems; ++u) {
-      c1[u] *= scale;
-      c2[u] *= scale;
+      am = max(am, mag[u]);
+      logs += (int)(mag[u] >> 20);
+    }
+    am = __reduce_max_sync(0xffffffffu, am);
+    logs = __reduce_add_sync(0xffffffffu, logs);
+    if (lane == 0) {
+      atomicMax(&s_max[chunk & 1], am);
+      atomicAdd(&s_log[chunk & 1], logs);
+    }
+    __syncthreads();
+    const NuClass cls = nu_class(s_max[chunk & 1], s_log[chunk & 1], left);
+    if (cls.rare) {  // the same for the whole CTA
+#pragma unroll
+      for (int u = 0; u < kNuItems; ++u) {
+        const bool in = (int)(mag[u] >> 20) >= cls.floor;
+        if (cls.floor) left -= __syncthreads_count(in);
+        c1[u] = in ? c1[u] * cls.more : 0.f;
+        c2[u] = in ? c2[u] * cls.more : 0.f;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kNuItems; ++u) {
+      c1[u] *= cls.up;
+      c2[u] *= cls.up;
+    }
+    if (cls.floor) {
+      ceil = cls.floor;
+    } else {
+      ceil = kNuAll;
+      c0 += kNuChunk;
+      left = min(kNuChunk, n - c0);
     }
     for (int kb = 0, b = 0; kb < (kBlocks ? nc * (M / bs) : nc); ++kb, ++pass) {
       const int k = kBlocks ? kb / (M / bs) : kb;
       if (kBlocks) b = kb - k * (M / bs);
       int* fl = flag[pass & 1];
       if (tid < kNuBlock / 8) flag[~pass & 1][tid] = 0;  // read before this pass
-      if (tid == 0) s_max[~chunk & 1] = 0u;
+      if (tid == 0) s_max[~chunk & 1] = 0u, s_log[~chunk & 1] = 0;
 #pragma unroll
       for (int u = 0; u < kNuItems; ++u) {
         const int idx = kBlocks ? cell[u] - b * bs : cell[u];
@@ -961,18 +1088,9 @@ __global__ void __launch_bounds__(kNuThreads, 3)
         const int i = o * 16 + (tid & 15);  // point i / 2, part i & 1
         float* g = to + 2 * ((b * bs + (i >> 1) - (kNuW / 2 - 1)) & (M - 1)) + (i & 1);
         const float old = *g;
-        long long t = 0;
-        for (int h = 0; h < (!kBlocks && o == 0 ? 2 : 1); ++h) {
-          const int ii = i + h * 2 * M;
-#pragma unroll
-          for (int w4 = 0; w4 < kNuCopies / 4; ++w4) {
-            const int w = ii * (kNuCopies / 4) + ((w4 + (ii >> 1)) & (kNuCopies / 4 - 1));
-            const int4 x = nsm[w];
-            nsm[w] = make_int4(0, 0, 0, 0);
-            t += (long long)(x.x + x.y) + (long long)(x.z + x.w);
-          }
-        }
-        *g = fmaf((float)t, unit, old);
+        long long t = nu_add_up(nsm, i * (kNuCopies / 4), i >> 1);
+        if (!kBlocks && o == 0) t += nu_add_up(nsm, (i + 2 * M) * (kNuCopies / 4), (i >> 1) + M);
+        *g = fmaf((float)t * cls.less, cls.down, old);
       }
       __syncthreads();
     }
@@ -1141,15 +1259,7 @@ __global__ void __cluster_dims__(kNuRanks, 1, 1) __launch_bounds__(kNuClThreads)
   }
 }
 
-// I0 by its power series (the terms are positive: no cancellation; beta < 20).
-double bessel_i0(double x) {
-  double t = 1.0, s = 1.0;
-  for (int k = 1; k < 200 && t > 1e-18 * s; ++k) {
-    t *= (0.5 * x / k) * (0.5 * x / k);
-    s += t;
-  }
-  return s;
-}
+double bessel_i0(double x) { return bessel_i0_of(0.25 * x * x); }
 
 double kb_kernel(double x) {
   const double z = 2.0 * x / kNuW, y = 1.0 - z * z;
