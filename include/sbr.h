@@ -304,7 +304,10 @@ sbr_status sbr_trace_counts(const sbr_scene* scene, const sbr_radar_cfg* radar,
 /* Synthesis (Section 3.2.2, Eq. 8)                                         */
 /* ------------------------------------------------------------------------ */
 
-/* Scratch bytes for sbr_synthesize / sbr_synthesize_bwd; 0 for a radar they do not support. */
+/* Scratch bytes for sbr_synthesize / sbr_synthesize_bwd in every mode; 0 for a
+ * radar they do not support.  A static scene and the adjoint take a buffer of the
+ * size asked for with n_chirps = 1, whatever the chirps; so does a moving scene,
+ * whose chirps then go one launch each instead of many at a time. */
 size_t sbr_synth_ws_bytes(const sbr_radar_cfg* radar, int64_t path_cap);
 
 /* d_cube [V][C][N_s] complex64 (interleaved re, im) =

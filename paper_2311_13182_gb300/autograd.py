@@ -62,7 +62,7 @@ class Simulator:
         self.bvh_refit = False
         self.paths = None if recompute else sim.PathBuffers(self.n_rays, max_bounces, radar.n_virt, device)
         cap = self.n_rays * max_bounces
-        self.synth_ws = torch.empty(sim.synth_ws_bytes(radar, cap), dtype=torch.uint8, device=device)
+        self.synth_ws = torch.empty(sim.synth_ws_bytes(radar, cap, phase_mode), dtype=torch.uint8, device=device)
         self.cube = torch.empty((radar.n_virt, radar.n_chirps, radar.n_samples, 2), dtype=torch.float32,
                                 device=device)
         self.points = torch.empty((cfar.k_max, 4), dtype=torch.float32, device=device)

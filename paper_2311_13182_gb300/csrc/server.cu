@@ -190,7 +190,9 @@ Sizes request_sizes(const sbr_radar_cfg* radar, const sbr_cfar_cfg* cfar, const 
   s.mesh = sbr_arena::round(sizeof(float) * 3 * (size_t)q->nv) + sbr_arena::round(sizeof(int32_t) * 3 * (size_t)q->nt);
   s.scene = sbr_arena::round(sbr_scene_bytes(q->nt));
   s.paths = sbr_arena::round(sbr_paths_bytes((int32_t)R, q->max_bounces, V));
-  s.ws = sbr_arena::round(sbr_synth_ws_bytes(radar, R * q->max_bounces));
+  sbr_radar_cfg one = *radar;  // scenes are static: room for one chirp
+  one.n_chirps = 1;
+  s.ws = sbr_arena::round(sbr_synth_ws_bytes(&one, R * q->max_bounces));
   s.cube = sbr_arena::round(sizeof(float) * 2 * (size_t)V * radar->n_chirps * radar->n_samples);
   s.pc = sbr_arena::round(sbr_pc_bytes(radar, cfar));
   s.points = sbr_arena::round(sizeof(float) * 4 * (size_t)cfar->k_max) + kAlign;

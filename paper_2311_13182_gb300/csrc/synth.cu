@@ -1631,25 +1631,34 @@ inline int nufft_grids(int V, int qn, int C, int Ns, int64_t cap) {
 }
 
 // Summed grids per antenna: none where a cluster finishes the rows.
-inline int nufft_sums(int qg, int Ns) { return 2 * Ns <= kNuClusterPoints ? 0 : qg; }
+inline int nufft_sums(int rows, int Ns) { return 2 * Ns <= kNuClusterPoints ? 0 : rows; }
 
-// Workspace: per-CTA partial sums of the direct kernels, the chirp-summed
-// upstream gradient of the adjoint, and, for the non-uniform FFT, the CTAs'
-// grids, their sum and the finishing counters.
-size_t ws_layout(const sbr_radar_cfg* radar, int64_t cap, int* Q, int* Qn = nullptr) {
+struct SynthWs {
+  float2* partial;        // per-CTA partial sums of the direct kernels
+  float2* gsum;           // chirp-summed upstream gradient of the adjoint
+  float2* grids;          // non-uniform FFT: the CTAs' grids, V * Qg
+  float2* bsum;           // non-uniform FFT: the rows' summed grids, nufft_sums
+  unsigned int* fin_cnt;  // non-uniform FFT: finishing counters, V * rows
+  float4* adj;            // adjoint: the antennas' grids
+  int Q, Qn, Qg, rows;    // per antenna: CTAs (direct, FFT), grids, chirps that one launch may finish
+};
+
+// The workspace in `mem` (or its size alone) with room for the launches of `chirps`
+// chirps of a moving scene.  One is all that a static scene and the adjoint use, and
+// enough for a moving scene too, whose chirps then go one launch each.
+size_t ws_layout(const sbr_radar_cfg* radar, int64_t cap, int chirps, void* mem, SynthWs* w) {
   const int V = radar->n_tx * radar->n_rx, Ns = radar->n_samples;
-  grid_shape(V, Ns, cap, Q);
-  int qn = 0;
-  nufft_shape(V, Ns, cap, &qn);
-  if (Qn) *Qn = qn;
-  Carver c(nullptr);
-  c.take<float2>((size_t)V * (*Q) * Ns);       // per-CTA partial sums
-  c.take<float2>((size_t)V * Ns);              // chirp-summed upstream gradient
-  const int qg = nufft_grids(V, qn, radar->n_chirps, Ns, cap);
-  c.take<float2>((size_t)V * qg * 2 * Ns);     // non-uniform FFT: the CTAs' grids
-  c.take<float2>((size_t)V * nufft_sums(qg, Ns) * 2 * Ns);  // non-uniform FFT: the rows' summed grids (a moving scene: V * chirps)
-  c.take<unsigned int>((size_t)V * qg);        // non-uniform FFT: finishing counters
-  c.take<float4>((size_t)V * (2 * Ns + kAdjMargin));  // adjoint: the antennas' grids
+  grid_shape(V, Ns, cap, &w->Q);
+  nufft_shape(V, Ns, cap, &w->Qn);
+  w->Qg = nufft_grids(V, w->Qn, chirps, Ns, cap);
+  w->rows = std::max(1, std::min(chirps, w->Qg));
+  Carver c(mem);
+  w->partial = c.take<float2>((size_t)V * w->Q * Ns);
+  w->gsum = c.take<float2>((size_t)V * Ns);
+  w->grids = c.take<float2>((size_t)V * w->Qg * 2 * Ns);
+  w->bsum = c.take<float2>((size_t)V * nufft_sums(w->rows, Ns) * 2 * Ns);
+  w->fin_cnt = c.take<unsigned int>((size_t)V * w->rows);
+  w->adj = c.take<float4>((size_t)V * (2 * Ns + kAdjMargin));
   return c.bytes();
 }
 
@@ -1665,41 +1674,20 @@ extern "C" size_t sbr_synth_ws_bytes(const sbr_radar_cfg* radar, int64_t path_ca
     set_error("sbr_synth_ws_bytes: n_samples=%d must be a power of two in [%d, %d]", Ns, kMinSamples, kMaxSamples);
     return 0;
   }
-  int Q;
-  return ws_layout(radar, path_cap, &Q);
+  SynthWs w;
+  return ws_layout(radar, path_cap, radar->n_chirps, nullptr, &w);
 }
 
 namespace {
-struct SynthWs {
-  float2* partial;
-  float2* gsum;
-  float2* grids;
-  float2* bsum;
-  unsigned int* fin_cnt;
-  float4* adj;
-  int Q, Qn, Qg;
-};
-
-sbr_status bind_ws(const sbr_radar_cfg* radar, int64_t cap, void* ws, size_t bytes, SynthWs* w,
+sbr_status bind_ws(const sbr_radar_cfg* radar, int64_t cap, bool moving, void* ws, size_t bytes, SynthWs* w,
                    const char* who) {
-  int Q, Qn;
-  const size_t need = ws_layout(radar, cap, &Q, &Qn);
   SBR_ARG(ws && aligned256(ws), "%s: workspace NULL or not 256-byte aligned", who);
+  if (moving && ws_layout(radar, cap, radar->n_chirps, ws, w) <= bytes) return SBR_OK;
+  const size_t need = ws_layout(radar, cap, 1, ws, w);
   if (bytes < need) {
     set_error("%s: workspace of %zu bytes, %zu needed", who, bytes, need);
     return SBR_ERR_OOM;
   }
-  const int V = radar->n_tx * radar->n_rx, Ns = radar->n_samples;
-  Carver c(ws);
-  w->partial = c.take<float2>((size_t)V * Q * Ns);
-  w->gsum = c.take<float2>((size_t)V * Ns);
-  w->Qg = nufft_grids(V, Qn, radar->n_chirps, Ns, cap);
-  w->grids = c.take<float2>((size_t)V * w->Qg * 2 * Ns);
-  w->bsum = c.take<float2>((size_t)V * nufft_sums(w->Qg, Ns) * 2 * Ns);
-  w->fin_cnt = c.take<unsigned int>((size_t)V * w->Qg);
-  w->adj = c.take<float4>((size_t)V * (2 * Ns + kAdjMargin));
-  w->Q = Q;
-  w->Qn = Qn;
   return SBR_OK;
 }
 
@@ -1725,7 +1713,7 @@ NufftArg nufft_arg(const sbr_paths* p, const sbr_radar_cfg* r, int Q, int c0, in
 
 // The non-uniform FFT of chirps [c0, c0 + chirps) of a moving scene, or of a static
 // scene's one chirp, written to all of them: spread by Q CTAs per antenna and chirp
-// (Q * chirps <= w.Qg), then finish.
+// (Q * chirps <= w.Qg, chirps <= w.rows), then finish.
 void launch_nufft(sbr_phase_mode mode, const sbr_paths* p, const sbr_radar_cfg* r, const SynthWs& w, bool moving, int Q,
                   int c0, int chirps, float2* cube, cudaStream_t st) {
   const int V = p->n_virt, Ns = r->n_samples, M = 2 * Ns;
@@ -1774,7 +1762,8 @@ sbr_status launch_moving(sbr_phase_mode mode, const sbr_paths* p, const sbr_rada
                          float2* cube, cudaStream_t st) {
   if (mode == SBR_PHASE_FP64 || (mode == SBR_PHASE_SPLIT && r->n_samples <= kNuMovingMaxSamples)) {
     const int C = r->n_chirps;
-    if (mode == SBR_PHASE_SPLIT && nufft_tiles(p->n_virt, C, r->n_samples, p->path_cap)) {
+    if (mode == SBR_PHASE_SPLIT && nufft_tiles(p->n_virt, C, r->n_samples, p->path_cap) &&
+        w.Qg >= w.Qn * std::min(C, kTile)) {
       launch_chirps(p, r, w, cube, st);
       return SBR_OK;
     }
@@ -1782,7 +1771,7 @@ sbr_status launch_moving(sbr_phase_mode mode, const sbr_paths* p, const sbr_rada
     int best = 1, group = 1;
     double cost = 1e30;
     for (int q = 1; q <= w.Qn; ++q) {
-      const int most = std::min(C, wave / q), launches = (C + most - 1) / most;
+      const int most = std::min(w.rows, wave / q), launches = (C + most - 1) / most;
       if (launches < cost * q) {
         cost = (double)launches / q;
         best = q;
@@ -1835,7 +1824,7 @@ extern "C" sbr_status sbr_synthesize(const sbr_paths* paths, const sbr_radar_cfg
   SBR_ARG(mode == SBR_PHASE_SPLIT || mode == SBR_PHASE_FP64 || mode == SBR_PHASE_NAIVE,
           "sbr_synthesize: unknown phase mode %d", (int)mode);
   SynthWs w;
-  rs = bind_ws(radar, paths->path_cap, d_ws, ws_bytes, &w, "sbr_synthesize");
+  rs = bind_ws(radar, paths->path_cap, moving, d_ws, ws_bytes, &w, "sbr_synthesize");
   if (rs != SBR_OK) return rs;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const int Ns = radar->n_samples, T = threads_for(Ns), M = Ns / T;
@@ -1949,7 +1938,7 @@ extern "C" sbr_status sbr_synthesize_bwd(const sbr_paths* paths, const sbr_radar
   if (rs != SBR_OK) return rs;
   SBR_ARG(paths->n_virt == radar->n_tx * radar->n_rx, "sbr_synthesize_bwd: V mismatch");
   SynthWs w;
-  rs = bind_ws(radar, paths->path_cap, d_ws, ws_bytes, &w, "sbr_synthesize_bwd");
+  rs = bind_ws(radar, paths->path_cap, false, d_ws, ws_bytes, &w, "sbr_synthesize_bwd");
   if (rs != SBR_OK) return rs;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const int V = paths->n_virt, Ns = radar->n_samples, C = radar->n_chirps;

@@ -32,7 +32,8 @@ class Forward:
         self.faces = faces.detach().contiguous()
         self.scene = sim.Scene(self.verts, self.faces)
         self.paths = sim.PathBuffers(grid.n_rays, max_bounces, radar.n_virt)
-        self.ws = torch.empty(sim.synth_ws_bytes(radar, self.paths.cap), dtype=torch.uint8, device=self.verts.device)
+        self.ws = torch.empty(sim.synth_ws_bytes(radar, self.paths.cap, mode), dtype=torch.uint8,
+                              device=self.verts.device)
         self.cube = torch.empty((radar.n_virt, radar.n_chirps, radar.n_samples, 2), device=self.verts.device)
         self.state = sim.PcState(radar, cfar)
         self.points = torch.empty((cfar.k_max, 4), device=self.verts.device)
@@ -147,7 +148,7 @@ class PipelinedForward:
         self.faces = faces.detach().contiguous()
         self.scenes = [sim.Scene(self.verts, self.faces), sim.Scene(self.verts, self.faces)]
         self.paths = [sim.PathBuffers(grid.n_rays, max_bounces, radar.n_virt) for _ in range(depth - 2)]
-        self.ws = torch.empty(sim.synth_ws_bytes(radar, self.paths[0].cap), dtype=torch.uint8, device=dev)
+        self.ws = torch.empty(sim.synth_ws_bytes(radar, self.paths[0].cap, mode), dtype=torch.uint8, device=dev)
         self.cubes = [torch.zeros((radar.n_virt, radar.n_chirps, radar.n_samples, 2), device=dev) for _ in range(2)]
         self.state = sim.PcState(radar, cfar)
         self.points = torch.empty((cfar.k_max, 4), device=dev)

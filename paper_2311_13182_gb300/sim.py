@@ -277,8 +277,17 @@ def trace_counts(scene: Scene, radar, grid, max_bounces: int, out: PathBuffers, 
     return c[0], c[1], c[2]
 
 
-def synth_ws_bytes(radar, path_cap: int) -> int:
-    return int(L.load().sbr_synth_ws_bytes(ctypes.byref(radar_struct(radar)), path_cap))
+def synth_ws_bytes(radar, path_cap: int, mode: int | None = None) -> int:
+    """Scratch bytes of ``synthesize`` and ``synthesize_bwd``: for every mode, or what ``mode`` uses
+    (without SYNTH_MOVING: less with many chirps)."""
+    return _ws_bytes(radar_struct(radar), path_cap, mode is None or bool(mode & SYNTH_MOVING))
+
+
+def _ws_bytes(r: L.RadarCfg, cap: int, moving: bool) -> int:
+    chirps, r.n_chirps = r.n_chirps, r.n_chirps if moving else 1
+    nb = int(L.load().sbr_synth_ws_bytes(ctypes.byref(r), cap))
+    r.n_chirps = chirps
+    return nb
 
 
 def synthesize(paths: PathBuffers, radar, mode: int = PHASE_SPLIT, out: torch.Tensor | None = None,
@@ -288,10 +297,10 @@ def synthesize(paths: PathBuffers, radar, mode: int = PHASE_SPLIT, out: torch.Te
     V, C, Ns = radar.n_virt, radar.n_chirps, radar.n_samples
     if out is None:
         out = torch.empty((V, C, Ns, 2), dtype=torch.float32, device=paths.mem.device)
-    nb = int(L.load().sbr_synth_ws_bytes(ctypes.byref(r), paths.cap))
-    if ws is None or ws.numel() < nb:
-        ws = torch.empty(nb, dtype=torch.uint8, device=paths.mem.device)
-    L.call("sbr_synthesize", ctypes.byref(paths.s), ctypes.byref(r), int(mode), _vp(out), _vp(ws), nb,
+    if ws is None or ws.numel() < _ws_bytes(r, paths.cap, False):
+        ws = torch.empty(_ws_bytes(r, paths.cap, bool(mode & SYNTH_MOVING)), dtype=torch.uint8,
+                         device=paths.mem.device)
+    L.call("sbr_synthesize", ctypes.byref(paths.s), ctypes.byref(r), int(mode), _vp(out), _vp(ws), ws.numel(),
            _stream(stream))
     return out
 
@@ -305,7 +314,7 @@ def synthesize_bwd(paths: PathBuffers, radar, gcube: torch.Tensor, ws: torch.Ten
     glen = torch.empty((paths.V, max(paths.cap, 1)), dtype=torch.float32, device=gcube.device)
     gamp = torch.empty_like(glen)
     gph = torch.empty_like(glen) if phase else None
-    nb = int(L.load().sbr_synth_ws_bytes(ctypes.byref(r), paths.cap))
+    nb = _ws_bytes(r, paths.cap, False)
     if ws is None or ws.numel() < nb:
         ws = torch.empty(nb, dtype=torch.uint8, device=gcube.device)
     L.call("sbr_synthesize_bwd", ctypes.byref(paths.s), ctypes.byref(r), _vp(gcube), _vp(glen), _vp(gamp),

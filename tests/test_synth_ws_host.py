@@ -31,3 +31,20 @@ def test_unsupported_sample_counts_have_no_workspace(n_samples):
 def test_workspace_grows_with_the_paths(n_samples):
     sizes = [size(n_samples, cap) for cap in (1, 1000, 100000, 1000000)]
     assert sizes[0] > 0 and sizes == sorted(sizes)
+
+
+@pytest.mark.parametrize("n_samples", [256, 512, 4096])
+def test_workspace_of_a_static_scene_does_not_grow_with_the_chirps(n_samples):
+    """What a mode uses: one chirp's room without motion, more with it."""
+    from types import SimpleNamespace
+
+    import numpy as np
+    from paper_2311_13182_gb300 import _lib, build, sim
+    build.build()
+    def rad(n_chirps):
+        return SimpleNamespace(f0=77e9, bandwidth=4e9, chirp_time=4e-5, chirp_rep=4e-5, n_samples=n_samples,
+                               n_chirps=n_chirps, n_tx=3, n_rx=4, tx=np.zeros((3, 3)), rx=np.zeros((4, 3)))
+    one = sim.synth_ws_bytes(rad(1), 100000)
+    assert sim.synth_ws_bytes(rad(128), 100000, 0) == one == size(n_samples, 100000)
+    assert sim.synth_ws_bytes(rad(128), 100000) == size(n_samples, 100000, 128)
+    assert sim.synth_ws_bytes(rad(128), 100000, _lib.SYNTH_MOVING) == size(n_samples, 100000, 128) >= one
