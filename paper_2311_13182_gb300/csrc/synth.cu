@@ -574,6 +574,7 @@ constexpr int kNuChunk = kNuThreads * kNuItems;
 constexpr int kNuBits = 25;    // 2 kNuChunk / 32 additions per copy of terms up to 0.98 2^25: below 2^31
 static_assert(kNuChunk / kNuCopies <= 1 << (31 - kNuBits), "a class's additions to one copy");
 constexpr int kNuSpan = 24;    // mean distance of a class's amplitudes from its largest, in eighths of an octave
+constexpr int kNuFar = 40;     // the same where many are close to it
 constexpr double kNuBeta = 2.3 * kNuW;
 
 struct NufftCoef {
@@ -645,15 +646,17 @@ constexpr int kNuAll = 2048;  // above every logarithm
 
 // The class of records that one pass rounds on one scale, 2^s for the largest amplitude
 // (its bits: top) to land in (0.49, 0.98] 2^kNuBits: all N that are left if their
-// logarithms (sum: logs) lie within kNuSpan of the largest's on average, else those
-// within kNuSpan of it.  The class's rms amplitude is then an eighth of its largest or
-// more, and the rounding stays near the error of the transform around it; on one scale
-// for all, a chunk's few strong records would cost its weak ones their bits (one record
-// in 1,024 a hundred times the others: 9e-7 to 1.4e-6 from FP64 instead of 1.8e-7; two in
-// 1,024 a thousand times the others and cancelling: 3e-5 instead of 1.9e-7).  Specular
-// returns of one chunk differ little, so more than one class is rare; where it is not it
-// costs passes, not accuracy.  The scale is a power of two, exact; one past a float's
-// range (amplitudes below 1e-31) is applied in two factors.
+// logarithms (sum: logs) lie within kNuSpan of the largest's on average, or within
+// kNuFar and a sixteenth of them within an octave of it (nu_near); else those within
+// kNuSpan of it.  The class's rms amplitude is then an eighth of its largest or more, and
+// the rounding stays near the error of the transform around it; on one scale for all, a
+// chunk's few strong records would cost its weak ones their bits (one record in 1,024 a
+// hundred times the others: 9e-7 to 1.4e-6 from FP64 instead of 1.8e-7; two in 1,024 a
+// thousand times the others and cancelling: 3e-5 instead of 1.9e-7).  The returns of one
+// chunk differ little: traced paths of superquadrics over a ground plane leave kNuSpan in
+// up to 9 % of the chunks (26 % in the worst of nine scenes), and need a second class in
+// up to 0.6 %.  The scale is a power of two, exact; one past a float's range (amplitudes
+// below 1e-31) is applied in two factors.
 // The two words per chunk that this takes, and the copies' sum in 64 bits, cost 12
 // antennas x 367,500 records 42.0 -> 43.0 us for the whole synthesis, 4 antennas x 3.1 M
 // records x 4096 samples 122.8 -> 126.4; moving chirps (no sign extensions in the sum)
@@ -676,6 +679,12 @@ __device__ __forceinline__ NuClass nu_class(uint32_t top, int logs, int N) {
   c.down = __int_as_float((127 - a) << 23);
   c.less = __int_as_float((127 - s + a) << 23);
   return c;
+}
+
+// Amplitudes within an octave of the largest, where a chunk has left kNuSpan.
+__device__ __forceinline__ bool nu_near(int log, const NuClass& c) { return log >= c.floor + kNuSpan - 8; }
+__device__ __forceinline__ bool nu_one_class(const NuClass& c, int near, int logs, int N) {
+  return 16 * near >= N && N * (c.floor + kNuSpan - kNuFar) <= logs;
 }
 
 // Grid words in shared memory are kept kNuZero off, so that the copies add up unsigned,
@@ -834,9 +843,16 @@ __global__ void __launch_bounds__(kNuThreads, 3)
       if (kBlocks) atomicOr(&s_blk[chunk & 1], blocks);
     }
     __syncthreads();  // the chunk's words; the turn before is added up
-    const NuClass cls = nu_class(s_max[chunk & 1], s_log[chunk & 1], left);
+    logs = s_log[chunk & 1];
+    NuClass cls = nu_class(s_max[chunk & 1], logs, left);
     blocks = kBlocks ? s_blk[chunk & 1] : 1u;
     if (cls.rare) {  // the same for the whole CTA
+      if (cls.floor) {
+        int near = 0;
+#pragma unroll
+        for (int u = 0; u < kNuItems; ++u) near += __syncthreads_count(nu_near(nu_log(rec[u].w), cls));
+        if (nu_one_class(cls, near, logs, left)) cls.floor = 0;
+      }
 #pragma unroll
       for (int u = 0; u < kNuItems; ++u) {
         const bool in = nu_log(rec[u].w) >= cls.floor;
@@ -1019,8 +1035,15 @@ __global__ void __launch_bounds__(kNuThreads, 3)
       atomicAdd(&s_log[chunk & 1], logs);
     }
     __syncthreads();
-    const NuClass cls = nu_class(s_max[chunk & 1], s_log[chunk & 1], left);
+    logs = s_log[chunk & 1];
+    NuClass cls = nu_class(s_max[chunk & 1], logs, left);
     if (cls.rare) {  // the same for the whole CTA
+      if (cls.floor) {
+        int near = 0;
+#pragma unroll
+        for (int u = 0; u < kNuItems; ++u) near += __syncthreads_count(nu_near((int)(mag[u] >> 20), cls));
+        if (nu_one_class(cls, near, logs, left)) cls.floor = 0;
+      }
 #pragma unroll
       for (int u = 0; u < kNuItems; ++u) {
         const bool in = (int)(mag[u] >> 20) >= cls.floor;
