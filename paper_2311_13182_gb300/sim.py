@@ -38,11 +38,17 @@ def _need_cuda(t: torch.Tensor, dtype, name):
 
 
 def _positions(field, pos, n):
-    """The first n antenna positions into a ctypes [.][3] double array, as one copy."""
-    a = np.ascontiguousarray(np.asarray(pos, dtype=np.float64)[:n, :3])
-    if a.shape != (n, 3):
-        raise IndexError(f"{n} antenna positions of 3 coordinates needed, got {a.shape}")
-    ctypes.memmove(field, a.tobytes(), 24 * n)
+    """The first n antenna positions into a ctypes [.][3] double array: an array of numbers as one
+    copy, anything else (lists, tensors on any device) value by value."""
+    if isinstance(pos, np.ndarray) and pos.dtype.kind in "fiu":
+        a = np.ascontiguousarray(pos[:n, :3], dtype=np.float64)
+        if a.shape != (n, 3):
+            raise IndexError(f"{n} antenna positions of 3 coordinates needed, got {a.shape}")
+        ctypes.memmove(field, a.tobytes(), 24 * n)
+        return
+    for t in range(n):
+        for j in range(3):
+            field[t][j] = float(pos[t][j])
 
 
 def radar_struct(radar) -> L.RadarCfg:
