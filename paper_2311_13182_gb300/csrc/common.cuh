@@ -25,6 +25,16 @@ void note_launch();
 // it.  next_may_start() lets the next kernel be dispatched from the moment all CTAs
 // of this one have begun; long kernels leave it out, as waiting CTAs hold registers
 // and shared memory that other streams could use.
+//
+// What a kernel reads through const __restrict__ pointers or __ldg counts as constant
+// for its lifetime, and the compiler may move such a load past a barrier that only
+// names memory.  Here it holds from the wait to the kernel's end (the writers have
+// finished, and whatever writes next waits for this kernel in turn), so no such load may
+// come before the wait.  Hence the loop around it, whose end depends on a value the
+// compiler does not know: it moves no load above a branch it cannot decide unless it
+// knows the address to be valid, which it does of no pointer argument.  Past the wait
+// nothing is stale: the memory operations of all earlier grids are visible to this one,
+// and none of its threads has touched their lines before.
 template <class T>
 struct same_type {
   using type = T;
@@ -44,7 +54,12 @@ inline cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, siz
   c.numAttrs = 1;
   return cudaLaunchKernelEx(&c, kernel, args...);
 }
-__device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void after_previous() {
+  unsigned again;  // 0, from the asm the wait is in: the loop is gone from the machine code
+  do {
+    asm volatile("griddepcontrol.wait;\n\tmov.u32 %0, 0;" : "=r"(again)::"memory");
+  } while (again);
+}
 __device__ __forceinline__ void next_may_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 constexpr double kC = 299792458.0;  // m/s
