@@ -12,6 +12,16 @@ namespace {
 thread_local char g_err[512] = "";
 std::atomic<unsigned long long> g_launches{0};
 }
+int sm_count() {
+  constexpr int kCached = 64;  // devices; those beyond are asked on every call
+  static std::atomic<int> cache[kCached] = {};
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) dev = 0;
+  if (dev < kCached && (n = cache[dev].load(std::memory_order_relaxed)) != 0) return n;
+  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 152;
+  if (dev < kCached) cache[dev].store(n, std::memory_order_relaxed);
+  return n;
+}
 void note_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
 void set_error(const char* fmt, ...) {
   va_list ap;

@@ -14,6 +14,9 @@ void set_error(const char* fmt, ...);
 // Host-side count of kernel launches issued by the library (sbr_launch_count).
 void note_launch();
 
+// Streaming multiprocessors of the current device.
+int sm_count();
+
 // ---- launches of a chain of dependent kernels ------------------------------
 //
 // Most calls are chains of kernels of a few microseconds, between which a plain

@@ -1505,16 +1505,6 @@ inline int current_device() {
   return dev;
 }
 
-int sm_count() {
-  static int cache[kDevCache] = {};
-  const int dev = current_device();
-  if (dev < kDevCache && cache[dev]) return cache[dev];
-  int n = 0;
-  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 152;
-  if (dev < kDevCache) cache[dev] = n;
-  return n;
-}
-
 // Grid: V * Q CTAs, Q the largest that keeps every CTA resident at once (one
 // wave), capped by the number of path chunks.
 // dynamic shared memory of the split kernel: the groups' reduction buffer

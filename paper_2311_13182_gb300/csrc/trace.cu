@@ -581,15 +581,16 @@ __device__ inline void record_hit(const float4* __restrict__ tris, Ray& r, const
 // warps decide, and two rows of grazing rays in one warp make them longer: tiles of 32 x 32
 // rays, a warp a row of 32 (250,000 rays on 5,120 triangles, row by row / 32 / 16: 147 / 135 /
 // 125 us; 360,000 on 150,000 triangles, four views: 405 407 426 292 / 363 383 429 308 / 391 409
-// 465 336).  In a single wave (152 SMs x 7 CTAs) nothing starts late, and a ray list is the
+// 465 336).  In a single wave (152 SMs x 7 CTAs: 136,192 rays) nothing starts late, and a ray list is the
 // caller's: both are taken in their order (47,157 triangles, 34,225 rays, the worst of four
 // views: 115 us, 129 in tiles of 32, 148 of 16).
 constexpr int kTraceThreads = 128;
-constexpr int64_t kOneWaveRays = 136192, kRowWarpRays = 400000;
+constexpr int64_t kRowWarpRays = 400000;
 constexpr int kInOrder = 0;  // in place of a tile size's logarithm
 
 inline int tile_log2(int64_t R, bool list) {
-  return list || R <= kOneWaveRays ? kInOrder : R <= kRowWarpRays ? 5 : 4;
+  const int64_t wave = (int64_t)sm_count() * SBR_TRACE_MIN_BLOCKS * kTraceThreads;
+  return list || R <= wave ? kInOrder : R <= kRowWarpRays ? 5 : 4;
 }
 __host__ __device__ inline int tiles_across(int G, int log2) { return (G + (1 << log2) - 1) >> log2; }
 
@@ -1234,13 +1235,7 @@ inline RayDump* dump_records(const sbr_paths* p) {
   return reinterpret_cast<RayDump*>(static_cast<char*>(p->scratch) + scan_part(p->n_rays) + kCtrBytes);
 }
 // warps of the straggler kernel: 16 per SM, each takes rays until none is left
-inline int coop_grid() {
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
-    sms = 152;
-  return 4 * sms;
-}
+inline int coop_grid() { return 4 * sm_count(); }
 
 size_t paths_layout(sbr_paths* p, void* mem, int32_t R, int32_t K, int32_t V) {
   Carver c(mem);
