@@ -713,6 +713,31 @@ __device__ __forceinline__ double split_rint(double x, int& n) {
   return x - (k - 6755399441055744.0);
 }
 
+// What a record's rate turns into over the chirps, as FP32 pairs: carrier cycles and
+// delta per (m/s) of dL/dt.  A product with a rate keeps the fraction of its cycles to
+// 2^-25 however many they are; rounded with its whole cycles it would lose a bit for each
+// doubling, and a tile's turns would add that up (the last of 16 chirps at up to 100 m/s:
+// 2.3e-6 from FP64, 7e-7 so; of 128 chirps at up to 8 m/s 1.7e-6 and 4e-7).
+struct Pair32 {
+  float hi, lo;
+  __device__ explicit Pair32(double x) : hi((float)x), lo((float)(x - (double)(float)x)) {}
+  __device__ __forceinline__ float rest(float r, float p) const { return fmaf(r, lo, fmaf(r, hi, -p)); }  // r x - p, p = r hi rounded
+};
+// r x modulo 1
+__device__ __forceinline__ float cycles_of(float r, const Pair32& x) {
+  const float p = r * x.hi;
+  return (p - rintf(p)) + x.rest(r, p);
+}
+// The record's phi0 and delta after a shift of r cyc and r eps; whole multiples of 2^-12
+// of the delta shift move into delta_hi (which stays exact).
+__device__ __forceinline__ void shift_record(float4& rec, float r, const Pair32& cyc, const Pair32& eps) {
+  const float ph = rec.x + cycles_of(r, cyc);
+  rec.x = ph - rintf(ph);
+  const float p = r * eps.hi, kq = rintf((p + rec.z) * 4096.f), dh = rec.y + kq * (1.f / 4096.f);
+  rec.y = dh - rintf(dh);
+  rec.z = (p - kq * (1.f / 4096.f)) + (rec.z + eps.rest(r, p));
+}
+
 // CTA (q, v, chirp) spreads its share of antenna v's records, P/Q consecutive
 // ones.  Writes the CTA's grid, grids[CTA][l].  kBlocks: M > kNuBlock.
 template <bool kFp64, bool kMoving, bool kBlocks>
@@ -730,7 +755,7 @@ __global__ void __launch_bounds__(kNuThreads, 3)
   const int tid = threadIdx.x, lane = tid & 31;
   const int cl = blockIdx.x % na.chirps, v = (blockIdx.x / na.chirps) % na.V, q = blockIdx.x / (na.chirps * na.V);
   const double dt = kMoving ? (double)(na.chirp0 + cl) * na.per_chirp : 0.0;  // path length change per (m/s)
-  const float cnu = (float)(dt * na.f0_c), ceps = (float)(dt * na.b_cn);
+  const Pair32 cyc(dt * na.f0_c), eps(dt * na.b_cn);
   float2* out = grids + (size_t)blockIdx.x * M;
   for (int i = tid; i < npts * (2 * kNuCopies / 4); i += kNuThreads) nsm[i] = nu_zero();
   for (int i = tid; i < 2 * npts; i += kNuThreads) sum[i] = 0.f;
@@ -796,14 +821,8 @@ __global__ void __launch_bounds__(kNuThreads, 3)
         bad |= !isfinite(x + t + r.w);
       } else {
         if (kMoving) {
-          // phi0 + dL/dt cnu and delta + dL/dt ceps, whole multiples of 2^-12 of the delta
-          // shift moved into delta_hi (which stays exact)
           const float ld = p < n ? __ldg(&rate[at + p]) : 0.f;
-          const float ph = fmaf(ld, cnu, r.x);
-          r.x = ph - rintf(ph);
-          const float dl = fmaf(ld, ceps, r.z), kq = rintf(dl * 4096.f), dh = r.y + kq * (1.f / 4096.f);
-          r.y = dh - rintf(dh);
-          r.z = dl - kq * (1.f / 4096.f);
+          shift_record(r, ld, cyc, eps);
         }
         x = na.half_n * r.y;  // exact
         x -= rintf(x);
@@ -946,7 +965,7 @@ __global__ void __launch_bounds__(kNuThreads, 3)
 // 12 antennas x 367,500 records x 128 chirps 3.5 ms against 5.0 in groups chirp by chirp
 // (8 chirps at a time 3.9, 4 at a time 4.6; a third of it adds the chunks' copies up), 512
 // samples, 12 x 8,600 records 843 -> 560 us.  The rounding of up to kTile - 1 turns adds
-// about 1e-7.  A chunk's sums go to the chirp's grid in global memory (L2), each point by
+// 3e-7 to 7e-7 to the last chirp's error.  A chunk's sums go to the chirp's grid in global memory (L2), each point by
 // one thread; kTile copies in shared memory would cost a resident CTA.
 constexpr int kTile = 16;  // chirps per launch
 template <bool kBlocks>
@@ -961,8 +980,8 @@ __global__ void __launch_bounds__(kNuThreads, 3)
   const int tid = threadIdx.x, lane = tid & 31;
   const int v = blockIdx.x % na.V, q = blockIdx.x / na.V, nc = na.chirps;
   const double dt = (double)na.chirp0 * na.per_chirp;  // path length change per (m/s)
-  const float cnu = (float)(dt * na.f0_c), ceps = (float)(dt * na.b_cn);
-  const float turn = (float)(na.per_chirp * na.cyc), move = (float)(na.per_chirp * na.cell);  // per (m/s) and chirp
+  const Pair32 cyc(dt * na.f0_c), eps(dt * na.b_cn), turn(na.per_chirp * na.cyc);
+  const float move = (float)(na.per_chirp * na.cell);  // per (m/s) and chirp, as turn
   float2* out = grids + (size_t)(q * na.V + v) * nc * M;
   for (int i = tid; i < npts * (2 * kNuCopies / 4); i += kNuThreads) nsm[i] = nu_zero();
   for (int i = tid; i < 2 * (kNuBlock / 8); i += kNuThreads) (&flag[0][0])[i] = 0;
@@ -986,21 +1005,15 @@ __global__ void __launch_bounds__(kNuThreads, 3)
 #pragma unroll
     for (int u = 0; u < kNuItems; ++u) {
       const int p = c0 + tid + u * kNuThreads;
-      const float4 r = p < n ? __ldg(&prep[at + p]) : make_float4(0.f, 0.f, 0.f, 0.f);
+      float4 r = p < n ? __ldg(&prep[at + p]) : make_float4(0.f, 0.f, 0.f, 0.f);
       const float ld = p < n ? __ldg(&rate[at + p]) : 0.f;
-      // the tile's first chirp: phi0 + dL/dt cnu and delta + dL/dt ceps, whole multiples of
-      // 2^-12 of the delta shift moved into delta_hi (which stays exact)
-      const float ph = fmaf(ld, cnu, r.x);
-      const float dl = fmaf(ld, ceps, r.z), kq = rintf(dl * 4096.f);
-      float dh = r.y + kq * (1.f / 4096.f);
-      dh -= rintf(dh);
-      const float dlo = dl - kq * (1.f / 4096.f);
-      float x = na.half_n * dh;  // exact
+      shift_record(r, ld, cyc, eps);  // the tile's first chirp
+      float x = na.half_n * r.y;  // exact
       x -= rintf(x);
-      x = fmaf(na.half_n, dlo, x) + (ph - rintf(ph));
-      const float uh = na.m * dh;  // exact
+      x = fmaf(na.half_n, r.z, x) + r.x;
+      const float uh = na.m * r.y;  // exact
       float fl = floorf(uh);
-      float t = fmaf(na.m, dlo, uh - fl);
+      float t = fmaf(na.m, r.z, uh - fl);
       int ce = (int)fl;
       bad |= !isfinite(x + t + r.w + ld);
       fl = floorf(t);
@@ -1013,7 +1026,7 @@ __global__ void __launch_bounds__(kNuThreads, 3)
       // sine negated, the swapped pair turns by the same formula
       c1[u] = r.w * (upper ? sn : cs);
       c2[u] = r.w * (upper ? cs : sn);
-      sincospif(2.f * (ld * turn), &sn, &cs);
+      sincospif(2.f * cycles_of(ld, turn), &sn, &cs);
       wr[u] = cs;
       wi[u] = upper ? -sn : sn;
       mag[u] = __float_as_uint(fabsf(r.w));
