@@ -241,7 +241,8 @@ extern "C" sbr_status sbr_chamfer(const float* d_pred, const int32_t* d_n_pred, 
           "sbr_chamfer: n_target=%d outside [0, %d]", n_target, kChamferMax);
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   ::sbr::note_launch();
-  launch_after(k_chamfer, 1, 1024, 0, st, reinterpret_cast<const float4*>(d_pred), d_n_pred, pred_cap, reinterpret_cast<const float4*>(d_target), n_target, d_loss, reinterpret_cast<float4*>(d_gpred));
+  launch_after(k_chamfer, 1, 1024, 0, st, reinterpret_cast<const float4*>(d_pred), d_n_pred, pred_cap,
+               reinterpret_cast<const float4*>(d_target), n_target, d_loss, reinterpret_cast<float4*>(d_gpred));
   SBR_CUDA(cudaGetLastError());
   return SBR_OK;
 }
@@ -300,7 +301,8 @@ extern "C" sbr_status sbr_laplacian(const float* d_verts, int32_t nv, const int3
   ::sbr::note_launch();
   launch_after(k_lap_delta, b, kLapThreads, 0, st, d_verts, nv, d_off, d_adj, delta, partial);
   ::sbr::note_launch();
-  launch_after(k_lap_grad, b, kLapThreads, 0, st, delta, nv, d_off, d_adj, 2.f * weight / (float)nv, d_gverts, partial, b, weight / (float)nv, d_loss);
+  launch_after(k_lap_grad, b, kLapThreads, 0, st, delta, nv, d_off, d_adj, 2.f * weight / (float)nv, d_gverts, partial,
+               b, weight / (float)nv, d_loss);
   SBR_CUDA(cudaGetLastError());
   return SBR_OK;
 }
@@ -313,7 +315,8 @@ extern "C" sbr_status sbr_adam_step(float* d_params, const float* d_grad, float*
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   if (n > 0) {
     ::sbr::note_launch();
-    launch_after(k_adam, (unsigned)((n + 255) / 256), 256, 0, st, d_params, d_grad, d_m, d_v, n, d_step, lr, beta1, beta2, eps);
+    launch_after(k_adam, (unsigned)((n + 255) / 256), 256, 0, st, d_params, d_grad, d_m, d_v, n, d_step, lr, beta1,
+                 beta2, eps);
   }
   ::sbr::note_launch();
   launch_after(k_step_inc, 1, 1, 0, st, d_step);

@@ -1153,21 +1153,26 @@ extern "C" sbr_status sbr_pointcloud(const float* d_cube, const sbr_radar_cfg* r
   if (cells <= kSortOneCta || cfar->k_max <= kSelMax) {
     SBR_CUDA(select_attr());
     ::sbr::note_launch();
-    launch_after(k_detect, cells / kDetThreads, kDetThreads, 0, st, L.power, ca, L.amax_key, L.argmax, nullptr, L.key, L.flag, L.off);
+    launch_after(k_detect, cells / kDetThreads, kDetThreads, 0, st, L.power, ca, L.amax_key, L.argmax, nullptr, L.key,
+                 L.flag, L.off);
     ::sbr::note_launch();
-    launch_after(k_select, 1, kSelThreads, cta::kSortSmemBytes, st, L.power, pa, L.amax_key, L.key, L.flag, L.off, L.skeys[0], L.svals[0], L.skeys[1], L.svals[1], reinterpret_cast<float4*>(d_points), L.peak_cell, L.n_points);
+    launch_after(k_select, 1, kSelThreads, cta::kSortSmemBytes, st, L.power, pa, L.amax_key, L.key, L.flag, L.off,
+                 L.skeys[0], L.svals[0], L.skeys[1], L.svals[1], reinterpret_cast<float4*>(d_points), L.peak_cell,
+                 L.n_points);
     SBR_CUDA(cudaGetLastError());
     return SBR_OK;
   }
   ::sbr::note_launch();
-  launch_after(k_detect, cells / kDetThreads, kDetThreads, 0, st, L.power, ca, L.amax_key, L.argmax, L.flag, L.key, nullptr, nullptr);
+  launch_after(k_detect, cells / kDetThreads, kDetThreads, 0, st, L.power, ca, L.amax_key, L.argmax, L.flag, L.key,
+               nullptr, nullptr);
   SBR_CUDA(exclusive_scan(L.flag, L.off, cells, nullptr, L.scan_scr, st));
   ::sbr::note_launch();
   launch_after(k_compact, (cells + 255) / 256, 256, 0, st, L.flag, L.off, L.key, cells, L.skeys[0], L.svals[0]);
   SBR_CUDA(radix_sort_pairs(L.skeys, L.svals, cells, L.off + cells, 32, L.sort_scr, st));
   // 8-9: refine and emit points
   ::sbr::note_launch();
-  launch_after(k_points, (cfar->k_max + 255) / 256, 256, 0, st, L.power, pa, L.argmax, L.svals[0], L.off + cells, reinterpret_cast<float4*>(d_points), L.peak_cell, L.n_points);
+  launch_after(k_points, (cfar->k_max + 255) / 256, 256, 0, st, L.power, pa, L.argmax, L.svals[0], L.off + cells,
+               reinterpret_cast<float4*>(d_points), L.peak_cell, L.n_points);
   SBR_CUDA(cudaGetLastError());
   return SBR_OK;
 }

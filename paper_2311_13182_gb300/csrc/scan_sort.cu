@@ -351,7 +351,8 @@ cudaError_t radix_sort_pairs(uint32_t* keys[2], int32_t* vals[2], int64_t n, con
     cudaError_t e = sort_small_attr();
     if (e != cudaSuccess) return e;
     ::sbr::note_launch();
-    launch_after(k_sort_small, 1, kSmallThreads, kSortSmemBytes, s, keys[0], vals[0], keys[1], vals[1], n, d_n, bits, d_hist);
+    launch_after(k_sort_small, 1, kSmallThreads, kSortSmemBytes, s, keys[0], vals[0], keys[1], vals[1], n, d_n, bits,
+                 d_hist);
     return cudaGetLastError();
   }
   const int nt = tiles_for(n < 1 ? 1 : n);
@@ -365,7 +366,8 @@ cudaError_t radix_sort_pairs(uint32_t* keys[2], int32_t* vals[2], int64_t n, con
     ::sbr::note_launch();
     launch_after(k_digit_scan, kDigits, kThreads, 0, s, hist, nt, total);
     ::sbr::note_launch();
-    launch_after(k_digit_scatter, nt, kThreads, 0, s, keys[cur], vals[cur], keys[cur ^ 1], vals[cur ^ 1], n, d_n, shift, mask, hist, total, nt);
+    launch_after(k_digit_scatter, nt, kThreads, 0, s, keys[cur], vals[cur], keys[cur ^ 1], vals[cur ^ 1], n, d_n, shift,
+                 mask, hist, total, nt);
     cur ^= 1;
   }
   if (cur == 1) {  // odd number of passes: copy back so the result is in buffer 0

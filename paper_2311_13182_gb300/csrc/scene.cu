@@ -1156,7 +1156,8 @@ sbr_status rebuild(sbr_scene* s, const float* verts, cudaStream_t st, bool refit
   launch_after(k_bounds, blocks(nt, 256), 256, 0, st, verts, nv, s->faces, nt, s->bounds, s->err);
   if (!refit) {
     ::sbr::note_launch();
-    launch_after(k_morton, blocks(nt, 256), 256, 0, st, verts, nv, s->faces, nt, s->bounds, s->keys[0], s->vals[0], nt <= kSortOneCta ? s->hist : nullptr, s->err);
+    launch_after(k_morton, blocks(nt, 256), 256, 0, st, verts, nv, s->faces, nt, s->bounds, s->keys[0], s->vals[0],
+                 nt <= kSortOneCta ? s->hist : nullptr, s->err);
     SBR_CUDA(radix_sort_pairs(s->keys, s->vals, nt, nullptr, 31, s->sort_scratch, st, s->hist));
   }
   ::sbr::note_launch();
@@ -1168,7 +1169,8 @@ sbr_status rebuild(sbr_scene* s, const float* verts, cudaStream_t st, bool refit
     }
     SBR_CUDA(cudaMemsetAsync(s->visits, 0, sizeof(uint32_t) * (nt - 1), st));
     ::sbr::note_launch();
-    launch_after(k_refit, blocks(nt, kRefitTile), kRefitTile, 0, st, s->tris, nt, s->nodes, s->parent, s->visits, s->bounds);
+    launch_after(k_refit, blocks(nt, kRefitTile), kRefitTile, 0, st, s->tris, nt, s->nodes, s->parent, s->visits,
+                 s->bounds);
     ::sbr::note_launch();
     launch_after(k_collapse4, blocks(nt - 1, 128), 128, 0, st, s->nodes, nt, s->nodes4);
   }

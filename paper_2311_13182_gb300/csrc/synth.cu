@@ -3,11 +3,11 @@
 // cube[v, c, n] = sum_p A_{p,v} exp(j 2 pi (f_c tau_{p,v} + mu tau_{p,v} t_n)),
 // t_n = n T / N_s, identical for every chirp c of a static scene.
 //
-// Split-phase mode (sbr_synthesize's default path): a type-1 non-uniform FFT.  Each (path, antenna) is spread onto a periodic grid of
-// 2 N_s points with a width-8 Kaiser-Bessel kernel, one FFT per antenna follows,
-// and the kernel's Fourier transform is divided out: 8 grid updates per (path,
-// antenna) instead of N_s phasors, less than 1e-6 from the FP64 sum (details at
-// k_nufft_spread).
+// Split-phase mode (sbr_synthesize's default path): a type-1 non-uniform FFT.  Each
+// (path, antenna) is spread onto a periodic grid of 2 N_s points with a width-8
+// Kaiser-Bessel kernel, one FFT per antenna follows, and the kernel's Fourier transform
+// is divided out: 8 grid updates per (path, antenna) instead of N_s phasors, less than
+// 1e-6 from the FP64 sum (details at k_nufft_spread).
 //
 // Tensor-core kernel (N_s = 256 or 512, run by the allocation-free entry
 // point): with n = 16 a + b (b < 16), Eq. 8 factorises per path into
@@ -635,7 +635,8 @@ constexpr double nu_outer(double x) {  // psi(x)
   return bessel_i0_of(0.25 * kNuBeta * kNuBeta * (1.0 - (2.0 * x / kNuW) * (2.0 * x / kNuW))) /
          bessel_i0_of(0.25 * kNuBeta * kNuBeta);
 }
-static_assert(0.98 * (1 << kNuBits) * nu_outer(kNuW / 2 - kNuSmall) < 0.99 * (1 << 22), "outer terms pass the FMA's range");
+static_assert(0.98 * (1 << kNuBits) * nu_outer(kNuW / 2 - kNuSmall) < 0.99 * (1 << 22),
+              "outer terms pass the FMA's range");
 __device__ __forceinline__ int nu_term(float c, float w, bool small) {
   return small ? __float_as_int(fmaf(c, w, 12582912.f)) - 0x4B400000 : __float2int_rn(c * w);
 }
@@ -721,7 +722,8 @@ __device__ __forceinline__ double split_rint(double x, int& n) {
 struct Pair32 {
   float hi, lo;
   __device__ explicit Pair32(double x) : hi((float)x), lo((float)(x - (double)(float)x)) {}
-  __device__ __forceinline__ float rest(float r, float p) const { return fmaf(r, lo, fmaf(r, hi, -p)); }  // r x - p, p = r hi rounded
+  // r x - p, p = r hi rounded
+  __device__ __forceinline__ float rest(float r, float p) const { return fmaf(r, lo, fmaf(r, hi, -p)); }
 };
 // r x modulo 1
 __device__ __forceinline__ float cycles_of(float r, const Pair32& x) {
@@ -965,13 +967,15 @@ __global__ void __launch_bounds__(kNuThreads, 3)
 // 12 antennas x 367,500 records x 128 chirps 3.5 ms against 5.0 in groups chirp by chirp
 // (8 chirps at a time 3.9, 4 at a time 4.6; a third of it adds the chunks' copies up), 512
 // samples, 12 x 8,600 records 843 -> 560 us.  The rounding of up to kTile - 1 turns adds
-// 3e-7 to 7e-7 to the last chirp's error.  A chunk's sums go to the chirp's grid in global memory (L2), each point by
-// one thread; kTile copies in shared memory would cost a resident CTA.
+// 3e-7 to 7e-7 to the last chirp's error.  A chunk's sums go to the chirp's grid in global
+// memory (L2), each point by one thread; kTile copies in shared memory would cost a
+// resident CTA.
 constexpr int kTile = 16;  // chirps per launch
 template <bool kBlocks>
 __global__ void __launch_bounds__(kNuThreads, 3)
     k_nufft_spread_chirps(const float4* __restrict__ prep, const float* __restrict__ rate, int64_t cap,
-                          const int32_t* __restrict__ d_P, const NufftArg na, const __grid_constant__ NufftCoef co, float2* __restrict__ grids) {
+                          const int32_t* __restrict__ d_P, const NufftArg na, const __grid_constant__ NufftCoef co,
+                          float2* __restrict__ grids) {
   extern __shared__ uint4 nsm[];  // [npts][re, im][kNuCopies]
   __shared__ uint32_t s_max[2];  // by the parity of the turn: largest amplitude
   __shared__ int s_log[2];       // and the sum of the amplitudes' logarithms
@@ -1753,11 +1757,13 @@ void launch_nufft(sbr_phase_mode mode, const sbr_paths* p, const sbr_radar_cfg* 
                p->phase_ofs, p->path_rate, p->path_cap, p->count, na, co, w.grids, w.fin_cnt);
   ::sbr::note_launch();
   if (M <= kNuClusterPoints) {
-    launch_after(k_nufft_finish_cluster, V * chirps * kNuRanks, kNuClThreads, nufft_cl_smem(Ns), st, w.grids, na, co, cube, r->n_chirps, moving);
+    launch_after(k_nufft_finish_cluster, V * chirps * kNuRanks, kNuClThreads, nufft_cl_smem(Ns), st, w.grids, na, co,
+                 cube, r->n_chirps, moving);
     return;
   }
   const int slices = M / kNuFinSlice;
-  launch_after(k_nufft_finish, V * chirps * slices, kNuFinThreads, nufft_fin_smem(Ns), st, w.grids, na, co, w.bsum, w.fin_cnt, cube, r->n_chirps, moving);
+  launch_after(k_nufft_finish, V * chirps * slices, kNuFinThreads, nufft_fin_smem(Ns), st, w.grids, na, co, w.bsum,
+               w.fin_cnt, cube, r->n_chirps, moving);
 }
 
 // The chirps of a moving scene, kTile at a time: a launch is one wave of CTAs, each with
@@ -1821,18 +1827,22 @@ void launch_fwd(sbr_phase_mode mode, const sbr_paths* p, const sbr_radar_cfg* r,
   const float4* prep = reinterpret_cast<const float4*>(p->prep);
   if (mode == SBR_PHASE_SPLIT && (Ns == 256 || Ns == 512)) {
     ::sbr::note_launch();
-    if (Ns == 256) launch_after(k_synth_mma<1>, grid, kMmaThreads, 0, st, prep, p->path_cap, p->count, V, w.Q, w.partial);
+    if (Ns == 256) launch_after(k_synth_mma<1>, grid, kMmaThreads, 0, st, prep, p->path_cap, p->count, V, w.Q,
+                                w.partial);
     else launch_after(k_synth_mma<2>, grid, kMmaThreads, 0, st, prep, p->path_cap, p->count, V, w.Q, w.partial);
   } else if (mode == SBR_PHASE_SPLIT) {
     ::sbr::note_launch();
-    launch_after(k_synth_split<M>, grid, kSplitThreads, split_smem(Ns), st, prep, p->path_cap, p->count, V, w.Q, Ns, w.partial);
+    launch_after(k_synth_split<M>, grid, kSplitThreads, split_smem(Ns), st, prep, p->path_cap, p->count, V, w.Q, Ns,
+                 w.partial);
   } else if (mode == SBR_PHASE_FP64) {
     ::sbr::note_launch();
-    launch_after(k_synth_fp64<M>, grid, T, 0, st, prep, reinterpret_cast<const float2*>(p->path_len), p->phase_ofs, p->path_cap, p->count, V, w.Q, Ns, r->f0, r->bandwidth / Ns, w.partial);
+    launch_after(k_synth_fp64<M>, grid, T, 0, st, prep, reinterpret_cast<const float2*>(p->path_len), p->phase_ofs,
+                 p->path_cap, p->count, V, w.Q, Ns, r->f0, r->bandwidth / Ns, w.partial);
   } else {
     const double mu = r->bandwidth / r->chirp_time, dt = r->chirp_time / Ns;
     ::sbr::note_launch();
-    launch_after(k_synth_naive<M>, grid, T, 0, st, prep, reinterpret_cast<const float2*>(p->path_len), p->phase_ofs, p->path_cap, p->count, V, w.Q, Ns, (float)r->f0, (float)mu, (float)dt, w.partial);
+    launch_after(k_synth_naive<M>, grid, T, 0, st, prep, reinterpret_cast<const float2*>(p->path_len), p->phase_ofs,
+                 p->path_cap, p->count, V, w.Q, Ns, (float)r->f0, (float)mu, (float)dt, w.partial);
   }
 }
 }  // namespace
@@ -1876,7 +1886,8 @@ extern "C" sbr_status sbr_synthesize(const sbr_paths* paths, const sbr_radar_cfg
   SBR_CUDA(cudaGetLastError());
   const int V = paths->n_virt;
   ::sbr::note_launch();
-  launch_after(k_reduce, reduce_grid(V, Ns, radar->n_chirps), 256, 0, st, w.partial, V, w.Q, Ns, radar->n_chirps, reinterpret_cast<float2*>(d_cube));
+  launch_after(k_reduce, reduce_grid(V, Ns, radar->n_chirps), 256, 0, st, w.partial, V, w.Q, Ns, radar->n_chirps,
+               reinterpret_cast<float2*>(d_cube));
   SBR_CUDA(cudaGetLastError());
   return SBR_OK;
 }
@@ -1951,7 +1962,8 @@ extern "C" sbr_status sbr_synthesize_noalloc(const sbr_paths* paths, const sbr_r
   }
   SBR_CUDA(cudaGetLastError());
   ::sbr::note_launch();
-  launch_after(k_reduce, reduce_grid(V, Ns, radar->n_chirps), 256, 0, st, w.partial, V, w.Q, Ns, radar->n_chirps, reinterpret_cast<float2*>(d_cube));
+  launch_after(k_reduce, reduce_grid(V, Ns, radar->n_chirps), 256, 0, st, w.partial, V, w.Q, Ns, radar->n_chirps,
+               reinterpret_cast<float2*>(d_cube));
   SBR_CUDA(cudaGetLastError());
   return SBR_OK;
 }
@@ -1994,7 +2006,9 @@ extern "C" sbr_status sbr_synthesize_bwd(const sbr_paths* paths, const sbr_radar
     // a wave of CTAs at most, at least one per antenna
     const int64_t need = (paths->path_cap + 255) / 256, wave = std::max(1, 8 * sm_count() / V);
     ::sbr::note_launch();
-    launch_after(k_synth_bwd_nufft, dim3((unsigned)std::min(need, wave), V), 256, 0, st, reinterpret_cast<const float4*>(paths->prep), paths->path_cap, paths->count, log_m, co, w.adj, (float)lam_inv, d_glen, d_gamp, d_gphase);
+    launch_after(k_synth_bwd_nufft, dim3((unsigned)std::min(need, wave), V), 256, 0, st,
+                 reinterpret_cast<const float4*>(paths->prep), paths->path_cap, paths->count, log_m, co, w.adj,
+                 (float)lam_inv, d_glen, d_gamp, d_gphase);
     SBR_CUDA(cudaGetLastError());
     return SBR_OK;
   }
@@ -2010,7 +2024,8 @@ extern "C" sbr_status sbr_synthesize_bwd(const sbr_paths* paths, const sbr_radar
     dim3 grid((unsigned)((cap + 255) / 256), (unsigned)V);
     const double bcn = radar->bandwidth / (kC * Ns);
     ::sbr::note_launch();
-    launch_after(k_synth_bwd, grid, 256, Ns * sizeof(float2), st, reinterpret_cast<const float4*>(paths->prep), cap, paths->count, Ns, gs, (float)lam_inv, (float)bcn, d_glen, d_gamp, d_gphase);
+    launch_after(k_synth_bwd, grid, 256, Ns * sizeof(float2), st, reinterpret_cast<const float4*>(paths->prep), cap,
+                 paths->count, Ns, gs, (float)lam_inv, (float)bcn, d_glen, d_gamp, d_gphase);
   }
   SBR_CUDA(cudaGetLastError());
   return SBR_OK;

@@ -1,9 +1,9 @@
 // Ray tracing with specular bounces (Section 3.2.1, Eq. 2-3) and path preparation.
 //
-// One thread per ray (up to 32,768 rays eight lanes, k_trace_warp).  The ray is carried in float-float (ff.cuh): its FP32 hi
-// parts drive a stack traversal of the 4-wide BVH collapsed from the LBVH (a
-// node's four child boxes and links as seven float4 loads, triangles as three
-// float4 loads) with the Moller-Trumbore (1997) test.  Every
+// One thread per ray (up to 32,768 rays eight lanes, k_trace_warp).  The ray is carried
+// in float-float (ff.cuh): its FP32 hi parts drive a stack traversal of the 4-wide BVH
+// collapsed from the LBVH (a node's four child boxes and links as seven float4 loads,
+// triangles as three float4 loads) with the Moller-Trumbore (1997) test.  Every
 // FP32 decision carries a forward error bound: a triangle is accepted or
 // rejected in FP32 only when the bound says exact arithmetic on the exact ray
 // would decide the same; otherwise the test is repeated in float-float
@@ -1208,19 +1208,24 @@ void launch_prep(int nb, cudaStream_t st, const float4* hp4, const sbr_paths* pa
                  const RadarArg& rd, const MatArg& mat, const MotionArg& mot, float4* prep, float2* plen) {
   switch (rd.ntx) {
     case 1:
-      launch_after(k_prep<1, kMotion>, nb, 128, 0, st, hp4, paths->hits, paths->ray_weight, paths->ray_first, (int)R, K, rd, mat, mot, paths->path_cap, prep, plen, paths->path_ray, paths->phase_ofs, paths->path_rate);
+      launch_after(k_prep<1, kMotion>, nb, 128, 0, st, hp4, paths->hits, paths->ray_weight, paths->ray_first, (int)R, K,
+                   rd, mat, mot, paths->path_cap, prep, plen, paths->path_ray, paths->phase_ofs, paths->path_rate);
       break;
     case 2:
-      launch_after(k_prep<2, kMotion>, nb, 128, 0, st, hp4, paths->hits, paths->ray_weight, paths->ray_first, (int)R, K, rd, mat, mot, paths->path_cap, prep, plen, paths->path_ray, paths->phase_ofs, paths->path_rate);
+      launch_after(k_prep<2, kMotion>, nb, 128, 0, st, hp4, paths->hits, paths->ray_weight, paths->ray_first, (int)R, K,
+                   rd, mat, mot, paths->path_cap, prep, plen, paths->path_ray, paths->phase_ofs, paths->path_rate);
       break;
     case 3:
-      launch_after(k_prep<3, kMotion>, nb, 128, 0, st, hp4, paths->hits, paths->ray_weight, paths->ray_first, (int)R, K, rd, mat, mot, paths->path_cap, prep, plen, paths->path_ray, paths->phase_ofs, paths->path_rate);
+      launch_after(k_prep<3, kMotion>, nb, 128, 0, st, hp4, paths->hits, paths->ray_weight, paths->ray_first, (int)R, K,
+                   rd, mat, mot, paths->path_cap, prep, plen, paths->path_ray, paths->phase_ofs, paths->path_rate);
       break;
     case 4:
-      launch_after(k_prep<4, kMotion>, nb, 128, 0, st, hp4, paths->hits, paths->ray_weight, paths->ray_first, (int)R, K, rd, mat, mot, paths->path_cap, prep, plen, paths->path_ray, paths->phase_ofs, paths->path_rate);
+      launch_after(k_prep<4, kMotion>, nb, 128, 0, st, hp4, paths->hits, paths->ray_weight, paths->ray_first, (int)R, K,
+                   rd, mat, mot, paths->path_cap, prep, plen, paths->path_ray, paths->phase_ofs, paths->path_rate);
       break;
     default:
-      launch_after(k_prep<0, kMotion>, nb, 128, 0, st, hp4, paths->hits, paths->ray_weight, paths->ray_first, (int)R, K, rd, mat, mot, paths->path_cap, prep, plen, paths->path_ray, paths->phase_ofs, paths->path_rate);
+      launch_after(k_prep<0, kMotion>, nb, 128, 0, st, hp4, paths->hits, paths->ray_weight, paths->ray_first, (int)R, K,
+                   rd, mat, mot, paths->path_cap, prep, plen, paths->path_ray, paths->phase_ofs, paths->path_rate);
   }
 }
 
@@ -1380,19 +1385,27 @@ static sbr_status trace_impl(const sbr_scene* scene, const sbr_radar_cfg* radar,
     const int nbw = blocks(R * kGroup, 128);
     ::sbr::note_launch();
     if (d_counts)
-      launch_after(k_trace_warp<true>, nbw, 128, 0, st, scene->tris, scene->nodes4, scene->nt, g, d_ray_ids, (int)R, max_bounces, paths->hits, hp, paths->ray_weight, paths->ray_first, d_counts);
+      launch_after(k_trace_warp<true>, nbw, 128, 0, st, scene->tris, scene->nodes4, scene->nt, g, d_ray_ids, (int)R,
+                   max_bounces, paths->hits, hp, paths->ray_weight, paths->ray_first, d_counts);
     else
-      launch_after(k_trace_warp<false>, nbw, 128, 0, st, scene->tris, scene->nodes4, scene->nt, g, d_ray_ids, (int)R, max_bounces, paths->hits, hp, paths->ray_weight, paths->ray_first, nullptr);
+      launch_after(k_trace_warp<false>, nbw, 128, 0, st, scene->tris, scene->nodes4, scene->nt, g, d_ray_ids, (int)R,
+                   max_bounces, paths->hits, hp, paths->ray_weight, paths->ray_first, nullptr);
   } else if (d_counts) {
     ::sbr::note_launch();
-    launch_after(k_trace<true>, trace_blocks(R, grid->G, tile), kTraceThreads, 0, st, scene->tris, scene->nodes4, scene->nt, g, d_ray_ids, (int)R, tile, max_bounces, paths->hits, hp, paths->ray_weight, paths->ray_first, dumps, dctr, d_counts, scene->top, scene->top_n);
+    launch_after(k_trace<true>, trace_blocks(R, grid->G, tile), kTraceThreads, 0, st, scene->tris, scene->nodes4,
+                 scene->nt, g, d_ray_ids, (int)R, tile, max_bounces, paths->hits, hp, paths->ray_weight,
+                 paths->ray_first, dumps, dctr, d_counts, scene->top, scene->top_n);
     ::sbr::note_launch();
-    launch_after(k_trace_coop<true>, coop_grid(), 128, 0, st, scene->tris, scene->nodes4, scene->nt, g, max_bounces, dumps, dctr, dctr + 1, paths->hits, hp, paths->ray_first, d_counts);
+    launch_after(k_trace_coop<true>, coop_grid(), 128, 0, st, scene->tris, scene->nodes4, scene->nt, g, max_bounces,
+                 dumps, dctr, dctr + 1, paths->hits, hp, paths->ray_first, d_counts);
   } else {
     ::sbr::note_launch();
-    launch_after(k_trace<false>, trace_blocks(R, grid->G, tile), kTraceThreads, 0, st, scene->tris, scene->nodes4, scene->nt, g, d_ray_ids, (int)R, tile, max_bounces, paths->hits, hp, paths->ray_weight, paths->ray_first, dumps, dctr, nullptr, scene->top, scene->top_n);
+    launch_after(k_trace<false>, trace_blocks(R, grid->G, tile), kTraceThreads, 0, st, scene->tris, scene->nodes4,
+                 scene->nt, g, d_ray_ids, (int)R, tile, max_bounces, paths->hits, hp, paths->ray_weight,
+                 paths->ray_first, dumps, dctr, nullptr, scene->top, scene->top_n);
     ::sbr::note_launch();
-    launch_after(k_trace_coop<false>, coop_grid(), 128, 0, st, scene->tris, scene->nodes4, scene->nt, g, max_bounces, dumps, dctr, dctr + 1, paths->hits, hp, paths->ray_first, nullptr);
+    launch_after(k_trace_coop<false>, coop_grid(), 128, 0, st, scene->tris, scene->nodes4, scene->nt, g, max_bounces,
+                 dumps, dctr, dctr + 1, paths->hits, hp, paths->ray_first, nullptr);
   }
   SBR_CUDA(cudaGetLastError());
   SBR_CUDA(exclusive_scan(paths->ray_first, paths->ray_first, R, nullptr, paths->scratch, st));

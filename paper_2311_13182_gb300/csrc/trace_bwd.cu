@@ -386,9 +386,13 @@ extern "C" sbr_status sbr_trace_bwd(const sbr_scene* scene, const float* d_verts
   const float4* hp = reinterpret_cast<const float4*>(paths->hit_pos);
   const float4* pr = reinterpret_cast<const float4*>(paths->prep);
   ::sbr::note_launch();
-  launch_after(k_trace_bwd<0>, (R + 127) / 128, 128, 0, st, d_verts, scene->nv, scene->faces, g, rd, mat, d_ray_ids, R, paths->max_bounces, paths->hits, hp, paths->ray_first, pr, paths->path_cap, d_glen, d_gamp, d_gphase, reparam, w.fs, w.fe);
+  launch_after(k_trace_bwd<0>, (R + 127) / 128, 128, 0, st, d_verts, scene->nv, scene->faces, g, rd, mat, d_ray_ids, R,
+               paths->max_bounces, paths->hits, hp, paths->ray_first, pr, paths->path_cap, d_glen, d_gamp, d_gphase,
+               reparam, w.fs, w.fe);
   ::sbr::note_launch();
-  launch_after(k_trace_bwd<1>, (R + 127) / 128, 128, 0, st, d_verts, scene->nv, scene->faces, g, rd, mat, d_ray_ids, R, paths->max_bounces, paths->hits, hp, paths->ray_first, pr, paths->path_cap, d_glen, d_gamp, d_gphase, reparam, w.fs, w.fe);
+  launch_after(k_trace_bwd<1>, (R + 127) / 128, 128, 0, st, d_verts, scene->nv, scene->faces, g, rd, mat, d_ray_ids, R,
+               paths->max_bounces, paths->hits, hp, paths->ray_first, pr, paths->path_cap, d_glen, d_gamp, d_gphase,
+               reparam, w.fs, w.fe);
   const int n3 = 3 * scene->nv;
   if (n3 > 0) {
     ::sbr::note_launch();
