@@ -556,8 +556,8 @@ __global__ void __launch_bounds__(256) k_synth_bwd(const float4* __restrict__ pr
 //
 // A CTA has a barrier for a chunk's largest amplitude and one before its sums are added
 // up; the next chunk's records are in flight meanwhile, and its preparation needs none.
-// Bound by issue slots (212 instructions per 32 records) and the conversion unit,
-// three CTAs per SM: 12 antennas x 367,500 records x 256 samples 35 us (109 us when
+// Bound by issue slots (211 instructions per 32 records) and the conversion unit,
+// three CTAs per SM: 12 antennas x 367,500 records x 256 samples 36 us (109 us when
 // each warp kept runs of equal cells in registers, eight lanes to a record, and
 // flushed them to its own FP32 grid, one group at a time; 93 us with the chunk sorted
 // by cell first), 71 MB of records at 2 TB/s.  A block of 512 cells, so that long
@@ -574,7 +574,7 @@ constexpr int kNuChunk = kNuThreads * kNuItems;
 constexpr int kNuBits = 25;    // 2 kNuChunk / 32 additions per copy of terms up to 0.98 2^25: below 2^31
 static_assert(kNuChunk / kNuCopies <= 1 << (31 - kNuBits), "a class's additions to one copy");
 constexpr int kNuSpan = 24;    // mean distance of a class's amplitudes from its largest, in eighths of an octave
-constexpr int kNuFar = 40;     // the same where many are close to it
+constexpr int kNuFar = 40;     // the same where their rms is near it all the same
 constexpr double kNuBeta = 2.3 * kNuW;
 
 struct NufftCoef {
@@ -648,44 +648,52 @@ constexpr int kNuAll = 2048;  // above every logarithm
 // The class of records that one pass rounds on one scale, 2^s for the largest amplitude
 // (its bits: top) to land in (0.49, 0.98] 2^kNuBits: all N that are left if their
 // logarithms (sum: logs) lie within kNuSpan of the largest's on average, or within
-// kNuFar and a sixteenth of them within an octave of it (nu_near); else those within
+// kNuFar with a rms amplitude of an eighth of it or more (nu_one_class); else those within
 // kNuSpan of it.  The class's rms amplitude is then an eighth of its largest or more, and
 // the rounding stays near the error of the transform around it; on one scale for all, a
 // chunk's few strong records would cost its weak ones their bits (one record in 1,024 a
 // hundred times the others: 9e-7 to 1.4e-6 from FP64 instead of 1.8e-7; two in 1,024 a
 // thousand times the others and cancelling: 3e-5 instead of 1.9e-7).  The returns of one
-// chunk differ little: traced paths of superquadrics over a ground plane leave kNuSpan in
-// up to 9 % of the chunks (26 % in the worst of nine scenes), and need a second class in
-// up to 0.6 %.  The scale is a power of two, exact; one past a float's range (amplitudes
+// chunk differ little: the traced paths of 28 scenes leave kNuSpan in up to 9 % of their
+// chunks (two of them in 26 and 39 %), and need a second class in up to 0.1 % (1 %).
+// The scale is a power of two, exact; one past a float's range (amplitudes
 // below 1e-31) is applied in two factors.
-// The two words per chunk that this takes, and the copies' sum in 64 bits, cost 12
-// antennas x 367,500 records 42.0 -> 43.0 us for the whole synthesis, 4 antennas x 3.1 M
-// records x 4096 samples 122.8 -> 126.4; moving chirps (no sign extensions in the sum)
-// 3.49 -> 3.41 ms.
+// The words per chunk that this takes cost 12 antennas x 367,500 records 41.8 -> 42.6 us
+// for the whole synthesis, 471,630 records in whose chunks the rms is looked at in 39 %
+// 55.4 -> 58.3, 4 antennas x 3.1 M records x 4096 samples 122.5 -> 125.8; moving chirps
+// (no sign extensions in the sum) 3.49 -> 3.45 ms.
 struct NuClass {
-  int floor;   // logarithms from here on belong to the class; 0: every record left
-  bool rare;   // floor or more matter
-  float up, more;    // 2^s = up more, more = 1 but for the smallest amplitudes
-  float down, less;  // their reciprocals
+  float up, down;    // 2^s and its reciprocal
+  float more, less;  // the scale's second factor and its reciprocal
+  int floor;         // logarithms from here on belong to the class; 0: every record left
+  bool rare;         // the fields above are nu_rare's to set
 };
 __device__ __forceinline__ NuClass nu_class(uint32_t top, int logs, int N) {
-  const int l = (int)(top >> 20);
   NuClass c;
-  c.floor = N * (l - kNuSpan) <= logs ? 0 : max(l - kNuSpan, 0);
-  // exponents of the largest's upper bound: one more from 1.96 on, 1 for all denormal numbers
-  const int s = 126 + kNuBits - max((int)((top + 0x51eb9u) >> 23), 1), a = min(s, 126);
-  c.rare = c.floor != 0 || s != a;
-  c.up = __int_as_float((127 + a) << 23);
-  c.more = __int_as_float((127 + s - a) << 23);
-  c.down = __int_as_float((127 - a) << 23);
-  c.less = __int_as_float((127 - s + a) << 23);
+  const int e = (int)((top + 0x51eb9u) >> 23);  // the largest's exponent, one more from 1.96 2^e on
+  c.up = __int_as_float((127 + 126 + kNuBits - e) << 23);
+  c.down = __int_as_float((e + 1 - kNuBits) << 23);
+  c.more = c.less = 1.f;
+  c.floor = 0;
+  c.rare = N * ((int)(top >> 20) - kNuSpan) > logs || e < kNuBits;
   return c;
 }
+__device__ __forceinline__ void nu_rare(NuClass& c, uint32_t top, int logs, int N) {
+  const int e = (int)((top + 0x51eb9u) >> 23), l = (int)(top >> 20) - kNuSpan;
+  if (e < kNuBits) {  // up would pass a float's range, down fall below it
+    c.up = __int_as_float((127 + 126) << 23);
+    c.down = __int_as_float((127 - 126) << 23);
+    c.more = __int_as_float((127 + kNuBits - e) << 23);
+    c.less = __int_as_float((127 - kNuBits + e) << 23);
+  }
+  c.floor = N * l > logs ? max(l, 0) : 0;
+}
 
-// Amplitudes within an octave of the largest, where a chunk has left kNuSpan.
-__device__ __forceinline__ bool nu_near(int log, const NuClass& c) { return log >= c.floor + kNuSpan - 8; }
-__device__ __forceinline__ bool nu_one_class(const NuClass& c, int near, int logs, int N) {
-  return 16 * near >= N && N * (c.floor + kNuSpan - kNuFar) <= logs;
+// Amplitude whose square counts for nu_one_class: the largest's is 15,000 to 63,000.
+__device__ __forceinline__ float nu_part(float a, const NuClass& c) { return a * c.more * c.up * 0x1p-17f; }
+__device__ __forceinline__ bool nu_one_class(const NuClass& c, uint32_t top, int power, int logs, int N) {
+  const float x = nu_part(__uint_as_float(top), c);
+  return power >= (N * (int)(x * x)) >> 6 && N * (c.floor + kNuSpan - kNuFar) <= logs;
 }
 
 // Grid words in shared memory are kept kNuZero off, so that the copies add up unsigned,
@@ -749,7 +757,7 @@ __global__ void __launch_bounds__(kNuThreads, 3)
                    const __grid_constant__ NufftCoef co, float2* __restrict__ grids, unsigned int* __restrict__ fin_cnt) {
   extern __shared__ uint4 nsm[];
   __shared__ uint32_t s_max[2], s_blk[2];     // by the parity of the chunk: largest amplitude, blocks
-  __shared__ int s_log[2];                    // and the sum of the amplitudes' logarithms
+  __shared__ int s_log[2], s_pow[2];          // and the sums of the amplitudes' logarithms and, rarely, powers
   __shared__ int flag[2][kNuBlock / 8];       // by the parity of the pass: a record of cells 8 o .. 8 o + 7
   const int M = 1 << na.log_m, bs = nu_cells(M), npts = nu_points(M);
   int* grid = reinterpret_cast<int*>(nsm);                            // [npts][re, im][kNuCopies]
@@ -762,7 +770,7 @@ __global__ void __launch_bounds__(kNuThreads, 3)
   for (int i = tid; i < npts * (2 * kNuCopies / 4); i += kNuThreads) nsm[i] = nu_zero();
   for (int i = tid; i < 2 * npts; i += kNuThreads) sum[i] = 0.f;
   for (int i = tid; i < 2 * (kNuBlock / 8); i += kNuThreads) (&flag[0][0])[i] = 0;
-  if (tid < 2) s_max[tid] = s_blk[tid] = 0u, s_log[tid] = 0;
+  if (tid < 2) s_max[tid] = s_blk[tid] = 0u, s_log[tid] = s_pow[tid] = 0;
   after_previous();
   if (blockIdx.x == 0)
     for (int i = tid; i < na.V * na.chirps; i += kNuThreads) fin_cnt[i] = 0u;  // the finishing kernel's counters
@@ -865,20 +873,30 @@ __global__ void __launch_bounds__(kNuThreads, 3)
     }
     __syncthreads();  // the chunk's words; the turn before is added up
     logs = s_log[chunk & 1];
-    NuClass cls = nu_class(s_max[chunk & 1], logs, left);
+    const uint32_t top = s_max[chunk & 1];
+    NuClass cls = nu_class(top, logs, left);
     blocks = kBlocks ? s_blk[chunk & 1] : 1u;
     if (cls.rare) {  // the same for the whole CTA
+      nu_rare(cls, top, logs, left);
       if (cls.floor) {
-        int near = 0;
+        float x = 0.f;
 #pragma unroll
-        for (int u = 0; u < kNuItems; ++u) near += __syncthreads_count(nu_near(nu_log(rec[u].w), cls));
-        if (nu_one_class(cls, near, logs, left)) cls.floor = 0;
+        for (int u = 0; u < kNuItems; ++u) {
+          const float y = nu_part(rec[u].w, cls);
+          x = fmaf(y, y, x);
+        }
+        const int power = __reduce_add_sync(0xffffffffu, (int)x);
+        if (lane == 0) atomicAdd(&s_pow[chunk & 1], power);
+        __syncthreads();
+        if (nu_one_class(cls, top, s_pow[chunk & 1], logs, left)) cls.floor = 0;
       }
+      if (cls.floor || cls.more != 1.f) {
 #pragma unroll
-      for (int u = 0; u < kNuItems; ++u) {
-        const bool in = nu_log(rec[u].w) >= cls.floor;
-        if (cls.floor) left -= __syncthreads_count(in);
-        rec[u].w = in ? rec[u].w * cls.more : 0.f;
+        for (int u = 0; u < kNuItems; ++u) {
+          const bool in = nu_log(rec[u].w) >= cls.floor;
+          if (cls.floor) left -= __syncthreads_count(in);
+          rec[u].w = in ? rec[u].w * cls.more : 0.f;
+        }
       }
     }
 #pragma unroll
@@ -901,7 +919,7 @@ __global__ void __launch_bounds__(kNuThreads, 3)
       int* fl = flag[pass & 1];
       // read before this pass: the other parity's flags and words
       if (tid < kNuBlock / 8) flag[~pass & 1][tid] = 0;
-      if (tid == 0) s_max[~chunk & 1] = s_blk[~chunk & 1] = 0u, s_log[~chunk & 1] = 0;
+      if (tid == 0) s_max[~chunk & 1] = s_blk[~chunk & 1] = 0u, s_log[~chunk & 1] = s_pow[~chunk & 1] = 0;
 #pragma unroll
       for (int u = 0; u < kNuItems; ++u) {
         const int idx = kBlocks ? cell[u] - b * bs : cell[u];
@@ -978,7 +996,7 @@ __global__ void __launch_bounds__(kNuThreads, 3)
                           float2* __restrict__ grids) {
   extern __shared__ uint4 nsm[];  // [npts][re, im][kNuCopies]
   __shared__ uint32_t s_max[2];  // by the parity of the turn: largest amplitude
-  __shared__ int s_log[2];       // and the sum of the amplitudes' logarithms
+  __shared__ int s_log[2], s_pow[2];  // and the sums of the amplitudes' logarithms and, rarely, powers
   __shared__ int flag[2][kNuBlock / 8];
   const int M = 1 << na.log_m, bs = nu_cells(M), npts = nu_points(M), oct = bs >> 3;
   const int tid = threadIdx.x, lane = tid & 31;
@@ -989,7 +1007,7 @@ __global__ void __launch_bounds__(kNuThreads, 3)
   float2* out = grids + (size_t)(q * na.V + v) * nc * M;
   for (int i = tid; i < npts * (2 * kNuCopies / 4); i += kNuThreads) nsm[i] = nu_zero();
   for (int i = tid; i < 2 * (kNuBlock / 8); i += kNuThreads) (&flag[0][0])[i] = 0;
-  if (tid < 2) s_max[tid] = 0u, s_log[tid] = 0;
+  if (tid < 2) s_max[tid] = 0u, s_log[tid] = s_pow[tid] = 0;
   after_previous();
   for (int i = tid; i < nc * M; i += kNuThreads) out[i] = make_float2(0.f, 0.f);
   const int64_t P = *d_P;
@@ -1053,20 +1071,30 @@ __global__ void __launch_bounds__(kNuThreads, 3)
     }
     __syncthreads();
     logs = s_log[chunk & 1];
-    NuClass cls = nu_class(s_max[chunk & 1], logs, left);
+    const uint32_t top = s_max[chunk & 1];
+    NuClass cls = nu_class(top, logs, left);
     if (cls.rare) {  // the same for the whole CTA
+      nu_rare(cls, top, logs, left);
       if (cls.floor) {
-        int near = 0;
+        float x = 0.f;
 #pragma unroll
-        for (int u = 0; u < kNuItems; ++u) near += __syncthreads_count(nu_near((int)(mag[u] >> 20), cls));
-        if (nu_one_class(cls, near, logs, left)) cls.floor = 0;
+        for (int u = 0; u < kNuItems; ++u) {
+          const float y = nu_part(__uint_as_float(mag[u]), cls);
+          x = fmaf(y, y, x);
+        }
+        const int power = __reduce_add_sync(0xffffffffu, (int)x);
+        if (lane == 0) atomicAdd(&s_pow[chunk & 1], power);
+        __syncthreads();
+        if (nu_one_class(cls, top, s_pow[chunk & 1], logs, left)) cls.floor = 0;
       }
+      if (cls.floor || cls.more != 1.f) {
 #pragma unroll
-      for (int u = 0; u < kNuItems; ++u) {
-        const bool in = (int)(mag[u] >> 20) >= cls.floor;
-        if (cls.floor) left -= __syncthreads_count(in);
-        c1[u] = in ? c1[u] * cls.more : 0.f;
-        c2[u] = in ? c2[u] * cls.more : 0.f;
+        for (int u = 0; u < kNuItems; ++u) {
+          const bool in = (int)(mag[u] >> 20) >= cls.floor;
+          if (cls.floor) left -= __syncthreads_count(in);
+          c1[u] = in ? c1[u] * cls.more : 0.f;
+          c2[u] = in ? c2[u] * cls.more : 0.f;
+        }
       }
     }
 #pragma unroll
@@ -1086,7 +1114,7 @@ __global__ void __launch_bounds__(kNuThreads, 3)
       if (kBlocks) b = kb - k * (M / bs);
       int* fl = flag[pass & 1];
       if (tid < kNuBlock / 8) flag[~pass & 1][tid] = 0;  // read before this pass
-      if (tid == 0) s_max[~chunk & 1] = 0u, s_log[~chunk & 1] = 0;
+      if (tid == 0) s_max[~chunk & 1] = 0u, s_log[~chunk & 1] = s_pow[~chunk & 1] = 0;
 #pragma unroll
       for (int u = 0; u < kNuItems; ++u) {
         const int idx = kBlocks ? cell[u] - b * bs : cell[u];
