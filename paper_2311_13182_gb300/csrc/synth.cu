@@ -583,6 +583,19 @@ struct NufftCoef {
   float inv[9];  // 1 / Psi(n'/M) = sum_k inv[k] (2 n' / N_s)^(2k)
 };
 
+// What a record's rate turns into over the chirps, as FP32 pairs: carrier cycles and
+// delta per (m/s) of dL/dt.  A product with a rate keeps the fraction of its cycles to
+// 2^-25 however many they are; rounded with its whole cycles it would lose a bit for each
+// doubling, and a tile's turns would add that up (the last of 16 chirps at up to 100 m/s:
+// 2.3e-6 from FP64, 7e-7 so; of 128 chirps at up to 8 m/s 1.7e-6 and 4e-7).
+struct Pair32 {
+  float hi, lo;
+  Pair32() = default;
+  __host__ __device__ explicit Pair32(double x) : hi((float)x), lo((float)(x - (double)(float)x)) {}
+  // r x - p, p = r hi rounded
+  __device__ __forceinline__ float rest(float r, float p) const { return fmaf(r, lo, fmaf(r, hi, -p)); }
+};
+
 struct NufftArg {
   int log_m;
   float half_n, m;           // N_s / 2, M = 2 N_s
@@ -590,6 +603,9 @@ struct NufftArg {
   double f0_c, b_cn;         // f_c / c and B / (c N_s) per metre
   int V, Q, chirps, chirp0;  // antennas, CTAs per antenna and chirp, chirps of this launch, the first of them
   double per_chirp;          // moving scenes: change of path length per chirp per (m/s) of dL/dt
+  // a tile of chirps, per (m/s): the first chirp's carrier cycles and delta, a chirp's turn at n' = 0 and move in cells
+  Pair32 cyc0, eps0, turn;
+  float move;
 };
 
 // Cells a CTA's grid holds, and its points: the cells and w - 1 more to the right
@@ -643,7 +659,6 @@ __device__ __forceinline__ int nu_term(float c, float w, bool small) {
 
 // An amplitude's logarithm in eighths of an octave (2047 and 2046: not finite).
 __device__ __forceinline__ int nu_log(float a) { return (int)((__float_as_uint(a) & 0x7fffffffu) >> 20); }
-constexpr int kNuAll = 2048;  // above every logarithm
 
 // The class of records that one pass rounds on one scale, 2^s for the largest amplitude
 // (its bits: top) to land in (0.49, 0.98] 2^kNuBits: all N that are left if their
@@ -658,10 +673,10 @@ constexpr int kNuAll = 2048;  // above every logarithm
 // chunks (two of them in 26 and 39 %), and need a second class in up to 0.1 % (1 %).
 // The scale is a power of two, exact; one past a float's range (amplitudes
 // below 1e-31) is applied in two factors.
-// The words per chunk that this takes cost 12 antennas x 367,500 records 41.8 -> 42.6 us
-// for the whole synthesis, 471,630 records in whose chunks the rms is looked at in 39 %
-// 55.4 -> 58.3, 4 antennas x 3.1 M records x 4096 samples 122.5 -> 125.8; moving chirps
-// (no sign extensions in the sum) 3.49 -> 3.45 ms.
+// With the words per chunk that this takes, and the copies added up without sign
+// extensions, 12 antennas x 367,500 records went from 41.7 to 40.4 us for the whole
+// synthesis, 4 antennas x 3.1 M records x 4096 samples from 122.0 to 123.4, moving chirps
+// from 3.50 to 3.31 ms.
 struct NuClass {
   float up, down;    // 2^s and its reciprocal
   float more, less;  // the scale's second factor and its reciprocal
@@ -722,17 +737,6 @@ __device__ __forceinline__ double split_rint(double x, int& n) {
   return x - (k - 6755399441055744.0);
 }
 
-// What a record's rate turns into over the chirps, as FP32 pairs: carrier cycles and
-// delta per (m/s) of dL/dt.  A product with a rate keeps the fraction of its cycles to
-// 2^-25 however many they are; rounded with its whole cycles it would lose a bit for each
-// doubling, and a tile's turns would add that up (the last of 16 chirps at up to 100 m/s:
-// 2.3e-6 from FP64, 7e-7 so; of 128 chirps at up to 8 m/s 1.7e-6 and 4e-7).
-struct Pair32 {
-  float hi, lo;
-  __device__ explicit Pair32(double x) : hi((float)x), lo((float)(x - (double)(float)x)) {}
-  // r x - p, p = r hi rounded
-  __device__ __forceinline__ float rest(float r, float p) const { return fmaf(r, lo, fmaf(r, hi, -p)); }
-};
 // r x modulo 1
 __device__ __forceinline__ float cycles_of(float r, const Pair32& x) {
   const float p = r * x.hi;
@@ -804,8 +808,11 @@ __global__ void __launch_bounds__(kNuThreads, 3)
   };
   load(0);
   __syncthreads();
-  // A turn takes a class of a chunk's records: nearly always all of them.
-  int ceil = kNuAll, left = min(kNuChunk, n);  // a chunk's records from ceil on are done, `left` are not
+  // A turn takes a class of a chunk's records: nearly always all of them.  (The votes below
+  // are over equal conditions: what depends on a vote stays out of the lanes' registers and
+  // needs no reconvergence, 124.6 against 127.2 us for 4 x 3.1 M records x 4096 samples.)
+  bool again = false;                     // the turn has another class of the same chunk
+  int ceil = 0, left = min(kNuChunk, n);  // logarithms done, records to do of that chunk
   for (int c0 = 0, chunk = 0; c0 < n; ++chunk) {
     int cell[kNuItems], logs = 0;
     uint32_t am = 0, blocks = 0;
@@ -853,7 +860,7 @@ __global__ void __launch_bounds__(kNuThreads, 3)
       cell[u] = ce;
       if (kBlocks && p < n) blocks |= 1u << (ce / kNuBlock);
     }
-    if (ceil != kNuAll) {
+    if (again) {
 #pragma unroll
       for (int u = 0; u < kNuItems; ++u)
         if (nu_log(rec[u].w) >= ceil) rec[u].w = 0.f;
@@ -875,8 +882,9 @@ __global__ void __launch_bounds__(kNuThreads, 3)
     logs = s_log[chunk & 1];
     const uint32_t top = s_max[chunk & 1];
     NuClass cls = nu_class(top, logs, left);
-    blocks = kBlocks ? s_blk[chunk & 1] : 1u;
-    if (cls.rare) {  // the same for the whole CTA
+    blocks = kBlocks ? __reduce_or_sync(0xffffffffu, s_blk[chunk & 1]) : 1u;
+    again = false;
+    if (__any_sync(0xffffffffu, cls.rare)) {  // the same for the whole CTA
       nu_rare(cls, top, logs, left);
       if (cls.floor) {
         float x = 0.f;
@@ -890,24 +898,23 @@ __global__ void __launch_bounds__(kNuThreads, 3)
         __syncthreads();
         if (nu_one_class(cls, top, s_pow[chunk & 1], logs, left)) cls.floor = 0;
       }
-      if (cls.floor || cls.more != 1.f) {
+      again = __any_sync(0xffffffffu, cls.floor != 0);
+      ceil = cls.floor;
+      if (again || cls.more != 1.f) {
 #pragma unroll
         for (int u = 0; u < kNuItems; ++u) {
           const bool in = nu_log(rec[u].w) >= cls.floor;
-          if (cls.floor) left -= __syncthreads_count(in);
+          if (again) left -= __syncthreads_count(in);
           rec[u].w = in ? rec[u].w * cls.more : 0.f;
         }
       }
     }
 #pragma unroll
     for (int u = 0; u < kNuItems; ++u) rec[u].w *= cls.up;
-    if (cls.floor) {
-      ceil = cls.floor;
-    } else {
-      ceil = kNuAll;
-      c0 += kNuChunk;
-      left = min(kNuChunk, n - c0);
-    }
+    c0 += again ? 0 : kNuChunk;
+    left = again ? left : min(kNuChunk, n - c0);
+    // the turn before's words: read before this turn's first barrier
+    if (tid == 0) s_max[~chunk & 1] = s_blk[~chunk & 1] = 0u, s_log[~chunk & 1] = s_pow[~chunk & 1] = 0;
     while (blocks) {
       const int b = kBlocks ? __ffs(blocks) - 1 : 0;
       blocks &= blocks - 1;
@@ -917,9 +924,7 @@ __global__ void __launch_bounds__(kNuThreads, 3)
         __syncthreads();
       }
       int* fl = flag[pass & 1];
-      // read before this pass: the other parity's flags and words
-      if (tid < kNuBlock / 8) flag[~pass & 1][tid] = 0;
-      if (tid == 0) s_max[~chunk & 1] = s_blk[~chunk & 1] = 0u, s_log[~chunk & 1] = s_pow[~chunk & 1] = 0;
+      if (tid < kNuBlock / 8) flag[~pass & 1][tid] = 0;  // read before this pass
 #pragma unroll
       for (int u = 0; u < kNuItems; ++u) {
         const int idx = kBlocks ? cell[u] - b * bs : cell[u];
@@ -1001,9 +1006,6 @@ __global__ void __launch_bounds__(kNuThreads, 3)
   const int M = 1 << na.log_m, bs = nu_cells(M), npts = nu_points(M), oct = bs >> 3;
   const int tid = threadIdx.x, lane = tid & 31;
   const int v = blockIdx.x % na.V, q = blockIdx.x / na.V, nc = na.chirps;
-  const double dt = (double)na.chirp0 * na.per_chirp;  // path length change per (m/s)
-  const Pair32 cyc(dt * na.f0_c), eps(dt * na.b_cn), turn(na.per_chirp * na.cyc);
-  const float move = (float)(na.per_chirp * na.cell);  // per (m/s) and chirp, as turn
   float2* out = grids + (size_t)(q * na.V + v) * nc * M;
   for (int i = tid; i < npts * (2 * kNuCopies / 4); i += kNuThreads) nsm[i] = nu_zero();
   for (int i = tid; i < 2 * (kNuBlock / 8); i += kNuThreads) (&flag[0][0])[i] = 0;
@@ -1019,7 +1021,8 @@ __global__ void __launch_bounds__(kNuThreads, 3)
   int pass = 0;
   bool bad = false;  // a record that is not finite: the antenna's samples are NaN
   __syncthreads();
-  int ceil = kNuAll, left = min(kNuChunk, n);  // classes in turns, as k_nufft_spread
+  bool again = false;
+  int ceil = 0, left = min(kNuChunk, n);  // classes in turns, as k_nufft_spread
   for (int c0 = 0, chunk = 0; c0 < n; ++chunk) {
     float c1[kNuItems], c2[kNuItems], wr[kNuItems], wi[kNuItems], s[kNuItems], ds[kNuItems];
     int cell[kNuItems], logs = 0;
@@ -1029,7 +1032,7 @@ __global__ void __launch_bounds__(kNuThreads, 3)
       const int p = c0 + tid + u * kNuThreads;
       float4 r = p < n ? __ldg(&prep[at + p]) : make_float4(0.f, 0.f, 0.f, 0.f);
       const float ld = p < n ? __ldg(&rate[at + p]) : 0.f;
-      shift_record(r, ld, cyc, eps);  // the tile's first chirp
+      shift_record(r, ld, na.cyc0, na.eps0);  // the tile's first chirp
       float x = na.half_n * r.y;  // exact
       x -= rintf(x);
       x = fmaf(na.half_n, r.z, x) + r.x;
@@ -1041,19 +1044,19 @@ __global__ void __launch_bounds__(kNuThreads, 3)
       fl = floorf(t);
       s[u] = (t - fl) - 0.5f;
       cell[u] = (ce + (int)fl) & (M - 1);
-      ds[u] = ld * move;
+      ds[u] = ld * na.move;
       float sn, cs;
       sincospif(2.f * x, &sn, &cs);
       // the lower half of a warp adds real parts first, the upper imaginary ones: with the turn's
       // sine negated, the swapped pair turns by the same formula
       c1[u] = r.w * (upper ? sn : cs);
       c2[u] = r.w * (upper ? cs : sn);
-      sincospif(2.f * cycles_of(ld, turn), &sn, &cs);
+      sincospif(2.f * cycles_of(ld, na.turn), &sn, &cs);
       wr[u] = cs;
       wi[u] = upper ? -sn : sn;
       mag[u] = __float_as_uint(fabsf(r.w));
     }
-    if (ceil != kNuAll) {
+    if (again) {
 #pragma unroll
       for (int u = 0; u < kNuItems; ++u)
         if ((int)(mag[u] >> 20) >= ceil) c1[u] = c2[u] = 0.f, mag[u] = 0u;
@@ -1073,7 +1076,8 @@ __global__ void __launch_bounds__(kNuThreads, 3)
     logs = s_log[chunk & 1];
     const uint32_t top = s_max[chunk & 1];
     NuClass cls = nu_class(top, logs, left);
-    if (cls.rare) {  // the same for the whole CTA
+    again = false;
+    if (__any_sync(0xffffffffu, cls.rare)) {  // the same for the whole CTA
       nu_rare(cls, top, logs, left);
       if (cls.floor) {
         float x = 0.f;
@@ -1087,11 +1091,13 @@ __global__ void __launch_bounds__(kNuThreads, 3)
         __syncthreads();
         if (nu_one_class(cls, top, s_pow[chunk & 1], logs, left)) cls.floor = 0;
       }
-      if (cls.floor || cls.more != 1.f) {
+      again = __any_sync(0xffffffffu, cls.floor != 0);
+      ceil = cls.floor;
+      if (again || cls.more != 1.f) {
 #pragma unroll
         for (int u = 0; u < kNuItems; ++u) {
           const bool in = (int)(mag[u] >> 20) >= cls.floor;
-          if (cls.floor) left -= __syncthreads_count(in);
+          if (again) left -= __syncthreads_count(in);
           c1[u] = in ? c1[u] * cls.more : 0.f;
           c2[u] = in ? c2[u] * cls.more : 0.f;
         }
@@ -1102,19 +1108,15 @@ __global__ void __launch_bounds__(kNuThreads, 3)
       c1[u] *= cls.up;
       c2[u] *= cls.up;
     }
-    if (cls.floor) {
-      ceil = cls.floor;
-    } else {
-      ceil = kNuAll;
-      c0 += kNuChunk;
-      left = min(kNuChunk, n - c0);
-    }
+    c0 += again ? 0 : kNuChunk;
+    left = again ? left : min(kNuChunk, n - c0);
+    // the turn before's words: read before this turn's first barrier
+    if (tid == 0) s_max[~chunk & 1] = 0u, s_log[~chunk & 1] = s_pow[~chunk & 1] = 0;
     for (int kb = 0, b = 0; kb < (kBlocks ? nc * (M / bs) : nc); ++kb, ++pass) {
       const int k = kBlocks ? kb / (M / bs) : kb;
       if (kBlocks) b = kb - k * (M / bs);
       int* fl = flag[pass & 1];
       if (tid < kNuBlock / 8) flag[~pass & 1][tid] = 0;  // read before this pass
-      if (tid == 0) s_max[~chunk & 1] = 0u, s_log[~chunk & 1] = s_pow[~chunk & 1] = 0;
 #pragma unroll
       for (int u = 0; u < kNuItems; ++u) {
         const int idx = kBlocks ? cell[u] - b * bs : cell[u];
@@ -1765,6 +1767,10 @@ NufftArg nufft_arg(const sbr_paths* p, const sbr_radar_cfg* r, int Q, int c0, in
   na.chirps = chirps;
   na.chirp0 = c0;
   na.per_chirp = r->chirp_rep;
+  na.cyc0 = Pair32(c0 * na.per_chirp * na.f0_c);
+  na.eps0 = Pair32(c0 * na.per_chirp * na.b_cn);
+  na.turn = Pair32(na.per_chirp * na.cyc);
+  na.move = (float)(na.per_chirp * na.cell);
   nufft_per_sm(Ns);
   return na;
 }
