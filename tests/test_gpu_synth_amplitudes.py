@@ -6,6 +6,8 @@ kernel's squares 1.9 in sum) is then 4e-7 of the class's samples, whatever the o
 with the other contributions (1.7e-7, tests/test_gpu_synth_records.py) 4.4e-7.  The tolerance is
 about twice that, and twice again for chirps whose shifts are rounded once more."""
 
+import math
+
 import numpy as np
 import pytest
 import torch
@@ -90,3 +92,32 @@ def test_moving(sbr, ns, nc, P, kind):
     ref = torch.stack([reference(phi + rate * (c * per * radar.f0), delta + rate * (c * per * radar.bandwidth / ns), A, ns)
                        for c in range(nc)], 1)
     assert rel(cube, ref) <= 2 * TOL
+
+
+@pytest.mark.parametrize("what", ["inf", "nan", "phase", "rate"])
+@pytest.mark.parametrize("ns,nc,P,mode", [(256, 1, 20000, "split"), (4096, 1, 5000, "split"), (256, 1, 3000, "fp64"),
+                                          (256, 4, 17000, "moving"), (512, 4, 17000, "moving"), (128, 2, 3000, "moving")])
+def test_not_finite(sbr, ns, nc, P, mode, what):
+    """A record that is not finite makes its antenna's samples NaN, and no others, among amplitudes
+    that need several classes."""
+    radar = radar_single_tx(ns, nc)
+    rng = np.random.default_rng(P)
+    A = amplitudes(rng, "decades", 4, P)
+    rate = rng.uniform(-8.0, 8.0, (4, P)).astype(np.float32)
+    delta, phi = rng.uniform(-0.5, 0.5, (4, P)), rng.uniform(-0.5, 0.5, (4, P))
+    L = rng.uniform(0.1, 0.999, (4, P)) * ns * C_LIGHT / radar.bandwidth
+    if what == "rate" and mode != "moving":
+        pytest.skip("no rates")
+    {"inf": A, "nan": A, "phase": L if mode == "fp64" else phi, "rate": rate}[what][2, 1030] = \
+        np.nan if what == "nan" else np.inf
+    if mode == "fp64":
+        paths = bind64(sbr, radar, P + 3, np.where(np.isfinite(L), L, 1.0), A)[0]
+        if what == "phase":
+            paths.phase_ofs()[:P].zero_()
+            raw = paths.mem[paths.s.path_len - paths.mem.data_ptr():][:8 * 4 * (P + 3)].view(torch.float32)
+            raw.view(4, P + 3, 2)[2, 1030, 0] = math.inf
+        cube = sbr.synthesize(paths, radar, sbr.PHASE_FP64)
+    else:
+        paths = bind(sbr, radar, P + 3, delta, phi, A, rate)[0]
+        cube = sbr.synthesize(paths, radar, sbr.PHASE_SPLIT | (sbr.SYNTH_MOVING if mode == "moving" else 0))
+    assert torch.isnan(cube[2]).all() and torch.isfinite(cube[[0, 1, 3]]).all()
