@@ -556,8 +556,8 @@ __global__ void __launch_bounds__(256) k_synth_bwd(const float4* __restrict__ pr
 //
 // A CTA has a barrier for a chunk's largest amplitude and one before its sums are added
 // up; the next chunk's records are in flight meanwhile, and its preparation needs none.
-// Bound by issue slots (211 instructions per 32 records) and the conversion unit,
-// three CTAs per SM: 12 antennas x 367,500 records x 256 samples 36 us (109 us when
+// Bound by issue slots (209 instructions per 32 records) and the conversion unit,
+// three CTAs per SM: 12 antennas x 367,500 records x 256 samples 35 us (109 us when
 // each warp kept runs of equal cells in registers, eight lanes to a record, and
 // flushed them to its own FP32 grid, one group at a time; 93 us with the chunk sorted
 // by cell first), 71 MB of records at 2 TB/s.  A block of 512 cells, so that long
@@ -1874,9 +1874,18 @@ void launch_fwd(sbr_phase_mode mode, const sbr_paths* p, const sbr_radar_cfg* r,
                  p->path_cap, p->count, V, w.Q, Ns, r->f0, r->bandwidth / Ns, w.partial);
   } else {
     const double mu = r->bandwidth / r->chirp_time, dt = r->chirp_time / Ns;
+    const float2* plen = reinterpret_cast<const float2*>(p->path_len);
+    const float f0 = (float)r->f0, fmu = (float)mu, fdt = (float)dt;
     ::sbr::note_launch();
-    launch_after(k_synth_naive<M>, grid, T, 0, st, prep, reinterpret_cast<const float2*>(p->path_len), p->phase_ofs,
-                 p->path_cap, p->count, V, w.Q, Ns, (float)r->f0, (float)mu, (float)dt, w.partial);
+    // Several of its small CTAs to an SM: placed while the kernel before still holds some SMs,
+    // they crowd the others for the whole launch (4 antennas x 800,000 records x 1024 samples
+    // 2.23 ms launched after it, 2.94 dispatched early; 12 x 150,000 x 256 0.89 and 1.14).
+    if (grid > sm_count())
+      k_synth_naive<M><<<grid, T, 0, st>>>(prep, plen, p->phase_ofs, p->path_cap, p->count, V, w.Q, Ns, f0, fmu, fdt,
+                                           w.partial);
+    else
+      launch_after(k_synth_naive<M>, grid, T, 0, st, prep, plen, p->phase_ofs, p->path_cap, p->count, V, w.Q, Ns, f0,
+                   fmu, fdt, w.partial);
   }
 }
 }  // namespace
