@@ -135,6 +135,7 @@ struct FixScatter {
   unsigned long long* acc;  // zeroed before pass 2
   unsigned int* max_bits;   // zeroed before pass 1
   int log2n;                // ceil(log2(a bound on the number of contributions))
+  int alone = 4;            // lanes of a warp with one index that add each for itself (fix_add_peers)
 };
 
 __host__ inline int ceil_log2(int64_t n) {
@@ -185,12 +186,13 @@ __device__ inline long long peer_sum(unsigned peers, long long x) {
 // one: rays of a warp mostly hit the same few triangles, and a large triangle's
 // corners take contributions from most of the launch, whose atomics would queue at one
 // address.  Integer sums: the result is that of one atomic per lane.  Each group of
-// peers runs its warp sums on its own, so small groups go straight to the atomics.
-constexpr int kPeersDirect = 4;
+// peers runs its warp sums on its own, so groups of up to fs.alone lanes go straight to
+// the atomics.
 template <int n>
-__device__ inline void fix_add_peers(unsigned long long* acc, int i, const float* x, int E) {
+__device__ inline void fix_add_peers(const FixScatter& fs, int i, const float* x, int E) {
+  unsigned long long* acc = fs.acc;
   const unsigned peers = __match_any_sync(__activemask(), i);
-  if (__popc(peers) <= kPeersDirect) {
+  if (__popc(peers) <= fs.alone) {
 #pragma unroll
     for (int c = 0; c < n; ++c) fix_add(&acc[(size_t)n * i + c], x[c], E);
     return;

@@ -32,8 +32,13 @@
 // What bounds it where many rays share a triangle (a ground plane's two) is the queue
 // of 64-bit atomics at its corners, so the lanes of a warp that add to one vertex add
 // as one (fix_add_peers), at the same bounce: 523,000 rays on 20,002 triangles,
-// integer pass 1214 -> 84 us; 4,096 rays on 5,120 triangles, where few lanes share a
-// vertex, 11.5 -> 11.9 us (38 us if groups of up to four were summed too).
+// integer pass 1214 -> 84 us.  Few rays make no queue worth the warp sums of a middling
+// group, whose latency is then the kernel's: up to 8,192 rays groups of up to 12 lanes add
+// lane by lane, up to 40,000 rays groups of up to 8, above of up to 4.  The whole call with
+// groups of 4 / 8 / 12, against an atomic per lane, in us: 1,089 rays on 320 triangles 18.2
+// / 14.2 / 13.5, 15.0; 8,100 on 5,120 19.2 / 14.9 / 14.8, 16.8; 8,100 on 20,002, two
+// bounces, 24.6 / 24.0 / 23.0, 40.4; 16,384 on 5,120 20.9 / 17.2 / 16.5, 17.8; 32,761 on
+// 5,002, two bounces, 31.5 / 27.0 / 28.5, 103; 65,536 on 320 22.7 / 27.5 / 37.0, 108.
 #include <math.h>
 
 #include "scene.cuh"
@@ -68,7 +73,7 @@ __device__ inline void scatter(const FixScatter& fs, int E, float& lmax, int vi,
     lmax = fmaxf(lmax, fmaxf(fabsf(d.x), fmaxf(fabsf(d.y), fabsf(d.z))));
   } else {
     const float x[3] = {d.x, d.y, d.z};
-    fix_add_peers<3>(fs.acc, vi, x, E);
+    fix_add_peers<3>(fs, vi, x, E);
   }
 }
 
@@ -79,7 +84,7 @@ __device__ inline void scatter_eps(const FixScatter& fe, int Ee, float& emax, in
     emax = fmaxf(emax, fmaxf(fabsf(dre), fabsf(dim)));
   } else {
     const float x[2] = {dre, dim};
-    fix_add_peers<2>(fe.acc, m, x, Ee);
+    fix_add_peers<2>(fe, m, x, Ee);
   }
 }
 
@@ -381,6 +386,8 @@ extern "C" sbr_status sbr_trace_bwd(const sbr_scene* scene, const float* d_verts
   bwd_ws_layout(d_ws, scene->nv, &w);
   w.fs.log2n = ceil_log2(3 * (int64_t)R * (paths->max_bounces + (reparam ? 1 : 0)));  // contributions per axis, at most
   w.fe.log2n = ceil_log2((int64_t)R * paths->max_bounces * paths->max_bounces);  // per material, at most
+  w.fs.alone = R <= 8192 ? 12 : R <= 40000 ? 8 : 4;  // see the head of the file
+  w.fe.alone = 4;                                    // few materials: large groups
   const MatArg mat = mat_arg(scene);
   SBR_CUDA(cudaMemsetAsync(d_ws, 0, sbr_trace_bwd_ws_bytes(scene->nv), st));
   const float4* hp = reinterpret_cast<const float4*>(paths->hit_pos);
