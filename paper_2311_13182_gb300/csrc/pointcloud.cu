@@ -978,7 +978,15 @@ void launch_angle_power(const float2* X, const Steer& xl, int V, int C, int Ns, 
   const size_t sm = sizeof(float2) * ((size_t)R * V + (size_t)V * kKT);
   dim3 grid(Ns / kKT, groups);
   ::sbr::note_launch();
-  launch_after(k_angle_power<APT>, grid, 256, sm, st, X, xl, V, C, Ns, (C + groups - 1) / groups, part);
+  const int dpg = (C + groups - 1) / groups;
+  // Its few CTAs, placed while the transforms still hold most SMs, come two or three to an
+  // SM, which is felt where a CTA is long: 32 antennas x 16 chirps x 256 samples x 64 angles,
+  // power map 32.4 us dispatched early, 21.8 after them (20 antennas 21.5 and 16.7; up to 16
+  // the early dispatch is the faster one, 4 antennas x 256 angles 14.6 and 17.2).
+  if (V > 16)
+    k_angle_power<APT><<<grid, 256, sm, st>>>(X, xl, V, C, Ns, dpg, part);
+  else
+    launch_after(k_angle_power<APT>, grid, 256, sm, st, X, xl, V, C, Ns, dpg, part);
 }
 
 template <int APT>
