@@ -432,7 +432,9 @@ __global__ void __launch_bounds__(256) k_synth_naive(const float4* __restrict__ 
 constexpr int kRedChirps = 16;
 __global__ void k_reduce(const float2* __restrict__ partial, int V, int Q, int Ns, int C,
                          float2* __restrict__ cube) {
-  next_may_start();
+  // with many chirps to write it is a long kernel: 12 antennas x 128 chirps x 512 samples,
+  // trace and synthesis of 1,089 rays 35.4 us with the next trace placed early, 29.1 without
+  if (C <= kRedChirps) next_may_start();
   after_previous();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= V * Ns) return;
