@@ -998,7 +998,10 @@ void launch_angle_bwd(const float2* X, const Steer& xl, const float* dpw, const 
   dim3 grid(Ns / kKT, C);
   if (sm > 48 * 1024) cudaFuncSetAttribute(k_angle_bwd<APT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   ::sbr::note_launch();
-  launch_after(k_angle_bwd<APT>, grid, 256, sm, st, X, xl, dpw, fs, V, C, Ns, dX);
+  // Not dispatched early: its long CTAs would crowd the SMs that the kernels before have left.
+  // Power map and image loss: 12 antennas x 16 chirps x 256 samples 36.6 us early, 30.5 after
+  // them; 20 antennas 57.2 and 35.9; 32 antennas 82.2 and 46.2; 4 x 32 samples 9.1 and 9.2.
+  k_angle_bwd<APT><<<grid, 256, sm, st>>>(X, xl, dpw, fs, V, C, Ns, dX);
 }
 
 // Eight points per thread: as many short rows per CTA as 256 threads hold (32 to 256
