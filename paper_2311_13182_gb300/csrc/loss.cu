@@ -41,8 +41,8 @@ __device__ inline float block_sum(float v, float* red) {
 __global__ void __launch_bounds__(1024) k_chamfer(const float4* __restrict__ P, const int32_t* __restrict__ d_n,
                                                   int cap, const float4* __restrict__ Q, int m,
                                                   float* __restrict__ loss, float4* __restrict__ gP) {
-  next_may_start();
   after_previous();
+  next_may_start();
   __shared__ int nn_p[kChamferMax], nn_q[kChamferMax];
   __shared__ float d2_p[kChamferMax], d2_q[kChamferMax];
   __shared__ float red[32];
@@ -123,8 +123,8 @@ __global__ void __launch_bounds__(kLapThreads) k_lap_delta(const float* __restri
                                                            const int32_t* __restrict__ off,
                                                            const int32_t* __restrict__ adj, float* __restrict__ delta,
                                                            float* __restrict__ partial) {
-  next_may_start();
   after_previous();
+  next_may_start();
   __shared__ float red[32];
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   float sq = 0.f;
@@ -166,8 +166,8 @@ __global__ void __launch_bounds__(kLapThreads) k_lap_grad(const float* __restric
                                                           const int32_t* __restrict__ adj, float scale,
                                                           float* __restrict__ g, const float* __restrict__ partial,
                                                           int nb, float lscale, float* __restrict__ loss) {
-  next_may_start();
   after_previous();
+  next_may_start();
   __shared__ float red[32];
   if (blockIdx.x == 0) {
     float s = 0.f;
@@ -206,8 +206,8 @@ __global__ void __launch_bounds__(kLapThreads) k_lap_grad(const float* __restric
 __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
                        float* __restrict__ v, int64_t n, const int32_t* __restrict__ step, float lr, float b1,
                        float b2, float eps) {
-  next_may_start();
   after_previous();
+  next_may_start();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const float t = (float)(*step + 1);
@@ -221,8 +221,8 @@ __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float
 }
 
 __global__ void k_step_inc(int32_t* step) {
-  next_may_start();
   after_previous();
+  next_may_start();
   *step += 1;
 }
 

@@ -32,14 +32,16 @@ using namespace fft;
 
 // FFT along the contiguous last axis: 2^logb rows of n points per CTA, eight points
 // per thread.  clear: words the first CTA zeroes for later kernels of the call, or NULL.
+constexpr int kFewCtas = 4;  // up to here the next kernel may come before the wait: there is nothing to crowd
 __global__ void k_fft_rows(const float2* __restrict__ in, float2* __restrict__ out, int rows, int logn, int logb,
                            float sign, unsigned long long* clear) {
-  next_may_start();
+  if (gridDim.x <= kFewCtas) next_may_start();  // one chirp of 256 samples to points 20.1 -> 19.2 us
   extern __shared__ float2 s[];  // [2^logb] rows of slots(n) points, slots(n / 2) twiddles
   const int n = 1 << logn, ld = slots(n);
   float2* tw = s + (ld << logb);
   fill_twiddles(tw, n, sign, blockDim.x, threadIdx.x);
   after_previous();
+  if (gridDim.x > kFewCtas) next_may_start();
   if (clear && blockIdx.x == 0 && threadIdx.x < 2) clear[threadIdx.x] = 0ull;
   const size_t at = (size_t)blockIdx.x << (logn + logb);
   const int cnt = min(1 << logb, rows - ((int)blockIdx.x << logb)) << logn;  // points of this CTA's rows
@@ -65,7 +67,6 @@ constexpr int kLogColTile = 4, kColTile = 1 << kLogColTile;
 // Columns sit an odd number of points apart in shared memory, so the 16 columns of
 // one chirp fall in different banks.
 __global__ void k_fft_cols(float2* __restrict__ x, int C, int logc, int Ns, float sign) {
-  next_may_start();
   extern __shared__ float2 s[];  // [kColTile][slots(C) | 1] points, slots(C / 2) twiddles
   const int ld = slots(C) | 1;
   float2* tw = s + kColTile * ld;
@@ -74,6 +75,7 @@ __global__ void k_fft_cols(float2* __restrict__ x, int C, int logc, int Ns, floa
   float2* base = x + (size_t)v * C * Ns + k0;
   fill_twiddles(tw, C, sign, blockDim.x, threadIdx.x);
   after_previous();
+  next_may_start();
   constexpr int kAhead = 8;  // loads in flight per thread
   for (int i0 = threadIdx.x; i0 < C * kColTile; i0 += kAhead * blockDim.x) {
     float2 y[kAhead];
@@ -132,8 +134,8 @@ template <int APT>
 __global__ void __launch_bounds__(256) k_angle_power(const float2* __restrict__ X,
                                                      const Steer xl, int V, int C,
                                                      int Ns, int dpg, float* __restrict__ part) {
-  next_may_start();
   after_previous();
+  next_may_start();
   extern __shared__ float2 sm[];
   constexpr int R = 8 * APT;
   float2* sw = sm;                // [R][V]
@@ -231,7 +233,6 @@ template <int NR>
 __global__ void __launch_bounds__(kTcThreads) k_angle_tc(const float2* __restrict__ X, const Steer xl, int R,
                                                          int V, int C, int Ns, float* __restrict__ part,
                                                          int* __restrict__ err) {
-  next_may_start();
   constexpr int kN = 2 * NR;                         // MMA N
   constexpr int kCols = tc_cols<NR>();
   constexpr uint32_t kTileW = (uint32_t)kN * kTcK * 4;  // steering operand bytes (hi or lo)
@@ -263,6 +264,7 @@ __global__ void __launch_bounds__(kTcThreads) k_angle_tc(const float2* __restric
     tc_put4(sw_hi, sw_lo, tc_off(2 * a + 1, 4 * j), make_float4(s0, c0, s1, c1));
   }
   after_previous();
+  next_may_start();
   // A: thread t takes range bin k0 + t; per Doppler bin and antenna pair one 16-byte chunk
   // (Re, Im of antenna 2j, Re, Im of antenna 2j + 1); antennas >= V and bins >= nd are zero.
   float2 xv[kTcDG][kTcK / 2];
@@ -340,8 +342,8 @@ __global__ void __launch_bounds__(kTcThreads) k_angle_tc(const float2* __restric
 // amax_key must be 0 on entry.
 __global__ void k_power_reduce(const float* __restrict__ part, int groups, int cells, float* __restrict__ Pw,
                                unsigned long long* __restrict__ amax_key) {
-  next_may_start();
   after_previous();
+  next_may_start();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   unsigned long long key = 0ull;
   if (i < cells) {
@@ -446,8 +448,8 @@ __global__ void __launch_bounds__(kDetThreads) k_detect(const float* __restrict_
                                                         int32_t* __restrict__ amax, int32_t* __restrict__ flag,
                                                         uint32_t* __restrict__ key, int32_t* __restrict__ cell,
                                                         int32_t* __restrict__ cnt) {
-  next_may_start();
   after_previous();
+  next_may_start();
   __shared__ int wn[kDetThreads / 32];
   const int i = blockIdx.x * kDetThreads + threadIdx.x;  // cells come in multiples of 256
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -481,8 +483,8 @@ __global__ void __launch_bounds__(kDetThreads) k_detect(const float* __restrict_
 __global__ void k_compact(const int32_t* __restrict__ flag, const int32_t* __restrict__ off,
                           const uint32_t* __restrict__ key, int cells, uint32_t* __restrict__ ko,
                           int32_t* __restrict__ vo) {
-  next_may_start();
   after_previous();
+  next_may_start();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= cells || !flag[i]) return;
   ko[off[i]] = key[i];
@@ -563,8 +565,8 @@ __global__ void k_points(const float* __restrict__ Pw, PointArg pa, const int32_
                          const int32_t* __restrict__ cand, const int32_t* __restrict__ n_cand,
                          float4* __restrict__ pts, int32_t* __restrict__ cell_out,
                          int32_t* __restrict__ n_out) {
-  next_may_start();
   after_previous();
+  next_may_start();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int n = min(*n_cand, pa.k_max);
   if (i == 0) *n_out = n;
@@ -641,8 +643,8 @@ __global__ void __launch_bounds__(kSelThreads) k_select(const float* __restrict_
                                                         uint32_t* k0, int32_t* v0, uint32_t* k1, int32_t* v1,
                                                         float4* __restrict__ pts, int32_t* __restrict__ cell_out,
                                                         int32_t* __restrict__ n_out) {
-  next_may_start();
   after_previous();
+  next_may_start();
   extern __shared__ __align__(16) uint32_t sel_sm[];  // cta::kSortSmemWords
   __shared__ uint32_t wt[32];
   const CfarArg& c = pa.c;
@@ -793,8 +795,8 @@ template <int kPass>
 __global__ void k_points_bwd(const float* __restrict__ Pw, PointArg pa, const int32_t* __restrict__ amax,
                              const int32_t* __restrict__ cells, const int32_t* __restrict__ n_pts,
                              const float4* __restrict__ gpts, FixScatter fs) {
-  next_may_start();
   after_previous();
+  next_may_start();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   float lmax = 0.f;
   const DpwScatter<kPass> sc{fs, kPass == 0 ? 0 : fix_exp(*fs.max_bits, fs.log2n), lmax};
@@ -810,8 +812,8 @@ __global__ void __launch_bounds__(256) k_angle_bwd(const float2* __restrict__ X,
                                                    const Steer xl,
                                                    const float* __restrict__ dPw, FixScatter fs, int V, int C,
                                                    int Ns, float2* __restrict__ dX) {
-  next_may_start();
   after_previous();
+  next_may_start();
   extern __shared__ float2 sm[];
   constexpr int R = 8 * APT;
   float2* sw = sm;               // [R][V]
@@ -1242,8 +1244,8 @@ constexpr int kMseThreads = 1024;
 __global__ void __launch_bounds__(kMseThreads) k_image_mse(const float* __restrict__ Pw, const float* __restrict__ T,
                                                            int cells, float* __restrict__ loss,
                                                            float* __restrict__ dpw) {
-  next_may_start();
   after_previous();
+  next_may_start();
   __shared__ float red[kMseThreads / 32];
   const float inv_n = 1.f / (float)cells;
   float s = 0.f;

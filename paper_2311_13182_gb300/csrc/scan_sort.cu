@@ -66,8 +66,8 @@ __device__ inline void load_items(const int32_t* in, int64_t base, int64_t n, in
 
 __global__ void k_tile_sums(const int32_t* __restrict__ in, int64_t cap, const int32_t* d_n,
                             int32_t* __restrict__ sums) {
-  next_may_start();
   after_previous();
+  next_may_start();
   __shared__ uint32_t wt[32];
   const int64_t n = clamp_n(cap, d_n);
   const int64_t base = (int64_t)blockIdx.x * kTile + (int64_t)threadIdx.x * kItems;
@@ -83,8 +83,8 @@ __global__ void k_tile_sums(const int32_t* __restrict__ in, int64_t cap, const i
 
 // In-place exclusive scan of m values with one CTA (m up to a few million).
 __global__ void k_scan_single(int32_t* __restrict__ a, int64_t m) {
-  next_may_start();
   after_previous();
+  next_may_start();
   __shared__ uint32_t wt[32];
   uint32_t carry = 0;
   for (int64_t base = 0; base < m; base += blockDim.x) {
@@ -99,8 +99,8 @@ __global__ void k_scan_single(int32_t* __restrict__ a, int64_t m) {
 
 __global__ void k_tile_scan(const int32_t* __restrict__ in, int32_t* __restrict__ out, int64_t cap,
                             const int32_t* d_n, const int32_t* __restrict__ sums) {
-  next_may_start();
   after_previous();
+  next_may_start();
   __shared__ uint32_t wt[32];
   const int64_t n = clamp_n(cap, d_n);
   if (n == 0) {
@@ -152,10 +152,10 @@ __device__ inline int64_t tile_item(int i) {
 __global__ void __launch_bounds__(kThreads) k_digit_hist(const uint32_t* __restrict__ keys, int64_t cap,
                                                          const int32_t* d_n, int shift, uint32_t mask,
                                                          int32_t* __restrict__ hist, int ntiles) {
-  next_may_start();
   __shared__ uint32_t cnt[kDigits];
   cnt[threadIdx.x] = 0;
   after_previous();
+  next_may_start();
   __syncthreads();
   const int64_t n = clamp_n(cap, d_n);
 #pragma unroll
@@ -173,8 +173,8 @@ __global__ void __launch_bounds__(kThreads) k_digit_hist(const uint32_t* __restr
 // CTA d: exclusive scan of digit d's counts over the tiles, in place; their sum to total[d].
 __global__ void __launch_bounds__(kThreads) k_digit_scan(int32_t* __restrict__ hist, int ntiles,
                                                          int32_t* __restrict__ total) {
-  next_may_start();
   after_previous();
+  next_may_start();
   __shared__ uint32_t wt[32];
   int32_t* row = hist + (size_t)blockIdx.x * ntiles;
   uint32_t carry = 0;
@@ -198,12 +198,12 @@ __global__ void __launch_bounds__(kThreads) k_digit_scatter(const uint32_t* __re
                                                             int64_t cap, const int32_t* d_n, int shift, uint32_t mask,
                                                             const int32_t* __restrict__ hist,
                                                             const int32_t* __restrict__ total, int ntiles) {
-  next_may_start();
   __shared__ uint32_t wt[32], cnt[kThreads / 32][kDigits], local[kDigits], skey[kTile];
   __shared__ int32_t sval[kTile], first[kDigits];  // first[d]: output position of the tile's slot 0, for digit d
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int i = threadIdx.x; i < kThreads / 32 * kDigits; i += kThreads) (&cnt[0][0])[i] = 0;
   after_previous();
+  next_may_start();
   const int64_t n = clamp_n(cap, d_n);
   uint32_t key[kItems], rank[kItems];
   int32_t val[kItems];
@@ -270,8 +270,8 @@ using cta::kSortSmemBytes;
 __global__ void __launch_bounds__(kSmallThreads) k_scan_small(const int32_t* __restrict__ in,
                                                               int32_t* __restrict__ out, int64_t cap,
                                                               const int32_t* d_n) {
-  next_may_start();
   after_previous();
+  next_may_start();
   __shared__ uint32_t wt[32];
   const int64_t n = clamp_n(cap, d_n);
   uint32_t carry = 0;
@@ -299,8 +299,8 @@ __global__ void __launch_bounds__(kSmallThreads) k_scan_small(const int32_t* __r
 __global__ void __launch_bounds__(kSmallThreads) k_sort_small(uint32_t* k0, int32_t* v0, uint32_t* k1,
                                                               int32_t* v1, int64_t cap, const int32_t* d_n,
                                                               int bits, const uint32_t* __restrict__ d_hist) {
-  next_may_start();
   after_previous();
+  next_may_start();
   extern __shared__ __align__(16) uint32_t sm[];  // kSortSmemWords
   cta::sort_pairs(k0, v0, k1, v1, clamp_n(cap, d_n), bits, d_hist, sm);
 }

@@ -27,8 +27,8 @@ __device__ inline int32_t ord(float f) {
 __device__ inline float unord(int32_t i) { return __int_as_float(i >= 0 ? i : i ^ 0x7fffffff); }
 
 __global__ void k_init_bounds(int32_t* b, int32_t* err, uint32_t* hist) {
-  next_may_start();
   after_previous();
+  next_may_start();
   if (threadIdx.x < 3) b[threadIdx.x] = 0x7fffffff;           // min x, y, z
   else if (threadIdx.x < 6) b[threadIdx.x] = (int32_t)0x80000000;  // max x, y, z
   else if (threadIdx.x == 6) b[6] = 0;                        // max |coord| (ordered, >= 0)
@@ -50,8 +50,8 @@ __device__ inline float3 vload(const float* v, int i) { return f3(v[3 * i], v[3 
 
 __global__ void __launch_bounds__(256) k_bounds(const float* __restrict__ verts, int nv, const int32_t* __restrict__ faces,
                          int nt, int32_t* bounds, int32_t* err) {
-  next_may_start();
   after_previous();
+  next_may_start();
   int f = blockIdx.x * blockDim.x + threadIdx.x;
   float3 lo = f3(INFINITY, INFINITY, INFINITY), hi = f3(-INFINITY, -INFINITY, -INFINITY);
   float mabs = 0.f;
@@ -129,8 +129,8 @@ __global__ void __launch_bounds__(256) k_morton(const float* __restrict__ verts,
                                                 const int32_t* __restrict__ faces, int nt,
                                                 const int32_t* __restrict__ bounds, uint32_t* keys,
                                                 int32_t* vals, uint32_t* hist, int32_t* err) {
-  next_may_start();
   after_previous();
+  next_may_start();
   __shared__ uint32_t h[4 * 256];
   for (int i = threadIdx.x; i < 4 * 256; i += blockDim.x) h[i] = 0u;
   __syncthreads();
@@ -161,8 +161,8 @@ __global__ void __launch_bounds__(256) k_morton(const float* __restrict__ verts,
 __global__ void k_pack(const float* __restrict__ verts, int nv, const int32_t* __restrict__ faces,
                        int nt, const int32_t* __restrict__ order, float4* __restrict__ tris,
                        int32_t* err) {
-  next_may_start();
   after_previous();
+  next_may_start();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= nt) return;
   int f = order[i];
@@ -212,8 +212,8 @@ __device__ inline void karras_node(const KeyAt& key, int n, int i, int* left, in
 }
 
 __global__ void k_karras(const uint32_t* __restrict__ keys, int n, Node* nodes, int32_t* parent) {
-  next_may_start();
   after_previous();
+  next_may_start();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n - 1) return;
   int left, right, lo, hi;
@@ -260,11 +260,11 @@ constexpr int kRefitTile = 512;
 __global__ void __launch_bounds__(kRefitTile) k_refit(const float4* __restrict__ tris, int n, Node* nodes,
                                                       const int32_t* __restrict__ parent, uint32_t* visits,
                                                       const int32_t* __restrict__ bounds) {
-  next_may_start();
   __shared__ uint32_t seen[kRefitTile];
   __shared__ float side_box[2][6][kRefitTile];  // the children's boxes
   seen[threadIdx.x] = 0u;
   after_previous();
+  next_may_start();
   __syncthreads();
   const int base = blockIdx.x * kRefitTile, l = base + threadIdx.x;
   if (l >= n) return;
@@ -969,8 +969,8 @@ __device__ inline void node_children(const Node* nodes, int i, Box& l, Box& r, i
 // Entry i of the 4-wide tree: binary node i's grandchildren, then greedy
 // expansion of the largest internal slot while fewer than four slots are used.
 __global__ void k_collapse4(const Node* __restrict__ nodes, int n, Node4* __restrict__ out) {
-  next_may_start();
   after_previous();
+  next_may_start();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n - 1) return;
   Box bx[4];

@@ -432,10 +432,8 @@ __global__ void __launch_bounds__(256) k_synth_naive(const float4* __restrict__ 
 constexpr int kRedChirps = 16;
 __global__ void k_reduce(const float2* __restrict__ partial, int V, int Q, int Ns, int C,
                          float2* __restrict__ cube) {
-  // with many chirps to write it is a long kernel: 12 antennas x 128 chirps x 512 samples,
-  // trace and synthesis of 1,089 rays 35.4 us with the next trace placed early, 29.1 without
-  if (C <= kRedChirps) next_may_start();
   after_previous();
+  if (C <= kRedChirps) next_may_start();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= V * Ns) return;
   const int v = i / Ns, n = i - v * Ns;
@@ -457,8 +455,8 @@ inline dim3 reduce_grid(int V, int Ns, int C) {
 
 __global__ void k_chirp_sum(const float2* __restrict__ g, int V, int C, int Ns,
                             float2* __restrict__ gs) {
-  next_may_start();
   after_previous();
+  next_may_start();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= V * Ns) return;
   const int v = i / Ns, n = i - v * Ns;
@@ -480,8 +478,8 @@ __global__ void __launch_bounds__(256) k_synth_bwd(const float4* __restrict__ pr
                                                    const float2* __restrict__ gs, float inv_lambda,
                                                    float b_over_cns, float* __restrict__ glen,
                                                    float* __restrict__ gamp, float* __restrict__ gphase) {
-  next_may_start();
   after_previous();
+  next_may_start();
   extern __shared__ float2 sg[];
   const int v = blockIdx.y;
   for (int n = threadIdx.x; n < Ns; n += blockDim.x) sg[n] = gs[(size_t)v * Ns + n];
@@ -1186,8 +1184,8 @@ __global__ void __launch_bounds__(kNuFinThreads) k_nufft_finish(const float2* __
                                                                 float2* __restrict__ bsum,
                                                                 unsigned int* __restrict__ cnt,
                                                                 float2* __restrict__ cube, int C, bool moving) {
-  next_may_start();
   after_previous();
+  next_may_start();
   extern __shared__ float2 sg[];  // slots(M) grid, slots(M / 2) twiddles, [kNuFinThreads] per-thread sums
   __shared__ int s_last;
   const int log_m = na.log_m, M = 1 << log_m, slice = M < kNuFinSlice ? M : kNuFinSlice, S = M / slice;
@@ -1268,7 +1266,6 @@ constexpr int kNuClThreads = 512;
 __global__ void __cluster_dims__(kNuRanks, 1, 1) __launch_bounds__(kNuClThreads)
     k_nufft_finish_cluster(const float2* __restrict__ grids, const NufftArg na, const __grid_constant__ NufftCoef co,
                            float2* __restrict__ cube, int C, bool moving) {
-  next_may_start();
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
   extern __shared__ float2 sg[];  // slots(M) grid, slots(M / 2) twiddles, [kNuClThreads] per-thread sums, [M / 8] this eighth
@@ -1284,6 +1281,7 @@ __global__ void __cluster_dims__(kNuRanks, 1, 1) __launch_bounds__(kNuClThreads)
   const int c0 = moving ? (rank == 0 ? 0 : 1) : C * rank / kNuRanks, c1 = moving ? 1 : C * (rank + 1) / kNuRanks;
   if (c0 < c1) fft::fill_twiddles(tw, M, 1.f, kNuClThreads, tid);
   after_previous();
+  next_may_start();
   float2 a0 = make_float2(0.f, 0.f), a1 = a0, a2 = a0, a3 = a0;
   int q = k0;
   for (; q + 3 * parts < Q; q += 4 * parts) {  // four loads in flight, four interleaved sums
@@ -1406,7 +1404,6 @@ constexpr int kAdjMargin = kNuW;  // the grid is stored with its wrap-around: en
 __global__ void __launch_bounds__(kAdjThreads) k_adj_grid(const float2* __restrict__ g, int V, int C, int Ns, int log_m,
                                                           float slope, const __grid_constant__ NufftCoef co,
                                                           float2* __restrict__ out) {
-  next_may_start();
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
   extern __shared__ float2 sa[];  // [N_s] this CTA's chirps summed, slots(M) grid, slots(M / 2) twiddles
@@ -1420,6 +1417,7 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_grid(const float2* __restri
     for (int i = threadIdx.x; i < fft::slots(M); i += kAdjThreads) s[i] = make_float2(0.f, 0.f);
   }
   after_previous();
+  next_may_start();
   for (int n = threadIdx.x; n < Ns; n += kAdjThreads) {
     float2 a = make_float2(0.f, 0.f);
 #pragma unroll 8

@@ -1002,8 +1002,8 @@ __global__ void __launch_bounds__(128) k_trace_warp(const float4* __restrict__ t
                                                     sbr_hit* __restrict__ hits, float4* __restrict__ hit_pos,
                                                     float* __restrict__ ray_w, int32_t* __restrict__ nvalid,
                                                     unsigned long long* __restrict__ counts) {
-  next_may_start();
   after_previous();
+  next_may_start();
   __shared__ int stacks[kGroupsPerCta][kGroupStack];
   const bool lead = (threadIdx.x & (kGroup - 1)) == 0;
   int* stack = stacks[threadIdx.x / kGroup];

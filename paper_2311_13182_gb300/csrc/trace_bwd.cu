@@ -303,8 +303,8 @@ __global__ void __launch_bounds__(128) k_trace_bwd(
 
 // gverts[i] += acc[i] 2^-E
 __global__ void k_fix_finish_add(FixScatter fs, int n, float* __restrict__ gverts) {
-  next_may_start();
   after_previous();
+  next_may_start();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   gverts[i] += fix_get(fs.acc[i], fix_exp(*fs.max_bits, fs.log2n));
